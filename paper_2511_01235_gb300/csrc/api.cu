@@ -156,6 +156,12 @@ T *dalloc_n(maxflow_ctx *c, int64_t count)
     return (T *)dalloc(c, sizeof(T) * (size_t)(count > 0 ? count : 1));
 }
 
+// Barrier and counter sets back to zero, after a launch that did not reach its end.
+cudaError_t clear_sync(MfCtrl *ctrl, cudaStream_t st)
+{
+    return cudaMemsetAsync(&ctrl->bar, 0, MF_CTRL_SYNC_BYTES, st);
+}
+
 int rc_cuda(cudaError_t e) { return e == cudaSuccess ? MAXFLOW_OK : MAXFLOW_ERR_CUDA; }
 
 #define MF_TRY(expr)                          \
@@ -356,9 +362,9 @@ void fill_stats(maxflow_ctx *c, const MfCtrl &h, float ms)
     maxflow_stats_t &s = c->st;
     s.iterations = h.iters;
     s.bfs_levels = h.bfs_levels;
-    s.pushes = h.pushes;
-    s.relabels = h.relabels;
-    s.steep_fixes = h.steep;
+    s.pushes = h.stat[ST_PUSHES];
+    s.relabels = h.stat[ST_RELABELS];
+    s.steep_fixes = h.stat[ST_STEEP];
     s.active_first = h.active_first;
     s.active_total = h.active_total;
     // algorithmic bytes of the paper's Bi-CSR (int32 per slot field, int64 excess), counted by the kernel:
@@ -372,11 +378,11 @@ void fill_stats(maxflow_ctx *c, const MfCtrl &h, float ms)
     //   apply: per applied update the record, the slot's cap, cf, pcap and its reverse's pcap
     //        (read-modify-write), rev and the dedup entry = 12 + 8 + 8 + 8 + 8 + 4 + 12 = 60 B;
     //        per slot read by the search or the source row 4 B; per clamp two c_f and two excess RMWs 48 B
-    s.bytes_bfs = 16 * h.slots_bfs + 12 * h.verts_bfs + 4 * h.hscan_bfs + 20 * h.lab_bfs;
-    s.bytes_discharge = 12 * h.slots_dis + 20 * h.cycles_dis + 48 * h.pushes;
-    s.bytes_fix = 12 * h.slots_fix + 20 * h.verts_fix + 48 * h.steep;
+    s.bytes_bfs = 16 * h.stat[ST_SLOTS_BFS] + 12 * h.stat[ST_VERTS_BFS] + 4 * h.stat[ST_HSCAN_BFS] + 20 * h.stat[ST_LAB_BFS];
+    s.bytes_discharge = 12 * h.stat[ST_SLOTS_DIS] + 20 * h.stat[ST_CYCLES_DIS] + 48 * h.stat[ST_PUSHES];
+    s.bytes_fix = 12 * h.stat[ST_SLOTS_FIX] + 20 * h.stat[ST_VERTS_FIX] + 48 * h.stat[ST_STEEP];
     s.bytes_worklist = c->opt.data_driven ? 0 : 16LL * c->n * (h.iters + 1);
-    s.bytes_apply = 60 * h.n_apply + 4 * h.slots_apply + 48 * h.clamps_apply;
+    s.bytes_apply = 60 * h.stat[ST_N_APPLY] + 4 * h.stat[ST_SLOTS_APPLY] + 48 * h.stat[ST_CLAMPS_APPLY];
     s.ms_last = ms;
     s.ms_bfs = h.ns_bfs * 1e-6;
     s.ms_discharge = h.ns_dis * 1e-6;
@@ -385,9 +391,9 @@ void fill_stats(maxflow_ctx *c, const MfCtrl &h, float ms)
     s.ms_apply = h.ns_apply * 1e-6;
     s.ms_kernel = (h.t_exit - h.t_entry) * 1e-6;
     s.ms_update = c->acc_ms;   // run_kernel has added this launch already
-    s.us_discharge_cta_rows = h.ns_dis_cta * 1e-3;
-    s.us_discharge_warp_rows = h.ns_dis_warp * 1e-3;
-    s.us_discharge_thread_rows = h.ns_dis_thread * 1e-3;
+    s.us_discharge_cta_rows = h.stat[ST_NS_CTA] * 1e-3;
+    s.us_discharge_warp_rows = h.stat[ST_NS_WARP] * 1e-3;
+    s.us_discharge_thread_rows = h.stat[ST_NS_THREAD] * 1e-3;
     s.discharge_rounds = h.rounds_total;
     s.barriers = h.barriers;
     s.kernel_cycles = c->kernel_cycles;
@@ -400,7 +406,7 @@ int run_kernel(maxflow_ctx *c, const MfParams &p, int *kerr, int *kstatus)
     MF_TRY(rc_cuda(cudaEventRecord(c->ev0, c->stream)));
     MF_TRY(counted(mf_launch(p, c->grid, (void *)c->stream), 1));
     MF_TRY(rc_cuda(cudaEventRecord(c->ev1, c->stream)));
-    MF_TRY(rc_cuda(cudaMemcpyAsync(c->hctrl, c->ctrl, sizeof(MfCtrl), cudaMemcpyDeviceToHost, c->stream)));
+    MF_TRY(rc_cuda(cudaMemcpyAsync(c->hctrl, c->ctrl, MF_CTRL_HOST_BYTES, cudaMemcpyDeviceToHost, c->stream)));
     MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, c->ev0, c->ev1);
@@ -410,7 +416,7 @@ int run_kernel(maxflow_ctx *c, const MfParams &p, int *kerr, int *kstatus)
     fill_stats(c, *c->hctrl, ms);
     if (*kerr != MF_E_NONE) {
         // a barrier may have been left half-way: reset it for the next launch
-        MF_TRY(rc_cuda(cudaMemsetAsync(c->ctrl, 0, 2 * sizeof(MfLine), c->stream)));
+        MF_TRY(rc_cuda(clear_sync(c->ctrl, c->stream)));
         MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
     }
     return MAXFLOW_OK;
@@ -1214,7 +1220,7 @@ int maxflow_solve_batched(maxflow_ctx *const *ctxs, int32_t count, const maxflow
     int abort_h = 0;
     MF_TRY(rc_cuda(cudaMemcpyAsync(&abort_h, abort_flag, sizeof(int), cudaMemcpyDeviceToHost, c0->stream)));
     for (int32_t i = 0; i < count; ++i)
-        MF_TRY(rc_cuda(cudaMemcpyAsync(ctxs[i]->hctrl, ctxs[i]->ctrl, sizeof(MfCtrl), cudaMemcpyDeviceToHost,
+        MF_TRY(rc_cuda(cudaMemcpyAsync(ctxs[i]->hctrl, ctxs[i]->ctrl, MF_CTRL_HOST_BYTES, cudaMemcpyDeviceToHost,
                                        c0->stream)));
     MF_TRY(rc_cuda(cudaStreamSynchronize(c0->stream)));
     float ms = 0.f;
@@ -1227,7 +1233,7 @@ int maxflow_solve_batched(maxflow_ctx *const *ctxs, int32_t count, const maxflow
         c->acc_ms = ms;
         fill_stats(c, *c->hctrl, ms);
         if (abort_h || kerr != MF_E_NONE) {
-            MF_TRY(rc_cuda(cudaMemsetAsync(c->ctrl, 0, 2 * sizeof(MfLine), c->stream)));
+            MF_TRY(rc_cuda(clear_sync(c->ctrl, c->stream)));
             MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
         }
         int rc;
@@ -1549,16 +1555,16 @@ int maxflow_update_pp(maxflow_ctx *c, const maxflow_batch *b, int32_t stop_after
     MF_TRY(rc_cuda(cudaEventRecord(c->ev1, c->stream)));
     int abort_h = 0;
     MF_TRY(rc_cuda(cudaMemcpyAsync(&abort_h, abort_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream)));
-    MF_TRY(rc_cuda(cudaMemcpyAsync(c->hctrl, c->ctrl, sizeof(MfCtrl), cudaMemcpyDeviceToHost, c->stream)));
-    MF_TRY(rc_cuda(cudaMemcpyAsync(c->pp.hctrl, c->pp.ctrl, sizeof(MfCtrl), cudaMemcpyDeviceToHost, c->stream)));
+    MF_TRY(rc_cuda(cudaMemcpyAsync(c->hctrl, c->ctrl, MF_CTRL_HOST_BYTES, cudaMemcpyDeviceToHost, c->stream)));
+    MF_TRY(rc_cuda(cudaMemcpyAsync(c->pp.hctrl, c->pp.ctrl, MF_CTRL_HOST_BYTES, cudaMemcpyDeviceToHost, c->stream)));
     MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
     float ms2 = 0.f;
     cudaEventElapsedTime(&ms2, c->ev0, c->ev1);
     ms += ms2;
     const int e0 = (int)c->hctrl->err.w[0], e1 = (int)c->pp.hctrl->err.w[0];
     if (abort_h || e0 != MF_E_NONE || e1 != MF_E_NONE) {
-        MF_TRY(rc_cuda(cudaMemsetAsync(c->ctrl, 0, 2 * sizeof(MfLine), c->stream)));
-        MF_TRY(rc_cuda(cudaMemsetAsync(c->pp.ctrl, 0, 2 * sizeof(MfLine), c->stream)));
+        MF_TRY(rc_cuda(clear_sync(c->ctrl, c->stream)));
+        MF_TRY(rc_cuda(clear_sync(c->pp.ctrl, c->stream)));
         MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
         c->st.ms_update = ms;
         if (abort_h) return MAXFLOW_ERR_INTERNAL;

@@ -13,6 +13,7 @@
 //              reads the reverse residual without a gather through rev.
 //   h[n]       heights (int32), e[n] excesses (int64)
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 #include <cuda_runtime.h>
 
@@ -69,79 +70,106 @@ struct alignas(128) MfLine {
     unsigned int w[32];
 };
 
-// Control block in device memory.  Fields that many CTAs update with atomics
-// sit on their own 128-byte lines.  Fields marked (hook) are written only by
-// the single thread that completes a grid barrier, while every other CTA
-// waits, and are read by all CTAs after it: every CTA sees the same value.
-// Hook-written values that the phases and the kernel's loop read.  They fill
-// one 128-byte line of their own; after every grid barrier one thread of each
-// CTA copies them into shared memory with 16-byte loads issued together, so a
-// phase pays one round trip to L2 for all of them instead of one per field.
-struct alignas(128) MfDesc {
+// Every word that many CTAs update with atomics during a phase sits on a line
+// of its own in a counter set.  Phase k (the stretch up to grid barrier k of a
+// launch) uses set k mod 3; behind the barrier every CTA reads the whole set
+// and works out by itself what comes next, so no CTA has to decide for the
+// others and publish the decision.  Set (k + 2) mod 3 was last read behind
+// barrier k - 1, before any CTA arrived at barrier k, so the first CTA can
+// clear it during phase k + 1, and nobody touches it before phase k + 2.
+enum MfLineId {
+    L_BFS = 0,            // regular frontier entries appended in this phase
+    L_HUB,                // frontier work items
+    L_LONG,               // long-row vertices (blong)
+    L_DEFER,              // bottom-up chunks deferred to the level's second pass
+    L_HEAD0,              // dynamic work heads
+    L_HEAD1,
+    L_HEAD2,
+    L_HEAD3,
+    L_WL,                 // [MF_NBIN] worklist entries per bin (built by the BFS)
+    L_AUX = L_WL + MF_NBIN,       // [MF_NBIN] next-round worklist entries per bin
+    L_FIX = L_AUX + MF_NBIN,      // [2] remove-invalid lists (warp / CTA)
+    L_ACT = L_FIX + 2,    // active vertices (only when the worklist is a pass of its own)
+    L_MISC,               // w[0] new pairs, w[1] a row without room, w[2] dedup entries, w[3] error (MF_E_*)
+    L_LAB,                // 64-bit: labelled vertices << 32 | their slots
+    L_TOTAL,              // 64-bit: used slots of the whole graph (summed by the BFS roots pass)
+    L_TIME,               // 64-bit: the first CTA's clock when it arrived at the barrier
+    MF_LINES
+};
+
+struct MfSet {
+    MfLine l[MF_LINES];
+};
+
+#define MF_MAX_CTAS 1024  // CTAs whose finish times and slots are traced (a grid is far smaller)
+
+// What the phases read, the same in every CTA (kept in shared memory).
+struct MfDesc {
     int status;
     int level;
-    int lvl_lo, lvl_hi;
-    int hub_lo, hub_hi;
+    int lvl_lo, lvl_hi;           // this level's regular frontier in border[]
+    int hub_lo, hub_hi;           // ... work items in bitem[]
+    int long_lo, long_hi;         // ... long-row vertices labelled by the last level (blong)
+    int app_bfs, app_hub, app_long;   // where this phase's entries of the three lists start
+    int wl_app[MF_NBIN];          // where this phase's worklist entries start
     int bfs_done;
-    int wl_sel;           // which worklist buffer the current round reads
+    int bu_mode;                  // the coming BFS level runs bottom-up
+    int bu_split;                 // the bottom-up level just scanned deferred long rows: their pass follows
+    int defer_n;                  // work items of that pass
+    int bfs_cta_mode;             // the coming top-down level is small: CTA 0 runs it (and the next small ones) alone
+    int expand;                   // the coming top-down level first splits long rows into work items
+    int need_total;               // the coming BFS roots pass sums the used slots (first BFS of a launch)
+    int wl_sel;                   // which worklist buffer the current round reads
     int wl_n[MF_NBIN];
-    int ins_n, touch_n;
-    int round;            // discharge round within the iteration
-    int dis_more;         // another discharge round follows
-    int fix_n[2];         // vertices for remove-invalid-edges (warp list, CTA list)
-    int qstamp, fstamp;   // dedupe stamps (never reset: they only grow across launches)
-    int bu_mode;          // the coming BFS level runs bottom-up
-    int bu_split;         // the bottom-up level just scanned deferred long rows: their pass follows
-    int bfs_cta_mode;     // the coming top-down level is small: CTA 0 runs it (and the next small ones) alone
-    int defer_n;          // work items of that pass
-    int need_total;       // the coming BFS initialisation sums the used slots (first BFS of a launch)
-    int pad0;
-    unsigned long long t_phase;   // when the last barrier's hook ran
-    int long_lo, long_hi;         // long-row vertices labelled by the last level (blong)
-    int expand;                   // the coming top-down level first splits them into work items
-    int pad1;
+    int ins_n, hused_n;           // batch: new pairs, dedup table entries
+    int round;                    // discharge round within the iteration
+    int dis_more;                 // another discharge round follows
+    int fix_n[2];                 // vertices for remove-invalid-edges (warp list, CTA list); grows over the rounds
+    int qstamp, fstamp;           // dedupe stamps (never reset: they only grow across launches)
 };
-static_assert(sizeof(MfDesc) == 128, "MfDesc is one 128-byte line, copied as 16-byte vectors");
+
+// The rest of what every CTA carries from barrier to barrier.  Decisions take
+// the first CTA's clock, read from the counter set, so all CTAs decide alike.
+struct MfState {
+    unsigned long long t_phase;   // this CTA's clock behind the last barrier (statistics only)
+    unsigned long long t_now;     // the first CTA's clock when it arrived at the last barrier
+    unsigned long long t_start, t_bfs0, t_dis0;   // t_now at the first barrier, at this iteration's BFS and discharge
+    unsigned long long ns_bfs, ns_dis, ns_fix, ns_wl, ns_apply;
+    long long vis_slots;          // slots of the vertices labelled so far in this BFS
+    long long lvl_slots, lvl_cnt; // slots and number of the vertices labelled by the level that is running
+    long long used_slots;         // used slots of the graph (0: not summed yet)
+    long long iters, bfs_levels, rounds_total, barriers, active_first, active_total;
+    int err;                      // MF_E_*
+    int trace_n;
+};
+
+// Work counters.  Each CTA keeps its own in shared memory and adds them to the
+// control block once, at the end of the launch.
+enum MfStat {
+    ST_PUSHES = 0, ST_RELABELS, ST_STEEP,
+    ST_SLOTS_BFS, ST_VERTS_BFS,
+    ST_HSCAN_BFS,         // heights read by the passes over all vertices of bottom-up levels
+    ST_LAB_BFS,           // vertices labelled by all BFS levels
+    ST_SLOTS_DIS, ST_CYCLES_DIS,
+    ST_SLOTS_FIX, ST_VERTS_FIX,
+    ST_N_APPLY,
+    ST_SLOTS_APPLY,       // slots read by the batch phases (slot search, source row)
+    ST_CLAMPS_APPLY,      // slots whose residual went negative and was sent back
+    ST_NS_CTA, ST_NS_WARP, ST_NS_THREAD,  // discharge time by row kind, summed over workers
+    MF_STATS
+};
 
 struct MfCtrl {
-    MfLine bar_count;     // w[0]: arrivals at the current barrier
-    MfLine bar_gen;       // w[0]: barrier generation
-    MfLine err;           // w[0]: sticky error (MF_E_*)
-    MfLine bfs_tail;      // w[0]: regular frontier append position
-    MfLine hub_tail;      // w[0]: frontier work-item append position
-    MfLine head0;         // w[0]: dynamic work head
-    MfLine head1;
-    MfLine head2;
-    MfLine head3;
-    // each counter that many warps bump at once on a line of its own: returning
-    // atomics on one line are served one after another
-    MfLine wl_tail[MF_NBIN + 1];   // [0..3]: worklist append positions per bin, [4]: active vertices
-    MfLine misc;          // w[0]: insert list tail, w[1]: touched tail, w[2]: overflow flag
-    MfLine aux_tail[MF_NBIN + 2];  // [0..3]: next-round worklist tails, [4]/[5]: remove-invalid lists (warp / CTA)
-    MfLine defer_tail;    // w[0]: bottom-up work items of long rows deferred to the level's second pass
-    MfLine long_tail;     // w[0]: append position of the long-row vertex list (blong)
-    MfLine bfs_acc;       // 64-bit words: [0] slots of the vertices labelled in this level, [1] their number,
-                          // [2] used slots of the whole graph (summed by the BFS initialisation)
-    // ---- (hook) snapshots: what the phases read, copied to shared memory once per barrier ----
-    MfDesc d;
-    unsigned long long t_bfs0, t_dis0;   // this iteration: BFS start, discharge start (adaptive rounds)
-    long long vis_slots;  // slots of the vertices labelled so far in this BFS
-    long long iters;
-    unsigned long long t_start;
-    // ---- results and statistics (atomics, flushed once per CTA per phase) ----
-    long long value;
-    long long pushes, relabels, steep, bfs_levels, active_total, active_first;
-    long long slots_bfs, verts_bfs, slots_dis, cycles_dis, slots_fix, verts_fix, verts_wl, n_apply;
-    long long lab_bfs;        // vertices labelled by all BFS levels
-    long long hscan_bfs;      // heights read by the passes over all vertices of bottom-up levels
-    long long slots_apply;    // slots read by the batch phases (slot search, source row)
-    long long clamps_apply;   // slots whose residual went negative and was sent back
+    // ---- read by the host after every launch ----
+    MfLine err;           // w[0]: error of the launch (MF_E_*)
+    MfDesc d;             // final; the stamps carry over to the next launch
+    long long iters, value;
+    long long bfs_levels, active_total, active_first;
+    long long stat[MF_STATS];     // MfStat, summed over the CTAs at the end of a launch
     unsigned long long ns_bfs, ns_dis, ns_fix, ns_wl, ns_apply;
-    unsigned long long ns_dis_cta, ns_dis_warp, ns_dis_thread;   // discharge time by row kind, summed over workers
     int active_hist[MF_ACTIVE_HIST];
     long long rounds_total;
-    // ---- tracing: kernel entry (block 0, before the first barrier), last hook, hook timeline ----
-    unsigned long long t_entry, t_exit;
+    unsigned long long t_entry, t_exit;   // kernel entry (first CTA), last barrier
     long long barriers;
     int trace_n;
     int trace_hook[MF_TRACE];
@@ -151,11 +179,21 @@ struct MfCtrl {
     // discharge round: bits 20..29 = CTA-bin (hub) vertices, bits 0..19 = vertices in the round's lists
     long long trace_slots[MF_TRACE];
     int trace_info[MF_TRACE];
-    // when the CTAs finished the phase that a barrier closes (ns after the previous barrier's release):
+    // when the CTAs finished the phase that a barrier closes (ns after the previous barrier):
     // the last one and the mean, per traced barrier
-    unsigned long long fin_max, fin_sum;
     unsigned trace_fin_max[MF_TRACE], trace_fin_mean[MF_TRACE];
+    // ---- device only ----
+    MfLine bar;           // w[0]: arrivals in this launch (the first CTA leaves it at zero)
+    MfSet set[3];
+    // the first CTA's state for the others, after it ran phases alone
+    MfDesc jd;
+    MfState js;
+    // per phase (mod 3) and CTA: finish time, slots scanned
+    unsigned fin[3][MF_MAX_CTAS], scanned[3][MF_MAX_CTAS];
 };
+// What the host copies back, and the part it clears after a launch that ended in a barrier that gave up.
+#define MF_CTRL_HOST_BYTES offsetof(MfCtrl, bar)
+#define MF_CTRL_SYNC_BYTES (sizeof(MfLine) + sizeof(MfSet) * 3)
 
 struct MfGraph {
     int32_t n;

@@ -13,7 +13,7 @@
 // MAXFLOW_NOALLOC_MAX_SLOTS slots), so every GPU that loads this library holds
 // about 14 MB for it until the process exits.
 // Every call uses the same array and it keeps the contents of the last call:
-// the barrier words of the control block are cleared before each launch, and
+// the barrier and counter sets of the control block are cleared before each launch, and
 // the kernel resets the rest itself.  Two calls whose work overlaps on the GPU
 // (different streams, or different host threads) race on the array.
 #include <cuda_runtime.h>
@@ -143,8 +143,8 @@ extern "C" int maxflow_global_relabel_noalloc(int32_t n, int32_t s, int32_t t, c
     if (cudaStreamSynchronize(st) != cudaSuccess) return MAXFLOW_ERR_CUDA;
     if (nslots < 0) return MAXFLOW_ERR_INVALID;
     if (nslots > MAXFLOW_NOALLOC_MAX_SLOTS) return MAXFLOW_ERR_TOO_LARGE;
-    // barrier words must start at zero (a previous call may have ended early)
-    if (cudaMemsetAsync(ctrl, 0, 2 * sizeof(MfLine), st) != cudaSuccess) return MAXFLOW_ERR_CUDA;
+    // barrier and counter sets must start at zero (a previous call may have ended early)
+    if (cudaMemsetAsync(&ctrl->bar, 0, MF_CTRL_SYNC_BYTES, st) != cudaSuccess) return MAXFLOW_ERR_CUDA;
     int maxg = ds->per_sm * ds->sms;
     int grid = (int)((n + 2047) / 2048);
     if (grid < 2) grid = 2;

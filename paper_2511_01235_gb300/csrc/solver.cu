@@ -161,30 +161,30 @@ __device__ __forceinline__ int warp_rank(int nctas, int skip)
     return r >= s ? r - s : r - s + nw;
 }
 
-// Per-CTA accumulators, flushed to global memory once per phase.
+// What a CTA keeps in shared memory: its accumulators, its copy of the launch's
+// state (the same in every CTA between two barriers), and work space of phases.
 struct Sh {
-    long long sink_e, src_e;
-    long long pushes, relabels, steep, slots, verts, cycles;
-    long long lab_slots, lab_cnt;     // BFS: slots and number of the vertices labelled this level
-    unsigned long long dis_cta_ns, dis_warp_ns, dis_thread_ns;   // discharge: time of this CTA's warps by row kind
+    long long sink_e, src_e;          // excess of the sink and the source, added to memory before every barrier
+    long long stat[MF_STATS];         // work counters, added to memory at the end of the launch
+    unsigned long long lab;           // BFS: vertices labelled this phase << 32 | their slots
     unsigned long long red[MF_WARPS];
     long long wsum[MF_WARPS];
     int wcnt[MF_WARPS];
-    long long bcast_rem;
-    int bcast_k;
     int bcast_i;
     long long tb_e[MF_BLOCK / (32 * MF_GROUP_WARPS)];   // per team (CTA: [0]; 4-warp groups: [g]) broadcasts
     int tb_h[MF_BLOCK / (32 * MF_GROUP_WARPS)];
     int tb_i[MF_BLOCK / (32 * MF_GROUP_WARPS)];
-    int bcast_h;
-    long long bcast_e;
     int ok;
-    unsigned gen;
-    MfDesc d;         // the hook's snapshot, copied after every barrier
+    unsigned phase;                   // barriers passed in this launch
+    MfSet *cs;                        // the counter set of the running phase
+    int tr_hook, tr_info;             // of the last barrier, for the trace
+    int4 cnt[MF_LINES];               // the counters of the phase that just ended
+    MfDesc d;
+    MfState hs;
 };
 
 enum Hook {
-    H_START = 0,
+    H_START = 0,          // unused (a launch starts without a barrier); keeps the trace ids
     H_NONE,
     H_APPLY_VALID,
     H_APPLY_LOCATED,
@@ -201,392 +201,435 @@ enum Hook {
     H_EXPANDED,
 };
 
-__device__ __forceinline__ int rd(const int &x) { return __ldcg(&x); }
-__device__ __forceinline__ unsigned rd(const unsigned &x) { return __ldcg(&x); }
-__device__ __forceinline__ long long rd(const long long &x) { return __ldcg(&x); }
-__device__ __forceinline__ unsigned long long rd(const unsigned long long &x) { return __ldcg(&x); }
+__device__ __forceinline__ void add_stat(Sh &sh, MfStat i, long long v)
+{
+    if (v) atomicAdd((unsigned long long *)&sh.stat[i], (unsigned long long)v);
+}
+
+__device__ __forceinline__ int cnt32(const Sh &sh, int line) { return sh.cnt[line].x; }
+__device__ __forceinline__ unsigned long long cnt64(const Sh &sh, int line)
+{
+    return (unsigned long long)(unsigned)sh.cnt[line].x | ((unsigned long long)(unsigned)sh.cnt[line].y << 32);
+}
 
 // The termination test of the loop (Alg. 1 / Alg. 5: stop when no active
 // vertex remains), taken right after a complete backward BFS.
-__device__ __forceinline__ void decide_iteration(const MfParams &P, MfCtrl *c, unsigned long long now,
-                                                 const unsigned (&wl)[MF_NBIN + 1], long long iters,
-                                                 unsigned long long t_start, int qstamp, int fstamp)
+__device__ __forceinline__ void decide_iteration(const MfParams &P, Sh &sh, int active)
 {
-    c->d.round = 0;
-    for (int i = 0; i < MF_NBIN + 2; ++i) c->aux_tail[i].w[0] = 0;
-    c->d.qstamp = qstamp + 1;
-    c->d.fstamp = fstamp + 1;
-    const int active = (int)wl[MF_NBIN];
-    c->t_dis0 = now;
-    for (int b = 0; b < MF_NBIN; ++b) c->d.wl_n[b] = (int)wl[b];
-    c->head0.w[0] = c->head1.w[0] = c->head2.w[0] = c->head3.w[0] = 0;
-    if (iters < MF_ACTIVE_HIST) c->active_hist[iters] = active;
-    if (iters == 0) c->active_first = active;
-    c->active_total = rd(c->active_total) + active;
+    MfDesc &d = sh.d;
+    MfState &st = sh.hs;
+    d.round = 0;
+    d.fix_n[0] = d.fix_n[1] = 0;
+    ++d.qstamp;
+    ++d.fstamp;
+    st.t_dis0 = st.t_now;
+    for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = d.wl_app[b];
+    if (vb() == 0 && st.iters < MF_ACTIVE_HIST) P.ctrl->active_hist[st.iters] = active;
+    if (st.iters == 0) st.active_first = active;
+    st.active_total += active;
     if (active == 0) {
-        c->d.status = MF_ST_CONVERGED;
-    } else if (iters >= P.max_iters || now - t_start > P.time_limit_ns) {
-        c->d.status = MF_ST_CAP;
+        d.status = MF_ST_CONVERGED;
+    } else if (st.iters >= P.max_iters || st.t_now - st.t_start > P.time_limit_ns) {
+        d.status = MF_ST_CAP;
     } else {
-        c->iters = iters + 1;
+        ++st.iters;
     }
 }
 
-// Hook work that opens an iteration of the loop (its BFS comes next).
-__device__ __forceinline__ void begin_iteration(MfCtrl *c, unsigned long long now)
+// Opens an iteration of the loop (its BFS comes next).
+__device__ __forceinline__ void begin_iteration(Sh &sh)
 {
-    c->t_bfs0 = now;
-    c->bfs_tail.w[0] = 0;
-    c->hub_tail.w[0] = 0;
-    c->long_tail.w[0] = 0;
-    // the used-slot total (acc word 2) only changes with insertions, which
-    // come before the first BFS: later iterations keep it
-    for (int i = 0; i < 4; ++i) c->bfs_acc.w[i] = 0;
-    c->d.need_total = rd(c->bfs_acc.w[4]) == 0 && rd(c->bfs_acc.w[5]) == 0;
-    c->d.bu_mode = 0;
-    for (int i = 0; i <= MF_NBIN; ++i) c->wl_tail[i].w[0] = 0;
-    c->head0.w[0] = c->head1.w[0] = c->head2.w[0] = c->head3.w[0] = 0;
+    MfDesc &d = sh.d;
+    sh.hs.t_bfs0 = sh.hs.t_now;
+    sh.hs.vis_slots = sh.hs.lvl_slots = sh.hs.lvl_cnt = 0;
+    d.lvl_lo = d.lvl_hi = d.hub_lo = d.hub_hi = d.long_lo = d.long_hi = 0;
+    d.app_bfs = d.app_hub = d.app_long = 0;
+    for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] = 0;
+    // the used-slot total only changes with insertions, which come before the
+    // first BFS: later iterations keep it
+    d.need_total = sh.hs.used_slots == 0;
+    d.bu_mode = 0;
 }
 
-// Executed by the one thread that completes a grid barrier, while every
-// other CTA waits for it.  All fields it needs are loaded first (through L2)
-// so the barrier's critical path holds one memory round trip.
-__device__ __noinline__ void run_hook(const MfParams &P, int hook)
+// What comes after a grid barrier: thread 0 of every CTA works it out from the
+// counters of the phase that ended (sh.cnt) and the state all CTAs share, in
+// shared memory only, so all of them arrive at the same answer.  t: the first
+// CTA's clock.
+__device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsigned long long t)
 {
-    MfCtrl *c = P.ctrl;
-    const unsigned long long now = gtimer();
-    if (hook == H_BU_SPLIT) {
-        // after the first pass of a bottom-up level: a second pass over the
-        // deferred long rows, or (none deferred) the level is complete
-        const unsigned dn = rd(c->defer_tail.w[0]);
-        if (dn == 0) {
-            c->d.bu_split = 0;
-            hook = H_BFS_NEXT;
-        } else {
-            c->d.bu_split = 1;
-            c->d.defer_n = (int)dn;
-            c->defer_tail.w[0] = 0;
-            c->head1.w[0] = 0;
+    MfDesc &d = sh.d;
+    MfState &st = sh.hs;
+    const unsigned long long now = gtimer(), dt = now - st.t_phase;
+    st.t_phase = now;
+    st.t_now = t;
+    if (st.barriers == 0) st.t_start = t;
+    ++st.barriers;
+    if (st.err == 0) st.err = sh.cnt[L_MISC].w;
+    int tinfo = 0;
+    const bool want_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
+    if (hook == H_BU_SPLIT || hook == H_BFS_START || hook == H_BFS_NEXT || hook == H_EXPANDED) {
+        // the lists grew by what the phase appended
+        st.ns_bfs += dt;
+        d.app_bfs += cnt32(sh, L_BFS);
+        d.app_hub += cnt32(sh, L_HUB);
+        d.app_long += cnt32(sh, L_LONG);
+        for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] += cnt32(sh, L_WL + b);
+        const unsigned long long lab = cnt64(sh, L_LAB);
+        st.lvl_slots += (long long)(lab & 0xffffffffull);
+        st.lvl_cnt += (long long)(lab >> 32);
+        if (hook == H_BU_SPLIT) {
+            // after the first pass of a bottom-up level: a second pass over the
+            // deferred long rows, or (none deferred) the level is complete
+            d.defer_n = cnt32(sh, L_DEFER);
+            d.bu_split = d.defer_n > 0 ? 1 : 0;
+            tinfo = (1 << 30) | min(d.defer_n, (1 << 20) - 1);
+            if (!d.bu_split) hook = H_BFS_NEXT;
         }
     }
-    const unsigned long long t_phase = rd(c->d.t_phase);
-    const int trace_n = hook == H_START ? 0 : rd(c->trace_n);
-    const long long barriers = hook == H_START ? 0 : rd(c->barriers);
-    const unsigned bfs_tail = rd(c->bfs_tail.w[0]), item_tail = rd(c->hub_tail.w[0]);
-    const int lvl_hi = rd(c->d.lvl_hi), hub_hi = rd(c->d.hub_hi), level = rd(c->d.level), hub_lo_old = rd(c->d.hub_lo);
-    const long long iters = rd(c->iters), bfs_levels = rd(c->bfs_levels);
-    const unsigned long long t_start = rd(c->t_start);
-    unsigned wl[MF_NBIN + 1], misc[4];
-    for (int i = 0; i <= MF_NBIN; ++i) wl[i] = rd(c->wl_tail[i].w[0]);
-    for (int i = 0; i < 4; ++i) misc[i] = rd(c->misc.w[i]);
-    unsigned aux[MF_NBIN + 2];
-    for (int i = 0; i < MF_NBIN + 2; ++i) aux[i] = rd(c->aux_tail[i].w[0]);
-    const int sel = rd(c->d.wl_sel), round = rd(c->d.round), qstamp = rd(c->d.qstamp), fstamp = rd(c->d.fstamp);
-    const long long rounds_total = rd(c->rounds_total);
-    const long long slots_all = rd(c->slots_bfs) + rd(c->slots_dis) + rd(c->slots_fix);
-    const unsigned long long fin_max = rd(c->fin_max), fin_sum = rd(c->fin_sum);
-    const int bu_prev = rd(c->d.bu_mode);
-    int wl_prev[MF_NBIN];
-    for (int b = 0; b < MF_NBIN; ++b) wl_prev[b] = rd(c->d.wl_n[b]);
-    int tinfo = 0;
-    unsigned err = rd(c->err.w[0]);
-    const unsigned long long dt = now - t_phase;
-    const bool want_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
-
-    c->d.t_phase = now;
-    c->barriers = barriers + 1;
-    c->t_exit = now;
-    c->trace_n = trace_n + 1;
     switch (hook) {
-    case H_START:
-        err = 0;
-        c->err.w[0] = 0;
-        c->d.status = MF_ST_RUNNING;
-        c->iters = 0;
-        c->value = 0;
-        c->pushes = c->relabels = c->steep = c->bfs_levels = c->active_total = c->active_first = 0;
-        c->slots_bfs = c->verts_bfs = c->slots_dis = c->cycles_dis = c->slots_fix = c->verts_fix = 0;
-        c->verts_wl = c->n_apply = 0;
-        c->lab_bfs = c->slots_apply = c->clamps_apply = c->hscan_bfs = 0;
-        c->fin_max = c->fin_sum = 0;
-        c->ns_bfs = c->ns_dis = c->ns_fix = c->ns_wl = c->ns_apply = 0;
-        c->ns_dis_cta = c->ns_dis_warp = c->ns_dis_thread = 0;
-        c->bfs_tail.w[0] = 0;
-        c->hub_tail.w[0] = 0;
-        c->long_tail.w[0] = 0;
-        c->defer_tail.w[0] = 0;
-        c->d.bu_split = 0;
-        c->head0.w[0] = c->head1.w[0] = c->head2.w[0] = c->head3.w[0] = 0;
-        for (int i = 0; i <= MF_NBIN; ++i) c->wl_tail[i].w[0] = 0;
-        for (int i = 0; i < 8; ++i) c->misc.w[i] = 0;
-        for (int i = 0; i < MF_ACTIVE_HIST; ++i) c->active_hist[i] = 0;
-        for (int i = 0; i < MF_NBIN + 2; ++i) c->aux_tail[i].w[0] = 0;
-        for (int i = 0; i < 8; ++i) c->bfs_acc.w[i] = 0;
-        c->d.bu_mode = 0;
-        c->d.bfs_cta_mode = 0;
-        c->d.need_total = 1;
-        c->d.round = 0;
-        c->d.dis_more = 0;
-        c->rounds_total = 0;
-        c->t_start = now;
-        break;
     case H_APPLY_VALID:
-        c->ns_apply = rd(c->ns_apply) + dt;
+        st.ns_apply += dt;
+        d.hused_n = sh.cnt[L_MISC].z;
         break;
     case H_APPLY_LOCATED:
-        c->ns_apply = rd(c->ns_apply) + dt;
-        c->d.ins_n = (int)misc[0];
-        if (misc[2] != 0 && err == 0) {      // a row has no room for its new pairs
-            err = MF_E_OVERFLOW;
-            c->err.w[0] = err;
-        }
+        st.ns_apply += dt;
+        d.ins_n = sh.cnt[L_MISC].x;
+        if (sh.cnt[L_MISC].y != 0 && st.err == 0) st.err = MF_E_OVERFLOW;   // a row has no room for its new pairs
         break;
     case H_APPLY_DELTA:
-        c->ns_apply = rd(c->ns_apply) + dt;
-        c->d.touch_n = (int)misc[1];
-        break;
     case H_NONE:
-        c->ns_apply = rd(c->ns_apply) + dt;
+        st.ns_apply += dt;
         break;
     case H_ITER:
-        c->ns_fix = rd(c->ns_fix) + dt;
-        begin_iteration(c, now);
+        if (P.mode & (MF_M_STATIC_INIT | MF_M_APPLY) && st.iters == 0) st.ns_apply += dt;
+        else st.ns_fix += dt;
+        begin_iteration(sh);
         break;
     case H_BFS_START:
     case H_BFS_NEXT: {
-        c->ns_bfs = rd(c->ns_bfs) + dt;
         const bool first = hook == H_BFS_START;
-        const int lo = first ? 0 : lvl_hi, hlo = first ? 0 : hub_hi, llo = first ? 0 : rd(c->d.long_hi);
-        const unsigned long_tail = rd(c->long_tail.w[0]);
-        const bool done = lo == (int)bfs_tail && hlo == (int)item_tail && llo == (int)long_tail;
-        if (!first && !done) c->bfs_levels = bfs_levels + 1;
-        c->d.level = first ? 0 : level + 1;
-        c->d.lvl_lo = lo;
-        c->d.lvl_hi = (int)bfs_tail;
-        c->d.hub_lo = hlo;
-        c->d.hub_hi = (int)item_tail;
-        c->d.long_lo = llo;
-        c->d.long_hi = (int)long_tail;
-        c->head0.w[0] = c->head1.w[0] = 0;
-        c->d.bfs_done = done;
-        {
-            // direction of the coming level (Beamer's test): bottom-up once the
-            // frontier's slots exceed 1/alpha of the unexplored slots, back to
-            // top-down once it holds fewer than n/beta vertices
-            const unsigned long long *acc = (const unsigned long long *)c->bfs_acc.w;
-            const long long fr = (long long)__ldcg(acc + 0), cnt = (long long)__ldcg(acc + 1);
-            const long long tot = (long long)__ldcg(acc + 2);
-            const long long vis = (first ? 0 : rd(c->vis_slots)) + fr;
-            tinfo = ((first ? 0 : bu_prev) << 30) | ((first ? 0 : min(hub_hi - hub_lo_old, 1023)) << 20) |
-                    (int)min(cnt, (long long)((1 << 20) - 1));
-            int bu = first ? 0 : rd(c->d.bu_mode);
-            if (P.bu_alpha <= 0) bu = 0;
-            else if (!bu && fr * P.bu_alpha > tot - vis) bu = 1;
-            else if (bu && cnt * P.bu_beta < (long long)P.g.n) bu = 0;
-            c->d.bu_mode = bu;
-            c->vis_slots = vis;
-            // a top-down level after one that labelled long rows first splits them
-            // into work items (a bottom-up level never reads them)
-            const int expand = (!done && !bu && (int)long_tail > llo) ? 1 : 0;
-            c->d.expand = expand;
-            // a small top-down frontier is expanded by CTA 0 alone: a level of a
-            // few hundred slots costs a grid barrier otherwise
-            c->d.bfs_cta_mode =
-                (!done && !bu && !expand && P.tail_slots > 0 && fr <= P.tail_slots && cnt <= P.tail_slots) ? 1 : 0;
-            c->bfs_acc.w[0] = c->bfs_acc.w[1] = c->bfs_acc.w[2] = c->bfs_acc.w[3] = 0;   // per level; [2] stays
+        if (first && d.need_total) st.used_slots = (long long)cnt64(sh, L_TOTAL);
+        const int items = d.hub_hi - d.hub_lo;
+        d.lvl_lo = d.lvl_hi;
+        d.hub_lo = d.hub_hi;
+        d.long_lo = d.long_hi;
+        d.lvl_hi = d.app_bfs;
+        d.hub_hi = d.app_hub;
+        d.long_hi = d.app_long;
+        const bool done = d.lvl_lo == d.lvl_hi && d.hub_lo == d.hub_hi && d.long_lo == d.long_hi;
+        if (!first && !done) ++st.bfs_levels;
+        d.level = first ? 0 : d.level + 1;
+        d.bfs_done = done;
+        // direction of the coming level (Beamer's test): bottom-up once the
+        // frontier's slots exceed 1/alpha of the unexplored slots, back to
+        // top-down once it holds fewer than n/beta vertices
+        const long long fr = st.lvl_slots, cnt = st.lvl_cnt;
+        st.vis_slots += fr;
+        st.lvl_slots = st.lvl_cnt = 0;
+        tinfo = ((first ? 0 : d.bu_mode) << 30) | ((first ? 0 : min(items, 1023)) << 20) |
+                (int)min(cnt, (long long)((1 << 20) - 1));
+        int bu = d.bu_mode;
+        if (P.bu_alpha <= 0) bu = 0;
+        else if (!bu && fr * P.bu_alpha > st.used_slots - st.vis_slots) bu = 1;
+        else if (bu && cnt * P.bu_beta < (long long)P.g.n) bu = 0;
+        d.bu_mode = bu;
+        d.bu_split = 0;
+        // a top-down level after one that labelled long rows first splits them
+        // into work items (a bottom-up level never reads them)
+        d.expand = (!done && !bu && d.long_hi > d.long_lo) ? 1 : 0;
+        // a small top-down frontier is expanded by CTA 0 alone: a level of a
+        // few hundred slots costs a grid barrier otherwise
+        d.bfs_cta_mode =
+            (!done && !bu && !d.expand && P.tail_slots > 0 && fr <= P.tail_slots && cnt <= P.tail_slots) ? 1 : 0;
+        if (done && want_wl) {
+            int active = 0;
+            for (int b = 0; b < MF_NBIN; ++b) active += d.wl_app[b];
+            decide_iteration(P, sh, active);
         }
-        if (done && want_wl) decide_iteration(P, c, now, wl, iters, t_start, qstamp, fstamp);
         break;
     }
     case H_WL:
-        c->ns_wl = rd(c->ns_wl) + dt;
-        decide_iteration(P, c, now, wl, iters, t_start, qstamp, fstamp);
+        st.ns_wl += dt;
+        for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] = cnt32(sh, L_WL + b);
+        decide_iteration(P, sh, cnt32(sh, L_ACT));
         break;
     case H_DIS: {
         // after a discharge round: run another one over the vertices that
         // became active during it, or end the discharge of this iteration
-        c->ns_dis = rd(c->ns_dis) + dt;
-        tinfo = (min(wl_prev[2] + wl_prev[3], 1023) << 20) |
-                min(wl_prev[0] + wl_prev[1] + wl_prev[2] + wl_prev[3], (1 << 20) - 1);
-        c->head0.w[0] = c->head1.w[0] = c->head2.w[0] = c->head3.w[0] = 0;
-        c->rounds_total = rounds_total + 1;
-        const unsigned nxt = aux[0] + aux[1] + aux[2] + aux[3];
+        st.ns_dis += dt;
+        tinfo = (min(d.wl_n[2] + d.wl_n[3], 1023) << 20) |
+                min(d.wl_n[0] + d.wl_n[1] + d.wl_n[2] + d.wl_n[3], (1 << 20) - 1);
+        ++st.rounds_total;
+        d.fix_n[0] += cnt32(sh, L_FIX);
+        d.fix_n[1] += cnt32(sh, L_FIX + 1);
+        int nxt = 0;
+        for (int b = 0; b < MF_NBIN; ++b) nxt += cnt32(sh, L_AUX + b);
         // fixed: P.rounds rounds; adaptive (P.rounds == 0): at least
         // MF_DEFAULT_ROUNDS, then more while this iteration's discharge has
         // taken less than half of its BFS -- a global relabel that costs much
         // (deep BFS, e.g. grids) is amortised over more rounds
-        bool more = nxt > 0 && err == 0 && round + 1 < MF_MAX_ROUNDS;
-        if (more && round + 1 >= (P.rounds > 0 ? P.rounds : MF_DEFAULT_ROUNDS)) {
-            if (P.rounds > 0) {
-                more = false;
-            } else {
-                const unsigned long long t_bfs0 = rd(c->t_bfs0), t_dis0 = rd(c->t_dis0);
-                more = 2 * (now - t_dis0) < t_dis0 - t_bfs0;
-            }
-        }
+        bool more = nxt > 0 && st.err == 0 && d.round + 1 < MF_MAX_ROUNDS;
+        if (more && d.round + 1 >= (P.rounds > 0 ? P.rounds : MF_DEFAULT_ROUNDS))
+            more = P.rounds > 0 ? false : 2 * (t - st.t_dis0) < st.t_dis0 - st.t_bfs0;
+        d.dis_more = more ? 1 : 0;
         if (more) {
-            c->d.wl_sel = sel ^ 1;
-            for (int b = 0; b < MF_NBIN; ++b) {
-                c->d.wl_n[b] = (int)aux[b];
-                c->aux_tail[b].w[0] = 0;
-            }
-            c->d.round = round + 1;
-            c->d.qstamp = qstamp + 1;
-            c->d.dis_more = 1;
-        } else {
-            c->d.dis_more = 0;
-            c->d.fix_n[0] = (int)aux[MF_NBIN];
-            c->d.fix_n[1] = (int)aux[MF_NBIN + 1];
+            d.wl_sel ^= 1;
+            for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = cnt32(sh, L_AUX + b);
+            ++d.round;
+            ++d.qstamp;
+        } else if (!P.fix_steep) {
             // without Alg. 3 the next iteration's BFS follows at once: this
             // barrier opens it
-            if (!P.fix_steep) begin_iteration(c, now);
+            begin_iteration(sh);
         }
         break;
     }
-    case H_FINAL:
-        break;
     case H_BFS_JOIN:
-        c->ns_bfs = rd(c->ns_bfs) + dt;
+        st.ns_bfs += dt;
         break;
     case H_EXPANDED:
         // the long rows' work items are written: the level takes them with the rest
-        c->ns_bfs = rd(c->ns_bfs) + dt;
-        c->d.hub_hi = (int)item_tail;
-        c->d.expand = 0;
-        c->head0.w[0] = c->head1.w[0] = 0;
+        d.hub_hi = d.app_hub;
+        d.expand = 0;
         break;
-    case H_BU_SPLIT:
-        c->ns_bfs = rd(c->ns_bfs) + dt;
-        tinfo = (1 << 30) | (int)min((long long)rd(c->d.defer_n), (long long)((1 << 20) - 1));
+    default:
         break;
     }
-    if (trace_n < MF_TRACE) {
-        c->trace_hook[trace_n] = hook;
-        c->trace_t[trace_n] = now;
-        c->trace_slots[trace_n] = slots_all;
-        c->trace_info[trace_n] = tinfo;
-        c->trace_fin_max[trace_n] = (unsigned)min(fin_max, 0xffffffffull);
-        c->trace_fin_mean[trace_n] = (unsigned)min(fin_sum / (unsigned long long)vn(), 0xffffffffull);
-    }
-    c->fin_max = 0;
-    c->fin_sum = 0;
-    if (err != 0) c->d.status = MF_ST_ERROR;
+    sh.tr_hook = hook;
+    sh.tr_info = tinfo;
+    ++st.trace_n;
+    if (st.err != 0) d.status = MF_ST_ERROR;
 }
 
-// The hook's snapshot into shared memory: eight 16-byte loads through L2,
-// issued together (one round trip).  Called by one thread, after the barrier's
-// acquire (or by the thread that ran the hook itself).
-__device__ __forceinline__ void load_desc(const MfCtrl *c, Sh &sh)
+// One entry of the hook timeline, written by the last warp of the first CTA
+// beside the phase that follows: the barrier, when it was reached, and from
+// what every CTA left before arriving when they finished and the slots scanned.
+__device__ __noinline__ void write_trace(const MfParams &P, Sh &sh, unsigned phase)
 {
-    constexpr int kN = (int)(sizeof(MfDesc) / sizeof(int4));
-    const int4 *src = reinterpret_cast<const int4 *>(&c->d);
-    int4 v[kN];
-#pragma unroll
-    for (int i = 0; i < kN; ++i) v[i] = __ldcg(src + i);
-    int4 *dst = reinterpret_cast<int4 *>(&sh.d);
-#pragma unroll
-    for (int i = 0; i < kN; ++i) dst[i] = v[i];
+    MfCtrl *c = P.ctrl;
+    const int lane = threadIdx.x & 31;
+    const int i = sh.hs.trace_n - 1;
+    if (i >= MF_TRACE) return;
+    const unsigned *fin = c->fin[phase % 3], *scn = c->scanned[phase % 3];
+    unsigned fmax = 0;
+    unsigned long long fsum = 0, slots = 0;
+    const int n = min(vn(), MF_MAX_CTAS);
+    for (int q = lane; q < n; q += 32) {
+        const unsigned f = __ldcg(fin + q);
+        fmax = max(fmax, f);
+        fsum += f;
+        slots += __ldcg(scn + q);
+    }
+    fmax = __reduce_max_sync(0xffffffffu, fmax);
+    fsum = (unsigned long long)warp_sum_ll((long long)fsum);
+    slots = (unsigned long long)warp_sum_ll((long long)slots);
+    if (lane == 0) {
+        c->trace_hook[i] = sh.tr_hook;
+        c->trace_t[i] = sh.hs.t_phase;
+        c->trace_slots[i] = (long long)slots;
+        c->trace_info[i] = sh.tr_info;
+        c->trace_fin_max[i] = fmax;
+        c->trace_fin_mean[i] = (unsigned)min(fsum / (unsigned long long)n, 0xffffffffull);
+    }
+}
+
+// A warp copies a structure between shared memory and device memory.
+__device__ __forceinline__ void words_out(int *dst, const int *sh_src, int words)
+{
+    for (int i = threadIdx.x & 31; i < words; i += 32) __stcg(dst + i, sh_src[i]);
+}
+__device__ __forceinline__ void words_in(int *sh_dst, const int *src, int words)
+{
+    for (int i = threadIdx.x & 31; i < words; i += 32) sh_dst[i] = __ldcg(src + i);
+}
+
+// Excess of sink and source and the BFS label counters go to memory, the
+// finish time and the slots scanned into this CTA's place; then the arrival.
+// Called by warp 0 after a __syncthreads.
+__device__ __forceinline__ void arrive(const MfParams &P, Sh &sh)
+{
+    MfCtrl *c = P.ctrl;
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) {
+        const unsigned long long now = gtimer();
+        const int s3 = (int)(sh.phase % 3u);
+        if (vb() < MF_MAX_CTAS) {
+            c->fin[s3][vb()] = (unsigned)(now > sh.hs.t_phase ? now - sh.hs.t_phase : 0);
+            c->scanned[s3][vb()] = (unsigned)(sh.stat[ST_SLOTS_BFS] + sh.stat[ST_SLOTS_DIS] + sh.stat[ST_SLOTS_FIX]);
+        }
+        if (vb() == 0) *(unsigned long long *)sh.cs->l[L_TIME].w = now;
+    } else if (lane == 1) {
+        if (sh.sink_e) atomic_add_ll(P.e + P.sink, sh.sink_e);
+        sh.sink_e = 0;
+    } else if (lane == 2) {
+        if (sh.src_e) atomic_add_ll(P.e + P.source, sh.src_e);
+        sh.src_e = 0;
+    } else if (lane == 3) {
+        if (sh.lab) atomicAdd((unsigned long long *)sh.cs->l[L_LAB].w, sh.lab);
+        sh.stat[ST_LAB_BFS] += (long long)(sh.lab >> 32);
+        sh.lab = 0;
+    }
+    __syncwarp();
+    if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&c->bar.w[0]) : "memory");
+}
+
+// Wait until every CTA has arrived at the current barrier; false after the
+// wait limit (MF_E_WAIT is recorded).  One thread.
+__device__ __forceinline__ bool wait_all(const MfParams &P, Sh &sh)
+{
+    MfCtrl *c = P.ctrl;
+    const unsigned target = (sh.phase + 1u) * (unsigned)vn();
+    unsigned long long t0 = 0;
+    unsigned spins = 0;
+    while ((int)(ld_acquire(&c->bar.w[0]) - target) < 0) {
+        if ((++spins & 255u) == 0) {
+            const unsigned long long now = gtimer();
+            if (t0 == 0) {
+                t0 = now;
+            } else if (now - t0 > P.wait_limit_ns) {
+                atomicCAS(&c->err.w[0], 0u, (unsigned)MF_E_WAIT);
+                return false;
+            }
+            if (spins > 4096) __nanosleep(100);
+        }
+    }
+    return true;
 }
 
 // Grid-wide barrier with a hook.  Returns false if this CTA gave up waiting
-// (the caller must return from the kernel at once).  Each CTA counts the
-// barrier generations it has passed (sh.gen), so arriving needs no read.
+// (the caller must return from the kernel at once).  One counter, which every
+// CTA raises and then watches: the arrival that completes it releases all of
+// them at once (304 CTAs: 1.4 us, against 2.5 us when the last one resets the
+// counter and publishes a generation word), and each works out the next step
+// from the counter set by itself (advance), where one thread running that
+// behind the barrier for all held them up for another 3 us.
 __device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh)
 {
     MfCtrl *c = P.ctrl;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        const unsigned gen = sh.gen;
-        __threadfence();
-        unsigned arrived = atomicAdd(&c->bar_count.w[0], 1u) + 1u;
-        if (arrived == vn()) {
-            atomicExch(&c->bar_count.w[0], 0u);
-            run_hook(P, hook);
-            __threadfence();
-            st_release(&c->bar_gen.w[0], gen + 1u);
-        } else {
-            unsigned long long t0 = 0;
-            unsigned spins = 0;
-            while (ld_acquire(&c->bar_gen.w[0]) == gen) {
-                ++spins;
-                if (spins > 64) __nanosleep(spins > 4096 ? 200 : 32);
-                if ((spins & 31u) == 0) {
-                    unsigned long long now = gtimer();
-                    if (t0 == 0) {
-                        t0 = now;
-                    } else if (now - t0 > P.wait_limit_ns) {
-                        atomicCAS(&c->err.w[0], 0u, (unsigned)MF_E_WAIT);
-                        ok = 0;
-                        break;
-                    }
-                }
-            }
+    const unsigned k = sh.phase;
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        if (hook == H_BFS_JOIN && vb() == 0) {
+            words_out((int *)&c->jd, (const int *)&sh.d, (int)(sizeof(MfDesc) / 4));
+            words_out((int *)&c->js, (const int *)&sh.hs, (int)(sizeof(MfState) / 4));
         }
-        __threadfence();
-        sh.gen = gen + 1u;
-        sh.ok = ok;
-        if (ok) load_desc(c, sh);
+        arrive(P, sh);
+        int ok = 0;
+        if (lane == 0) ok = wait_all(P, sh) ? 1 : 0;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        __syncwarp();
+        if (ok) {
+            if (lane < MF_LINES) {
+                sh.cnt[lane] = __ldcg(reinterpret_cast<const int4 *>(&sh.cs->l[lane]));
+                if (vb() == 0) __stcg(reinterpret_cast<int4 *>(&c->set[(k + 2u) % 3u].l[lane]), make_int4(0, 0, 0, 0));
+            }
+            if (hook == H_BFS_JOIN && vb() != 0) {
+                words_in((int *)&sh.d, (const int *)&c->jd, (int)(sizeof(MfDesc) / 4));
+                words_in((int *)&sh.hs, (const int *)&c->js, (int)(sizeof(MfState) / 4));
+            }
+            __syncwarp();
+            if (lane == 0) advance(P, hook, sh, cnt64(sh, L_TIME));
+        }
+        if (lane == 0) {
+            sh.ok = ok;
+            sh.phase = k + 1u;
+            sh.cs = &c->set[(k + 1u) % 3u];
+        }
     }
     __syncthreads();
+    if (vb() == 0 && (threadIdx.x >> 5) == (blockDim.x >> 5) - 1 && sh.ok) write_trace(P, sh, k);
     return sh.ok != 0;
 }
 
-
-// Flush per-CTA accumulators (excess of sink/source and counters).
-__device__ void flush_acc(const MfParams &P, Sh &sh, int phase)
+// The same step inside a run of small levels that the first CTA does alone
+// (nobody else touches the counter set meanwhile).
+__device__ __noinline__ void solo_step(const MfParams &P, int hook, Sh &sh)
 {
     __syncthreads();
-    if (threadIdx.x == 0) {
-        MfCtrl *c = P.ctrl;
-        {
-            // when this CTA finished the phase, after the release of the barrier that opened it
-            const unsigned long long t0 = sh.d.t_phase, now = gtimer();
-            const unsigned long long d = now > t0 ? now - t0 : 0;
-            atomicMax(&c->fin_max, d);
-            atomicAdd(&c->fin_sum, d);
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        if (lane < MF_LINES) {
+            int4 *p = reinterpret_cast<int4 *>(&sh.cs->l[lane]);
+            sh.cnt[lane] = __ldcg(p);
+            __stcg(p, make_int4(0, 0, 0, 0));
         }
-        if (sh.sink_e) atomic_add_ll(P.e + P.sink, sh.sink_e);
-        if (sh.src_e) atomic_add_ll(P.e + P.source, sh.src_e);
-        if (sh.pushes) atomic_add_ll(&c->pushes, sh.pushes);
-        if (sh.relabels) atomic_add_ll(&c->relabels, sh.relabels);
-        if (sh.steep) atomic_add_ll(&c->steep, sh.steep);
-        if (sh.slots || sh.verts || sh.cycles) {
-            if (phase == 0) {
-                atomic_add_ll(&c->slots_bfs, sh.slots);
-                atomic_add_ll(&c->verts_bfs, sh.verts);
-                atomic_add_ll(&c->hscan_bfs, sh.cycles);
-            } else if (phase == 1) {
-                atomic_add_ll(&c->slots_dis, sh.slots);
-                atomic_add_ll(&c->cycles_dis, sh.cycles);
-            } else if (phase == 2) {
-                atomic_add_ll(&c->slots_fix, sh.slots);
-                atomic_add_ll(&c->verts_fix, sh.verts);
-            } else if (phase == 3) {
-                atomic_add_ll(&c->verts_wl, sh.verts);
-            } else {
-                atomic_add_ll(&c->n_apply, sh.verts);
-                atomic_add_ll(&c->slots_apply, sh.slots);
-                atomic_add_ll(&c->clamps_apply, sh.cycles);
+        __syncwarp();
+        if (lane == 0) {
+            sh.cnt[L_LAB] = make_int4((int)(unsigned)sh.lab, (int)(sh.lab >> 32), 0, 0);
+            sh.stat[ST_LAB_BFS] += (long long)(sh.lab >> 32);
+            sh.lab = 0;
+            advance(P, hook, sh, gtimer());
+            const int i = sh.hs.trace_n - 1;
+            if (i < MF_TRACE) {
+                MfCtrl *c = P.ctrl;
+                c->trace_hook[i] = sh.tr_hook;
+                c->trace_t[i] = sh.hs.t_phase;
+                c->trace_slots[i] = sh.stat[ST_SLOTS_BFS] + sh.stat[ST_SLOTS_DIS] + sh.stat[ST_SLOTS_FIX];
+                c->trace_info[i] = sh.tr_info;
+                c->trace_fin_max[i] = c->trace_fin_mean[i] = 0;
             }
         }
-        if (sh.dis_cta_ns || sh.dis_warp_ns || sh.dis_thread_ns) {
-            atomicAdd(&c->ns_dis_cta, sh.dis_cta_ns);
-            atomicAdd(&c->ns_dis_warp, sh.dis_warp_ns);
-            atomicAdd(&c->ns_dis_thread, sh.dis_thread_ns);
-            sh.dis_cta_ns = sh.dis_warp_ns = sh.dis_thread_ns = 0;
-        }
-        if (sh.lab_cnt) {
-            atomic_add_ll(&c->lab_bfs, sh.lab_cnt);
-            unsigned long long *acc = (unsigned long long *)c->bfs_acc.w;
-            atomicAdd(acc + 0, (unsigned long long)sh.lab_slots);
-            atomicAdd(acc + 1, (unsigned long long)sh.lab_cnt);
-        }
-        sh.sink_e = sh.src_e = 0;
-        sh.pushes = sh.relabels = sh.steep = sh.slots = sh.verts = sh.cycles = 0;
-        sh.lab_slots = sh.lab_cnt = 0;
     }
     __syncthreads();
+}
+
+// The end of a launch: the counters go to the control block, every CTA arrives
+// once more, and the first one alone waits for the others, writes the results
+// down and leaves barrier and counter sets at zero for the next launch.
+__device__ __noinline__ bool finish(const MfParams &P, Sh &sh)
+{
+    MfCtrl *c = P.ctrl;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        if (lane < MF_STATS && sh.stat[lane]) atomic_add_ll(&c->stat[lane], sh.stat[lane]);
+        __syncwarp();
+        arrive(P, sh);
+        if (vb() == 0) {
+            int ok = 0;
+            if (lane == 0) ok = wait_all(P, sh) ? 1 : 0;
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            __syncwarp();
+            if (lane == 0) {
+                sh.ok = ok;
+                MfState &st = sh.hs;
+                st.t_phase = gtimer();
+                ++st.barriers;
+                ++st.trace_n;
+                sh.tr_hook = H_FINAL;
+                sh.tr_info = 0;
+            }
+            __syncwarp();
+            if (ok) {
+                write_trace(P, sh, sh.phase);
+                const int4 zero = make_int4(0, 0, 0, 0);
+                if (lane < MF_LINES)
+                    for (int q = 0; q < 3; ++q) __stcg(reinterpret_cast<int4 *>(&c->set[q].l[lane]), zero);
+                if (lane == 0) {
+                    const MfState &st = sh.hs;
+                    c->bar.w[0] = 0;
+                    c->d = sh.d;
+                    c->err.w[0] = (unsigned)st.err;
+                    c->iters = st.iters;
+                    c->bfs_levels = st.bfs_levels;
+                    c->active_total = st.active_total;
+                    c->active_first = st.active_first;
+                    c->ns_bfs = st.ns_bfs;
+                    c->ns_dis = st.ns_dis;
+                    c->ns_fix = st.ns_fix;
+                    c->ns_wl = st.ns_wl;
+                    c->ns_apply = st.ns_apply;
+                    c->rounds_total = st.rounds_total;
+                    c->barriers = st.barriers;
+                    c->trace_n = st.trace_n;
+                    c->t_exit = st.t_phase;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    return vb() != 0 || sh.ok != 0;
 }
 
 // Add d to the excess of z (sink and source go to the CTA accumulators).
@@ -744,9 +787,9 @@ __device__ __forceinline__ bool batch_entry(const MfParams &P, long long i, int 
 
 // Validate every entry; insert the directed key into the dedup table, where
 // the largest batch index (the last update of the pair) wins.
-__device__ __noinline__ void phase_apply_validate(const MfParams &P)
+__device__ __noinline__ void phase_apply_validate(const MfParams &P, Sh &sh)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int bits = P.sc.hash_bits;
     const unsigned mask = (1u << bits) - 1u;
     const int lane = threadIdx.x & 31;
@@ -758,7 +801,7 @@ __device__ __noinline__ void phase_apply_validate(const MfParams &P)
         int u, v, c;
         if (i < P.bcount) {
             if (!batch_entry(P, i, u, v, c)) {
-                atomicCAS(&ctl->err.w[0], 0u, (unsigned)MF_E_INVALID);
+                atomicCAS(&cs->l[L_MISC].w[3], 0u, (unsigned)MF_E_INVALID);
             } else if (u != v) {
                 unsigned long long key = ((unsigned long long)(unsigned)u << 32) | (unsigned)v;
                 pos = hash_slot(key, bits);
@@ -773,7 +816,7 @@ __device__ __noinline__ void phase_apply_validate(const MfParams &P)
                 }
             }
         }
-        warp_append(&ctl->misc.w[3], P.sc.hused, fresh, (int)pos);   // positions to clear afterwards
+        warp_append(&cs->l[L_MISC].w[2], P.sc.hused, fresh, (int)pos);   // positions to clear afterwards
     }
 }
 
@@ -842,7 +885,7 @@ __device__ __forceinline__ unsigned hash_find(const unsigned long long *keys, in
 // is refused whole.
 __device__ __noinline__ void phase_apply_locate(const MfParams &P, Sh &sh)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int bits = P.sc.hash_bits;
     const unsigned mask = (1u << bits) - 1u;
     const int lane = threadIdx.x & 31;
@@ -869,7 +912,7 @@ __device__ __noinline__ void phase_apply_locate(const MfParams &P, Sh &sh)
                 if (rp != 0xffffffffu) crev = __ldcg(P.bc + __ldcg(P.sc.hval + rp));
                 else if (x >= 0) crev = ldg_cg(P.g.cap + ldg_cg(P.g.rev + x));
                 if ((long long)c + crev > (long long)INT32_MAX)
-                    atomicCAS(&ctl->err.w[0], 0u, (unsigned)MF_E_TOO_LARGE);
+                    atomicCAS(&cs->l[L_MISC].w[3], 0u, (unsigned)MF_E_TOO_LARGE);
             }
             if (x < 0) {
                 const int a = min(u, v), b = max(u, v);
@@ -885,7 +928,7 @@ __device__ __noinline__ void phase_apply_locate(const MfParams &P, Sh &sh)
                         const int nb = atomicAdd(P.sc.ins_need + b, 1) + 1;
                         if (na > P.g.off[a + 1] - P.g.off[a] - ldg_cg(P.g.deg + a) ||
                             nb > P.g.off[b + 1] - P.g.off[b] - ldg_cg(P.g.deg + b))
-                            atomicExch(&ctl->misc.w[2], 1u);
+                            atomicExch(&cs->l[L_MISC].w[1], 1u);
                         break;
                     }
                     if (prev == pk) break;
@@ -893,9 +936,9 @@ __device__ __noinline__ void phase_apply_locate(const MfParams &P, Sh &sh)
                 }
             }
         }
-        warp_append(&ctl->misc.w[0], P.sc.ins_list, fresh, (int)pp);   // each new pair once
+        warp_append(&cs->l[L_MISC].w[0], P.sc.ins_list, fresh, (int)pp);   // each new pair once
     }
-    if (probes) atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)probes);
+    add_stat(sh, ST_SLOTS_APPLY, probes);
 }
 
 // Winning new capacity of the directed pair (a, b) in the batch, or -1 if the
@@ -965,17 +1008,16 @@ __device__ __noinline__ void phase_apply_change(const MfParams &P, Sh &sh)
             ++clamped;
         }
     }
-    if (applied) atomicAdd((unsigned long long *)&sh.verts, (unsigned long long)applied);
-    if (clamped) atomicAdd((unsigned long long *)&sh.cycles, (unsigned long long)clamped);
+    add_stat(sh, ST_N_APPLY, applied);
+    add_stat(sh, ST_CLAMPS_APPLY, clamped);
 }
 
 // keep_need: leave ins_need[] as it is (the rows' demand of spare slots after
 // an overflow; the rebuild that follows reads and clears it).
-__device__ __noinline__ void phase_apply_cleanup(const MfParams &P, bool keep_need)
+__device__ __noinline__ void phase_apply_cleanup(const MfParams &P, const Sh &sh, bool keep_need)
 {
-    MfCtrl *ctl = P.ctrl;
-    const int nused = (int)*(volatile unsigned *)&ctl->misc.w[3];
-    const int nins = (int)*(volatile unsigned *)&ctl->misc.w[0];
+    const int nused = sh.d.hused_n;
+    const int nins = sh.d.ins_n;
     for (int k = vb() * blockDim.x + threadIdx.x; k < nused; k += vn() * blockDim.x) {
         int pos = __ldcg(P.sc.hused + k);
         P.sc.hkey[pos] = kEmpty;
@@ -1002,7 +1044,7 @@ __device__ __noinline__ void phase_resaturate(const MfParams &P, Sh &sh)
     const int r0 = P.g.off[s];
     const int d = ldg_cg(P.g.deg + s);
     long long acc = 0;
-    if (vb() == 0 && threadIdx.x == 0) atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)d);
+    if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_SLOTS_APPLY, d);
     for (int j = vb() * blockDim.x + threadIdx.x; j < d; j += vn() * blockDim.x) {
         int x = r0 + j;
         int c = ldg_cg(P.cf + x);
@@ -1042,7 +1084,7 @@ __device__ __forceinline__ void frontier_push(const MfParams &P, Sh &sh, const b
                                               const int (&d)[R], const long long (&ev)[R], bool with_wl, int sel,
                                               bool eager = false)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int lane = threadIdx.x & 31;
     // long rows go to the long-row list, to be split into work items only if a
     // top-down level follows (a bottom-up level never reads them); `eager`
@@ -1080,10 +1122,8 @@ __device__ __forceinline__ void frontier_push(const MfParams &P, Sh &sh, const b
     // slots and number of the vertices labelled (the BFS direction test reads them)
     lab_slots = warp_sum_ll(lab_slots);
     const long long lab_cnt = warp_sum_ll((long long)lab_n);
-    if (lane == 0 && lab_cnt) {      // per CTA in shared memory, flushed with the phase's counters
-        atomicAdd((unsigned long long *)&sh.lab_slots, (unsigned long long)lab_slots);
-        atomicAdd((unsigned long long *)&sh.lab_cnt, (unsigned long long)lab_cnt);
-    }
+    if (lane == 0 && lab_cnt)        // per CTA in shared memory, added to the counter set at the barrier
+        atomicAdd(&sh.lab, ((unsigned long long)lab_cnt << 32) | (unsigned long long)lab_slots);
     if (total == 0 && ctot == 0) return;
     static_assert(MF_NBIN == 4, "one reservation per worklist bin below");
     // One lane reserves room in every list the warp appends to.  The
@@ -1094,14 +1134,13 @@ __device__ __forceinline__ void frontier_push(const MfParams &P, Sh &sh, const b
                    k4 = (unsigned)((total >> 32) & 0xffull);
     unsigned b0 = 0, b1 = 0, b2 = 0, b3 = 0, b4 = 0, bi = 0;
     if (lane == 0) {
-        if (k0) b0 = atomicAdd(&ctl->bfs_tail.w[0], k0);
-        if (k1) b1 = atomicAdd(&ctl->wl_tail[0].w[0], k1);
-        if (k2) b2 = atomicAdd(&ctl->wl_tail[1].w[0], k2);
-        if (k3) b3 = atomicAdd(&ctl->wl_tail[2].w[0], k3);
-        if (k4) b4 = atomicAdd(&ctl->wl_tail[3].w[0], k4);
-        if (ctot) bi = atomicAdd(lazy ? &ctl->long_tail.w[0] : &ctl->hub_tail.w[0], (unsigned)ctot);
-        const unsigned act = k1 + k2 + k3 + k4;
-        if (act) atomicAdd(&ctl->wl_tail[MF_NBIN].w[0], act);
+        if (k0) b0 = sh.d.app_bfs + atomicAdd(&cs->l[L_BFS].w[0], k0);
+        if (k1) b1 = sh.d.wl_app[0] + atomicAdd(&cs->l[L_WL].w[0], k1);
+        if (k2) b2 = sh.d.wl_app[1] + atomicAdd(&cs->l[L_WL + 1].w[0], k2);
+        if (k3) b3 = sh.d.wl_app[2] + atomicAdd(&cs->l[L_WL + 2].w[0], k3);
+        if (k4) b4 = sh.d.wl_app[3] + atomicAdd(&cs->l[L_WL + 3].w[0], k4);
+        if (ctot)
+            bi = (lazy ? sh.d.app_long : sh.d.app_hub) + atomicAdd(&cs->l[lazy ? L_LONG : L_HUB].w[0], (unsigned)ctot);
     }
     unsigned pos[MF_NBIN + 1];
     pos[0] = __shfl_sync(0xffffffffu, b0, 0) + (unsigned)(excl & 0xffull);
@@ -1187,7 +1226,7 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
     long long total = 0;
     const int lane = threadIdx.x & 31;
     const long long gs = (long long)vn() * blockDim.x;
-    if (vb() == 0 && threadIdx.x == 0) sh.verts += n;     // every vertex: e read, h written
+    if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_VERTS_BFS, n);     // every vertex: e read, h written
     for (long long base = (long long)vb() * blockDim.x + threadIdx.x - lane; base < n; base += gs) {
         const int v = (int)base + lane;
         bool root[1] = {false};
@@ -1217,7 +1256,7 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
         if (threadIdx.x == 0) {
             long long t = 0;
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh.wsum[w];
-            if (t) atomicAdd((unsigned long long *)P.ctrl->bfs_acc.w + 2, (unsigned long long)t);
+            if (t) atomicAdd((unsigned long long *)sh.cs->l[L_TOTAL].w, (unsigned long long)t);
         }
         __syncthreads();
     }
@@ -1265,14 +1304,14 @@ constexpr int kBR = 4;
 // long-row vertices 32 at a time and write their items together.
 __device__ __noinline__ void phase_bfs_expand(const MfParams &P, Sh &sh)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int lane = threadIdx.x & 31;
     const int lo = sh.d.long_lo, cnt = sh.d.long_hi - lo;
     const int nwarps = vn() * (int)(blockDim.x >> 5);
     const int rank = warp_rank(vn(), 0);
     bool first = true;
     for (;;) {
-        const int b = warp_deal(&ctl->head0.w[0], cnt, 32u, rank, nwarps, first);
+        const int b = warp_deal(&cs->l[L_HEAD0].w[0], cnt, 32u, rank, nwarps, first);
         if (b >= cnt) break;
         const int k = b + lane;
         const int z = k < cnt ? __ldcg(P.sc.blong + lo + k) : -1;
@@ -1288,7 +1327,7 @@ __device__ __noinline__ void phase_bfs_expand(const MfParams &P, Sh &sh)
         }
         const int tot = __shfl_sync(0xffffffffu, incl, 31);
         unsigned bi = 0;
-        if (lane == 0 && tot) bi = atomicAdd(&ctl->hub_tail.w[0], (unsigned)tot);
+        if (lane == 0 && tot) bi = sh.d.app_hub + atomicAdd(&cs->l[L_HUB].w[0], (unsigned)tot);
         bi = __shfl_sync(0xffffffffu, bi, 0);
         write_items<1>(P, nc, x0, d, bi, incl - nc[0], tot);
     }
@@ -1296,7 +1335,7 @@ __device__ __noinline__ void phase_bfs_expand(const MfParams &P, Sh &sh)
 
 __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int L = sh.d.level;
     const int sel = sh.d.wl_sel;
     const int lane = threadIdx.x & 31;
@@ -1308,7 +1347,7 @@ __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
     bool first = true;
     const int rank_i = warp_rank(nctas, 0);
     for (;;) {
-        const int i = warp_deal(&ctl->head1.w[0], icnt, 1u, rank_i, nwarps, first);
+        const int i = warp_deal(&cs->l[L_HEAD1].w[0], icnt, 1u, rank_i, nwarps, first);
         if (i >= icnt) break;
         const int2 it = __ldcg(P.sc.bitem + ilo + i);
         if (lane == 0) slots += it.y;
@@ -1333,7 +1372,7 @@ __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
     first = true;
     const int rank_f = warp_rank(nctas, icnt);
     for (;;) {
-        const int b = warp_deal(&ctl->head0.w[0], cnt, (unsigned)take, rank_f, nwarps, first);
+        const int b = warp_deal(&cs->l[L_HEAD0].w[0], cnt, (unsigned)take, rank_f, nwarps, first);
         if (b >= cnt) break;
         int idx = b + lane;
         int u = (lane < take && idx < cnt) ? __ldcg(P.sc.border + lo + idx) : -1;
@@ -1369,7 +1408,7 @@ __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
             bfs_visit<kBR>(P, sh, xs, vs, L, sel);
         }
     }
-    if (slots) atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)slots);
+    add_stat(sh, ST_SLOTS_BFS, slots);
 }
 
 // A BFS level bottom-up (direction-optimising BFS): every unlabelled vertex v
@@ -1382,7 +1421,7 @@ __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
 // rows, which pays off once the frontier holds most of the graph.
 __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int n = P.g.n;
     const int L = sh.d.level;
     const int sel = sh.d.wl_sel;
@@ -1401,7 +1440,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
     constexpr int kA = 4;
     const int cap = P.sc.bdefer != nullptr ? MF_BU_SCAN : 0x7fffffff;
     long long slots = 0, unl = 0;
-    if (vb() == 0 && threadIdx.x == 0) sh.cycles += n;    // every vertex's height is read
+    if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_HSCAN_BFS, n);    // every vertex's height is read
     for (long long base = (long long)vb() * blockDim.x + threadIdx.x - lane; base < n; base += gs) {
         const int v = (int)base + lane;
         const bool ok = v < n && v != skip;
@@ -1485,13 +1524,13 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
             }
             const int tot = __shfl_sync(0xffffffffu, ic, 31);
             unsigned at = 0;
-            if (lane == 0) at = atomicAdd(&ctl->defer_tail.w[0], (unsigned)tot);
+            if (lane == 0) at = atomicAdd(&cs->l[L_DEFER].w[0], (unsigned)tot);
             at = __shfl_sync(0xffffffffu, at, 0) + (unsigned)(ic - nitem);
             for (int cc = 0; cc < nitem; ++cc) P.sc.bdefer[at + cc] = make_int2(v, x0 + cc * MF_BU_CHUNK);
         }
     }
-    if (slots) atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)slots);
-    if (unl) atomicAdd((unsigned long long *)&sh.verts, (unsigned long long)unl);
+    add_stat(sh, ST_SLOTS_BFS, slots);
+    add_stat(sh, ST_VERTS_BFS, unl);
 }
 
 // Second pass of a bottom-up level: the deferred chunks of long rows whose
@@ -1501,7 +1540,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
 // chunks of the same row may find one too).
 __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int n = P.g.n;
     const int L = sh.d.level;
     const int sel = sh.d.wl_sel;
@@ -1515,7 +1554,7 @@ __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
     const int rank = warp_rank(vn(), 0);
     bool first = true;
     for (;;) {
-        const int i = warp_deal(&ctl->head1.w[0], cnt, 1u, rank, nwarps, first);
+        const int i = warp_deal(&cs->l[L_HEAD1].w[0], cnt, 1u, rank, nwarps, first);
         if (i >= cnt) break;
         const int2 it = __ldcg(P.sc.bdefer + i);
         const int v = it.x;
@@ -1548,7 +1587,7 @@ __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
             if (__any_sync(0xffffffffu, won[0])) frontier_push<1>(P, sh, won, zv, dv, ev, with_wl, sel);
         }
     }
-    if (slots) atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)slots);
+    add_stat(sh, ST_SLOTS_BFS, slots);
 }
 
 // ---------------------------------------------------------------------------
@@ -1557,7 +1596,7 @@ __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
 
 __device__ __noinline__ void phase_worklist(const MfParams &P, Sh &sh)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int sel = sh.d.wl_sel;
     const int n = P.g.n;
     const int lane = threadIdx.x & 31;
@@ -1571,9 +1610,9 @@ __device__ __noinline__ void phase_worklist(const MfParams &P, Sh &sh)
         int bin = 0;
         if (listed) bin = row_bin(P, ldg_cg(P.g.deg + v));
         unsigned am = __ballot_sync(0xffffffffu, act);
-        if (lane == 0 && am) atomicAdd(&ctl->wl_tail[MF_NBIN].w[0], (unsigned)__popc(am));
+        if (lane == 0 && am) atomicAdd(&cs->l[L_ACT].w[0], (unsigned)__popc(am));
 #pragma unroll
-        for (int b = 0; b < MF_NBIN; ++b) warp_append(&ctl->wl_tail[b].w[0], P.sc.wl[sel][b], listed && bin == b, v);
+        for (int b = 0; b < MF_NBIN; ++b) warp_append(&cs->l[L_WL + b].w[0], P.sc.wl[sel][b], listed && bin == b, v);
     }
 }
 
@@ -1590,6 +1629,8 @@ struct DisCtx {
     int qstamp;      // stamp of this round's queue
     int fstamp;      // stamp of this iteration's remove-invalid lists
     bool queue;      // a next round follows, so queue newly active vertices
+    MfSet *cs;       // this phase's counter set
+    int fix0, fix1;  // where this round's entries of the remove-invalid lists start
 };
 
 // z just became active (its excess went from <= 0 to > 0 during this round):
@@ -1600,7 +1641,7 @@ __device__ __forceinline__ void enqueue_active(const MfParams &P, int z, const D
     const int dz = ldg_cg(P.g.deg + z);      // in flight together with the stamp exchange
     if (atomicExch(P.sc.vmark + z, dc.qstamp) == dc.qstamp) return;
     const int bin = row_bin(P, dz);
-    const unsigned pos = atomicAdd(&P.ctrl->aux_tail[bin].w[0], 1u);
+    const unsigned pos = atomicAdd(&dc.cs->l[L_AUX + bin].w[0], 1u);
     P.sc.wl[dc.nsel][bin][pos] = z;
 }
 
@@ -1622,7 +1663,7 @@ __device__ __forceinline__ void note_relabel(const MfParams &P, int u, const Dis
     if (atomicExch(P.sc.fixmark + u, dc.fstamp) == dc.fstamp) return;
     const int d = ldg_cg(P.g.deg + u);
     const int li = d > P.hub_deg ? 1 : 0;
-    const unsigned pos = atomicAdd(&P.ctrl->aux_tail[MF_NBIN + li].w[0], 1u);
+    const unsigned pos = (li ? dc.fix1 : dc.fix0) + atomicAdd(&dc.cs->l[L_FIX + li].w[0], 1u);
     P.sc.fixl[li][pos] = u;
 }
 
@@ -1903,7 +1944,7 @@ __device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, 
                 hu = (best == kEmpty || best_h >= n - 1) ? n : best_h + 1;
                 P.h[u] = hu;
                 lifted = true;
-                atomicAdd((unsigned long long *)&sh.relabels, 1ull);
+                add_stat(sh, ST_RELABELS, 1);
                 ++cyc;
                 if (hu >= n || cyc >= P.kernel_cycles) continue;
             }
@@ -1946,7 +1987,7 @@ __device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, 
                 hu = (best == kEmpty || best_h >= n - 1) ? n : best_h + 1;
                 P.h[u] = hu;
                 lifted = true;
-                atomicAdd((unsigned long long *)&sh.relabels, 1ull);
+                add_stat(sh, ST_RELABELS, 1);
                 ++cyc;
                 if (hu >= n || cyc >= P.kernel_cycles) continue;
             }
@@ -1975,10 +2016,10 @@ __device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, 
         }
     }
     if (scans) {
-        atomicAdd((unsigned long long *)&sh.cycles, (unsigned long long)scans);
-        atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)(gscan + fused));
+        add_stat(sh, ST_CYCLES_DIS, scans);
+        add_stat(sh, ST_SLOTS_DIS, gscan + fused);
     }
-    if (moves) atomicAdd((unsigned long long *)&sh.pushes, (unsigned long long)moves);
+    add_stat(sh, ST_PUSHES, moves);
     return lifted;
 }
 
@@ -2029,7 +2070,7 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
             lifted = true;
             if (lane == 0) {
                 P.h[u] = hu;
-                atomicAdd((unsigned long long *)&sh.relabels, 1ull);
+                add_stat(sh, ST_RELABELS, 1);
             }
             ++cyc;
             if (hu >= n || cyc >= kcyc) {
@@ -2144,10 +2185,10 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
     fused = warp_sum_ll(fused);
     if (lane == 0) {
         if (scans) {
-            atomicAdd((unsigned long long *)&sh.cycles, (unsigned long long)scans);
-            atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)(gscan + fused));
+            add_stat(sh, ST_CYCLES_DIS, scans);
+            add_stat(sh, ST_SLOTS_DIS, gscan + fused);
         }
-        if (moves) atomicAdd((unsigned long long *)&sh.pushes, (unsigned long long)moves);
+        add_stat(sh, ST_PUSHES, moves);
     }
     return lifted;
 }
@@ -2235,8 +2276,8 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
         }
         const int best_h = b == kEmpty ? 0x7fffffff : (int)(b >> 32);
         if (T.tid == 0) {
-            atomicAdd((unsigned long long *)&sh.cycles, 1ull);
-            if (global_scan) atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)d);
+            add_stat(sh, ST_CYCLES_DIS, 1);
+            if (global_scan) add_stat(sh, ST_SLOTS_DIS, d);
         }
         bool go = b != kEmpty && hu > best_h;
         if (!go) {
@@ -2244,7 +2285,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
             const int nh = (b == kEmpty || best_h >= n - 1) ? n : best_h + 1;
             if (T.tid == 0) {
                 P.h[u] = nh;
-                atomicAdd((unsigned long long *)&sh.relabels, 1ull);
+                add_stat(sh, ST_RELABELS, 1);
             }
             lifted = true;
             ++cyc;
@@ -2311,7 +2352,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
                         }
                     }
                     if (T.tid == 0)
-                        atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)(seg * T.n));
+                        add_stat(sh, ST_SLOTS_DIS, seg * T.n);
                 }
                 long long incl = tsum;
                 int cincl = tcnt;
@@ -2374,7 +2415,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
             }
             if (T.tid == 0) {
                 if (sent) atomic_add_ll(P.e + u, PULL ? sent : -sent);
-                if (k) atomicAdd((unsigned long long *)&sh.pushes, (unsigned long long)k);
+                add_stat(sh, ST_PUSHES, k);
             }
             // staged: a pass that found only stale entries corrected them and costs no cycle (bounded)
             if (k > 0) cyc += k;
@@ -2382,7 +2423,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
         }
         T.sync();
     }
-    if (cand) atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)cand);
+    if (cand) add_stat(sh, ST_SLOTS_DIS, cand);
     return lifted;
 }
 
@@ -2411,13 +2452,16 @@ __device__ __forceinline__ bool discharge_group(const MfParams &P, Sh &sh, int u
 template <bool PULL>
 __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int lane = threadIdx.x & 31;
     const int sel = sh.d.wl_sel;
     DisCtx dc;
     dc.nsel = sel ^ 1;
     dc.qstamp = sh.d.qstamp;
     dc.fstamp = sh.d.fstamp;
+    dc.cs = cs;
+    dc.fix0 = sh.d.fix_n[0];
+    dc.fix1 = sh.d.fix_n[1];
     // queue the vertices that become active for a next round if one may follow
     // (adaptive rounds: the hook decides after this round)
     dc.queue = sh.d.round + 1 < (P.rounds > 0 ? P.rounds : MF_MAX_ROUNDS);
@@ -2428,8 +2472,8 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
     const int nh = sh.d.wl_n[3];
     for (;;) {
         if (threadIdx.x == 0) {
-            unsigned cur = *(volatile unsigned *)&ctl->head2.w[0];
-            sh.bcast_i = (int)(cur >= (unsigned)nh ? cur : atomicAdd(&ctl->head2.w[0], 1u));
+            unsigned cur = *(volatile unsigned *)&cs->l[L_HEAD2].w[0];
+            sh.bcast_i = (int)(cur >= (unsigned)nh ? cur : atomicAdd(&cs->l[L_HEAD2].w[0], 1u));
         }
         __syncthreads();
         int i = sh.bcast_i;
@@ -2451,8 +2495,8 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
         const int ng = sh.d.wl_n[2];
         for (;;) {
             if (T.tid == 0) {
-                unsigned cur = *(volatile unsigned *)&ctl->head3.w[0];
-                sh.tb_i[T.g] = (int)(cur >= (unsigned)ng ? cur : atomicAdd(&ctl->head3.w[0], 1u));
+                unsigned cur = *(volatile unsigned *)&cs->l[L_HEAD3].w[0];
+                sh.tb_i[T.g] = (int)(cur >= (unsigned)ng ? cur : atomicAdd(&cs->l[L_HEAD3].w[0], 1u));
             }
             T.sync();
             const int i = sh.tb_i[T.g];
@@ -2467,7 +2511,7 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
         }
     }
     const unsigned long long t_b = gtimer();
-    if (lane == 0) atomicAdd((unsigned long long *)&sh.dis_cta_ns, t_b - t_a);
+    if (lane == 0) add_stat(sh, ST_NS_CTA, (long long)(t_b - t_a));
     // mid-degree rows: one warp each, on a slice of its own group's quarter of
     // the snapshot buffer (free once the group has left the loop above, while
     // the other groups may still be on their rows)
@@ -2478,7 +2522,7 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
     int *wstage = stage != nullptr && wcap > 0
                       ? stage + (wid / MF_GROUP_WARPS) * gq + (wid % MF_GROUP_WARPS) * wcap : nullptr;
     for (;;) {
-        const int i = warp_grab(&ctl->head1.w[0], nm, 1u);
+        const int i = warp_grab(&cs->l[L_HEAD1].w[0], nm, 1u);
         if (i >= nm) break;
         const int u = __ldcg(wl1 + i);
         const bool lifted = discharge_warp<PULL>(P, sh, u, dc, wstage, wcap);
@@ -2491,7 +2535,7 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
     // small rows: one thread each, 32 per grab
     const int ns = sh.d.wl_n[0];
     for (;;) {
-        const int b = warp_grab(&ctl->head0.w[0], ns, 32u);
+        const int b = warp_grab(&cs->l[L_HEAD0].w[0], ns, 32u);
         if (b >= ns) break;
         if (b + lane < ns) {
             const int u = __ldcg(wl0 + b + lane);
@@ -2502,9 +2546,9 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
     __syncwarp();
     const unsigned long long t_d = gtimer();
     if (lane == 0) {
-        // per warp, into the CTA's accumulators (one global atomic per CTA and phase)
-        atomicAdd((unsigned long long *)&sh.dis_warp_ns, t_c - t_b);
-        atomicAdd((unsigned long long *)&sh.dis_thread_ns, t_d - t_c);
+        // per warp, into the CTA's counters
+        add_stat(sh, ST_NS_WARP, (long long)(t_c - t_b));
+        add_stat(sh, ST_NS_THREAD, (long long)(t_d - t_c));
     }
 }
 
@@ -2543,7 +2587,7 @@ __device__ __forceinline__ long long fix_scan(const MfParams &P, Sh &sh, int hu,
                     if (old > 0) {
                         atomicAdd(P.cf + x, old);
                         add_excess(P, sh, z[r], -(long long)old);
-                        atomicAdd((unsigned long long *)&sh.steep, 1ull);
+                        add_stat(sh, ST_STEEP, 1);
                         out -= old;
                     }
                 } else {
@@ -2551,7 +2595,7 @@ __device__ __forceinline__ long long fix_scan(const MfParams &P, Sh &sh, int hu,
                     if (old > 0) {
                         atomicAdd(P.cf + ldg_cg(P.g.rev + x), old);
                         add_excess(P, sh, z[r], (long long)old);
-                        atomicAdd((unsigned long long *)&sh.steep, 1ull);
+                        add_stat(sh, ST_STEEP, 1);
                         out += old;
                     }
                 }
@@ -2564,15 +2608,15 @@ __device__ __forceinline__ long long fix_scan(const MfParams &P, Sh &sh, int hu,
 template <bool PULL>
 __device__ __noinline__ void phase_fix(const MfParams &P, Sh &sh)
 {
-    MfCtrl *ctl = P.ctrl;
+    MfSet *cs = sh.cs;
     const int lane = threadIdx.x & 31;
     long long slots = 0, verts = 0;
     // rows above hub_deg: one CTA each
     const int nh = sh.d.fix_n[1];
     for (;;) {
         if (threadIdx.x == 0) {
-            unsigned cur = *(volatile unsigned *)&ctl->head2.w[0];
-            sh.bcast_i = (int)(cur >= (unsigned)nh ? cur : atomicAdd(&ctl->head2.w[0], 1u));
+            unsigned cur = *(volatile unsigned *)&cs->l[L_HEAD2].w[0];
+            sh.bcast_i = (int)(cur >= (unsigned)nh ? cur : atomicAdd(&cs->l[L_HEAD2].w[0], 1u));
         }
         __syncthreads();
         int i = sh.bcast_i;
@@ -2588,7 +2632,7 @@ __device__ __noinline__ void phase_fix(const MfParams &P, Sh &sh)
     // the others: one warp each
     const int nw = sh.d.fix_n[0];
     for (;;) {
-        const int i = warp_grab(&ctl->head1.w[0], nw, 1u);
+        const int i = warp_grab(&cs->l[L_HEAD1].w[0], nw, 1u);
         if (i >= nw) break;
         const int u = __ldcg(P.sc.fixl[0] + i);
         const int hu = ldg_cg(P.h + u);
@@ -2600,8 +2644,8 @@ __device__ __noinline__ void phase_fix(const MfParams &P, Sh &sh)
             ++verts;
         }
     }
-    if (slots) atomicAdd((unsigned long long *)&sh.slots, (unsigned long long)slots);
-    if (verts) atomicAdd((unsigned long long *)&sh.verts, (unsigned long long)verts);
+    add_stat(sh, ST_SLOTS_FIX, slots);
+    add_stat(sh, ST_VERTS_FIX, verts);
 }
 
 // ---------------------------------------------------------------------------
@@ -2629,95 +2673,100 @@ __device__ __noinline__ void phase_value(const MfParams &P)
 // CTAs together.
 __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
 {
-    if (vb() == 0 && threadIdx.x == 0) P.ctrl->t_entry = gtimer();
+    __syncthreads();          // the parameters are in shared memory
+    if (threadIdx.x < MF_STATS) sh.stat[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
-        sh.gen = ld_acquire(&P.ctrl->bar_gen.w[0]);   // nobody can pass the first barrier before all have read it
+        MfCtrl *c = P.ctrl;
         sh.sink_e = sh.src_e = 0;
-        sh.pushes = sh.relabels = sh.steep = sh.slots = sh.verts = sh.cycles = 0;
-        sh.lab_slots = sh.lab_cnt = 0;
-        sh.dis_cta_ns = sh.dis_warp_ns = sh.dis_thread_ns = 0;
+        sh.lab = 0;
+        sh.phase = 0;
+        sh.cs = &c->set[0];
+        sh.d = MfDesc{};
+        sh.hs = MfState{};
+        sh.d.qstamp = __ldcg(&c->d.qstamp);
+        sh.d.fstamp = __ldcg(&c->d.fstamp);
+        sh.hs.t_phase = gtimer();
     }
+    if (vb() == 0) {
+        // results start at zero; the other CTAs add to them at the end of the launch
+        MfCtrl *c = P.ctrl;
+        if (threadIdx.x < MF_STATS) c->stat[threadIdx.x] = 0;
+        if (threadIdx.x < MF_ACTIVE_HIST) c->active_hist[threadIdx.x] = 0;
+        if (threadIdx.x == 0) {
+            c->value = 0;
+            c->err.w[0] = 0;
+            c->t_entry = gtimer();
+        }
+    }
+    __syncthreads();
     // a CTA that never arrives (tests only): the others give up after
     // wait_limit_ns, record MF_E_WAIT and leave the kernel
     if (P.test_skip_cta == vb()) return true;
-    if (!grid_sync(P, H_START, sh)) return false;
 
+    const bool loops = (P.mode & (MF_M_SOLVE | MF_M_BFS_ONLY)) != 0;
+    bool opened = false;      // the last barrier opened the first iteration
     if (P.mode & MF_M_STATIC_INIT) {
+        const bool sat = !(P.mode & MF_M_NO_SRC_SAT), sink = (P.mode & MF_M_SAT_SINK) != 0;
         phase_static_reset(P);
-        if (!grid_sync(P, H_NONE, sh)) return false;
-        if (!(P.mode & MF_M_NO_SRC_SAT)) {
+        if (!grid_sync(P, sat || sink || !loops ? H_NONE : H_ITER, sh)) return false;
+        if (sat) {
             phase_saturate_source(P, sh);
-            flush_acc(P, sh, 4);
-            if (!grid_sync(P, H_NONE, sh)) return false;
+            if (!grid_sync(P, sink || !loops ? H_NONE : H_ITER, sh)) return false;
         }
-        if (P.mode & MF_M_SAT_SINK) {
+        if (sink) {
             phase_saturate_sink(P, sh);
-            flush_acc(P, sh, 4);
-            if (!grid_sync(P, H_NONE, sh)) return false;
+            if (!grid_sync(P, loops ? H_ITER : H_NONE, sh)) return false;
         }
+        opened = loops;
     }
     if (P.mode & MF_M_APPLY) {
-        phase_apply_validate(P);
+        phase_apply_validate(P, sh);
         if (!grid_sync(P, H_APPLY_VALID, sh)) return false;
         if (sh.d.status != MF_ST_RUNNING) {
-            phase_apply_cleanup(P, false);
-            return grid_sync(P, H_FINAL, sh);
+            phase_apply_cleanup(P, sh, false);
+            return finish(P, sh);
         }
         phase_apply_locate(P, sh);
-        flush_acc(P, sh, 4);
         if (!grid_sync(P, H_APPLY_LOCATED, sh)) return false;
         if (sh.d.status != MF_ST_RUNNING) {
             // a row overflow keeps the rows' demand for the rebuild that follows;
             // a refused batch (pair sum) leaves nothing behind
-            phase_apply_cleanup(P, *(volatile unsigned *)&P.ctrl->err.w[0] == MF_E_OVERFLOW);
-            return grid_sync(P, H_FINAL, sh);
+            phase_apply_cleanup(P, sh, sh.hs.err == MF_E_OVERFLOW);
+            return finish(P, sh);
         }
         phase_apply_change(P, sh);
-        flush_acc(P, sh, 4);
         if (!grid_sync(P, H_APPLY_DELTA, sh)) return false;
         // the source step reads the final residuals; the tables are cleared beside it
-        phase_apply_cleanup(P, false);
+        phase_apply_cleanup(P, sh, false);
         if (!(P.mode & MF_M_SKIP_SOURCE_SAT)) phase_resaturate(P, sh);
-        flush_acc(P, sh, 4);
         // straight on to the loop: this barrier opens its first iteration
-        if (!(P.mode & MF_M_CUT) && (P.mode & (MF_M_SOLVE | MF_M_BFS_ONLY))) {
-            if (!grid_sync(P, H_ITER, sh)) return false;
-            if (sh.d.status != MF_ST_RUNNING) return true;
-            goto loop;
-        }
-        if (!grid_sync(P, H_NONE, sh)) return false;
+        opened = loops && !(P.mode & MF_M_CUT);
+        if (!opened && !(P.mode & MF_M_CUT) && !loops) return finish(P, sh);
+        if (!grid_sync(P, opened ? H_ITER : H_NONE, sh)) return false;
         if (P.mode & MF_M_CUT) {
             phase_cut_side(P);
             if (!grid_sync(P, H_NONE, sh)) return false;
             phase_saturate_cut(P, sh);
-            flush_acc(P, sh, 4);
             if (!grid_sync(P, H_NONE, sh)) return false;
         }
-        if (sh.d.status != MF_ST_RUNNING) return true;
+        if (sh.d.status != MF_ST_RUNNING) return finish(P, sh);
     }
-    if (!(P.mode & (MF_M_SOLVE | MF_M_BFS_ONLY))) return true;
+    if (!loops) return finish(P, sh);
 
-    if (!grid_sync(P, H_ITER, sh)) return false;
-loop:
+    if (!opened && !grid_sync(P, H_ITER, sh)) return false;
     for (;;) {
         // backward BFS
         phase_bfs_init(P, sh);
-        flush_acc(P, sh, 0);               // the roots' label counters feed the first level's direction
         if (!grid_sync(P, H_BFS_START, sh)) return false;
         while (!sh.d.bfs_done) {
             if (sh.d.bfs_cta_mode) {
-                // small levels: CTA 0 alone, its own thread 0 running the level
-                // hook; the other CTAs wait at the next grid barrier
+                // small levels: CTA 0 alone; the others wait at the next grid
+                // barrier and take its state there
                 if (vb() == 0) {
                     int run = 0;
                     do {
                         phase_bfs_level(P, sh);
-                        flush_acc(P, sh, 0);
-                        if (threadIdx.x == 0) {
-                            run_hook(P, H_BFS_NEXT);
-                            load_desc(P.ctrl, sh);
-                        }
-                        __syncthreads();
+                        solo_step(P, H_BFS_NEXT, sh);
                     } while (++run < MF_TAIL_RUN && !sh.d.bfs_done && sh.d.bfs_cta_mode);
                 }
                 if (!grid_sync(P, H_BFS_JOIN, sh)) return false;
@@ -2725,11 +2774,9 @@ loop:
             }
             if (sh.d.bu_mode) {
                 phase_bfs_bottom_up(P, sh);
-                flush_acc(P, sh, 0);
                 if (!grid_sync(P, H_BU_SPLIT, sh)) return false;     // ends the level if nothing was deferred
                 if (sh.d.bu_split) {
                     phase_bfs_bottom_up_long(P, sh);
-                    flush_acc(P, sh, 0);
                     if (!grid_sync(P, H_BFS_NEXT, sh)) return false;
                 }
             } else {
@@ -2738,11 +2785,10 @@ loop:
                     if (!grid_sync(P, H_EXPANDED, sh)) return false;
                 }
                 phase_bfs_level(P, sh);
-                flush_acc(P, sh, 0);
                 if (!grid_sync(P, H_BFS_NEXT, sh)) return false;
             }
         }
-        if (P.mode & MF_M_BFS_ONLY) return true;
+        if (P.mode & MF_M_BFS_ONLY) return finish(P, sh);
         // worklist and termination test (built during the BFS when data-driven)
         if (!P.data_driven) {
             phase_worklist(P, sh);
@@ -2753,30 +2799,30 @@ loop:
         do {
             if (P.pull) phase_discharge<true>(P, sh);
             else phase_discharge<false>(P, sh);
-            flush_acc(P, sh, 1);
             if (!grid_sync(P, H_DIS, sh)) return false;
         } while (sh.d.dis_more);
         if (P.fix_steep) {
             if (P.pull) phase_fix<true>(P, sh);
             else phase_fix<false>(P, sh);
-            flush_acc(P, sh, 2);
             if (!grid_sync(P, H_ITER, sh)) return false;
         }
     }
-    if (sh.d.status == MF_ST_ERROR) return true;
-    if (!(P.mode & MF_M_NO_VALUE)) phase_value(P);
-    return grid_sync(P, H_FINAL, sh);
+    if (sh.d.status != MF_ST_ERROR && !(P.mode & MF_M_NO_VALUE)) phase_value(P);
+    return finish(P, sh);
 }
 
-__global__ void __launch_bounds__(MF_BLOCK, 2) mf_solve_kernel(MfParams P)
+__global__ void __launch_bounds__(MF_BLOCK, 2) mf_solve_kernel(const __grid_constant__ MfParams P)
 {
     __shared__ Sh sh;
+    __shared__ MfParams sP;       // the phases read the parameters often: from shared memory
+    for (int i = threadIdx.x; i < (int)(sizeof(MfParams) / 4); i += blockDim.x)
+        reinterpret_cast<int *>(&sP)[i] = reinterpret_cast<const int *>(&P)[i];
     if (threadIdx.x == 0) {
         g_vb = blockIdx.x;
         g_vn = gridDim.x;
     }
     __syncthreads();
-    solve_instance(P, sh);
+    solve_instance(sP, sh);
 }
 
 // Barrier of one group of CTAs (no hook): w[0] arrivals, w[1] generation.
@@ -2828,6 +2874,7 @@ __global__ void __launch_bounds__(MF_BLOCK, 2) mf_multi_kernel(const MfParams *_
                                                                unsigned long long wait_ns, int *abort)
 {
     __shared__ Sh sh;
+    __shared__ MfParams sP;
     __shared__ unsigned ggen;
     const int grp = blockIdx.x / gsize;
     unsigned *gw = gstate + 32 * grp;
@@ -2842,7 +2889,9 @@ __global__ void __launch_bounds__(MF_BLOCK, 2) mf_multi_kernel(const MfParams *_
         if (!group_sync(gw, ggen, wait_ns, abort)) return;
         const int i = (int)__ldcg(gw + 2);
         if (i >= count) return;
-        if (!solve_instance(plist[i], sh)) {
+        for (int w = threadIdx.x; w < (int)(sizeof(MfParams) / 4); w += blockDim.x)
+            reinterpret_cast<int *>(&sP)[w] = __ldcg(reinterpret_cast<const int *>(plist + i) + w);
+        if (!solve_instance(sP, sh)) {
             atomicExch(abort, 1);
             return;
         }
