@@ -303,12 +303,14 @@ int alloc_vertex_scratch(maxflow_ctx *c)
         for (int b = 0; b < MF_NBIN; ++b) c->sc.wl[q][b] = dalloc_n<int32_t>(c, n);
     c->sc.vmark = dalloc_n<int32_t>(c, n);
     c->sc.fixmark = dalloc_n<int32_t>(c, n);
+    c->sc.par = dalloc_n<int32_t>(c, n);
+    c->sc.dem = dalloc_n<long long>(c, n);
     c->sc.fixl[0] = dalloc_n<int32_t>(c, n);
     c->sc.fixl[1] = dalloc_n<int32_t>(c, n);
     c->sc.ins_need = dalloc_n<int32_t>(c, n);
     c->sc.blong = dalloc_n<int32_t>(c, n);
     if (!c->sc.border || !c->sc.vmark || !c->sc.fixmark || !c->sc.fixl[0] || !c->sc.fixl[1] || !c->sc.ins_need ||
-        !c->sc.blong)
+        !c->sc.blong || !c->sc.par || !c->sc.dem)
         return MAXFLOW_ERR_OOM;
     for (int q = 0; q < 2; ++q)
         for (int b = 0; b < MF_NBIN; ++b)

@@ -38,6 +38,10 @@
 #define MF_BU_SCAN 256        // bottom-up BFS: slots of a row its warp scans before deferring the rest
 #define MF_BU_CHUNK 256       // bottom-up BFS: slots per deferred work item (one warp, 8 per lane)
 #define MF_TAIL_SLOTS 2048    // BFS default: frontiers up to this many slots run in one CTA
+#define MF_NEAR_SINK 8        // near iterations: the sink's row holds at most 1/8 of the vertices
+#define MF_NEAR_SLOTS 65536   // near iterations: graphs of at least this many reserved slots
+#define MF_NEAR_STEP 3        // near iterations: a cut that settled less than half asks for 2^3 times the excess next
+#define MF_NEAR_SUB 8192      // walks: residuals up to this are taken with one atomic subtraction
 #define MF_TAIL_RUN 256       // BFS: levels CTA 0 runs alone before the grid meets once (bounds the others' wait)
 
 // Solve-kernel status (ctrl->status)
@@ -93,6 +97,8 @@ enum MfLineId {
     L_MISC,               // w[0] new pairs, w[1] a row without room, w[2] dedup entries, w[3] error (MF_E_*)
     L_LAB,                // 64-bit: labelled vertices << 32 | their slots
     L_TOTAL,              // 64-bit: used slots of the whole graph (summed by the BFS roots pass)
+    L_EXC,                // 64-bit: excess of the vertices labelled in this phase (near iterations)
+    L_DEM,                // 64-bit: what the roots can take (BFS roots pass, near iterations)
     L_TIME,               // 64-bit: the first CTA's clock when it arrived at the barrier
     MF_LINES
 };
@@ -124,6 +130,8 @@ struct MfDesc {
     int ins_n, hused_n;           // batch: new pairs, dedup table entries
     int round;                    // discharge round within the iteration
     int dis_more;                 // another discharge round follows
+    int near;                     // this launch may cut its global relabels short and walk the excess down
+    int cut;                      // ... and this iteration's was cut short
     int fix_n[2];                 // vertices for remove-invalid-edges (warp list, CTA list); grows over the rounds
     int qstamp, fstamp;           // dedupe stamps (never reset: they only grow across launches)
 };
@@ -138,6 +146,8 @@ struct MfState {
     long long vis_slots;          // slots of the vertices labelled so far in this BFS
     long long lvl_slots, lvl_cnt; // slots and number of the vertices labelled by the level that is running
     long long used_slots;         // used slots of the graph (0: not summed yet)
+    long long sup, dem, dem_prev; // this BFS: excess labelled, what the roots can take (and the BFS before)
+    int cut_prev, cut_shift;      // the iteration before was cut short; how much more excess a cut asks for
     long long iters, bfs_levels, rounds_total, barriers, active_first, active_total;
     int err;                      // MF_E_*
     int trace_n;
@@ -215,6 +225,8 @@ struct MfScratch {
                               // 4-warp group, CTA
     int32_t *vmark;           // [n] round stamp of the last time a vertex was queued
     int32_t *fixmark;         // [n] iteration stamp of the last time a vertex was listed for Alg. 3
+    int32_t *par;             // [n] slot (v, parent) of the vertices labelled by a near BFS (nullptr: never near)
+    long long *dem;           // [n] what a root can still take in a near iteration
     int32_t *fixl[2];         // [n] vertices relabelled this iteration: rows <= MF_HUB_DEG, rows above
     // batch apply
     int64_t batch_cap;

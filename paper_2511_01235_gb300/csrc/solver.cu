@@ -167,6 +167,7 @@ struct Sh {
     long long sink_e, src_e;          // excess of the sink and the source, added to memory before every barrier
     long long stat[MF_STATS];         // work counters, added to memory at the end of the launch
     unsigned long long lab;           // BFS: vertices labelled this phase << 32 | their slots
+    unsigned long long exc, dem;      // near BFS: excess labelled, what the roots can take, this phase
     unsigned long long red[MF_WARPS];
     long long wsum[MF_WARPS];
     int wcnt[MF_WARPS];
@@ -236,12 +237,25 @@ __device__ __forceinline__ void decide_iteration(const MfParams &P, Sh &sh, int 
     }
 }
 
+// Whether the launch may run near iterations: a push solve with the default
+// schedule, and a sink that can be reached from few vertices directly.  With a
+// longer sink row (grids: every pixel has an edge to t) what the sink can take
+// exceeds any excess, no relabel would be cut, and the bookkeeping would only
+// cost.
+__device__ __forceinline__ int near_allowed(const MfParams &P)
+{
+    if (P.sc.par == nullptr || !(P.mode & MF_M_SOLVE) || (P.mode & MF_M_NO_DEFICIT_ROOTS) || P.pull ||
+        P.side_root >= 0 || P.rounds != 0 || P.fix_steep || !P.data_driven || P.g.slot_cap < MF_NEAR_SLOTS)
+        return 0;
+    return (long long)ldg_cg(P.g.deg + P.sink) * MF_NEAR_SINK <= (long long)P.g.n ? 1 : 0;
+}
+
 // Opens an iteration of the loop (its BFS comes next).
 __device__ __forceinline__ void begin_iteration(Sh &sh)
 {
     MfDesc &d = sh.d;
     sh.hs.t_bfs0 = sh.hs.t_now;
-    sh.hs.vis_slots = sh.hs.lvl_slots = sh.hs.lvl_cnt = 0;
+    sh.hs.vis_slots = sh.hs.lvl_slots = sh.hs.lvl_cnt = sh.hs.sup = 0;
     d.lvl_lo = d.lvl_hi = d.hub_lo = d.hub_hi = d.long_lo = d.long_hi = 0;
     d.app_bfs = d.app_hub = d.app_long = 0;
     for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] = 0;
@@ -277,6 +291,7 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         const unsigned long long lab = cnt64(sh, L_LAB);
         st.lvl_slots += (long long)(lab & 0xffffffffull);
         st.lvl_cnt += (long long)(lab >> 32);
+        st.sup += (long long)cnt64(sh, L_EXC);
         if (hook == H_BU_SPLIT) {
             // after the first pass of a bottom-up level: a second pass over the
             // deferred long rows, or (none deferred) the level is complete
@@ -309,6 +324,14 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
     case H_BFS_NEXT: {
         const bool first = hook == H_BFS_START;
         if (first && d.need_total) st.used_slots = (long long)cnt64(sh, L_TOTAL);
+        if (first && d.near) {
+            // a cut-short relabel whose walks settled less than half of what was
+            // open looks for more excess this time, so that after a few of them
+            // the relabel is a complete one
+            st.dem = (long long)cnt64(sh, L_DEM);
+            if (st.cut_prev && 2 * st.dem > st.dem_prev) st.cut_shift = min(st.cut_shift + MF_NEAR_STEP, 60);
+            st.dem_prev = st.dem;
+        }
         const int items = d.hub_hi - d.hub_lo;
         d.lvl_lo = d.lvl_hi;
         d.hub_lo = d.hub_hi;
@@ -341,7 +364,11 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         // few hundred slots costs a grid barrier otherwise
         d.bfs_cta_mode =
             (!done && !bu && !d.expand && P.tail_slots > 0 && fr <= P.tail_slots && cnt <= P.tail_slots) ? 1 : 0;
-        if (done && want_wl) {
+        // near iterations: the levels so far hold as much excess as the roots can take
+        d.cut = d.near && !done && st.sup > 0 && (st.sup >> st.cut_shift) >= st.dem ? 1 : 0;
+        st.cut_prev = d.cut;
+        if (d.cut) d.bfs_done = 1;
+        if (d.bfs_done && want_wl) {
             int active = 0;
             for (int b = 0; b < MF_NBIN; ++b) active += d.wl_app[b];
             decide_iteration(P, sh, active);
@@ -369,7 +396,11 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         // taken less than half of its BFS -- a global relabel that costs much
         // (deep BFS, e.g. grids) is amortised over more rounds
         bool more = nxt > 0 && st.err == 0 && d.round + 1 < MF_MAX_ROUNDS;
-        if (more && d.round + 1 >= (P.rounds > 0 ? P.rounds : MF_DEFAULT_ROUNDS))
+        if (d.near && d.round == 0) {
+            // the walks: rounds follow only a complete relabel, and only while
+            // they are cheap beside it
+            more = more && !d.cut && 2 * (t - st.t_dis0) < st.t_dis0 - st.t_bfs0;
+        } else if (more && d.round + 1 >= (P.rounds > 0 ? P.rounds : MF_DEFAULT_ROUNDS))
             more = P.rounds > 0 ? false : 2 * (t - st.t_dis0) < st.t_dis0 - st.t_bfs0;
         d.dis_more = more ? 1 : 0;
         if (more) {
@@ -468,6 +499,12 @@ __device__ __forceinline__ void arrive(const MfParams &P, Sh &sh)
         if (sh.lab) atomicAdd((unsigned long long *)sh.cs->l[L_LAB].w, sh.lab);
         sh.stat[ST_LAB_BFS] += (long long)(sh.lab >> 32);
         sh.lab = 0;
+    } else if (lane == 4) {
+        if (sh.exc) atomicAdd((unsigned long long *)sh.cs->l[L_EXC].w, sh.exc);
+        sh.exc = 0;
+    } else if (lane == 5) {
+        if (sh.dem) atomicAdd((unsigned long long *)sh.cs->l[L_DEM].w, sh.dem);
+        sh.dem = 0;
     }
     __syncwarp();
     if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&c->bar.w[0]) : "memory");
@@ -559,6 +596,8 @@ __device__ __noinline__ void solo_step(const MfParams &P, int hook, Sh &sh)
             sh.cnt[L_LAB] = make_int4((int)(unsigned)sh.lab, (int)(sh.lab >> 32), 0, 0);
             sh.stat[ST_LAB_BFS] += (long long)(sh.lab >> 32);
             sh.lab = 0;
+            sh.cnt[L_EXC] = make_int4((int)(unsigned)sh.exc, (int)(sh.exc >> 32), 0, 0);
+            sh.exc = 0;
             advance(P, hook, sh, gtimer());
             const int i = sh.hs.trace_n - 1;
             if (i < MF_TRACE) {
@@ -1094,7 +1133,7 @@ __device__ __forceinline__ void frontier_push(const MfParams &P, Sh &sh, const b
     // bins; and this lane's long rows (lazy) or their work items
     unsigned long long packed = 0;
     int nch = 0;
-    long long lab_slots = 0;
+    long long lab_slots = 0, exc = 0;
     int lab_n = 0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -1103,8 +1142,12 @@ __device__ __forceinline__ void frontier_push(const MfParams &P, Sh &sh, const b
         ++lab_n;
         if (d[r] > P.bfs_hub) nch += lazy ? 1 : (d[r] + MF_BFS_CHUNK - 1) / MF_BFS_CHUNK;
         else packed += 1ull;
-        if (with_wl && ev[r] > 0) packed += 1ull << (8 * (row_bin(P, d[r]) + 1));
+        if (with_wl && ev[r] > 0) {
+            packed += 1ull << (8 * (row_bin(P, d[r]) + 1));
+            exc += ev[r];
+        }
     }
+    if (exc && sh.d.near) atomicAdd(&sh.exc, (unsigned long long)exc);
     unsigned long long incl = packed;
     int cincl = nch;
 #pragma unroll
@@ -1223,9 +1266,15 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
     const bool deficit_roots = (P.mode & MF_M_NO_DEFICIT_ROOTS) == 0;
     const bool pull = P.pull != 0;
     const bool need_total = sh.d.need_total != 0;
-    long long total = 0;
+    const bool near = sh.d.near != 0;
+    long long total = 0, take = 0;        // near: what the roots can take
     const int lane = threadIdx.x & 31;
     const long long gs = (long long)vn() * blockDim.x;
+    if (near) {
+        const int r0 = P.g.off[P.sink], d = ldg_cg(P.g.deg + P.sink);
+        for (long long j = (long long)vb() * blockDim.x + threadIdx.x; j < d; j += gs)
+            take += ldg_cg(P.g.pcap + r0 + j) - ldg_cg(P.cf + r0 + j);
+    }
     if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_VERTS_BFS, n);     // every vertex: e read, h written
     for (long long base = (long long)vb() * blockDim.x + threadIdx.x - lane; base < n; base += gs) {
         const int v = (int)base + lane;
@@ -1240,14 +1289,21 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
             const bool side_ok = P.side_root < 0 || P.side[v] == P.side_root;
             if (pull)
                 root[0] = (v == P.source) || (v != P.sink && side_ok && ldg_cg(P.e + v) > 0);
-            else
-                root[0] = (v == P.sink) || (deficit_roots && v != P.source && side_ok && ldg_cg(P.e + v) < 0);
+            else {
+                const long long e = (deficit_roots && v != P.source && v != P.sink && side_ok) ? ldg_cg(P.e + v) : 0;
+                root[0] = v == P.sink || e < 0;
+                if (near && e < 0) {
+                    P.sc.dem[v] = -e;
+                    take -= e;
+                }
+            }
             P.h[v] = root[0] ? 0 : n;
             if (root[0]) dv[0] = need_total ? dall : ldg_cg(P.g.deg + v);
         }
         total += dall;
         if (__any_sync(0xffffffffu, root[0])) frontier_push<1>(P, sh, root, zv, dv, ev, false, 0, true);
     }
+    if (take) atomicAdd(&sh.dem, (unsigned long long)take);
     if (need_total) {
         // one atomic per CTA for the used-slot total
         total = warp_sum_ll(total);
@@ -1274,6 +1330,8 @@ __device__ __forceinline__ void bfs_visit(const MfParams &P, Sh &sh, const int (
     const bool with_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
     const bool pull = P.pull != 0;
     const int skip = pull ? P.sink : P.source;     // the terminal a BFS never labels
+    const bool near = sh.d.near != 0;
+    const int t0 = near && L == 0 ? P.g.off[P.sink] : 0, t1 = near && L == 0 ? t0 + ldg_cg(P.g.deg + P.sink) : 0;
     const int n = P.g.n;
     int z[BR], rc[BR], hz[BR], d[BR];
     bool claim[BR];
@@ -1293,6 +1351,10 @@ __device__ __forceinline__ void bfs_visit(const MfParams &P, Sh &sh, const int (
         d[r] = claim[r] ? ldg_cg(P.g.deg + z[r]) : 0;
         const bool term = z[r] == P.sink || z[r] == P.source;
         ev[r] = (with_wl && claim[r] && !term) ? (pull ? -ldg_cg(P.e + z[r]) : ldg_cg(P.e + z[r])) : 0;
+        if (near && claim[r]) {
+            P.sc.par[z[r]] = ldg_cg(P.g.rev + x[r]);
+            if (x[r] >= t0 && x[r] < t1) P.sc.dem[z[r]] = rc[r];     // z's own edge into the sink
+        }
     }
     frontier_push<BR>(P, sh, claim, z, d, ev, with_wl, sel);
 }
@@ -1411,6 +1473,15 @@ __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
     add_stat(sh, ST_SLOTS_BFS, slots);
 }
 
+// Near BFS, bottom-up: slot x = (v, z) with residual c leads v down to z at
+// level L.  Several lanes may find a slot for the same v; any of them will do
+// (there is one slot (v, sink) at most, so dem[v] fits par[v] either way).
+__device__ __forceinline__ void note_parent(const MfParams &P, int v, int x, int z, int c, int L)
+{
+    P.sc.par[v] = x;
+    if (L == 0 && z == P.sink) P.sc.dem[v] = c;
+}
+
 // A BFS level bottom-up (direction-optimising BFS): every unlabelled vertex v
 // looks through its own row for a neighbour u of the current level with a
 // residual edge towards it -- c_f(v, u) > 0, v's own slot, for the push
@@ -1439,6 +1510,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
     // warp walks a very long row alone.
     constexpr int kA = 4;
     const int cap = P.sc.bdefer != nullptr ? MF_BU_SCAN : 0x7fffffff;
+    const bool near = sh.d.near != 0;
     long long slots = 0, unl = 0;
     if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_HSCAN_BFS, n);    // every vertex's height is read
     for (long long base = (long long)vb() * blockDim.x + threadIdx.x - lane; base < n; base += gs) {
@@ -1462,7 +1534,11 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
                 z[r] = in ? ldg_cg(P.g.dst + x) : 0;
             }
 #pragma unroll
-            for (int r = 0; r < kA; ++r) take[0] |= c[r] > 0 && ldg_cg(P.h + z[r]) == L;
+            for (int r = 0; r < kA; ++r) {
+                const bool hitr = c[r] > 0 && ldg_cg(P.h + z[r]) == L;
+                take[0] |= hitr;
+                if (near && hitr) note_parent(P, v, r0 + r, z[r], c[r], L);
+            }
             slots += d < kA ? d : kA;
         }
         // the warp-cooperative scan of the rows still open
@@ -1479,7 +1555,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
         const unsigned pend = __ballot_sync(0xffffffffu, rem > 0);
         unsigned hit = 0;
         for (int kb = 0; kb < T && (pend & ~hit) != 0; kb += 32 * kA) {
-            int c[kA], z[kA], ow[kA];
+            int c[kA], z[kA], ow[kA], xs[kA];
 #pragma unroll
             for (int r = 0; r < kA; ++r) {
                 const int k = kb + r * 32 + lane;
@@ -1494,6 +1570,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
                 const int eb = __shfl_sync(0xffffffffu, excl, owner);
                 const bool live = k < T && !((hit >> owner) & 1u);
                 const int x = rb + kA + (k - eb);
+                xs[r] = x;
                 ow[r] = owner;
                 c[r] = live ? (pull ? ldg_cg(P.g.pcap + x) - ldg_cg(P.cf + x) : ldg_cg(P.cf + x)) : 0;
                 z[r] = live ? ldg_cg(P.g.dst + x) : 0;
@@ -1502,7 +1579,10 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
             unsigned mine = 0;
 #pragma unroll
             for (int r = 0; r < kA; ++r)
-                if (c[r] > 0 && ldg_cg(P.h + z[r]) == L) mine |= 1u << ow[r];
+                if (c[r] > 0 && ldg_cg(P.h + z[r]) == L) {
+                    mine |= 1u << ow[r];
+                    if (near) note_parent(P, (int)base + ow[r], xs[r], z[r], c[r], L);
+                }
             hit |= __reduce_or_sync(0xffffffffu, mine);
         }
         if ((hit >> lane) & 1u) take[0] = true;
@@ -1548,6 +1628,7 @@ __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
     const bool with_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
     const int lane = threadIdx.x & 31;
     const int cnt = sh.d.defer_n;
+    const bool near = sh.d.near != 0;
     constexpr int kR = MF_BU_CHUNK / 32;
     long long slots = 0;
     const int nwarps = vn() * (int)(blockDim.x >> 5);
@@ -1573,7 +1654,11 @@ __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
             z[r] = ok ? ldg_cg(P.g.dst + x) : 0;
         }
 #pragma unroll
-        for (int r = 0; r < kR; ++r) hit |= c[r] > 0 && ldg_cg(P.h + z[r]) == L;
+        for (int r = 0; r < kR; ++r) {
+            const bool hitr = c[r] > 0 && ldg_cg(P.h + z[r]) == L;
+            hit |= hitr;
+            if (near && hitr) note_parent(P, v, it.y + r * 32 + lane, z[r], c[r], L);
+        }
         if (lane == 0) slots += len;
         bool won[1] = {false};
         int zv[1] = {v}, dv[1] = {d};
@@ -2553,6 +2638,109 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
 }
 
 // ---------------------------------------------------------------------------
+// Near iterations: the excess walks down the BFS forest
+// ---------------------------------------------------------------------------
+
+// Take up to a from the residual of slot y; returns what was there to take.
+// One subtraction, and what was not there is given back: other walkers see less
+// than there is meanwhile, never more.  Large residuals go by compare and swap,
+// because the overdraft of all walkers at once has to stay within int32 (at
+// most 2^18 threads times MF_NEAR_SUB = 2^13).
+__device__ __forceinline__ int draw(int *cf, long long a)
+{
+    int c = ldg_cg(cf);
+    if (c <= 0) return 0;
+    if (c <= MF_NEAR_SUB) {
+        const int g = a < c ? (int)a : c;
+        const int old = atomicSub(cf, g);
+        const int got = old >= g ? g : (old > 0 ? old : 0);
+        if (got < g) atomicAdd(cf, g - got);
+        return got;
+    }
+    for (;;) {
+        const int g = a < c ? (int)a : c;
+        const int old = atomicCAS(cf, c, c - g);
+        if (old == c) return g;
+        c = old;
+        if (c <= 0) return 0;
+    }
+}
+
+// One thread per active vertex.  It climbs the BFS forest to its root -- a
+// deficient vertex, or the neighbour through which its tree enters the sink --
+// reserves there what the root can still take, and carries that much down,
+// parent by parent; where an edge holds less, the rest stays as that vertex's
+// excess.  Heights do not change meanwhile, every step goes from height k to
+// k - 1 along residual capacity, so these are pushes Alg. 2 could make.
+//
+// What bounds it is one chain of dependent accesses per step (parent slot, its
+// head and reverse, the residual's atomic), a few steps long, with every
+// active vertex under way at once.  A discharge round over the same vertices
+// scans their whole rows: on R-MAT 20 with 10 K updates two rounds read some
+// 5 M slots of hub rows and took 120-190 us, the walks take about 10 us.
+__device__ __noinline__ void phase_walk(const MfParams &P, Sh &sh)
+{
+    const int sel = sh.d.wl_sel;
+    DisCtx dc;
+    dc.nsel = sel ^ 1;
+    dc.qstamp = sh.d.qstamp;
+    dc.fstamp = sh.d.fstamp;
+    dc.cs = sh.cs;
+    dc.fix0 = dc.fix1 = 0;
+    dc.queue = !sh.d.cut;      // discharge rounds may follow a complete relabel
+    int n0 = sh.d.wl_n[0], n1 = n0 + sh.d.wl_n[1], n2 = n1 + sh.d.wl_n[2], total = n2 + sh.d.wl_n[3];
+    long long pushes = 0;
+    for (long long i = spread_thread(); i < total; i += (long long)vn() * blockDim.x) {
+        const int k = (int)i;
+        const int u = __ldcg(k < n0 ? P.sc.wl[sel][0] + k
+                                    : (k < n1 ? P.sc.wl[sel][1] + (k - n0)
+                                              : (k < n2 ? P.sc.wl[sel][2] + (k - n1) : P.sc.wl[sel][3] + (k - n2))));
+        const long long eu = ldg_cg(P.e + u);
+        if (eu <= 0) continue;
+        int root = u;
+        for (;;) {
+            const int w = ldg_cg(P.g.dst + ldg_cg(P.sc.par + root));
+            if (w == P.sink) break;
+            const bool top = ldg_cg(P.h + w) == 0;
+            root = w;
+            if (top) break;
+        }
+        long long a = ldg_cg(P.sc.dem + root);
+        a = a < eu ? a : eu;
+        if (a > 0) {
+            const long long old = atomic_add_ll(P.sc.dem + root, -a);
+            const long long got = old >= a ? a : (old > 0 ? old : 0);
+            if (got < a) atomic_add_ll(P.sc.dem + root, a - got);
+            a = got;
+        }
+        if (a <= 0) {
+            if (dc.queue) enqueue_active(P, u, dc);
+            continue;
+        }
+        atomic_add_ll(P.e + u, -a);
+        if (dc.queue && eu > a) enqueue_active(P, u, dc);
+        int v = u;
+        do {
+            const int y = ldg_cg(P.sc.par + v);
+            const int w = ldg_cg(P.g.dst + y), r = ldg_cg(P.g.rev + y);
+            const int g = draw(P.cf + y, a);
+            if (g > 0) {
+                atomicAdd(P.cf + r, g);
+                ++pushes;
+            }
+            if (g < a) {
+                atomic_add_ll(P.e + v, a - g);
+                if (dc.queue) enqueue_active(P, v, dc);
+            }
+            a = g;
+            v = w;
+        } while (a > 0 && v != P.sink && ldg_cg(P.h + v) > 0);
+        if (a > 0) add_excess(P, sh, v, a);
+    }
+    add_stat(sh, ST_PUSHES, pushes);
+}
+
+// ---------------------------------------------------------------------------
 // Remove invalid edges (Alg. 3)
 // ---------------------------------------------------------------------------
 
@@ -2678,13 +2866,14 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
     if (threadIdx.x == 0) {
         MfCtrl *c = P.ctrl;
         sh.sink_e = sh.src_e = 0;
-        sh.lab = 0;
+        sh.lab = sh.exc = sh.dem = 0;
         sh.phase = 0;
         sh.cs = &c->set[0];
         sh.d = MfDesc{};
         sh.hs = MfState{};
         sh.d.qstamp = __ldcg(&c->d.qstamp);
         sh.d.fstamp = __ldcg(&c->d.fstamp);
+        sh.d.near = near_allowed(P);
         sh.hs.t_phase = gtimer();
     }
     if (vb() == 0) {
@@ -2797,7 +2986,8 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         if (sh.d.status != MF_ST_RUNNING) break;
         // discharge rounds, then remove-invalid-edges
         do {
-            if (P.pull) phase_discharge<true>(P, sh);
+            if (sh.d.near && sh.d.round == 0) phase_walk(P, sh);
+            else if (P.pull) phase_discharge<true>(P, sh);
             else phase_discharge<false>(P, sh);
             if (!grid_sync(P, H_DIS, sh)) return false;
         } while (sh.d.dis_more);
