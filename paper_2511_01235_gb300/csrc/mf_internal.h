@@ -37,12 +37,20 @@
 #define MF_ROW_ALIGN 4        // rows start on multiples of this many slots (16-byte loads of slot fields)
 #define MF_BU_SCAN 256        // bottom-up BFS: slots of a row its warp scans before deferring the rest
 #define MF_BU_CHUNK 256       // bottom-up BFS: slots per deferred work item (one warp, 8 per lane)
-#define MF_TAIL_SLOTS 2048    // BFS default: frontiers up to this many slots run in one CTA
 #define MF_NEAR_SINK 8        // near iterations: the sink's row holds at most 1/8 of the vertices
-#define MF_NEAR_SLOTS 65536   // near iterations: graphs of at least this many reserved slots
+#define MF_LARGE_SLOTS 65536  // near iterations and short rounds: graphs of at least this many reserved slots
 #define MF_NEAR_STEP 3        // near iterations: a cut that settled less than half asks for 2^3 times the excess next
 #define MF_NEAR_SUB 8192      // walks: residuals up to this are taken with one atomic subtraction
-#define MF_TAIL_RUN 256       // BFS: levels CTA 0 runs alone before the grid meets once (bounds the others' wait)
+#define MF_Q_BFS 8192         // on-chip queue of a CTA: labelled vertices of one BFS phase,
+#define MF_Q_LONG 2048        // ... those with long rows,
+#define MF_Q_WL 4096          // ... worklist entries of one phase (vertex; bin and place)
+#define MF_Q_INTS (MF_Q_BFS + MF_Q_LONG + 2 * MF_Q_WL)
+#define MF_SOLO_CAP 4096      // queue entries of a run of small phases that the first CTA does alone
+#define MF_SOLO_INTS (6 * MF_SOLO_CAP)   // its shared memory: two queues of vertex, row start, row length
+#define MF_SOLO_LEVEL 256     // BFS levels of at most this many vertices ...
+#define MF_SOLO_SLOTS 2048    // ... and slots run alone
+#define MF_SOLO_ACTIVE 256    // discharge rounds of at most this many vertices run alone
+#define MF_SHORT_ROW 512      // rounds of one cycle per vertex: the longest row
 
 // Solve-kernel status (ctrl->status)
 #define MF_ST_RUNNING 0
@@ -84,7 +92,6 @@ struct alignas(128) MfLine {
 enum MfLineId {
     L_BFS = 0,            // regular frontier entries appended in this phase
     L_HUB,                // frontier work items
-    L_LONG,               // long-row vertices (blong)
     L_DEFER,              // bottom-up chunks deferred to the level's second pass
     L_HEAD0,              // dynamic work heads
     L_HEAD1,
@@ -115,15 +122,15 @@ struct MfDesc {
     int level;
     int lvl_lo, lvl_hi;           // this level's regular frontier in border[]
     int hub_lo, hub_hi;           // ... work items in bitem[]
-    int long_lo, long_hi;         // ... long-row vertices labelled by the last level (blong)
-    int app_bfs, app_hub, app_long;   // where this phase's entries of the three lists start
+    int app_bfs, app_hub;         // where this phase's entries of the two lists start
     int wl_app[MF_NBIN];          // where this phase's worklist entries start
     int bfs_done;
     int bu_mode;                  // the coming BFS level runs bottom-up
     int bu_split;                 // the bottom-up level just scanned deferred long rows: their pass follows
     int defer_n;                  // work items of that pass
-    int bfs_cta_mode;             // the coming top-down level is small: CTA 0 runs it (and the next small ones) alone
-    int expand;                   // the coming top-down level first splits long rows into work items
+    int bfs_solo;                 // the coming top-down level is small: the first CTA runs it, and the next small ones, alone
+    int dis_short;                // the coming discharge round has short rows only: one cycle per vertex
+    int dis_solo;                 // ... and few of them: the first CTA runs it, and the next small ones, alone
     int need_total;               // the coming BFS roots pass sums the used slots (first BFS of a launch)
     int wl_sel;                   // which worklist buffer the current round reads
     int wl_n[MF_NBIN];
@@ -217,8 +224,6 @@ struct MfGraph {
 struct MfScratch {
     int32_t *border;          // [n] BFS order (level segments)
     int2 *bitem;              // [n + slot_cap / MF_BFS_CHUNK + 64] frontier work items (first slot, length)
-    int32_t *blong;           // [n] vertices with rows longer than bfs_hub labelled by the BFS, split into
-                              // work items only if a top-down level follows; nullptr: items at once
     int2 *bdefer;             // [n + slot_cap / MF_BFS_CHUNK + 64] bottom-up deferred chunks (vertex, first slot);
                               // nullptr: bottom-up threads scan whole rows themselves
     int32_t *wl[2][MF_NBIN];  // [n] worklists (two buffers for discharge rounds) per row kind: thread, warp,
@@ -273,7 +278,7 @@ struct MfParams {
     int32_t requeue;          // discharge rounds: a vertex still active after its cycles joins the next round
     int32_t cycle_div;        // > 0: a row of d slots gets max(kernel_cycles, d / cycle_div) cycles
     int32_t tail_slots;       // BFS: a top-down level whose frontier holds at most this many slots (and
-                              // vertices) runs in CTA 0 alone, without grid barriers; 0: never
+                              // vertices) runs in CTA 0 alone, without grid barriers; 0: MF_SOLO_SLOTS
     int32_t stage_slots;      // dynamic shared memory of the launch in ints: the discharge's on-chip row snapshot
                               // (a CTA keeps rows up to this many slots; 0: none)
     long long max_iters;

@@ -179,6 +179,12 @@ struct Sh {
     unsigned phase;                   // barriers passed in this launch
     MfSet *cs;                        // the counter set of the running phase
     int tr_hook, tr_info;             // of the last barrier, for the trace
+    // a run of small phases in the first CTA: entries of the next queue, of the
+    // next lists per bin, work items
+    int so_cnt, so_wl[MF_NBIN], so_hub, so_go;
+    // on-chip queue of a phase (place_labelled, place_active): entries taken, per kind
+    int q_bfs, q_long, q_wn, q_wl[MF_NBIN];
+    int q_base[MF_NBIN + 1];
     int4 cnt[MF_LINES];               // the counters of the phase that just ended
     MfDesc d;
     MfState hs;
@@ -198,8 +204,8 @@ enum Hook {
     H_DIS,
     H_FINAL,
     H_BU_SPLIT,
-    H_BFS_JOIN,
-    H_EXPANDED,
+    H_JOIN,               // the first CTA has run small phases alone: the others take its state
+    H_EXPANDED,           // unused (long rows are split into work items as they are queued); keeps the trace ids
 };
 
 __device__ __forceinline__ void add_stat(Sh &sh, MfStat i, long long v)
@@ -211,6 +217,27 @@ __device__ __forceinline__ int cnt32(const Sh &sh, int line) { return sh.cnt[lin
 __device__ __forceinline__ unsigned long long cnt64(const Sh &sh, int line)
 {
     return (unsigned long long)(unsigned)sh.cnt[line].x | ((unsigned long long)(unsigned)sh.cnt[line].y << 32);
+}
+
+// A top-down level of cnt vertices with fr slots, none of them long, that the
+// first CTA runs alone (solo_bfs).
+__device__ __forceinline__ bool solo_level(const MfParams &P, long long cnt, long long fr)
+{
+    return cnt <= MF_SOLO_LEVEL && fr <= (P.tail_slots > 0 ? P.tail_slots : MF_SOLO_SLOTS) && !P.pull &&
+           P.stage_slots >= MF_SOLO_INTS;
+}
+
+// How the coming discharge round over the worklists in d runs.  Short: a push
+// with the default schedule over rows of at most MF_SHORT_ROW slots gets one
+// cycle per vertex (phase_discharge_short), and a few vertices are left to the
+// first CTA (solo_discharge).
+__device__ __forceinline__ void pick_round(const MfParams &P, MfDesc &d)
+{
+    d.dis_short = P.rounds == 0 && !P.pull && !P.fix_steep && P.data_driven && P.requeue &&
+                          P.stage_slots >= MF_SOLO_INTS && P.hub_deg <= MF_SHORT_ROW &&
+                          P.g.slot_cap >= MF_LARGE_SLOTS && d.wl_n[2] + d.wl_n[3] == 0
+                      ? 1 : 0;
+    d.dis_solo = d.dis_short && d.wl_n[0] + d.wl_n[1] <= MF_SOLO_ACTIVE ? 1 : 0;
 }
 
 // The termination test of the loop (Alg. 1 / Alg. 5: stop when no active
@@ -225,6 +252,8 @@ __device__ __forceinline__ void decide_iteration(const MfParams &P, Sh &sh, int 
     ++d.fstamp;
     st.t_dis0 = st.t_now;
     for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = d.wl_app[b];
+    pick_round(P, d);
+    if (d.near) d.dis_short = d.dis_solo = 0;        // a near iteration starts with the walks
     if (vb() == 0 && st.iters < MF_ACTIVE_HIST) P.ctrl->active_hist[st.iters] = active;
     if (st.iters == 0) st.active_first = active;
     st.active_total += active;
@@ -245,7 +274,7 @@ __device__ __forceinline__ void decide_iteration(const MfParams &P, Sh &sh, int 
 __device__ __forceinline__ int near_allowed(const MfParams &P)
 {
     if (P.sc.par == nullptr || !(P.mode & MF_M_SOLVE) || (P.mode & MF_M_NO_DEFICIT_ROOTS) || P.pull ||
-        P.side_root >= 0 || P.rounds != 0 || P.fix_steep || !P.data_driven || P.g.slot_cap < MF_NEAR_SLOTS)
+        P.side_root >= 0 || P.rounds != 0 || P.fix_steep || !P.data_driven || P.g.slot_cap < MF_LARGE_SLOTS)
         return 0;
     return (long long)ldg_cg(P.g.deg + P.sink) * MF_NEAR_SINK <= (long long)P.g.n ? 1 : 0;
 }
@@ -256,8 +285,8 @@ __device__ __forceinline__ void begin_iteration(Sh &sh)
     MfDesc &d = sh.d;
     sh.hs.t_bfs0 = sh.hs.t_now;
     sh.hs.vis_slots = sh.hs.lvl_slots = sh.hs.lvl_cnt = sh.hs.sup = 0;
-    d.lvl_lo = d.lvl_hi = d.hub_lo = d.hub_hi = d.long_lo = d.long_hi = 0;
-    d.app_bfs = d.app_hub = d.app_long = 0;
+    d.lvl_lo = d.lvl_hi = d.hub_lo = d.hub_hi = 0;
+    d.app_bfs = d.app_hub = 0;
     for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] = 0;
     // the used-slot total only changes with insertions, which come before the
     // first BFS: later iterations keep it
@@ -281,12 +310,11 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
     if (st.err == 0) st.err = sh.cnt[L_MISC].w;
     int tinfo = 0;
     const bool want_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
-    if (hook == H_BU_SPLIT || hook == H_BFS_START || hook == H_BFS_NEXT || hook == H_EXPANDED) {
+    if (hook == H_BU_SPLIT || hook == H_BFS_START || hook == H_BFS_NEXT) {
         // the lists grew by what the phase appended
         st.ns_bfs += dt;
         d.app_bfs += cnt32(sh, L_BFS);
         d.app_hub += cnt32(sh, L_HUB);
-        d.app_long += cnt32(sh, L_LONG);
         for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] += cnt32(sh, L_WL + b);
         const unsigned long long lab = cnt64(sh, L_LAB);
         st.lvl_slots += (long long)(lab & 0xffffffffull);
@@ -335,11 +363,9 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         const int items = d.hub_hi - d.hub_lo;
         d.lvl_lo = d.lvl_hi;
         d.hub_lo = d.hub_hi;
-        d.long_lo = d.long_hi;
         d.lvl_hi = d.app_bfs;
         d.hub_hi = d.app_hub;
-        d.long_hi = d.app_long;
-        const bool done = d.lvl_lo == d.lvl_hi && d.hub_lo == d.hub_hi && d.long_lo == d.long_hi;
+        const bool done = d.lvl_lo == d.lvl_hi && d.hub_lo == d.hub_hi;
         if (!first && !done) ++st.bfs_levels;
         d.level = first ? 0 : d.level + 1;
         d.bfs_done = done;
@@ -357,13 +383,7 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         else if (bu && cnt * P.bu_beta < (long long)P.g.n) bu = 0;
         d.bu_mode = bu;
         d.bu_split = 0;
-        // a top-down level after one that labelled long rows first splits them
-        // into work items (a bottom-up level never reads them)
-        d.expand = (!done && !bu && d.long_hi > d.long_lo) ? 1 : 0;
-        // a small top-down frontier is expanded by CTA 0 alone: a level of a
-        // few hundred slots costs a grid barrier otherwise
-        d.bfs_cta_mode =
-            (!done && !bu && !d.expand && P.tail_slots > 0 && fr <= P.tail_slots && cnt <= P.tail_slots) ? 1 : 0;
+        d.bfs_solo = !done && !bu && d.hub_hi == d.hub_lo && solo_level(P, cnt, fr) ? 1 : 0;
         // near iterations: the levels so far hold as much excess as the roots can take
         d.cut = d.near && !done && st.sup > 0 && (st.sup >> st.cut_shift) >= st.dem ? 1 : 0;
         st.cut_prev = d.cut;
@@ -408,6 +428,7 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
             for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = cnt32(sh, L_AUX + b);
             ++d.round;
             ++d.qstamp;
+            pick_round(P, d);
         } else if (!P.fix_steep) {
             // without Alg. 3 the next iteration's BFS follows at once: this
             // barrier opens it
@@ -415,13 +436,7 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         }
         break;
     }
-    case H_BFS_JOIN:
-        st.ns_bfs += dt;
-        break;
-    case H_EXPANDED:
-        // the long rows' work items are written: the level takes them with the rest
-        d.hub_hi = d.app_hub;
-        d.expand = 0;
+    case H_JOIN:
         break;
     default:
         break;
@@ -430,6 +445,20 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
     sh.tr_info = tinfo;
     ++st.trace_n;
     if (st.err != 0) d.status = MF_ST_ERROR;
+}
+
+// advance() for the first CTA alone (one thread; sh.cnt filled in), with its entry in the timeline.
+__device__ __noinline__ void solo_advance(const MfParams &P, int hook, Sh &sh)
+{
+    advance(P, hook, sh, gtimer());
+    const int i = sh.hs.trace_n - 1;
+    if (i >= MF_TRACE) return;
+    MfCtrl *c = P.ctrl;
+    c->trace_hook[i] = sh.tr_hook;
+    c->trace_t[i] = sh.hs.t_phase;
+    c->trace_slots[i] = sh.stat[ST_SLOTS_BFS] + sh.stat[ST_SLOTS_DIS] + sh.stat[ST_SLOTS_FIX];
+    c->trace_info[i] = sh.tr_info;
+    c->trace_fin_max[i] = c->trace_fin_mean[i] = 0;
 }
 
 // One entry of the hook timeline, written by the last warp of the first CTA
@@ -502,6 +531,9 @@ __device__ __forceinline__ void arrive(const MfParams &P, Sh &sh)
     } else if (lane == 4) {
         if (sh.exc) atomicAdd((unsigned long long *)sh.cs->l[L_EXC].w, sh.exc);
         sh.exc = 0;
+    } else if (lane == 6) {
+        sh.q_bfs = sh.q_long = sh.q_wn = 0;
+        for (int b = 0; b < MF_NBIN; ++b) sh.q_wl[b] = 0;
     } else if (lane == 5) {
         if (sh.dem) atomicAdd((unsigned long long *)sh.cs->l[L_DEM].w, sh.dem);
         sh.dem = 0;
@@ -547,7 +579,7 @@ __device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh)
     const unsigned k = sh.phase;
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
-        if (hook == H_BFS_JOIN && vb() == 0) {
+        if (hook == H_JOIN && vb() == 0) {
             words_out((int *)&c->jd, (const int *)&sh.d, (int)(sizeof(MfDesc) / 4));
             words_out((int *)&c->js, (const int *)&sh.hs, (int)(sizeof(MfState) / 4));
         }
@@ -561,7 +593,7 @@ __device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh)
                 sh.cnt[lane] = __ldcg(reinterpret_cast<const int4 *>(&sh.cs->l[lane]));
                 if (vb() == 0) __stcg(reinterpret_cast<int4 *>(&c->set[(k + 2u) % 3u].l[lane]), make_int4(0, 0, 0, 0));
             }
-            if (hook == H_BFS_JOIN && vb() != 0) {
+            if (hook == H_JOIN && vb() != 0) {
                 words_in((int *)&sh.d, (const int *)&c->jd, (int)(sizeof(MfDesc) / 4));
                 words_in((int *)&sh.hs, (const int *)&c->js, (int)(sizeof(MfState) / 4));
             }
@@ -577,40 +609,6 @@ __device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh)
     __syncthreads();
     if (vb() == 0 && (threadIdx.x >> 5) == (blockDim.x >> 5) - 1 && sh.ok) write_trace(P, sh, k);
     return sh.ok != 0;
-}
-
-// The same step inside a run of small levels that the first CTA does alone
-// (nobody else touches the counter set meanwhile).
-__device__ __noinline__ void solo_step(const MfParams &P, int hook, Sh &sh)
-{
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        if (lane < MF_LINES) {
-            int4 *p = reinterpret_cast<int4 *>(&sh.cs->l[lane]);
-            sh.cnt[lane] = __ldcg(p);
-            __stcg(p, make_int4(0, 0, 0, 0));
-        }
-        __syncwarp();
-        if (lane == 0) {
-            sh.cnt[L_LAB] = make_int4((int)(unsigned)sh.lab, (int)(sh.lab >> 32), 0, 0);
-            sh.stat[ST_LAB_BFS] += (long long)(sh.lab >> 32);
-            sh.lab = 0;
-            sh.cnt[L_EXC] = make_int4((int)(unsigned)sh.exc, (int)(sh.exc >> 32), 0, 0);
-            sh.exc = 0;
-            advance(P, hook, sh, gtimer());
-            const int i = sh.hs.trace_n - 1;
-            if (i < MF_TRACE) {
-                MfCtrl *c = P.ctrl;
-                c->trace_hook[i] = sh.tr_hook;
-                c->trace_t[i] = sh.hs.t_phase;
-                c->trace_slots[i] = sh.stat[ST_SLOTS_BFS] + sh.stat[ST_SLOTS_DIS] + sh.stat[ST_SLOTS_FIX];
-                c->trace_info[i] = sh.tr_info;
-                c->trace_fin_max[i] = c->trace_fin_mean[i] = 0;
-            }
-        }
-    }
-    __syncthreads();
 }
 
 // The end of a launch: the counters go to the control block, every CTA arrives
@@ -1101,163 +1099,112 @@ __device__ __noinline__ void phase_resaturate(const MfParams &P, Sh &sh)
 // Backward BFS (Alg. 4 / Alg. 6)
 // ---------------------------------------------------------------------------
 
-template <int R>
-__device__ __forceinline__ void write_items(const MfParams &P, const int (&nc)[R], const int (&x0)[R],
-                                            const int (&d)[R], unsigned ibase, int cexcl, int ctot);
-
-// Labelled vertices enter the next frontier either as one entry of the
-// regular list (rows of at most bfs_hub slots, expanded warp-cooperatively)
-// or, for longer rows, as ceil(deg / MF_BFS_CHUNK) work items (first slot,
-// length) that any warp can take: no row is ever walked by one warp alone.
-// With with_wl, a labelled vertex that has excess (and is neither the sink
-// nor the source) also joins the worklist of the coming discharge (Sec. 5.2.1
-// O1): it is active exactly when this BFS labels it, so no separate pass over
-// all vertices is needed.
-//
-// Each lane brings R candidates; the six lists (regular frontier, four
-// worklist bins, work items) are reserved with one warp scan and one round of
-// atomics issued together, so a warp pays one append round trip per R slots.
-// Called by the whole warp.
-template <int R>
-__device__ __forceinline__ void frontier_push(const MfParams &P, Sh &sh, const bool (&take)[R], const int (&z)[R],
-                                              const int (&d)[R], const long long (&ev)[R], bool with_wl, int sel,
-                                              bool eager = false)
+// The work items of vertex z (d slots from r0), by one thread: where a queue has no room.
+__device__ __forceinline__ void put_items(const MfParams &P, int r0, int d, unsigned at)
 {
-    MfSet *cs = sh.cs;
-    const int lane = threadIdx.x & 31;
-    // long rows go to the long-row list, to be split into work items only if a
-    // top-down level follows (a bottom-up level never reads them); `eager`
-    // (the roots: the first level is top-down) or no list: items at once
-    const bool lazy = !eager && P.sc.blong != nullptr;
-    // per-lane counts packed 8 bits each: [0] regular, [1..MF_NBIN] worklist
-    // bins; and this lane's long rows (lazy) or their work items
-    unsigned long long packed = 0;
-    int nch = 0;
-    long long lab_slots = 0, exc = 0;
-    int lab_n = 0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        if (!take[r]) continue;
-        lab_slots += d[r];
-        ++lab_n;
-        if (d[r] > P.bfs_hub) nch += lazy ? 1 : (d[r] + MF_BFS_CHUNK - 1) / MF_BFS_CHUNK;
-        else packed += 1ull;
-        if (with_wl && ev[r] > 0) {
-            packed += 1ull << (8 * (row_bin(P, d[r]) + 1));
-            exc += ev[r];
-        }
-    }
-    if (exc && sh.d.near) atomicAdd(&sh.exc, (unsigned long long)exc);
-    unsigned long long incl = packed;
-    int cincl = nch;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
-        const int yc = __shfl_up_sync(0xffffffffu, cincl, o);
-        if (lane >= o) {
-            incl += y;
-            cincl += yc;
-        }
-    }
-    const unsigned long long total = __shfl_sync(0xffffffffu, incl, 31);
-    const int ctot = __shfl_sync(0xffffffffu, cincl, 31);
-    const unsigned long long excl = incl - packed;
-    // slots and number of the vertices labelled (the BFS direction test reads them)
-    lab_slots = warp_sum_ll(lab_slots);
-    const long long lab_cnt = warp_sum_ll((long long)lab_n);
-    if (lane == 0 && lab_cnt)        // per CTA in shared memory, added to the counter set at the barrier
-        atomicAdd(&sh.lab, ((unsigned long long)lab_cnt << 32) | (unsigned long long)lab_slots);
-    if (total == 0 && ctot == 0) return;
-    static_assert(MF_NBIN == 4, "one reservation per worklist bin below");
-    // One lane reserves room in every list the warp appends to.  The
-    // reservations are independent, so they are issued back to back and the
-    // warp waits for one round trip, not one per list.
-    const unsigned k0 = (unsigned)(total & 0xffull), k1 = (unsigned)((total >> 8) & 0xffull),
-                   k2 = (unsigned)((total >> 16) & 0xffull), k3 = (unsigned)((total >> 24) & 0xffull),
-                   k4 = (unsigned)((total >> 32) & 0xffull);
-    unsigned b0 = 0, b1 = 0, b2 = 0, b3 = 0, b4 = 0, bi = 0;
-    if (lane == 0) {
-        if (k0) b0 = sh.d.app_bfs + atomicAdd(&cs->l[L_BFS].w[0], k0);
-        if (k1) b1 = sh.d.wl_app[0] + atomicAdd(&cs->l[L_WL].w[0], k1);
-        if (k2) b2 = sh.d.wl_app[1] + atomicAdd(&cs->l[L_WL + 1].w[0], k2);
-        if (k3) b3 = sh.d.wl_app[2] + atomicAdd(&cs->l[L_WL + 2].w[0], k3);
-        if (k4) b4 = sh.d.wl_app[3] + atomicAdd(&cs->l[L_WL + 3].w[0], k4);
-        if (ctot)
-            bi = (lazy ? sh.d.app_long : sh.d.app_hub) + atomicAdd(&cs->l[lazy ? L_LONG : L_HUB].w[0], (unsigned)ctot);
-    }
-    unsigned pos[MF_NBIN + 1];
-    pos[0] = __shfl_sync(0xffffffffu, b0, 0) + (unsigned)(excl & 0xffull);
-    pos[1] = __shfl_sync(0xffffffffu, b1, 0) + (unsigned)((excl >> 8) & 0xffull);
-    pos[2] = __shfl_sync(0xffffffffu, b2, 0) + (unsigned)((excl >> 16) & 0xffull);
-    pos[3] = __shfl_sync(0xffffffffu, b3, 0) + (unsigned)((excl >> 24) & 0xffull);
-    pos[4] = __shfl_sync(0xffffffffu, b4, 0) + (unsigned)((excl >> 32) & 0xffull);
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        if (!take[r]) continue;
-        if (d[r] <= P.bfs_hub) P.sc.border[pos[0]++] = z[r];
-        if (with_wl && ev[r] > 0) {
-            const int bin = row_bin(P, d[r]);
-            P.sc.wl[sel][bin][pos[bin + 1]++] = z[r];
-        }
-    }
-    if (ctot == 0) return;
-    const unsigned ibase = __shfl_sync(0xffffffffu, bi, 0);
-    const int cexcl = cincl - nch;
-    if (lazy) {
-        unsigned at = ibase + (unsigned)cexcl;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (take[r] && d[r] > P.bfs_hub) P.sc.blong[at++] = z[r];
-        return;
-    }
-    int x0[R], nc[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const bool big = take[r] && d[r] > P.bfs_hub;
-        nc[r] = big ? (d[r] + MF_BFS_CHUNK - 1) / MF_BFS_CHUNK : 0;
-        x0[r] = big ? P.g.off[z[r]] : 0;
-    }
-    write_items<R>(P, nc, x0, d, ibase, cexcl, ctot);
+    for (int j = 0; j < d; j += MF_BFS_CHUNK)
+        P.sc.bitem[at++] = make_int2(r0 + j, d - j < MF_BFS_CHUNK ? d - j : MF_BFS_CHUNK);
 }
 
-// Long rows: ceil(deg / MF_BFS_CHUNK) work items each (first slot, length),
-// which any warp can take.  A hub of 10^5 slots has hundreds of items, so the
-// warp writes all its rows' items together, 32 at a time (each lane finds the
-// row that owns its item), at ibase + [0, ctot); lane L's rows own the items
-// from cexcl (the exclusive prefix of nc over the lanes).  Called by the whole warp.
-template <int R>
-__device__ __forceinline__ void write_items(const MfParams &P, const int (&nc)[R], const int (&x0)[R],
-                                            const int (&d)[R], unsigned ibase, int cexcl, int ctot)
+__device__ __forceinline__ int chunks_of(int d) { return (d + MF_BFS_CHUNK - 1) / MF_BFS_CHUNK; }
+
+// z (a row of d slots) joins a worklist: the BFS's own (line L_WL, the lists
+// wl[sel]) or the next round's (L_AUX, wl[sel ^ 1]).  The entry waits in the
+// CTA's queue until the phase ends, so that each CTA, not each warp, takes its
+// room in the shared lists with one atomic per list: returning atomics on one
+// word are served one after another, about 2.4 clocks each, and a level whose
+// 4864 warps append alone spends some 5 us on that.
+__device__ __forceinline__ void place_active(const MfParams &P, Sh &sh, int z, int d, int line, int sel,
+                                             const int *app)
 {
-    const int lane = threadIdx.x & 31;
-    for (int i0 = 0; i0 < ctot; i0 += 32) {         // the same trip count in every lane
-        const int i = i0 + lane;
-        int owner = 0;
-#pragma unroll
-        for (int st = 16; st >= 1; st >>= 1) {
-            const int cand = owner + st;
-            const int ec = __shfl_sync(0xffffffffu, cexcl, cand & 31);
-            if (cand < 32 && ec <= i) owner = cand;
-        }
-        int j = i - __shfl_sync(0xffffffffu, cexcl, owner);
-        int ix = 0, idg = 0, ic = -1;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int ncr = __shfl_sync(0xffffffffu, nc[r], owner);
-            const int xr = __shfl_sync(0xffffffffu, x0[r], owner);
-            const int dr = __shfl_sync(0xffffffffu, d[r], owner);
-            if (ic < 0 && j >= 0 && j < ncr) {
-                ic = j;
-                ix = xr;
-                idg = dr;
-            }
-            j -= ncr;
-        }
-        if (i < ctot) {
-            const int len = idg - ic * MF_BFS_CHUNK;
-            P.sc.bitem[ibase + (unsigned)i] = make_int2(ix + ic * MF_BFS_CHUNK, len < MF_BFS_CHUNK ? len : MF_BFS_CHUNK);
+    const int bin = row_bin(P, d);
+    if (P.stage_slots >= MF_Q_INTS) {
+        const int j = atomicAdd(&sh.q_wn, 1);
+        if (j < MF_Q_WL) {
+            int *q = mf_stage + MF_Q_BFS + MF_Q_LONG;
+            q[j] = z;
+            q[MF_Q_WL + j] = (bin << 28) | atomicAdd(&sh.q_wl[bin], 1);
+            return;
         }
     }
+    P.sc.wl[sel][bin][(app ? app[bin] : 0) + atomicAdd(&sh.cs->l[line + bin].w[0], 1u)] = z;
+}
+
+// A labelled vertex enters the next frontier either as one entry of the regular
+// list (rows of at most bfs_hub slots, expanded warp-cooperatively) or, for
+// longer rows, as ceil(deg / MF_BFS_CHUNK) work items (first slot, length) that
+// any warp can take: no row is ever walked by one warp alone.  One that has
+// excess (ev > 0; never the sink or the source) also joins the worklist of the
+// coming discharge (Sec. 5.2.1 O1): it is active exactly when this BFS labels
+// it, so no separate pass over all vertices is needed.  The entries wait in the
+// CTA's queue (flush_labelled).
+__device__ __forceinline__ void place_labelled(const MfParams &P, Sh &sh, int z, int d, long long ev)
+{
+    const bool room = P.stage_slots >= MF_Q_INTS;
+    if (d > P.bfs_hub) {
+        const int i = room ? atomicAdd(&sh.q_long, 1) : MF_Q_LONG;
+        if (i < MF_Q_LONG)
+            mf_stage[MF_Q_BFS + i] = z;
+        else
+            put_items(P, P.g.off[z], d, sh.d.app_hub + atomicAdd(&sh.cs->l[L_HUB].w[0], (unsigned)chunks_of(d)));
+    } else {
+        const int i = room ? atomicAdd(&sh.q_bfs, 1) : MF_Q_BFS;
+        if (i < MF_Q_BFS)
+            mf_stage[i] = z;
+        else
+            P.sc.border[sh.d.app_bfs + atomicAdd(&sh.cs->l[L_BFS].w[0], 1u)] = z;
+    }
+    if (ev > 0) {
+        place_active(P, sh, z, d, L_WL, sh.d.wl_sel, sh.d.wl_app);
+        if (sh.d.near) atomicAdd(&sh.exc, (unsigned long long)ev);
+    }
+}
+
+// The end of a phase: the CTA's queue goes onto the shared lists, and what its
+// threads labelled (vertices, slots) to the counters.  Long rows' work items
+// are written here by whole warps.
+__device__ __forceinline__ void flush_queue(const MfParams &P, Sh &sh, int line, int sel, const int *app, int lab,
+                                            unsigned lab_slots)
+{
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
+    __syncwarp();
+    lab = __reduce_add_sync(0xffffffffu, lab);
+    lab_slots = __reduce_add_sync(0xffffffffu, lab_slots);
+    if (lane == 0 && lab) atomicAdd(&sh.lab, ((unsigned long long)(unsigned)lab << 32) | lab_slots);
+    __syncthreads();
+    const int nb = min(sh.q_bfs, MF_Q_BFS), nl = min(sh.q_long, MF_Q_LONG), nw = min(sh.q_wn, MF_Q_WL);
+    if (nb + nw > 0) {
+        // a lane per list, so the reservations are in flight together
+        if (tid < MF_NBIN) {
+            if (sh.q_wl[tid])
+                sh.q_base[tid] = (app ? app[tid] : 0) + (int)atomicAdd(&sh.cs->l[line + tid].w[0], (unsigned)sh.q_wl[tid]);
+        } else if (tid == MF_NBIN) {
+            if (nb) sh.q_base[MF_NBIN] = sh.d.app_bfs + (int)atomicAdd(&sh.cs->l[L_BFS].w[0], (unsigned)nb);
+        }
+        __syncthreads();
+        for (int i = tid; i < nb; i += nt) P.sc.border[sh.q_base[MF_NBIN] + i] = mf_stage[i];
+        const int *q = mf_stage + MF_Q_BFS + MF_Q_LONG;
+        for (int i = tid; i < nw; i += nt) {
+            const int b = q[MF_Q_WL + i];
+            P.sc.wl[sel][b >> 28][sh.q_base[b >> 28] + (b & 0x0fffffff)] = q[i];
+        }
+    }
+    for (int i = wid; i < nl; i += nt >> 5) {
+        const int z = mf_stage[MF_Q_BFS + i];
+        const int r0 = P.g.off[z], d = ldg_cg(P.g.deg + z), nc = chunks_of(d);
+        unsigned at = 0;
+        if (lane == 0) at = sh.d.app_hub + atomicAdd(&sh.cs->l[L_HUB].w[0], (unsigned)nc);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        for (int c = lane; c < nc; c += 32) {
+            const int len = d - c * MF_BFS_CHUNK;
+            P.sc.bitem[at + c] = make_int2(r0 + c * MF_BFS_CHUNK, len < MF_BFS_CHUNK ? len : MF_BFS_CHUNK);
+        }
+    }
+}
+
+__device__ __forceinline__ void flush_labelled(const MfParams &P, Sh &sh, int lab, unsigned lab_slots)
+{
+    flush_queue(P, sh, L_WL, sh.d.wl_sel, sh.d.wl_app, lab, lab_slots);
 }
 
 __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
@@ -1268,6 +1215,8 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
     const bool need_total = sh.d.need_total != 0;
     const bool near = sh.d.near != 0;
     long long total = 0, take = 0;        // near: what the roots can take
+    int lab = 0;
+    unsigned lab_slots = 0;
     const int lane = threadIdx.x & 31;
     const long long gs = (long long)vn() * blockDim.x;
     if (near) {
@@ -1278,9 +1227,7 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
     if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_VERTS_BFS, n);     // every vertex: e read, h written
     for (long long base = (long long)vb() * blockDim.x + threadIdx.x - lane; base < n; base += gs) {
         const int v = (int)base + lane;
-        bool root[1] = {false};
-        int zv[1] = {v}, dv[1] = {0};
-        long long ev[1] = {0};
+        bool root = false;
         int dall = 0;
         if (v < n) {
             if (need_total) dall = ldg_cg(P.g.deg + v);
@@ -1288,22 +1235,27 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
             // overflowing vertices; with a side given, only that side's
             const bool side_ok = P.side_root < 0 || P.side[v] == P.side_root;
             if (pull)
-                root[0] = (v == P.source) || (v != P.sink && side_ok && ldg_cg(P.e + v) > 0);
+                root = (v == P.source) || (v != P.sink && side_ok && ldg_cg(P.e + v) > 0);
             else {
                 const long long e = (deficit_roots && v != P.source && v != P.sink && side_ok) ? ldg_cg(P.e + v) : 0;
-                root[0] = v == P.sink || e < 0;
+                root = v == P.sink || e < 0;
                 if (near && e < 0) {
                     P.sc.dem[v] = -e;
                     take -= e;
                 }
             }
-            P.h[v] = root[0] ? 0 : n;
-            if (root[0]) dv[0] = need_total ? dall : ldg_cg(P.g.deg + v);
+            P.h[v] = root ? 0 : n;
+            if (root) {
+                const int d = need_total ? dall : ldg_cg(P.g.deg + v);
+                ++lab;
+                lab_slots += (unsigned)d;
+                place_labelled(P, sh, v, d, 0);
+            }
         }
         total += dall;
-        if (__any_sync(0xffffffffu, root[0])) frontier_push<1>(P, sh, root, zv, dv, ev, false, 0, true);
     }
     if (take) atomicAdd(&sh.dem, (unsigned long long)take);
+    flush_labelled(P, sh, lab, lab_slots);
     if (need_total) {
         // one atomic per CTA for the used-slot total
         total = warp_sum_ll(total);
@@ -1325,7 +1277,7 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
 // lane keeps BR independent requests in flight.
 template <int BR>
 __device__ __forceinline__ void bfs_visit(const MfParams &P, Sh &sh, const int (&x)[BR], const bool (&valid)[BR], int L,
-                                          int sel)
+                                          int &lab, unsigned &lab_slots)
 {
     const bool with_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
     const bool pull = P.pull != 0;
@@ -1356,53 +1308,26 @@ __device__ __forceinline__ void bfs_visit(const MfParams &P, Sh &sh, const int (
             if (x[r] >= t0 && x[r] < t1) P.sc.dem[z[r]] = rc[r];     // z's own edge into the sink
         }
     }
-    frontier_push<BR>(P, sh, claim, z, d, ev, with_wl, sel);
+#pragma unroll
+    for (int r = 0; r < BR; ++r) {
+        if (!claim[r]) continue;
+        ++lab;
+        lab_slots += (unsigned)d[r];
+        place_labelled(P, sh, z[r], d[r], ev[r]);
+    }
 }
 
 constexpr int kBR = 4;
-
-// Before a top-down level that follows one which labelled long rows: each
-// long row becomes its ceil(deg / MF_BFS_CHUNK) work items.  Warps take the
-// long-row vertices 32 at a time and write their items together.
-__device__ __noinline__ void phase_bfs_expand(const MfParams &P, Sh &sh)
-{
-    MfSet *cs = sh.cs;
-    const int lane = threadIdx.x & 31;
-    const int lo = sh.d.long_lo, cnt = sh.d.long_hi - lo;
-    const int nwarps = vn() * (int)(blockDim.x >> 5);
-    const int rank = warp_rank(vn(), 0);
-    bool first = true;
-    for (;;) {
-        const int b = warp_deal(&cs->l[L_HEAD0].w[0], cnt, 32u, rank, nwarps, first);
-        if (b >= cnt) break;
-        const int k = b + lane;
-        const int z = k < cnt ? __ldcg(P.sc.blong + lo + k) : -1;
-        int d[1], x0[1], nc[1];
-        d[0] = z >= 0 ? ldg_cg(P.g.deg + z) : 0;
-        x0[0] = z >= 0 ? P.g.off[z] : 0;
-        nc[0] = (d[0] + MF_BFS_CHUNK - 1) / MF_BFS_CHUNK;
-        int incl = nc[0];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const int tot = __shfl_sync(0xffffffffu, incl, 31);
-        unsigned bi = 0;
-        if (lane == 0 && tot) bi = sh.d.app_hub + atomicAdd(&cs->l[L_HUB].w[0], (unsigned)tot);
-        bi = __shfl_sync(0xffffffffu, bi, 0);
-        write_items<1>(P, nc, x0, d, bi, incl - nc[0], tot);
-    }
-}
 
 __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
 {
     MfSet *cs = sh.cs;
     const int L = sh.d.level;
-    const int sel = sh.d.wl_sel;
     const int lane = threadIdx.x & 31;
     long long slots = 0;
-    const int nctas = sh.d.bfs_cta_mode ? 1 : vn();      // CTA 0 alone runs the small levels
+    const int nctas = vn();
+    int lab = 0;
+    unsigned lab_slots = 0;
     const int nwarps = nctas * (int)(blockDim.x >> 5);
     // chunks of long rows: one warp per item (at most MF_BFS_CHUNK slots)
     const int ilo = sh.d.hub_lo, icnt = sh.d.hub_hi - ilo;
@@ -1422,15 +1347,17 @@ __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
                 vs[r] = k < it.y;
                 xs[r] = it.x + k;
             }
-            bfs_visit<kBR>(P, sh, xs, vs, L, sel);
+            bfs_visit<kBR>(P, sh, xs, vs, L, lab, lab_slots);
         }
     }
     // regular frontier: warps take up to 32 vertices at a time and expand their
-    // rows together (each lane finds the vertex that owns its slot); a small
-    // frontier is dealt out fewer vertices per warp, so that its rows spread
-    // over many warps instead of queueing in one
+    // rows together (each lane finds the vertex that owns its slot); a frontier
+    // of fewer is dealt out evenly and at once, so that its rows spread over all
+    // warps and nobody comes back for more (a level of 5116 vertices, one for
+    // each of 4864 warps and a rush of all of them on the head for the rest,
+    // took 19 us, one of 4438 took 11)
     const int lo = sh.d.lvl_lo, cnt = sh.d.lvl_hi - lo;
-    const int take = max(1, min(32, cnt / max(1, nwarps)));
+    const int take = max(1, min(32, (cnt + nwarps - 1) / nwarps));
     first = true;
     const int rank_f = warp_rank(nctas, icnt);
     for (;;) {
@@ -1467,10 +1394,11 @@ __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
                 vs[r] = k < T;
                 xs[r] = rb + (k - eb);
             }
-            bfs_visit<kBR>(P, sh, xs, vs, L, sel);
+            bfs_visit<kBR>(P, sh, xs, vs, L, lab, lab_slots);
         }
     }
     add_stat(sh, ST_SLOTS_BFS, slots);
+    flush_labelled(P, sh, lab, lab_slots);
 }
 
 // Near BFS, bottom-up: slot x = (v, z) with residual c leads v down to z at
@@ -1495,7 +1423,6 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
     MfSet *cs = sh.cs;
     const int n = P.g.n;
     const int L = sh.d.level;
-    const int sel = sh.d.wl_sel;
     const bool pull = P.pull != 0;
     const int skip = pull ? P.sink : P.source;
     const bool with_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
@@ -1512,6 +1439,8 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
     const int cap = P.sc.bdefer != nullptr ? MF_BU_SCAN : 0x7fffffff;
     const bool near = sh.d.near != 0;
     long long slots = 0, unl = 0;
+    int lab = 0;
+    unsigned lab_slots = 0;
     if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_HSCAN_BFS, n);    // every vertex's height is read
     for (long long base = (long long)vb() * blockDim.x + threadIdx.x - lane; base < n; base += gs) {
         const int v = (int)base + lane;
@@ -1520,9 +1449,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
         const int r0 = ok ? P.g.off[v] : 0;
         const int d = ok ? ldg_cg(P.g.deg + v) : 0;
         const bool open = ok && hv == n;
-        bool take[1] = {false};
-        int zv[1] = {v}, dv[1] = {d};
-        long long ev[1] = {0};
+        bool take = false;
         if (open) {
             ++unl;
             int c[kA], z[kA];
@@ -1536,14 +1463,14 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
 #pragma unroll
             for (int r = 0; r < kA; ++r) {
                 const bool hitr = c[r] > 0 && ldg_cg(P.h + z[r]) == L;
-                take[0] |= hitr;
+                take |= hitr;
                 if (near && hitr) note_parent(P, v, r0 + r, z[r], c[r], L);
             }
             slots += d < kA ? d : kA;
         }
         // the warp-cooperative scan of the rows still open
         const int lim = d < cap ? d : cap;
-        const int rem = (open && !take[0] && lim > kA) ? lim - kA : 0;
+        const int rem = (open && !take && lim > kA) ? lim - kA : 0;
         int incl = rem;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1585,16 +1512,18 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
                 }
             hit |= __reduce_or_sync(0xffffffffu, mine);
         }
-        if ((hit >> lane) & 1u) take[0] = true;
+        if ((hit >> lane) & 1u) take = true;
         int nitem = 0, x0 = 0;
-        if (take[0]) {
+        if (take) {
             P.h[v] = L + 1;
-            if (with_wl && v != P.sink && v != P.source) ev[0] = pull ? -ldg_cg(P.e + v) : ldg_cg(P.e + v);
+            const long long ev = with_wl && v != P.sink && v != P.source ? (pull ? -ldg_cg(P.e + v) : ldg_cg(P.e + v)) : 0;
+            ++lab;
+            lab_slots += (unsigned)d;
+            place_labelled(P, sh, v, d, ev);
         } else if (open && d > lim) {
             nitem = (d - lim + MF_BU_CHUNK - 1) / MF_BU_CHUNK;
             x0 = r0 + lim;
         }
-        if (__any_sync(0xffffffffu, take[0])) frontier_push<1>(P, sh, take, zv, dv, ev, with_wl, sel);
         if (__any_sync(0xffffffffu, nitem > 0)) {
             int ic = nitem;
 #pragma unroll
@@ -1610,6 +1539,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
         }
     }
     add_stat(sh, ST_SLOTS_BFS, slots);
+    flush_labelled(P, sh, lab, lab_slots);
     add_stat(sh, ST_VERTS_BFS, unl);
 }
 
@@ -1623,7 +1553,6 @@ __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
     MfSet *cs = sh.cs;
     const int n = P.g.n;
     const int L = sh.d.level;
-    const int sel = sh.d.wl_sel;
     const bool pull = P.pull != 0;
     const bool with_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
     const int lane = threadIdx.x & 31;
@@ -1631,6 +1560,8 @@ __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
     const bool near = sh.d.near != 0;
     constexpr int kR = MF_BU_CHUNK / 32;
     long long slots = 0;
+    int lab = 0;
+    unsigned lab_slots = 0;
     const int nwarps = vn() * (int)(blockDim.x >> 5);
     const int rank = warp_rank(vn(), 0);
     bool first = true;
@@ -1660,19 +1591,16 @@ __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
             if (near && hitr) note_parent(P, v, it.y + r * 32 + lane, z[r], c[r], L);
         }
         if (lane == 0) slots += len;
-        bool won[1] = {false};
-        int zv[1] = {v}, dv[1] = {d};
-        long long ev[1] = {0};
-        if (__any_sync(0xffffffffu, hit)) {
-            if (lane == 0) {
-                won[0] = atomicCAS(P.h + v, n, L + 1) == n;
-                if (won[0] && with_wl && v != P.sink && v != P.source)
-                    ev[0] = pull ? -ldg_cg(P.e + v) : ldg_cg(P.e + v);
-            }
-            if (__any_sync(0xffffffffu, won[0])) frontier_push<1>(P, sh, won, zv, dv, ev, with_wl, sel);
+        if (__any_sync(0xffffffffu, hit) && lane == 0 && atomicCAS(P.h + v, n, L + 1) == n) {
+            const long long ev = with_wl && v != P.sink && v != P.source ? (pull ? -ldg_cg(P.e + v) : ldg_cg(P.e + v)) : 0;
+            ++lab;
+            lab_slots += (unsigned)d;
+            place_labelled(P, sh, v, d, ev);
         }
+        __syncwarp();
     }
     add_stat(sh, ST_SLOTS_BFS, slots);
+    flush_labelled(P, sh, lab, lab_slots);
 }
 
 // ---------------------------------------------------------------------------
@@ -2638,6 +2566,506 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
 }
 
 // ---------------------------------------------------------------------------
+// Short rounds and small phases
+// ---------------------------------------------------------------------------
+//
+// On grids, geometric and layered graphs most BFS levels hold a few hundred
+// vertices and most discharge rounds a few dozen, all with short rows.
+//
+// A short round (phase_discharge_short) gives each of its vertices one cycle of
+// Alg. 2, on values read in that round: a chain of four dependent accesses
+// (the vertex's state beside its row, the heads' heights, the receivers'
+// excess), against KERNEL_CYCLES such chains in phase_discharge.  The flow
+// moves one step per round either way, so the number of rounds hardly changes
+// (grid 1024: 1172 rounds of one cycle, 1066 of two).
+//
+// What a smaller phase still costs across the grid is the barrier and the
+// round trips around it, not its work.  The first CTA runs consecutive small
+// ones alone, with its queues in shared memory and __syncthreads between
+// them, and the others wait at one grid barrier, where they take its state
+// (H_JOIN).  What bounds it there is the SM's one scattered access per clock,
+// some 14 per vertex: up to MF_SOLO_LEVEL vertices (3 to 4 us a level) it beats
+// the grid; at 1000 a level took 13 us alone, against 9.5 us across the grid.
+
+// Whether the first CTA should go back to the grid: it has held up the others
+// for a quarter of the longest wait at a barrier.
+__device__ __forceinline__ bool solo_timeout(const MfParams &P, unsigned long long t0)
+{
+    return gtimer() - t0 > P.wait_limit_ns / 4;
+}
+
+// The queues of a run of small phases: vertex, row start and row length of the
+// next phase's entries.
+struct SoloQ {
+    int *v, *r, *d;
+};
+__device__ __forceinline__ SoloQ solo_q(int which)
+{
+    SoloQ q;
+    q.v = mf_stage + which * MF_SOLO_CAP;
+    q.r = q.v + 2 * MF_SOLO_CAP;
+    q.d = q.r + 2 * MF_SOLO_CAP;
+    return q;
+}
+__device__ __forceinline__ void solo_put(const SoloQ &q, int i, int v, int r0, int d)
+{
+    q.v[i] = v;
+    q.r[i] = r0;
+    q.d[i] = d;
+}
+
+// bfs_visit for a level that the first CTA runs alone: labelled vertices go
+// straight into its next queue (and onto the shared frontier list, should the
+// grid take over).
+template <int BR>
+__device__ __forceinline__ void solo_visit(const MfParams &P, Sh &sh, const int (&x)[BR], const bool (&valid)[BR],
+                                           int L, const SoloQ &nq, int &lab, unsigned &lab_slots)
+{
+    const bool want_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY), near = sh.d.near != 0;
+    const int n = P.g.n;
+    int z[BR], rc[BR], d[BR], r0[BR];
+    bool claim[BR];
+    long long ev[BR];
+#pragma unroll
+    for (int r = 0; r < BR; ++r) {
+        z[r] = valid[r] ? ldg_cg(P.g.dst + x[r]) : P.source;
+        rc[r] = valid[r] ? ldg_cg(P.g.pcap + x[r]) - ldg_cg(P.cf + x[r]) : 0;
+    }
+#pragma unroll
+    for (int r = 0; r < BR; ++r) claim[r] = rc[r] > 0 && z[r] != P.source && ldg_cg(P.h + z[r]) == n;
+#pragma unroll
+    for (int r = 0; r < BR; ++r) {
+        // in flight together with the claims
+        d[r] = claim[r] ? ldg_cg(P.g.deg + z[r]) : 0;
+        r0[r] = claim[r] ? P.g.off[z[r]] : 0;
+        ev[r] = claim[r] && want_wl ? ldg_cg(P.e + z[r]) : 0;
+        if (claim[r]) claim[r] = atomicCAS(P.h + z[r], n, L + 1) == n;
+    }
+#pragma unroll
+    for (int r = 0; r < BR; ++r) {
+        if (!claim[r]) continue;
+        ++lab;
+        lab_slots += (unsigned)d[r];
+        if (near) {
+            const int y = ldg_cg(P.g.rev + x[r]);
+            P.sc.par[z[r]] = y;
+            if (L == 0 && ldg_cg(P.g.dst + y) == P.sink) P.sc.dem[z[r]] = rc[r];
+        }
+        if (d[r] > P.bfs_hub) {
+            put_items(P, r0[r], d[r], sh.d.app_hub + atomicAdd(&sh.so_hub, chunks_of(d[r])));
+        } else {
+            const int i = atomicAdd(&sh.so_cnt, 1);
+            P.sc.border[sh.d.app_bfs + i] = z[r];
+            if (i < MF_SOLO_CAP) solo_put(nq, i, z[r], r0[r], d[r]);
+        }
+        if (ev[r] > 0 && z[r] != P.sink) {
+            const int bin = row_bin(P, d[r]);
+            P.sc.wl[sh.d.wl_sel][bin][sh.d.wl_app[bin] + atomicAdd(&sh.so_wl[bin], 1)] = z[r];
+            if (near) atomicAdd(&sh.exc, (unsigned long long)ev[r]);
+        }
+    }
+}
+
+// Top-down BFS levels, one after another, while they stay small.
+__device__ __noinline__ void solo_bfs(const MfParams &P, Sh &sh)
+{
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nwarps = nt >> 5;
+    const unsigned long long t0 = gtimer();
+    int cur = 0;
+    {
+        const int lo = sh.d.lvl_lo, cnt = sh.d.lvl_hi - lo;
+        const SoloQ q = solo_q(0);
+        for (int i = tid; i < cnt; i += nt) {
+            const int v = __ldcg(P.sc.border + lo + i);
+            solo_put(q, i, v, P.g.off[v], ldg_cg(P.g.deg + v));
+        }
+    }
+    if (tid < MF_NBIN) sh.so_wl[tid] = 0;
+    if (tid == 0) sh.so_cnt = sh.so_hub = 0;
+    __syncthreads();
+    for (;;) {
+        const int L = sh.d.level, cnt = sh.d.lvl_hi - sh.d.lvl_lo;
+        const SoloQ cq = solo_q(cur), nq = solo_q(cur ^ 1);
+        int lab = 0;
+        unsigned lab_slots = 0;
+        long long scanned = 0;
+        const int take = max(1, min(32, (cnt + nwarps - 1) / nwarps));
+        for (int b = wid * take; b < cnt; b += nwarps * take) {
+            const bool in = lane < take && b + lane < cnt;
+            const int d = in ? cq.d[b + lane] : 0, r0 = in ? cq.r[b + lane] : 0;
+            int incl = d;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int excl = incl - d;
+            const int T = __shfl_sync(0xffffffffu, incl, 31);
+            scanned += T;
+            for (int kb = 0; kb < T; kb += 32 * kBR) {
+                int xs[kBR];
+                bool vs[kBR];
+#pragma unroll
+                for (int r = 0; r < kBR; ++r) {
+                    const int k = kb + r * 32 + lane;
+                    int owner = 0;
+#pragma unroll
+                    for (int st = 16; st >= 1; st >>= 1) {
+                        const int cand = owner + st;
+                        const int ec = __shfl_sync(0xffffffffu, excl, cand & 31);
+                        if (cand < 32 && ec <= k) owner = cand;
+                    }
+                    const int rb = __shfl_sync(0xffffffffu, r0, owner), eb = __shfl_sync(0xffffffffu, excl, owner);
+                    vs[r] = k < T;
+                    xs[r] = rb + (k - eb);
+                }
+                solo_visit<kBR>(P, sh, xs, vs, L, nq, lab, lab_slots);
+            }
+        }
+        __syncwarp();
+        lab = __reduce_add_sync(0xffffffffu, lab);
+        lab_slots = __reduce_add_sync(0xffffffffu, lab_slots);
+        if (lane == 0) {
+            if (lab) atomicAdd(&sh.lab, ((unsigned long long)(unsigned)lab << 32) | lab_slots);
+            add_stat(sh, ST_SLOTS_BFS, scanned);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            MfDesc &d = sh.d;
+            MfState &st = sh.hs;
+            const int c = sh.so_cnt;
+            const long long fr = (long long)(unsigned)(sh.lab & 0xffffffffull), lab_n = (long long)(sh.lab >> 32);
+            const long long vis = st.vis_slots + fr, sup = st.sup + (long long)sh.exc;
+            sh.stat[ST_LAB_BFS] += lab_n;
+            const bool go = c > 0 && sh.so_hub == 0 && solo_level(P, c, fr) &&
+                            !(P.bu_alpha > 0 && fr * P.bu_alpha > st.used_slots - vis) &&
+                            !(d.near && sup > 0 && (sup >> st.cut_shift) >= st.dem) && !solo_timeout(P, t0);
+            if (go) {
+                // what advance() does for a level that is followed by another small one
+                ++d.level;
+                ++st.bfs_levels;
+                d.lvl_lo = d.lvl_hi;
+                d.app_bfs += c;
+                d.lvl_hi = d.app_bfs;
+                st.vis_slots = vis;
+                st.sup = sup;
+                for (int q = 0; q < MF_NBIN; ++q) d.wl_app[q] += sh.so_wl[q];
+            } else {
+                for (int q = 0; q < MF_LINES; ++q) sh.cnt[q] = make_int4(0, 0, 0, 0);
+                sh.cnt[L_BFS].x = c;
+                sh.cnt[L_HUB].x = sh.so_hub;
+                for (int q = 0; q < MF_NBIN; ++q) sh.cnt[L_WL + q].x = sh.so_wl[q];
+                sh.cnt[L_LAB] = make_int4((int)(unsigned)sh.lab, (int)(sh.lab >> 32), 0, 0);
+                sh.cnt[L_EXC] = make_int4((int)(unsigned)sh.exc, (int)(sh.exc >> 32), 0, 0);
+                solo_advance(P, H_BFS_NEXT, sh);
+            }
+            sh.lab = sh.exc = 0;
+            sh.so_cnt = sh.so_hub = 0;
+            for (int q = 0; q < MF_NBIN; ++q) sh.so_wl[q] = 0;
+            sh.so_go = go ? 1 : 0;
+        }
+        __syncthreads();
+        if (!sh.so_go) return;
+        cur ^= 1;
+    }
+}
+
+// z received flow and became active, or stays active after its cycle: into the
+// next round.  Alone (SOLO): into the first CTA's queue, or, when that is full
+// or z's row is long, onto the grid's lists; else into the CTA's queue of
+// worklist entries.
+template <bool SOLO>
+__device__ __forceinline__ void short_enqueue(const MfParams &P, Sh &sh, int z, int r0, int d, const SoloQ &nq)
+{
+    if (!SOLO) {
+        place_active(P, sh, z, d, L_AUX, sh.d.wl_sel ^ 1, nullptr);
+        return;
+    }
+    if (d <= MF_SHORT_ROW) {
+        const int i = atomicAdd(&sh.so_cnt, 1);
+        if (i < MF_SOLO_CAP) {
+            solo_put(nq, i, z, r0, d);
+            return;
+        }
+    }
+    const int bin = row_bin(P, d);
+    P.sc.wl[sh.d.wl_sel ^ 1][bin][atomicAdd(&sh.so_wl[bin], 1)] = z;
+}
+
+// g units along slot x = (u, z), y its reverse.  Every vertex is in a round's
+// lists at most once and lowers its own excess once, at its end, so z's excess
+// rises from <= 0 to > 0 at most once in a round: whoever makes it do so
+// queues it, and no stamp is needed.
+template <bool SOLO>
+__device__ __forceinline__ void short_push(const MfParams &P, Sh &sh, int x, int z, int y, int g, const SoloQ &nq)
+{
+    atomicSub(P.cf + x, g);
+    atomicAdd(P.cf + y, g);
+    if (z == P.sink) {
+        atomicAdd((unsigned long long *)&sh.sink_e, (unsigned long long)g);
+    } else if (z == P.source) {
+        atomicAdd((unsigned long long *)&sh.src_e, (unsigned long long)g);
+    } else {
+        const int d = ldg_cg(P.g.deg + z), r0 = SOLO ? P.g.off[z] : 0;     // in flight together with the excess
+        const long long old = atomic_add_ll(P.e + z, (long long)g);
+        if (old <= 0 && old + g > 0) short_enqueue<SOLO>(P, sh, z, r0, d, nq);
+    }
+}
+
+// u's new height when its lowest residual neighbour has height best (INT_MAX:
+// none): Alg. 2's relabel if u is not above it.
+__device__ __forceinline__ int short_lift(const MfParams &P, Sh &sh, int u, int hu, int best, bool write)
+{
+    const int n = P.g.n;
+    if (best < hu) return hu;
+    const int nh = best >= n - 1 ? n : best + 1;
+    if (write) {
+        P.h[u] = nh;
+        add_stat(sh, ST_RELABELS, 1);
+    }
+    return nh;
+}
+
+// One cycle of Alg. 2 for u by one thread (rows of at most 8 slots): relabel if
+// needed, then push to the lowest neighbours in slot order.
+template <bool SOLO>
+__device__ __forceinline__ int short_thread(const MfParams &P, Sh &sh, int u, int r0, int d, const SoloQ &nq)
+{
+    const int4 none = make_int4(0, 0, 0, 0);
+    const long long eu = ldg_cg(P.e + u);
+    int hu = ldg_cg(P.h + u);
+    int z[8], c[8], hz[8];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const bool in = 4 * q < d;
+        const int4 cf = in ? __ldcg(reinterpret_cast<const int4 *>(P.cf + r0) + q) : none;
+        const int4 dz = in ? __ldcg(reinterpret_cast<const int4 *>(P.g.dst + r0) + q) : none;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            c[4 * q + k] = 4 * q + k < d ? comp4(cf, k) : 0;
+            z[4 * q + k] = comp4(dz, k);
+        }
+    }
+    if (eu <= 0 || hu >= P.g.n) return 0;
+    int best = 0x7fffffff;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) hz[k] = c[k] > 0 ? ldg_cg(P.h + z[k]) : 0x7fffffff;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) best = min(best, hz[k]);
+    hu = short_lift(P, sh, u, hu, best, true);
+    if (hu >= P.g.n) return 0;
+    long long rem = eu;
+    int pushes = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        if (hz[k] != best || rem <= 0) continue;
+        const int g = rem < (long long)c[k] ? (int)rem : c[k];
+        short_push<SOLO>(P, sh, r0 + k, z[k], ldg_cg(P.g.rev + r0 + k), g, nq);
+        rem -= g;
+        ++pushes;
+    }
+    const long long old = atomic_add_ll(P.e + u, rem - eu);
+    if (old + rem - eu > 0) short_enqueue<SOLO>(P, sh, u, r0, d, nq);
+    return pushes;
+}
+
+// The same by one warp (rows of up to MF_SHORT_ROW slots): every lane holds four
+// slots of each 128, and a prefix sum over the lanes deals out the excess.
+template <bool SOLO>
+__device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int r0, int d, const SoloQ &nq)
+{
+    constexpr int kQ = MF_SHORT_ROW / 128;
+    const int lane = threadIdx.x & 31;
+    const int4 none = make_int4(0, 0, 0, 0);
+    const long long eu = ldg_cg(P.e + u);
+    int hu = ldg_cg(P.h + u);
+    if (eu <= 0 || hu >= P.g.n) return 0;                 // the same in every lane
+    int c[4 * kQ], hz[4 * kQ];
+    int best = 0x7fffffff;
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) {
+        const int j = q * 128 + lane * 4;
+        const bool in = j < d;
+        const int4 cf = in ? __ldcg(reinterpret_cast<const int4 *>(P.cf + r0 + j)) : none;
+        const int4 dz = in ? __ldcg(reinterpret_cast<const int4 *>(P.g.dst + r0 + j)) : none;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            c[4 * q + k] = j + k < d ? comp4(cf, k) : 0;
+            hz[4 * q + k] = c[4 * q + k] > 0 ? ldg_cg(P.h + comp4(dz, k)) : 0x7fffffff;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4 * kQ; ++k) best = min(best, hz[k]);
+    best = __reduce_min_sync(0xffffffffu, best);
+    hu = short_lift(P, sh, u, hu, best, lane == 0);
+    if (hu >= P.g.n) return 0;
+    long long mine = 0;
+#pragma unroll
+    for (int k = 0; k < 4 * kQ; ++k) mine += hz[k] == best ? c[k] : 0;
+    long long incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const long long total = __shfl_sync(0xffffffffu, incl, 31);
+    long long rem = eu - (incl - mine);                   // what is left when this lane's turn comes
+    int pushes = 0;
+#pragma unroll
+    for (int k = 0; k < 4 * kQ; ++k) {
+        if (hz[k] != best || rem <= 0) continue;
+        const int g = rem < (long long)c[k] ? (int)rem : c[k];
+        const int x = r0 + (k >> 2) * 128 + lane * 4 + (k & 3);
+        short_push<SOLO>(P, sh, x, ldg_cg(P.g.dst + x), ldg_cg(P.g.rev + x), g, nq);
+        rem -= g;
+        ++pushes;
+    }
+    __syncwarp();
+    pushes = __reduce_add_sync(0xffffffffu, pushes);
+    if (lane == 0) {
+        const long long sent = total < eu ? total : eu;
+        const long long old = atomic_add_ll(P.e + u, -sent);
+        if (old - sent > 0) short_enqueue<SOLO>(P, sh, u, r0, d, nq);
+    }
+    __syncwarp();
+    return pushes;
+}
+
+// A discharge round of one cycle per vertex across the grid: a thread for a row
+// of at most 8 slots, a warp for a longer one.
+__device__ __noinline__ void phase_discharge_short(const MfParams &P, Sh &sh)
+{
+    const int lane = threadIdx.x & 31;
+    const int sel = sh.d.wl_sel, n0 = sh.d.wl_n[0], n1 = sh.d.wl_n[1], cnt = n0 + n1;
+    const SoloQ none{};
+    long long pushes = 0, slots = 0, scans = 0;
+    for (long long k = spread_thread(); k < cnt; k += (long long)vn() * blockDim.x) {
+        const int i = (int)k;
+        const int u = __ldcg(i < n0 ? P.sc.wl[sel][0] + i : P.sc.wl[sel][1] + (i - n0));
+        const int d = ldg_cg(P.g.deg + u), r0 = P.g.off[u];
+        if (d > 8) continue;
+        pushes += short_thread<false>(P, sh, u, r0, d, none);
+        slots += d;
+        ++scans;
+    }
+    __syncwarp();
+    const int lo = P.small_deg <= 8 ? n0 : 0;          // the first list holds rows of at most small_deg slots
+    for (int i = lo + warp_rank(vn(), 0); i < cnt; i += vn() * (int)(blockDim.x >> 5)) {
+        const int u = __ldcg(i < n0 ? P.sc.wl[sel][0] + i : P.sc.wl[sel][1] + (i - n0));
+        const int d = ldg_cg(P.g.deg + u), r0 = P.g.off[u];
+        if (d <= 8) continue;
+        const int p = short_warp<false>(P, sh, u, r0, d, none);
+        if (lane == 0) {
+            pushes += p;
+            slots += d;
+            ++scans;
+        }
+    }
+    add_stat(sh, ST_PUSHES, pushes);
+    add_stat(sh, ST_SLOTS_DIS, slots);
+    add_stat(sh, ST_CYCLES_DIS, scans);
+    flush_queue(P, sh, L_AUX, sel ^ 1, nullptr, 0, 0u);
+}
+
+// Discharge rounds, one after another, while few vertices are active.  Ends when
+// none is left, when the rounds have taken their share of the time (as the
+// grid's do), or with the lists of the next grid round written.
+__device__ __noinline__ void solo_discharge(const MfParams &P, Sh &sh)
+{
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
+    const unsigned long long t0 = gtimer();
+    int cur = 0;
+    {
+        const int sel = sh.d.wl_sel, n0 = sh.d.wl_n[0], cnt = n0 + sh.d.wl_n[1];
+        const SoloQ q = solo_q(0);
+        for (int i = tid; i < cnt; i += nt) {
+            const int v = __ldcg(i < n0 ? P.sc.wl[sel][0] + i : P.sc.wl[sel][1] + (i - n0));
+            solo_put(q, i, v, P.g.off[v], ldg_cg(P.g.deg + v));
+        }
+        if (tid < MF_NBIN) sh.so_wl[tid] = 0;
+        if (tid == 0) {
+            sh.so_cnt = 0;
+            sh.bcast_i = cnt;
+        }
+    }
+    __syncthreads();
+    for (;;) {
+        const int cnt = sh.bcast_i;
+        const SoloQ cq = solo_q(cur), nq = solo_q(cur ^ 1);
+        long long slots = 0, pushes = 0, scans = 0;
+        for (int i = tid; i < cnt; i += nt) {
+            const int d = cq.d[i];
+            if (d > 8) continue;
+            pushes += short_thread<true>(P, sh, cq.v[i], cq.r[i], d, nq);
+            slots += d;
+            ++scans;
+        }
+        __syncwarp();
+        for (int i = wid; i < cnt; i += nt >> 5) {
+            const int d = cq.d[i];
+            if (d <= 8) continue;
+            const int p = short_warp<true>(P, sh, cq.v[i], cq.r[i], d, nq);
+            if (lane == 0) {
+                pushes += p;
+                slots += d;
+                ++scans;
+            }
+        }
+        add_stat(sh, ST_PUSHES, pushes);
+        add_stat(sh, ST_SLOTS_DIS, slots);
+        add_stat(sh, ST_CYCLES_DIS, scans);
+        __syncthreads();
+        if (tid == 0) {
+            MfDesc &d = sh.d;
+            MfState &st = sh.hs;
+            const int c = min(sh.so_cnt, MF_SOLO_CAP);
+            int spill = 0;
+            for (int q = 0; q < MF_NBIN; ++q) spill += sh.so_wl[q];
+            const unsigned long long now = gtimer();
+            const bool over = d.round + 1 >= MF_DEFAULT_ROUNDS && 2 * (now - st.t_dis0) >= st.t_dis0 - st.t_bfs0;
+            sh.so_go = c + spill == 0 || d.round + 1 >= MF_MAX_ROUNDS || over ? 0
+                       : spill > 0 || c > MF_SOLO_ACTIVE || solo_timeout(P, t0) ? 2 : 1;
+            if (sh.so_go) ++d.round;
+            ++st.rounds_total;
+            sh.bcast_i = c;
+            sh.so_cnt = 0;
+        }
+        __syncthreads();
+        const int go = sh.so_go, c = sh.bcast_i;
+        if (go == 1) {
+            cur ^= 1;
+            continue;
+        }
+        if (go == 2) {
+            // the next round is the grid's again: the queue goes onto its lists
+            for (int i = tid; i < c; i += nt) {
+                const int bin = row_bin(P, nq.d[i]);
+                P.sc.wl[sh.d.wl_sel ^ 1][bin][atomicAdd(&sh.so_wl[bin], 1)] = nq.v[i];
+            }
+            __syncthreads();
+        }
+        if (tid == 0) {
+            MfDesc &d = sh.d;
+            MfState &st = sh.hs;
+            const unsigned long long now = gtimer();
+            st.ns_dis += now - st.t_phase;
+            st.t_phase = st.t_now = now;
+            ++d.qstamp;
+            d.dis_more = go ? 1 : 0;
+            if (go) {
+                d.wl_sel ^= 1;
+                for (int q = 0; q < MF_NBIN; ++q) d.wl_n[q] = sh.so_wl[q];
+                pick_round(P, d);
+            } else {
+                begin_iteration(sh);
+            }
+        }
+        __syncthreads();
+        return;
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Near iterations: the excess walks down the BFS forest
 // ---------------------------------------------------------------------------
 
@@ -2867,6 +3295,8 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         MfCtrl *c = P.ctrl;
         sh.sink_e = sh.src_e = 0;
         sh.lab = sh.exc = sh.dem = 0;
+        sh.q_bfs = sh.q_long = sh.q_wn = 0;
+        for (int b = 0; b < MF_NBIN; ++b) sh.q_wl[b] = 0;
         sh.phase = 0;
         sh.cs = &c->set[0];
         sh.d = MfDesc{};
@@ -2948,17 +3378,10 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         phase_bfs_init(P, sh);
         if (!grid_sync(P, H_BFS_START, sh)) return false;
         while (!sh.d.bfs_done) {
-            if (sh.d.bfs_cta_mode) {
-                // small levels: CTA 0 alone; the others wait at the next grid
-                // barrier and take its state there
-                if (vb() == 0) {
-                    int run = 0;
-                    do {
-                        phase_bfs_level(P, sh);
-                        solo_step(P, H_BFS_NEXT, sh);
-                    } while (++run < MF_TAIL_RUN && !sh.d.bfs_done && sh.d.bfs_cta_mode);
-                }
-                if (!grid_sync(P, H_BFS_JOIN, sh)) return false;
+            if (sh.d.bfs_solo) {
+                // the others wait at the next grid barrier and take the first CTA's state there
+                if (vb() == 0) solo_bfs(P, sh);
+                if (!grid_sync(P, H_JOIN, sh)) return false;
                 continue;
             }
             if (sh.d.bu_mode) {
@@ -2969,10 +3392,6 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
                     if (!grid_sync(P, H_BFS_NEXT, sh)) return false;
                 }
             } else {
-                if (sh.d.expand) {
-                    phase_bfs_expand(P, sh);
-                    if (!grid_sync(P, H_EXPANDED, sh)) return false;
-                }
                 phase_bfs_level(P, sh);
                 if (!grid_sync(P, H_BFS_NEXT, sh)) return false;
             }
@@ -2986,7 +3405,13 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         if (sh.d.status != MF_ST_RUNNING) break;
         // discharge rounds, then remove-invalid-edges
         do {
+            if (sh.d.dis_solo) {
+                if (vb() == 0) solo_discharge(P, sh);
+                if (!grid_sync(P, H_JOIN, sh)) return false;
+                continue;
+            }
             if (sh.d.near && sh.d.round == 0) phase_walk(P, sh);
+            else if (sh.d.dis_short) phase_discharge_short(P, sh);
             else if (P.pull) phase_discharge<true>(P, sh);
             else phase_discharge<false>(P, sh);
             if (!grid_sync(P, H_DIS, sh)) return false;
