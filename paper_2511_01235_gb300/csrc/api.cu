@@ -57,9 +57,11 @@ struct maxflow_ctx {
     MfGraph g{};
     MfScratch sc{};
     MfCtrl *ctrl = nullptr;
-    MfCtrl *hctrl = nullptr;      // pinned
+    MfReport *rep = nullptr;      // pinned (the block holds hbuf and hside too): what launches report
     long long *dbuf = nullptr;    // device scratch for aux outputs (16 entries)
     long long *hbuf = nullptr;    // pinned mirror
+    uint8_t *hside = nullptr;     // pinned, [n]: the side of a query
+    int32_t *hbatch = nullptr;    // pinned, [3 * MF_PACK]: a small host batch on its way to the device
     int32_t *x_cf = nullptr, *x_cf2 = nullptr, *x_h = nullptr;
     long long *x_e = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -91,7 +93,7 @@ struct maxflow_ctx {
     // solve scratch) and the sides of the last cut; allocated on first use
     struct {
         MfCtrl *ctrl = nullptr;
-        MfCtrl *hctrl = nullptr;       // pinned
+        MfReport *rep = nullptr;       // pinned
         MfScratch sc{};
         int32_t *h = nullptr;
         uint8_t *side = nullptr;
@@ -176,6 +178,7 @@ MfParams base_params(maxflow_ctx *c)
     p.g = c->g;
     p.sc = c->sc;
     p.ctrl = c->ctrl;
+    p.rep = c->rep;
     p.cf = c->g.cf;
     p.h = c->g.h;
     p.e = c->g.e;
@@ -218,7 +221,7 @@ int ensure_batch(maxflow_ctx *c, int64_t count)
     while ((1LL << bits) < 2 * cap) ++bits;
     MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
     void *olds[] = {c->sc.hkey, c->sc.hval, c->sc.pkey, c->sc.pval, c->sc.bslot, c->sc.ins_list,
-                    c->sc.hused, c->sc.clamp, c->sc.bu, c->sc.bv, c->sc.bc};
+                    c->sc.hused, c->sc.bu};
     for (void *p : olds) dfree(c, p);
     int64_t hs = 1LL << bits;
     c->sc.hkey = dalloc_n<unsigned long long>(c, hs);
@@ -228,12 +231,9 @@ int ensure_batch(maxflow_ctx *c, int64_t count)
     c->sc.bslot = dalloc_n<int32_t>(c, cap);
     c->sc.ins_list = dalloc_n<int32_t>(c, cap);
     c->sc.hused = dalloc_n<int32_t>(c, cap);
-    c->sc.clamp = dalloc_n<int32_t>(c, cap);
-    c->sc.bu = dalloc_n<int32_t>(c, cap);
-    c->sc.bv = dalloc_n<int32_t>(c, cap);
-    c->sc.bc = dalloc_n<int32_t>(c, cap);
+    c->sc.bu = dalloc_n<int32_t>(c, 3 * cap);
     if (!c->sc.hkey || !c->sc.hval || !c->sc.pkey || !c->sc.pval || !c->sc.bslot || !c->sc.ins_list ||
-        !c->sc.hused || !c->sc.clamp || !c->sc.bu || !c->sc.bv || !c->sc.bc)
+        !c->sc.hused || !c->sc.bu)
         return MAXFLOW_ERR_OOM;
     MF_TRY(rc_cuda(cudaMemsetAsync(c->sc.hkey, 0xff, sizeof(unsigned long long) * hs, c->stream)));
     MF_TRY(rc_cuda(cudaMemsetAsync(c->sc.hval, 0xff, sizeof(int32_t) * hs, c->stream)));
@@ -241,6 +241,48 @@ int ensure_batch(maxflow_ctx *c, int64_t count)
     MF_TRY(rc_cuda(cudaMemsetAsync(c->sc.pval, 0xff, sizeof(int32_t) * hs, c->stream)));
     c->sc.batch_cap = cap;
     c->sc.hash_bits = bits;
+    return MAXFLOW_OK;
+}
+
+// The context's pinned memory, one block: report, mirror of the small results,
+// packed batch, side.
+int alloc_pinned(maxflow_ctx *c)
+{
+    auto round = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t a = round(sizeof(MfReport)), b = round(16 * sizeof(long long)),
+                 d = round(3 * MF_PACK * sizeof(int32_t));
+    char *p = nullptr;
+    MF_TRY(rc_cuda(cudaMallocHost((void **)&p, a + b + d + round((size_t)c->n))));
+    std::memset(p, 0, a + b);
+    c->rep = (MfReport *)p;
+    c->hbuf = (long long *)(p + a);
+    c->hbatch = (int32_t *)(p + a + b);
+    c->hside = (uint8_t *)(p + a + b + d);
+    return MAXFLOW_OK;
+}
+
+// A host batch onto the device (the caller has sized the scratch): tails, heads
+// and capacities one after the other.  A small one is packed into pinned memory
+// first, so that it takes one asynchronous copy instead of three that each wait
+// for their pageable source; the launch that reads it is waited for before the
+// next batch is packed.
+int upload_batch(maxflow_ctx *c, const maxflow_batch *b, cudaStream_t st, MfParams *p)
+{
+    const size_t k = (size_t)b->count, bytes = sizeof(int32_t) * k;
+    int32_t *d = c->sc.bu;
+    if (k > 0 && k <= MF_PACK) {
+        std::memcpy(c->hbatch, b->u, bytes);
+        std::memcpy(c->hbatch + k, b->v, bytes);
+        std::memcpy(c->hbatch + 2 * k, b->new_cap, bytes);
+        MF_TRY(rc_cuda(cudaMemcpyAsync(d, c->hbatch, 3 * bytes, cudaMemcpyHostToDevice, st)));
+    } else if (k > 0) {
+        MF_TRY(rc_cuda(cudaMemcpyAsync(d, b->u, bytes, cudaMemcpyHostToDevice, st)));
+        MF_TRY(rc_cuda(cudaMemcpyAsync(d + k, b->v, bytes, cudaMemcpyHostToDevice, st)));
+        MF_TRY(rc_cuda(cudaMemcpyAsync(d + 2 * k, b->new_cap, bytes, cudaMemcpyHostToDevice, st)));
+    }
+    p->bu = d;
+    p->bv = d + k;
+    p->bc = d + 2 * k;
     return MAXFLOW_OK;
 }
 
@@ -358,7 +400,7 @@ void note_incremental(maxflow_ctx *c)
     c->inc_ms = c->st.ms_last;
 }
 
-void fill_stats(maxflow_ctx *c, const MfCtrl &h, float ms)
+void fill_stats(maxflow_ctx *c, const MfReport &h, float ms)
 {
     maxflow_stats_t &s = c->st;
     s.iterations = h.iters;
@@ -404,17 +446,17 @@ void fill_stats(maxflow_ctx *c, const MfCtrl &h, float ms)
 // (MF_E_*) in *kerr and its status in *kstatus.
 int run_kernel(maxflow_ctx *c, const MfParams &p, int *kerr, int *kstatus)
 {
+    c->rep->err = MF_E_INTERNAL;      // stands if the kernel does not get to its end
     MF_TRY(rc_cuda(cudaEventRecord(c->ev0, c->stream)));
     MF_TRY(counted(mf_launch(p, c->grid, (void *)c->stream), 1));
     MF_TRY(rc_cuda(cudaEventRecord(c->ev1, c->stream)));
-    MF_TRY(rc_cuda(cudaMemcpyAsync(c->hctrl, c->ctrl, MF_CTRL_HOST_BYTES, cudaMemcpyDeviceToHost, c->stream)));
     MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, c->ev0, c->ev1);
     c->acc_ms += ms;
-    *kerr = (int)c->hctrl->err.w[0];
-    *kstatus = c->hctrl->d.status;
-    fill_stats(c, *c->hctrl, ms);
+    *kerr = c->rep->err;
+    *kstatus = c->rep->status;
+    fill_stats(c, *c->rep, ms);
     if (*kerr != MF_E_NONE) {
         // a barrier may have been left half-way: reset it for the next launch
         MF_TRY(rc_cuda(clear_sync(c->ctrl, c->stream)));
@@ -442,7 +484,7 @@ int run_solve(maxflow_ctx *c, MfParams p)
     int rc = status_to_rc(kerr, kst);
     c->st.solves++;
     if (rc == MAXFLOW_OK || rc == MAXFLOW_ERR_NOT_CONVERGED) {
-        c->value = c->hctrl->value;
+        c->value = c->rep->value;
         c->st.value = c->value;
         c->solved = (rc == MAXFLOW_OK);
     }
@@ -548,11 +590,12 @@ int rebuild_device(maxflow_ctx *c)
 
 int check_host_batch(maxflow_ctx *c, const maxflow_batch *b)
 {
-    for (int64_t i = 0; i < b->count; ++i) {
-        int32_t u = b->u[i], v = b->v[i], w = b->new_cap[i];
-        if (u < 0 || u >= c->n || v < 0 || v >= c->n || w < 0) return MAXFLOW_ERR_INVALID;
-    }
-    return MAXFLOW_OK;
+    // one pass without branches (a batch is refused rarely)
+    const uint32_t n = (uint32_t)c->n;
+    uint32_t bad = 0;
+    for (int64_t i = 0; i < b->count; ++i)
+        bad |= (uint32_t)((uint32_t)b->u[i] >= n) | (uint32_t)((uint32_t)b->v[i] >= n) | (uint32_t)(b->new_cap[i] < 0);
+    return bad ? MAXFLOW_ERR_INVALID : MAXFLOW_OK;
 }
 
 // Apply (and optionally solve) a batch.
@@ -572,13 +615,7 @@ int do_batch(maxflow_ctx *c, const maxflow_batch *b, int mode)
             p.bv = b->v;
             p.bc = b->new_cap;
         } else {
-            size_t bytes = sizeof(int32_t) * (size_t)b->count;
-            MF_TRY(rc_cuda(cudaMemcpyAsync(c->sc.bu, b->u, bytes, cudaMemcpyHostToDevice, c->stream)));
-            MF_TRY(rc_cuda(cudaMemcpyAsync(c->sc.bv, b->v, bytes, cudaMemcpyHostToDevice, c->stream)));
-            MF_TRY(rc_cuda(cudaMemcpyAsync(c->sc.bc, b->new_cap, bytes, cudaMemcpyHostToDevice, c->stream)));
-            p.bu = c->sc.bu;
-            p.bv = c->sc.bv;
-            p.bc = c->sc.bc;
+            MF_TRY(upload_batch(c, b, c->stream, &p));
         }
     }
     for (int attempt = 0; attempt < 2; ++attempt) {
@@ -596,7 +633,7 @@ int do_batch(maxflow_ctx *c, const maxflow_batch *b, int mode)
         if (mode & MF_M_SOLVE) {
             c->st.solves++;
             if (rc == MAXFLOW_OK || rc == MAXFLOW_ERR_NOT_CONVERGED) {
-                c->value = c->hctrl->value;
+                c->value = c->rep->value;
                 c->st.value = c->value;
                 c->solved = (rc == MAXFLOW_OK);
             }
@@ -629,7 +666,7 @@ int ensure_pp(maxflow_ctx *c)
 {
     auto &q = c->pp;
     const int32_t n = c->n;
-    if (!q.hctrl) MF_TRY(rc_cuda(cudaMallocHost((void **)&q.hctrl, sizeof(MfCtrl))));
+    if (!q.rep) MF_TRY(rc_cuda(cudaMallocHost((void **)&q.rep, sizeof(MfReport))));
     if (!q.ctrl) {
         q.ctrl = (MfCtrl *)dalloc(c, sizeof(MfCtrl));
         q.h = dalloc_n<int32_t>(c, n);
@@ -747,9 +784,8 @@ void maxflow_destroy(maxflow_ctx *c)
         if (c->stream) cudaStreamSynchronize(c->stream);
         while (!c->allocs.empty()) dfree(c, c->allocs.back().first);
         park_free(c);
-        if (c->pp.hctrl) cudaFreeHost(c->pp.hctrl);
-        if (c->hctrl) cudaFreeHost(c->hctrl);
-        if (c->hbuf) cudaFreeHost(c->hbuf);
+        if (c->pp.rep) cudaFreeHost(c->pp.rep);
+        if (c->rep) cudaFreeHost(c->rep);
         if (c->ev0) cudaEventDestroy(c->ev0);
         if (c->ev1) cudaEventDestroy(c->ev1);
     }
@@ -802,8 +838,7 @@ int maxflow_init(maxflow_ctx **out, const maxflow_graph *g, int32_t s, int32_t t
     c->group_deg = std::max<int32_t>(c->hub_deg, c->stage_slots / (MF_BLOCK / (32 * MF_GROUP_WARPS)));
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaEventCreate(&c->ev0));
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaEventCreate(&c->ev1));
-    if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMallocHost((void **)&c->hctrl, sizeof(MfCtrl)));
-    if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMallocHost((void **)&c->hbuf, 16 * sizeof(long long)));
+    if (rc == MAXFLOW_OK) rc = alloc_pinned(c);
     if (rc == MAXFLOW_OK) rc = upload_graph(c, hg);
     hg.release();
     if (rc == MAXFLOW_OK) {
@@ -816,6 +851,7 @@ int maxflow_init(maxflow_ctx **out, const maxflow_graph *g, int32_t s, int32_t t
     }
     if (rc == MAXFLOW_OK) rc = alloc_vertex_scratch(c);
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemsetAsync(c->ctrl, 0, sizeof(MfCtrl), c->stream));
+    if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemsetAsync(c->dbuf, 0, 16 * sizeof(long long), c->stream));
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemsetAsync(c->g.h, 0, sizeof(int32_t) * c->n, c->stream));
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemsetAsync(c->g.e, 0, sizeof(long long) * c->n, c->stream));
     if (rc == MAXFLOW_OK) rc = ensure_batch(c, 1024);
@@ -908,22 +944,16 @@ int maxflow_query(maxflow_ctx *c, int64_t *value, uint8_t *side, int64_t *cut_ca
     if (c->evicted && (side || cut_cap)) return MAXFLOW_ERR_STATE;
     DeviceGuard dg(c->device);
     if (!dg.ok) return MAXFLOW_ERR_CUDA;
-    MfParams p = base_params(c);
-    if (side) {
-        uint8_t *ds = (uint8_t *)dalloc(c, (size_t)c->n);
-        if (!ds) return MAXFLOW_ERR_OOM;
-        int rc = counted(mf_launch_aux(MF_AUX_SIDE, p, (void *)c->stream, nullptr, ds), 1);
-        if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemcpyAsync(side, ds, (size_t)c->n, cudaMemcpyDeviceToHost, c->stream));
-        if (rc == MAXFLOW_OK) rc = rc_cuda(cudaStreamSynchronize(c->stream));
-        dfree(c, ds);
-        MF_TRY(rc);
-    }
-    if (cut_cap) {
-        MF_TRY(rc_cuda(cudaMemsetAsync(c->dbuf, 0, sizeof(long long), c->stream)));
-        MF_TRY(counted(mf_launch_aux(MF_AUX_CUT, p, (void *)c->stream, c->dbuf, nullptr), 1));
-        MF_TRY(rc_cuda(cudaMemcpyAsync(c->hbuf, c->dbuf, sizeof(long long), cudaMemcpyDeviceToHost, c->stream)));
+    if (side || cut_cap) {
+        MfAnswer a{};
+        a.side = side ? c->hside : nullptr;
+        a.cut = cut_cap ? c->hbuf : nullptr;
+        a.acc = c->dbuf + 8;
+        a.from_sink = 2 * c->rep->cut_slots < c->rep->used_slots ? 1 : 0;
+        MF_TRY(counted(mf_launch_aux(MF_AUX_ANSWER, base_params(c), (void *)c->stream, nullptr, &a), 1));
         MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
-        *cut_cap = c->hbuf[0];
+        if (side) std::memcpy(side, c->hside, (size_t)c->n);
+        if (cut_cap) *cut_cap = c->hbuf[0];
     }
     if (value) *value = c->value;
     return MAXFLOW_OK;
@@ -932,7 +962,7 @@ int maxflow_query(maxflow_ctx *c, int64_t *value, uint8_t *side, int64_t *cut_ca
 int maxflow_trace(maxflow_ctx *c, int32_t *boundary, double *t_us, int32_t cap, int32_t *count)
 {
     if (!c || !count || cap < 0) return MAXFLOW_ERR_INVALID;
-    const MfCtrl &h = *c->hctrl;
+    const MfReport &h = *c->rep;
     int k = std::min<int>(h.trace_n, std::min<int>(cap, MF_TRACE));
     for (int i = 0; i < k; ++i) {
         if (boundary) boundary[i] = h.trace_hook[i];
@@ -946,7 +976,7 @@ int maxflow_trace_work(maxflow_ctx *c, int64_t *slots, int32_t *info, double *ct
                        int32_t cap, int32_t *count)
 {
     if (!c || !count || cap < 0) return MAXFLOW_ERR_INVALID;
-    const MfCtrl &h = *c->hctrl;
+    const MfReport &h = *c->rep;
     int k = std::min<int>(h.trace_n, std::min<int>(cap, MF_TRACE));
     for (int i = 0; i < k; ++i) {
         if (slots) slots[i] = h.trace_slots[i];
@@ -1001,13 +1031,11 @@ int stage_and_features(maxflow_ctx *c, const maxflow_batch *b, maxflow_batch *de
     MF_TRY(ensure_batch(c, b->count));
     *dev_view = *b;
     if (!b->on_device && b->count > 0) {
-        size_t bytes = sizeof(int32_t) * (size_t)b->count;
-        MF_TRY(rc_cuda(cudaMemcpyAsync(c->sc.bu, b->u, bytes, cudaMemcpyHostToDevice, c->stream)));
-        MF_TRY(rc_cuda(cudaMemcpyAsync(c->sc.bv, b->v, bytes, cudaMemcpyHostToDevice, c->stream)));
-        MF_TRY(rc_cuda(cudaMemcpyAsync(c->sc.bc, b->new_cap, bytes, cudaMemcpyHostToDevice, c->stream)));
-        dev_view->u = c->sc.bu;
-        dev_view->v = c->sc.bv;
-        dev_view->new_cap = c->sc.bc;
+        MfParams q{};
+        MF_TRY(upload_batch(c, b, c->stream, &q));
+        dev_view->u = q.bu;
+        dev_view->v = q.bv;
+        dev_view->new_cap = q.bc;
         dev_view->on_device = 1;
     }
     MfFeatIn f{};
@@ -1173,25 +1201,22 @@ int maxflow_solve_batched(maxflow_ctx *const *ctxs, int32_t count, const maxflow
     for (int32_t i = 0; i < count; ++i) order[(size_t)i] = i;
     std::sort(order.begin(), order.end(),
               [&](int32_t a, int32_t b) { return ctxs[a]->g.slot_cap > ctxs[b]->g.slot_cap; });
+    // every batch is checked, and its scratch sized, before any of them is on its way
+    for (int32_t i = 0; batches && i < count; ++i) {
+        const maxflow_batch *b = &batches[i];
+        if (b->count < 0 || (b->count > 0 && (!b->u || !b->v || !b->new_cap))) return MAXFLOW_ERR_INVALID;
+        if (!b->on_device) MF_TRY(check_host_batch(ctxs[i], b));
+    }
+    for (int32_t i = 0; batches && i < count; ++i) MF_TRY(ensure_batch(ctxs[i], batches[i].count));
     std::vector<MfParams> plist((size_t)count);
     for (int32_t k = 0; k < count; ++k) {
         maxflow_ctx *c = ctxs[order[(size_t)k]];
         MfParams p = base_params(c);
         if (batches) {
             const maxflow_batch *b = &batches[order[(size_t)k]];
-            if (b->count < 0 || (b->count > 0 && (!b->u || !b->v || !b->new_cap))) return MAXFLOW_ERR_INVALID;
-            if (!b->on_device) MF_TRY(check_host_batch(c, b));
-            MF_TRY(ensure_batch(c, b->count));
-            p = base_params(c);
             p.bcount = b->count;
             if (b->count > 0 && !b->on_device) {
-                size_t bytes = sizeof(int32_t) * (size_t)b->count;
-                MF_TRY(rc_cuda(cudaMemcpyAsync(c->sc.bu, b->u, bytes, cudaMemcpyHostToDevice, c0->stream)));
-                MF_TRY(rc_cuda(cudaMemcpyAsync(c->sc.bv, b->v, bytes, cudaMemcpyHostToDevice, c0->stream)));
-                MF_TRY(rc_cuda(cudaMemcpyAsync(c->sc.bc, b->new_cap, bytes, cudaMemcpyHostToDevice, c0->stream)));
-                p.bu = c->sc.bu;
-                p.bv = c->sc.bv;
-                p.bc = c->sc.bc;
+                MF_TRY(upload_batch(c, b, c0->stream, &p));
             } else {
                 p.bu = b->u;
                 p.bv = b->v;
@@ -1201,6 +1226,7 @@ int maxflow_solve_batched(maxflow_ctx *const *ctxs, int32_t count, const maxflow
         } else {
             p.mode = MF_M_STATIC_INIT | MF_M_SOLVE;
         }
+        c->rep->err = MF_E_INTERNAL;  // stands if the instance does not get to its end
         plist[(size_t)k] = p;
     }
     const int maxg = c0->per_sm * c0->sms;
@@ -1220,9 +1246,6 @@ int maxflow_solve_batched(maxflow_ctx *const *ctxs, int32_t count, const maxflow
     MF_TRY(rc_cuda(cudaEventRecord(c0->ev1, c0->stream)));
     int abort_h = 0;
     MF_TRY(rc_cuda(cudaMemcpyAsync(&abort_h, abort_flag, sizeof(int), cudaMemcpyDeviceToHost, c0->stream)));
-    for (int32_t i = 0; i < count; ++i)
-        MF_TRY(rc_cuda(cudaMemcpyAsync(ctxs[i]->hctrl, ctxs[i]->ctrl, MF_CTRL_HOST_BYTES, cudaMemcpyDeviceToHost,
-                                       c0->stream)));
     MF_TRY(rc_cuda(cudaStreamSynchronize(c0->stream)));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, c0->ev0, c0->ev1);
@@ -1230,9 +1253,9 @@ int maxflow_solve_batched(maxflow_ctx *const *ctxs, int32_t count, const maxflow
     int first_rc = MAXFLOW_OK;
     for (int32_t i = 0; i < count; ++i) {
         maxflow_ctx *c = ctxs[i];
-        const int kerr = (int)c->hctrl->err.w[0], kst = c->hctrl->d.status;
+        const int kerr = c->rep->err, kst = c->rep->status;
         c->acc_ms = ms;
-        fill_stats(c, *c->hctrl, ms);
+        fill_stats(c, *c->rep, ms);
         if (abort_h || kerr != MF_E_NONE) {
             MF_TRY(rc_cuda(clear_sync(c->ctrl, c->stream)));
             MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
@@ -1244,7 +1267,7 @@ int maxflow_solve_batched(maxflow_ctx *const *ctxs, int32_t count, const maxflow
             rc = abort_h ? MAXFLOW_ERR_INTERNAL : status_to_rc(kerr, kst);
             c->st.solves++;
             if (rc == MAXFLOW_OK || rc == MAXFLOW_ERR_NOT_CONVERGED) {
-                c->value = c->hctrl->value;
+                c->value = c->rep->value;
                 c->st.value = c->value;
                 c->solved = (rc == MAXFLOW_OK);
                 if (batches) c->st.updates++;
@@ -1461,6 +1484,7 @@ int maxflow_restore(maxflow_ctx *c)
         rc = counted(mf_launch_aux(MF_AUX_PCAP, base_params(c), (void *)c->stream, nullptr, nullptr), 1);
     if (rc == MAXFLOW_OK) rc = alloc_vertex_scratch(c);
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemsetAsync(c->ctrl, 0, sizeof(MfCtrl), c->stream));
+    if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemsetAsync(c->dbuf, 0, 16 * sizeof(long long), c->stream));
     if (rc == MAXFLOW_OK)
         rc = rc_cuda(cudaMemcpyAsync(c->g.h, v.h, sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
     if (rc == MAXFLOW_OK)
@@ -1542,6 +1566,8 @@ int maxflow_update_pp(maxflow_ctx *c, const maxflow_batch *b, int32_t stop_after
     pl[1].side_root = 0;
     pl[1].h = c->pp.h;
     pl[1].ctrl = c->pp.ctrl;
+    pl[1].rep = c->pp.rep;
+    c->rep->err = c->pp.rep->err = MF_E_INTERNAL;   // stand if a part does not get to its end
     pl[1].sc = c->pp.sc;
     const int maxg = c->per_sm * c->sms;
     const int gsize = std::max(1, std::min(c->grid, maxg) / 2);
@@ -1556,13 +1582,11 @@ int maxflow_update_pp(maxflow_ctx *c, const maxflow_batch *b, int32_t stop_after
     MF_TRY(rc_cuda(cudaEventRecord(c->ev1, c->stream)));
     int abort_h = 0;
     MF_TRY(rc_cuda(cudaMemcpyAsync(&abort_h, abort_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream)));
-    MF_TRY(rc_cuda(cudaMemcpyAsync(c->hctrl, c->ctrl, MF_CTRL_HOST_BYTES, cudaMemcpyDeviceToHost, c->stream)));
-    MF_TRY(rc_cuda(cudaMemcpyAsync(c->pp.hctrl, c->pp.ctrl, MF_CTRL_HOST_BYTES, cudaMemcpyDeviceToHost, c->stream)));
     MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
     float ms2 = 0.f;
     cudaEventElapsedTime(&ms2, c->ev0, c->ev1);
     ms += ms2;
-    const int e0 = (int)c->hctrl->err.w[0], e1 = (int)c->pp.hctrl->err.w[0];
+    const int e0 = c->rep->err, e1 = c->pp.rep->err;
     if (abort_h || e0 != MF_E_NONE || e1 != MF_E_NONE) {
         MF_TRY(rc_cuda(clear_sync(c->ctrl, c->stream)));
         MF_TRY(rc_cuda(clear_sync(c->pp.ctrl, c->stream)));
@@ -1573,7 +1597,7 @@ int maxflow_update_pp(maxflow_ctx *c, const maxflow_batch *b, int32_t stop_after
     }
     if (stop_after == 2) {
         c->st.ms_update = ms;
-        return status_to_rc(MF_E_NONE, c->hctrl->d.status == MF_ST_CAP || c->pp.hctrl->d.status == MF_ST_CAP
+        return status_to_rc(MF_E_NONE, c->rep->status == MF_ST_CAP || c->pp.rep->status == MF_ST_CAP
                                            ? MF_ST_CAP : MF_ST_CONVERGED);
     }
     // 3: a push solve over the whole graph finishes what the two parts left
@@ -1665,8 +1689,7 @@ int maxflow_clone(maxflow_ctx *src, maxflow_ctx **out)
     const int64_t S = src->g.slot_cap;
     int rc = rc_cuda(cudaEventCreate(&c->ev0));
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaEventCreate(&c->ev1));
-    if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMallocHost((void **)&c->hctrl, sizeof(MfCtrl)));
-    if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMallocHost((void **)&c->hbuf, 16 * sizeof(long long)));
+    if (rc == MAXFLOW_OK) rc = alloc_pinned(c);
     if (rc == MAXFLOW_OK) {
         c->g.n = n;
         c->g.slot_cap = S;
@@ -1707,6 +1730,7 @@ int maxflow_clone(maxflow_ctx *src, maxflow_ctx **out)
             if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemcpyAsync(cp.d, cp.s, cp.b, cudaMemcpyDeviceToDevice, c->stream));
     }
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemsetAsync(c->ctrl, 0, sizeof(MfCtrl), c->stream));
+    if (rc == MAXFLOW_OK) rc = rc_cuda(cudaMemsetAsync(c->dbuf, 0, 16 * sizeof(long long), c->stream));
     if (rc == MAXFLOW_OK) rc = ensure_batch(c, std::max<int64_t>(1024, src->sc.batch_cap));
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaStreamSynchronize(c->stream));
     if (rc != MAXFLOW_OK) {

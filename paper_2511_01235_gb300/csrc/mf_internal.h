@@ -27,7 +27,6 @@
 #define MF_GROUP_WARPS 4      // warps of a group; a group keeps rows up to a quarter of the snapshot
 #define MF_BFS_HUB 256        // BFS: rows above this many slots enter the frontier as work items
 #define MF_BFS_CHUNK 256      // BFS: slots per work item
-#define MF_ACTIVE_HIST 64
 #define MF_DEFAULT_ROUNDS 2   // adaptive discharge rounds: the minimum per iteration
 #define MF_MAX_ROUNDS 1024    // adaptive rounds: upper bound per iteration
 #define MF_TRACE 256          // hook timeline entries kept per launch
@@ -114,6 +113,7 @@ struct MfSet {
     MfLine l[MF_LINES];
 };
 
+#define MF_PACK 16384     // host batches of up to this many updates are packed into pinned memory
 #define MF_MAX_CTAS 1024  // CTAs whose finish times and slots are traced (a grid is far smaller)
 
 // What the phases read, the same in every CTA (kept in shared memory).
@@ -176,17 +176,19 @@ enum MfStat {
     MF_STATS
 };
 
-struct MfCtrl {
-    // ---- read by the host after every launch ----
-    MfLine err;           // w[0]: error of the launch (MF_E_*)
-    MfDesc d;             // final; the stamps carry over to the next launch
+// What the host reads of a launch.  The kernel's first CTA writes it straight to
+// the context's pinned memory (MfParams.rep), so nothing has to be copied back.
+struct MfReport {
+    int err;              // MF_E_*
+    int status;           // MF_ST_*
     long long iters, value;
     long long bfs_levels, active_total, active_first;
+    long long cut_slots, used_slots;      // slots of the vertices the last BFS labelled; of all
     long long stat[MF_STATS];     // MfStat, summed over the CTAs at the end of a launch
     unsigned long long ns_bfs, ns_dis, ns_fix, ns_wl, ns_apply;
-    int active_hist[MF_ACTIVE_HIST];
     long long rounds_total;
-    unsigned long long t_entry, t_exit;   // kernel entry (first CTA), last barrier
+    unsigned long long t_entry;   // kernel entry (first CTA), last barrier
+    unsigned long long t_exit;
     long long barriers;
     int trace_n;
     int trace_hook[MF_TRACE];
@@ -199,7 +201,14 @@ struct MfCtrl {
     // when the CTAs finished the phase that a barrier closes (ns after the previous barrier):
     // the last one and the mean, per traced barrier
     unsigned trace_fin_max[MF_TRACE], trace_fin_mean[MF_TRACE];
-    // ---- device only ----
+};
+
+struct MfCtrl {
+    MfReport rep;         // of launches without pinned memory to report to
+    MfLine err;           // w[0]: a barrier gave up (MF_E_WAIT)
+    int qstamp, fstamp;   // carried over from launch to launch
+    long long value;
+    long long stat[MF_STATS];
     MfLine bar;           // w[0]: arrivals in this launch (the first CTA leaves it at zero)
     MfSet set[3];
     // the first CTA's state for the others, after it ran phases alone
@@ -208,8 +217,7 @@ struct MfCtrl {
     // per phase (mod 3) and CTA: finish time, slots scanned
     unsigned fin[3][MF_MAX_CTAS], scanned[3][MF_MAX_CTAS];
 };
-// What the host copies back, and the part it clears after a launch that ended in a barrier that gave up.
-#define MF_CTRL_HOST_BYTES offsetof(MfCtrl, bar)
+// The part the host clears after a launch that ended in a barrier that gave up.
 #define MF_CTRL_SYNC_BYTES (sizeof(MfLine) + sizeof(MfSet) * 3)
 
 struct MfGraph {
@@ -243,15 +251,15 @@ struct MfScratch {
     int32_t *bslot;           // [batch_cap] slot of each update (-2: superseded or ignored)
     int32_t *ins_list;        // [batch_cap] new-pair table positions
     int32_t *hused;           // [batch_cap] dedup table positions in use
-    int32_t *clamp;           // [batch_cap] updates that lowered a capacity
     int32_t *ins_need;        // [n]
-    int32_t *bu, *bv, *bc;    // [batch_cap] staging of a host batch
+    int32_t *bu;              // [3 * batch_cap] a host batch: tails, heads, capacities one after the other
 };
 
 struct MfParams {
     MfGraph g;
     MfScratch sc;
     MfCtrl *ctrl;
+    MfReport *rep;            // where the launch reports (pinned host memory, or ctrl->rep)
     int32_t *cf;              // residual array of this run (g.cf, or a copy for extraction)
     int32_t *h;
     long long *e;
@@ -315,13 +323,19 @@ int mf_launch_aux(int which, const MfParams &p, void *stream, long long *dev_out
 #define MF_AUX_SET_FLOW 2         // extra = {count, u, v, f} device arrays; validate into dev_out[0] or apply
 #define MF_AUX_EXCESS 3           // e = sum(cf - cap) per row
 #define MF_AUX_CHECK 4            // dev_out[0..5]
-#define MF_AUX_SIDE 5             // extra = uint8_t* side (device)
-#define MF_AUX_CUT 6              // dev_out[0] = cut capacity
+#define MF_AUX_ANSWER 5           // extra = MfAnswer: the source side and the capacity of the cut
 #define MF_AUX_REVERSE_CF 7       // extra = int32_t* out: out[x] = cf[rev[x]]
 #define MF_AUX_CLEAR_SCRATCH 8    // reset hash tables and ins_need
 #define MF_AUX_DUMP 9             // extra = int32_t* rowid per slot (u of each slot index)
 #define MF_AUX_NEGATE_E 10        // e = -e
 #define MF_AUX_PCAP 11            // pcap = cap + cap[rev] on every used slot (after a restore)
+
+struct MfAnswer {
+    uint8_t *side;        // [n] 1: source side (device-accessible; nullptr: not wanted)
+    long long *cut;       // capacity of the cut (device-accessible; nullptr: not wanted)
+    long long *acc;       // device, [2], zero before and after
+    int from_sink;        // sum over the sink side's rows instead of the source side's
+};
 
 // device-side rebuild (rows grow, flows and excesses stay in place); noff holds
 // n + 1 row starts followed by the scan's tile totals: mf_rebuild_scratch(n) int64

@@ -117,6 +117,7 @@ extern "C" int maxflow_global_relabel_noalloc(int32_t n, int32_t s, int32_t t, c
     p.sc.bitem = (int2 *)(base + kCtrlBytes + kListBytes);
     p.sc.bdefer = nullptr;          // bottom-up threads scan whole rows (no deferred chunks: no room for them)
     p.ctrl = ctrl;
+    p.rep = &ctrl->rep;
     p.cf = p.g.cf;
     p.h = h;
     p.e = p.g.e;
@@ -153,7 +154,7 @@ extern "C" int maxflow_global_relabel_noalloc(int32_t n, int32_t s, int32_t t, c
     if (rc != MAXFLOW_OK) return rc;
     mf_note_launches(1);
     unsigned err = 0;
-    if (cudaMemcpyAsync(&err, &ctrl->err.w[0], sizeof(err), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    if (cudaMemcpyAsync(&err, &ctrl->rep.err, sizeof(err), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return MAXFLOW_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return MAXFLOW_ERR_CUDA;
     return err == MF_E_NONE ? MAXFLOW_OK : MAXFLOW_ERR_INTERNAL;

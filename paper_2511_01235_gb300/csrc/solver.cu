@@ -254,7 +254,6 @@ __device__ __forceinline__ void decide_iteration(const MfParams &P, Sh &sh, int 
     for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = d.wl_app[b];
     pick_round(P, d);
     if (d.near) d.dis_short = d.dis_solo = 0;        // a near iteration starts with the walks
-    if (vb() == 0 && st.iters < MF_ACTIVE_HIST) P.ctrl->active_hist[st.iters] = active;
     if (st.iters == 0) st.active_first = active;
     st.active_total += active;
     if (active == 0) {
@@ -453,7 +452,7 @@ __device__ __noinline__ void solo_advance(const MfParams &P, int hook, Sh &sh)
     advance(P, hook, sh, gtimer());
     const int i = sh.hs.trace_n - 1;
     if (i >= MF_TRACE) return;
-    MfCtrl *c = P.ctrl;
+    MfReport *c = P.rep;
     c->trace_hook[i] = sh.tr_hook;
     c->trace_t[i] = sh.hs.t_phase;
     c->trace_slots[i] = sh.stat[ST_SLOTS_BFS] + sh.stat[ST_SLOTS_DIS] + sh.stat[ST_SLOTS_FIX];
@@ -484,12 +483,13 @@ __device__ __noinline__ void write_trace(const MfParams &P, Sh &sh, unsigned pha
     fsum = (unsigned long long)warp_sum_ll((long long)fsum);
     slots = (unsigned long long)warp_sum_ll((long long)slots);
     if (lane == 0) {
-        c->trace_hook[i] = sh.tr_hook;
-        c->trace_t[i] = sh.hs.t_phase;
-        c->trace_slots[i] = (long long)slots;
-        c->trace_info[i] = sh.tr_info;
-        c->trace_fin_max[i] = fmax;
-        c->trace_fin_mean[i] = (unsigned)min(fsum / (unsigned long long)n, 0xffffffffull);
+        MfReport *r = P.rep;
+        r->trace_hook[i] = sh.tr_hook;
+        r->trace_t[i] = sh.hs.t_phase;
+        r->trace_slots[i] = (long long)slots;
+        r->trace_info[i] = sh.tr_info;
+        r->trace_fin_max[i] = fmax;
+        r->trace_fin_mean[i] = (unsigned)min(fsum / (unsigned long long)n, 0xffffffffull);
     }
 }
 
@@ -556,7 +556,8 @@ __device__ __forceinline__ bool wait_all(const MfParams &P, Sh &sh)
             if (t0 == 0) {
                 t0 = now;
             } else if (now - t0 > P.wait_limit_ns) {
-                atomicCAS(&c->err.w[0], 0u, (unsigned)MF_E_WAIT);
+                atomicExch(&c->err.w[0], (unsigned)MF_E_WAIT);
+                *(volatile int *)&P.rep->err = MF_E_WAIT;
                 return false;
             }
             if (spins > 4096) __nanosleep(100);
@@ -643,24 +644,31 @@ __device__ __noinline__ bool finish(const MfParams &P, Sh &sh)
                 const int4 zero = make_int4(0, 0, 0, 0);
                 if (lane < MF_LINES)
                     for (int q = 0; q < 3; ++q) __stcg(reinterpret_cast<int4 *>(&c->set[q].l[lane]), zero);
+                MfReport *r = P.rep;
+                if (lane < MF_STATS) r->stat[lane] = __ldcg(&c->stat[lane]);
                 if (lane == 0) {
                     const MfState &st = sh.hs;
                     c->bar.w[0] = 0;
-                    c->d = sh.d;
-                    c->err.w[0] = (unsigned)st.err;
-                    c->iters = st.iters;
-                    c->bfs_levels = st.bfs_levels;
-                    c->active_total = st.active_total;
-                    c->active_first = st.active_first;
-                    c->ns_bfs = st.ns_bfs;
-                    c->ns_dis = st.ns_dis;
-                    c->ns_fix = st.ns_fix;
-                    c->ns_wl = st.ns_wl;
-                    c->ns_apply = st.ns_apply;
-                    c->rounds_total = st.rounds_total;
-                    c->barriers = st.barriers;
-                    c->trace_n = st.trace_n;
-                    c->t_exit = st.t_phase;
+                    c->qstamp = sh.d.qstamp;
+                    c->fstamp = sh.d.fstamp;
+                    r->err = st.err;
+                    r->status = sh.d.status;
+                    r->value = __ldcg(&c->value);
+                    r->iters = st.iters;
+                    r->bfs_levels = st.bfs_levels;
+                    r->active_total = st.active_total;
+                    r->active_first = st.active_first;
+                    r->cut_slots = st.vis_slots;
+                    r->used_slots = st.used_slots;
+                    r->ns_bfs = st.ns_bfs;
+                    r->ns_dis = st.ns_dis;
+                    r->ns_fix = st.ns_fix;
+                    r->ns_wl = st.ns_wl;
+                    r->ns_apply = st.ns_apply;
+                    r->rounds_total = st.rounds_total;
+                    r->barriers = st.barriers;
+                    r->trace_n = st.trace_n;
+                    r->t_exit = st.t_phase;
                 }
             }
         }
@@ -3301,8 +3309,8 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         sh.cs = &c->set[0];
         sh.d = MfDesc{};
         sh.hs = MfState{};
-        sh.d.qstamp = __ldcg(&c->d.qstamp);
-        sh.d.fstamp = __ldcg(&c->d.fstamp);
+        sh.d.qstamp = __ldcg(&c->qstamp);
+        sh.d.fstamp = __ldcg(&c->fstamp);
         sh.d.near = near_allowed(P);
         sh.hs.t_phase = gtimer();
     }
@@ -3310,11 +3318,9 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         // results start at zero; the other CTAs add to them at the end of the launch
         MfCtrl *c = P.ctrl;
         if (threadIdx.x < MF_STATS) c->stat[threadIdx.x] = 0;
-        if (threadIdx.x < MF_ACTIVE_HIST) c->active_hist[threadIdx.x] = 0;
         if (threadIdx.x == 0) {
             c->value = 0;
-            c->err.w[0] = 0;
-            c->t_entry = gtimer();
+            P.rep->t_entry = gtimer();
         }
     }
     __syncthreads();
@@ -3595,27 +3601,119 @@ __global__ void k_check(MfParams P, long long *out)
     atomicAdd((unsigned long long *)&out[5], (unsigned long long)val);
 }
 
-__global__ void k_side(MfParams P, uint8_t *side)
+// The answer of a solve: the source side A = {h = n} and the capacity of the
+// cut.  Both come from one pass over the heights, four vertices per lane; the
+// side goes straight to the caller's (pinned) memory in 128-byte pieces.  The
+// cut is summed over the rows of whichever side has fewer slots: from A the
+// capacities c(u, v) of its slots into the other side, from the other side
+// c(u, v) = pcap - c(v, u) of its slots (v, u) into A, without a gather through
+// rev.  Warps take the rows of 32 vertices as one concatenated range; a row of
+// more than kAnswerLong slots goes to its whole CTA, and the terminal's row,
+// which on grids holds an edge to every pixel, to all CTAs (one warp per row
+// took 1.5 ms for the 262 K slots of a 512 x 512 grid's source).  The last CTA
+// to finish writes the sum and leaves the accumulators at zero.
+constexpr int kAnswerThreads = 256, kAnswerLong = 1024, kAnswerList = 128;
+
+__device__ __forceinline__ long long answer_slot(const MfParams &P, int x, bool from_sink)
 {
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < P.g.n;
-         v += (long long)gridDim.x * blockDim.x)
-        side[v] = (P.h[v] == P.g.n) ? 1 : 0;
+    const int hz = ldg_cg(P.h + ldg_cg(P.g.dst + x));
+    if (from_sink) return hz == P.g.n ? (long long)ldg_cg(P.g.pcap + x) - ldg_cg(P.g.cap + x) : 0;
+    return hz < P.g.n ? ldg_cg(P.g.cap + x) : 0;
 }
 
-__global__ void k_cut(MfParams P, long long *out)
+__global__ void __launch_bounds__(kAnswerThreads) k_answer(MfParams P, MfAnswer A)
 {
-    const int n = P.g.n;
-    const int lane = threadIdx.x & 31;
-    long long cut = 0;
-    for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n;
-         w += ((long long)gridDim.x * blockDim.x) >> 5) {
-        if (P.h[w] != n) continue;
-        int r0 = P.g.off[w], d = P.g.deg[w];
-        for (int j = lane; j < d; j += 32)
-            if (P.h[P.g.dst[r0 + j]] < n) cut += P.g.cap[r0 + j];
+    __shared__ int longs[kAnswerList];
+    __shared__ int nlong;
+    __shared__ long long part[kAnswerThreads / 32];
+    const int n = P.g.n, tid = threadIdx.x, lane = tid & 31;
+    const bool want = A.cut != nullptr, fs = A.from_sink != 0;
+    const int term = fs ? P.sink : P.source;
+    if (tid == 0) nlong = 0;
+    __syncthreads();
+    long long sum = 0;
+    const long long nw = (long long)gridDim.x * (kAnswerThreads / 32);
+    for (long long w = (long long)blockIdx.x * (kAnswerThreads / 32) + (tid >> 5); w * 128 < n; w += nw) {
+        const int v0 = (int)(w * 128) + 4 * lane;
+        int h[4];
+        if (v0 + 4 <= n) {
+            const int4 q = __ldcg(reinterpret_cast<const int4 *>(P.h + v0));
+            h[0] = q.x, h[1] = q.y, h[2] = q.z, h[3] = q.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) h[k] = v0 + k < n ? ldg_cg(P.h + v0 + k) : -1;
+        }
+        if (A.side) {
+            if (v0 + 4 <= n) {
+                *reinterpret_cast<uchar4 *>(A.side + v0) = make_uchar4(h[0] == n, h[1] == n, h[2] == n, h[3] == n);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (v0 + k < n) A.side[v0 + k] = h[k] == n;
+            }
+        }
+        if (!want) continue;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int v = v0 + k;
+            const bool mine = h[k] >= 0 && (h[k] == n) != fs && v != term;
+            if (!__any_sync(0xffffffffu, mine)) continue;
+            const int r0 = mine ? P.g.off[v] : 0;
+            int d = mine ? ldg_cg(P.g.deg + v) : 0;
+            if (d > kAnswerLong) {
+                const int i = atomicAdd(&nlong, 1);
+                if (i < kAnswerList) {
+                    longs[i] = v;
+                    d = 0;
+                }
+            }
+            int incl = d;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int excl = incl - d, T = __shfl_sync(0xffffffffu, incl, 31);
+            for (int kb = 0; kb < T; kb += 128) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int j = kb + r * 32 + lane;
+                    int owner = 0;
+#pragma unroll
+                    for (int st = 16; st >= 1; st >>= 1) {
+                        const int cand = owner + st;
+                        const int ec = __shfl_sync(0xffffffffu, excl, cand & 31);
+                        if (cand < 32 && ec <= j) owner = cand;
+                    }
+                    const int rb = __shfl_sync(0xffffffffu, r0, owner), eb = __shfl_sync(0xffffffffu, excl, owner);
+                    if (j < T) sum += answer_slot(P, rb + (j - eb), fs);
+                }
+            }
+        }
     }
-    cut = warp_sum_ll(cut);
-    if (lane == 0 && cut) atomicAdd((unsigned long long *)out, (unsigned long long)cut);
+    if (!want) return;
+    const int t0 = P.g.off[term], td = ldg_cg(P.g.deg + term);
+    for (long long j = (long long)blockIdx.x * kAnswerThreads + tid; j < td; j += (long long)gridDim.x * kAnswerThreads)
+        sum += answer_slot(P, t0 + (int)j, fs);
+    __syncthreads();
+    for (int i = 0; i < min(nlong, kAnswerList); ++i) {
+        const int r0 = P.g.off[longs[i]], d = ldg_cg(P.g.deg + longs[i]);
+        for (int j = tid; j < d; j += kAnswerThreads) sum += answer_slot(P, r0 + j, fs);
+    }
+    sum = warp_sum_ll(sum);
+    if (lane == 0) part[tid >> 5] = sum;
+    __syncthreads();
+    if (tid == 0) {
+        long long t = 0;
+        for (int i = 0; i < kAnswerThreads / 32; ++i) t += part[i];
+        if (t) atomic_add_ll(A.acc, t);
+        __threadfence();
+        if (atomic_add_ll(A.acc + 1, 1) + 1 == (long long)gridDim.x) {
+            __threadfence();
+            *A.cut = __ldcg(A.acc);
+            A.acc[0] = A.acc[1] = 0;
+        }
+    }
 }
 
 __global__ void k_reverse_cf(MfParams P, const int32_t *in, int32_t *out)
@@ -3981,14 +4079,13 @@ int mf_launch_aux(int which, const MfParams &p, void *stream, long long *dev_out
         if (cudaGetLastError() != cudaSuccess) return MAXFLOW_ERR_CUDA;
         k_excess<<<gv, B, 0, st>>>(p, dev_out + 1);
         break;
-    case MF_AUX_SIDE:
-        k_side<<<gv, B, 0, st>>>(p, (uint8_t *)extra);
-        break;
-    case MF_AUX_CUT: {
-        int g = (int)((nv * 32 + B - 1) / B);
-        if (g > 65535) g = 65535;
-        if (g < 1) g = 1;
-        k_cut<<<g, B, 0, st>>>(p, dev_out);
+    case MF_AUX_ANSWER: {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return MAXFLOW_ERR_CUDA;
+        const long long blocks = (nv + 4 * kAnswerThreads - 1) / (4 * kAnswerThreads);
+        k_answer<<<(int)(blocks < 8ll * sms ? blocks : 8ll * sms), kAnswerThreads, 0, st>>>(p, *(const MfAnswer *)extra);
         break;
     }
     case MF_AUX_REVERSE_CF: {

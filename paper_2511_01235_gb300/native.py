@@ -315,10 +315,10 @@ def maxflow_apply(h, u, v, c):
 def maxflow_query(h, n: int, side: bool = False, cut: bool = False):
     val = C.c_int64()
     cc = C.c_int64()
-    sd = np.zeros(n, np.uint8) if side else None
+    sd = np.empty(n, np.uint8) if side else None       # written whole by the call
     rc = load().maxflow_query(h, C.byref(val), _p(sd) if side else None, C.byref(cc) if cut else None)
     _check(rc, "maxflow_query")
-    return int(val.value), (sd.astype(bool) if side else None), (int(cc.value) if cut else None)
+    return int(val.value), (sd.view(np.bool_) if side else None), (int(cc.value) if cut else None)
 
 
 def maxflow_resolve_static(h):
