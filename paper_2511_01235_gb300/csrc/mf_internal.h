@@ -28,6 +28,8 @@
 #define MF_BFS_HUB 256        // BFS: rows above this many slots enter the frontier as work items
 #define MF_BFS_CHUNK 256      // BFS: slots per work item
 #define MF_DEFAULT_ROUNDS 2   // adaptive discharge rounds: the minimum per iteration
+#define MF_DIS_PARTS 1        // adaptive rounds: the discharge may take MF_DIS_PARTS / MF_BFS_PARTS
+#define MF_BFS_PARTS 1        // of its BFS's time
 #define MF_MAX_ROUNDS 1024    // adaptive rounds: upper bound per iteration
 #define MF_TRACE 256          // hook timeline entries kept per launch
 #define MF_BU_ALPHA 14        // BFS default: go bottom-up when the frontier's slots exceed the unexplored slots / alpha

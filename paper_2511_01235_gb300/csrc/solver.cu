@@ -157,7 +157,7 @@ __device__ __forceinline__ int warp_rank(int nctas, int skip)
 {
     const int nw = nctas * (int)(blockDim.x >> 5);
     const int r = (int)(threadIdx.x >> 5) * nctas + vb();
-    const int s = skip % nw;
+    const int s = skip < nw ? skip : skip % nw;
     return r >= s ? r - s : r - s + nw;
 }
 
@@ -179,6 +179,8 @@ struct Sh {
     unsigned phase;                   // barriers passed in this launch
     MfSet *cs;                        // the counter set of the running phase
     int tr_hook, tr_info;             // of the last barrier, for the trace
+    // of the parameters, for advance(): BFS direction switch, worklist wanted, longest level run alone (slots; 0: none)
+    int k_alpha, k_beta, k_wl, k_solo;
     // a run of small phases in the first CTA: entries of the next queue, of the
     // next lists per bin, work items
     int so_cnt, so_wl[MF_NBIN], so_hub, so_go;
@@ -221,10 +223,15 @@ __device__ __forceinline__ unsigned long long cnt64(const Sh &sh, int line)
 
 // A top-down level of cnt vertices with fr slots, none of them long, that the
 // first CTA runs alone (solo_bfs).
-__device__ __forceinline__ bool solo_level(const MfParams &P, long long cnt, long long fr)
+__device__ __forceinline__ bool solo_level(const Sh &sh, long long cnt, long long fr)
 {
-    return cnt <= MF_SOLO_LEVEL && fr <= (P.tail_slots > 0 ? P.tail_slots : MF_SOLO_SLOTS) && !P.pull &&
-           P.stage_slots >= MF_SOLO_INTS;
+    return cnt <= MF_SOLO_LEVEL && fr <= sh.k_solo;
+}
+
+// Adaptive rounds: whether this iteration's discharge may still take time beside its BFS.
+__device__ __forceinline__ bool rounds_left(const MfState &st, unsigned long long t)
+{
+    return MF_BFS_PARTS * (t - st.t_dis0) < MF_DIS_PARTS * (st.t_dis0 - st.t_bfs0);
 }
 
 // How the coming discharge round over the worklists in d runs.  Short: a push
@@ -235,7 +242,8 @@ __device__ __forceinline__ void pick_round(const MfParams &P, MfDesc &d)
 {
     d.dis_short = P.rounds == 0 && !P.pull && !P.fix_steep && P.data_driven && P.requeue &&
                           P.stage_slots >= MF_SOLO_INTS && P.hub_deg <= MF_SHORT_ROW &&
-                          P.g.slot_cap >= MF_LARGE_SLOTS && d.wl_n[2] + d.wl_n[3] == 0
+                          (P.g.slot_cap >= MF_LARGE_SLOTS || d.round >= MF_DEFAULT_ROUNDS) &&
+                          d.wl_n[2] + d.wl_n[3] == 0
                       ? 1 : 0;
     d.dis_solo = d.dis_short && d.wl_n[0] + d.wl_n[1] <= MF_SOLO_ACTIVE ? 1 : 0;
 }
@@ -293,6 +301,87 @@ __device__ __forceinline__ void begin_iteration(Sh &sh)
     d.bu_mode = 0;
 }
 
+// After a phase of the BFS.  On the critical path of every level: all it needs
+// is read before anything is written, so its shared-memory accesses overlap
+// instead of following one another.  Returns what the trace shows.
+__device__ __forceinline__ int advance_bfs(const MfParams &P, int &hook, Sh &sh)
+{
+    MfDesc &d = sh.d;
+    MfState &st = sh.hs;
+    const int c_bfs = cnt32(sh, L_BFS), c_hub = cnt32(sh, L_HUB), c_defer = cnt32(sh, L_DEFER);
+    const int c_w0 = cnt32(sh, L_WL), c_w1 = cnt32(sh, L_WL + 1), c_w2 = cnt32(sh, L_WL + 2), c_w3 = cnt32(sh, L_WL + 3);
+    const unsigned long long lab = cnt64(sh, L_LAB), exc = cnt64(sh, L_EXC);
+    const int alpha = sh.k_alpha, beta = sh.k_beta, want_wl = sh.k_wl, n = P.g.n, near = d.near;
+    const int app_bfs = d.app_bfs + c_bfs, app_hub = d.app_hub + c_hub;
+    const int w0 = d.wl_app[0] + c_w0, w1 = d.wl_app[1] + c_w1, w2 = d.wl_app[2] + c_w2, w3 = d.wl_app[3] + c_w3;
+    const int lvl_hi = d.lvl_hi, hub_hi = d.hub_hi, hub_lo = d.hub_lo, level = d.level, bu_was = d.bu_mode;
+    const long long fr = st.lvl_slots + (long long)(lab & 0xffffffffull), cnt = st.lvl_cnt + (long long)(lab >> 32);
+    const long long sup = st.sup + (long long)exc, levels = st.bfs_levels;
+    long long used = st.used_slots, dem = st.dem;
+    const long long vis = st.vis_slots + fr;
+    int shift = st.cut_shift;
+    // the lists grew by what the phase appended
+    d.app_bfs = app_bfs;
+    d.app_hub = app_hub;
+    d.wl_app[0] = w0;
+    d.wl_app[1] = w1;
+    d.wl_app[2] = w2;
+    d.wl_app[3] = w3;
+    st.sup = sup;
+    if (hook == H_BU_SPLIT) {
+        // after the first pass of a bottom-up level: a second pass over the
+        // deferred long rows, or (none deferred) the level is complete
+        d.defer_n = c_defer;
+        d.bu_split = c_defer > 0 ? 1 : 0;
+        if (c_defer > 0) {
+            st.lvl_slots = fr;
+            st.lvl_cnt = cnt;
+            return (1 << 30) | min(c_defer, (1 << 20) - 1);
+        }
+        hook = H_BFS_NEXT;
+    }
+    const bool first = hook == H_BFS_START;
+    if (first) {
+        if (d.need_total) st.used_slots = used = (long long)cnt64(sh, L_TOTAL);
+        if (near) {
+            // a cut-short relabel whose walks settled less than half of what was
+            // open looks for more excess this time, so that after a few of them
+            // the relabel is a complete one
+            dem = (long long)cnt64(sh, L_DEM);
+            if (st.cut_prev && 2 * dem > st.dem_prev) shift = min(shift + MF_NEAR_STEP, 60);
+            st.cut_shift = shift;
+            st.dem = st.dem_prev = dem;
+        }
+    }
+    const bool done = lvl_hi == app_bfs && hub_hi == app_hub;
+    if (!first && !done) st.bfs_levels = levels + 1;
+    d.lvl_lo = lvl_hi;
+    d.hub_lo = hub_hi;
+    d.lvl_hi = app_bfs;
+    d.hub_hi = app_hub;
+    d.level = first ? 0 : level + 1;
+    st.vis_slots = vis;
+    st.lvl_slots = st.lvl_cnt = 0;
+    // direction of the coming level (Beamer's test): bottom-up once the
+    // frontier's slots exceed 1/alpha of the unexplored slots, back to
+    // top-down once it holds fewer than n/beta vertices
+    int bu = bu_was;
+    if (alpha <= 0) bu = 0;
+    else if (!bu && fr * alpha > used - vis) bu = 1;
+    else if (bu && cnt * beta < (long long)n) bu = 0;
+    d.bu_mode = bu;
+    d.bu_split = 0;
+    d.bfs_solo = !done && !bu && app_hub == hub_hi && solo_level(sh, cnt, fr) ? 1 : 0;
+    // near iterations: the levels so far hold as much excess as the roots can take
+    const int cut = near && !done && sup > 0 && (sup >> shift) >= dem ? 1 : 0;
+    d.cut = cut;
+    st.cut_prev = cut;
+    d.bfs_done = done || cut ? 1 : 0;
+    if ((done || cut) && want_wl) decide_iteration(P, sh, w0 + w1 + w2 + w3);
+    return ((first ? 0 : bu_was) << 30) | ((first ? 0 : min(hub_hi - hub_lo, 1023)) << 20) |
+           (int)min(cnt, (long long)((1 << 20) - 1));
+}
+
 // What comes after a grid barrier: thread 0 of every CTA works it out from the
 // counters of the phase that ended (sh.cnt) and the state all CTAs share, in
 // shared memory only, so all of them arrive at the same answer.  t: the first
@@ -301,32 +390,23 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
 {
     MfDesc &d = sh.d;
     MfState &st = sh.hs;
+    const int trace_n = st.trace_n, perr = sh.cnt[L_MISC].w;
+    const int err = st.err == 0 ? perr : st.err;
+    const long long barriers = st.barriers;
     const unsigned long long now = gtimer(), dt = now - st.t_phase;
     st.t_phase = now;
     st.t_now = t;
-    if (st.barriers == 0) st.t_start = t;
-    ++st.barriers;
-    if (st.err == 0) st.err = sh.cnt[L_MISC].w;
+    if (barriers == 0) st.t_start = t;
+    st.barriers = barriers + 1;
+    st.trace_n = trace_n + 1;
+    st.err = err;
     int tinfo = 0;
-    const bool want_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
     if (hook == H_BU_SPLIT || hook == H_BFS_START || hook == H_BFS_NEXT) {
-        // the lists grew by what the phase appended
         st.ns_bfs += dt;
-        d.app_bfs += cnt32(sh, L_BFS);
-        d.app_hub += cnt32(sh, L_HUB);
-        for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] += cnt32(sh, L_WL + b);
-        const unsigned long long lab = cnt64(sh, L_LAB);
-        st.lvl_slots += (long long)(lab & 0xffffffffull);
-        st.lvl_cnt += (long long)(lab >> 32);
-        st.sup += (long long)cnt64(sh, L_EXC);
-        if (hook == H_BU_SPLIT) {
-            // after the first pass of a bottom-up level: a second pass over the
-            // deferred long rows, or (none deferred) the level is complete
-            d.defer_n = cnt32(sh, L_DEFER);
-            d.bu_split = d.defer_n > 0 ? 1 : 0;
-            tinfo = (1 << 30) | min(d.defer_n, (1 << 20) - 1);
-            if (!d.bu_split) hook = H_BFS_NEXT;
-        }
+        sh.tr_info = advance_bfs(P, hook, sh);
+        sh.tr_hook = hook;
+        if (err != 0) d.status = MF_ST_ERROR;
+        return;
     }
     switch (hook) {
     case H_APPLY_VALID:
@@ -347,53 +427,6 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         else st.ns_fix += dt;
         begin_iteration(sh);
         break;
-    case H_BFS_START:
-    case H_BFS_NEXT: {
-        const bool first = hook == H_BFS_START;
-        if (first && d.need_total) st.used_slots = (long long)cnt64(sh, L_TOTAL);
-        if (first && d.near) {
-            // a cut-short relabel whose walks settled less than half of what was
-            // open looks for more excess this time, so that after a few of them
-            // the relabel is a complete one
-            st.dem = (long long)cnt64(sh, L_DEM);
-            if (st.cut_prev && 2 * st.dem > st.dem_prev) st.cut_shift = min(st.cut_shift + MF_NEAR_STEP, 60);
-            st.dem_prev = st.dem;
-        }
-        const int items = d.hub_hi - d.hub_lo;
-        d.lvl_lo = d.lvl_hi;
-        d.hub_lo = d.hub_hi;
-        d.lvl_hi = d.app_bfs;
-        d.hub_hi = d.app_hub;
-        const bool done = d.lvl_lo == d.lvl_hi && d.hub_lo == d.hub_hi;
-        if (!first && !done) ++st.bfs_levels;
-        d.level = first ? 0 : d.level + 1;
-        d.bfs_done = done;
-        // direction of the coming level (Beamer's test): bottom-up once the
-        // frontier's slots exceed 1/alpha of the unexplored slots, back to
-        // top-down once it holds fewer than n/beta vertices
-        const long long fr = st.lvl_slots, cnt = st.lvl_cnt;
-        st.vis_slots += fr;
-        st.lvl_slots = st.lvl_cnt = 0;
-        tinfo = ((first ? 0 : d.bu_mode) << 30) | ((first ? 0 : min(items, 1023)) << 20) |
-                (int)min(cnt, (long long)((1 << 20) - 1));
-        int bu = d.bu_mode;
-        if (P.bu_alpha <= 0) bu = 0;
-        else if (!bu && fr * P.bu_alpha > st.used_slots - st.vis_slots) bu = 1;
-        else if (bu && cnt * P.bu_beta < (long long)P.g.n) bu = 0;
-        d.bu_mode = bu;
-        d.bu_split = 0;
-        d.bfs_solo = !done && !bu && d.hub_hi == d.hub_lo && solo_level(P, cnt, fr) ? 1 : 0;
-        // near iterations: the levels so far hold as much excess as the roots can take
-        d.cut = d.near && !done && st.sup > 0 && (st.sup >> st.cut_shift) >= st.dem ? 1 : 0;
-        st.cut_prev = d.cut;
-        if (d.cut) d.bfs_done = 1;
-        if (d.bfs_done && want_wl) {
-            int active = 0;
-            for (int b = 0; b < MF_NBIN; ++b) active += d.wl_app[b];
-            decide_iteration(P, sh, active);
-        }
-        break;
-    }
     case H_WL:
         st.ns_wl += dt;
         for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] = cnt32(sh, L_WL + b);
@@ -418,9 +451,9 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         if (d.near && d.round == 0) {
             // the walks: rounds follow only a complete relabel, and only while
             // they are cheap beside it
-            more = more && !d.cut && 2 * (t - st.t_dis0) < st.t_dis0 - st.t_bfs0;
+            more = more && !d.cut && rounds_left(st, t);
         } else if (more && d.round + 1 >= (P.rounds > 0 ? P.rounds : MF_DEFAULT_ROUNDS))
-            more = P.rounds > 0 ? false : 2 * (t - st.t_dis0) < st.t_dis0 - st.t_bfs0;
+            more = P.rounds > 0 ? false : rounds_left(st, t);
         d.dis_more = more ? 1 : 0;
         if (more) {
             d.wl_sel ^= 1;
@@ -442,7 +475,6 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
     }
     sh.tr_hook = hook;
     sh.tr_info = tinfo;
-    ++st.trace_n;
     if (st.err != 0) d.status = MF_ST_ERROR;
 }
 
@@ -470,18 +502,21 @@ __device__ __noinline__ void write_trace(const MfParams &P, Sh &sh, unsigned pha
     const int i = sh.hs.trace_n - 1;
     if (i >= MF_TRACE) return;
     const unsigned *fin = c->fin[phase % 3], *scn = c->scanned[phase % 3];
-    unsigned fmax = 0;
-    unsigned long long fsum = 0, slots = 0;
+    // hardware reductions of 32-bit words: times in units of 16 ns, the slot counts in halves
+    unsigned fmax = 0, fsum = 0, lo = 0, hi = 0;
     const int n = min(vn(), MF_MAX_CTAS);
     for (int q = lane; q < n; q += 32) {
-        const unsigned f = __ldcg(fin + q);
+        const unsigned f = __ldcg(fin + q), c2 = __ldcg(scn + q);
         fmax = max(fmax, f);
-        fsum += f;
-        slots += __ldcg(scn + q);
+        fsum += min(f, 1u << 25) >> 4;
+        lo += c2 & 0xffffu;
+        hi += c2 >> 16;
     }
     fmax = __reduce_max_sync(0xffffffffu, fmax);
-    fsum = (unsigned long long)warp_sum_ll((long long)fsum);
-    slots = (unsigned long long)warp_sum_ll((long long)slots);
+    fsum = __reduce_add_sync(0xffffffffu, fsum);
+    lo = __reduce_add_sync(0xffffffffu, lo);
+    hi = __reduce_add_sync(0xffffffffu, hi);
+    const unsigned long long slots = (unsigned long long)lo + ((unsigned long long)hi << 16);
     if (lane == 0) {
         MfReport *r = P.rep;
         r->trace_hook[i] = sh.tr_hook;
@@ -489,7 +524,7 @@ __device__ __noinline__ void write_trace(const MfParams &P, Sh &sh, unsigned pha
         r->trace_slots[i] = (long long)slots;
         r->trace_info[i] = sh.tr_info;
         r->trace_fin_max[i] = fmax;
-        r->trace_fin_mean[i] = (unsigned)min(fsum / (unsigned long long)n, 0xffffffffull);
+        r->trace_fin_mean[i] = (unsigned)((unsigned long long)fsum * 16u / (unsigned)n);
     }
 }
 
@@ -2745,7 +2780,7 @@ __device__ __noinline__ void solo_bfs(const MfParams &P, Sh &sh)
             const long long fr = (long long)(unsigned)(sh.lab & 0xffffffffull), lab_n = (long long)(sh.lab >> 32);
             const long long vis = st.vis_slots + fr, sup = st.sup + (long long)sh.exc;
             sh.stat[ST_LAB_BFS] += lab_n;
-            const bool go = c > 0 && sh.so_hub == 0 && solo_level(P, c, fr) &&
+            const bool go = c > 0 && sh.so_hub == 0 && solo_level(sh, c, fr) &&
                             !(P.bu_alpha > 0 && fr * P.bu_alpha > st.used_slots - vis) &&
                             !(d.near && sup > 0 && (sup >> st.cut_shift) >= st.dem) && !solo_timeout(P, t0);
             if (go) {
@@ -3030,7 +3065,7 @@ __device__ __noinline__ void solo_discharge(const MfParams &P, Sh &sh)
             int spill = 0;
             for (int q = 0; q < MF_NBIN; ++q) spill += sh.so_wl[q];
             const unsigned long long now = gtimer();
-            const bool over = d.round + 1 >= MF_DEFAULT_ROUNDS && 2 * (now - st.t_dis0) >= st.t_dis0 - st.t_bfs0;
+            const bool over = d.round + 1 >= MF_DEFAULT_ROUNDS && !rounds_left(st, now);
             sh.so_go = c + spill == 0 || d.round + 1 >= MF_MAX_ROUNDS || over ? 0
                        : spill > 0 || c > MF_SOLO_ACTIVE || solo_timeout(P, t0) ? 2 : 1;
             if (sh.so_go) ++d.round;
@@ -3312,6 +3347,10 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         sh.d.qstamp = __ldcg(&c->qstamp);
         sh.d.fstamp = __ldcg(&c->fstamp);
         sh.d.near = near_allowed(P);
+        sh.k_alpha = P.bu_alpha;
+        sh.k_beta = P.bu_beta;
+        sh.k_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY) ? 1 : 0;
+        sh.k_solo = P.pull || P.stage_slots < MF_SOLO_INTS ? 0 : (P.tail_slots > 0 ? P.tail_slots : MF_SOLO_SLOTS);
         sh.hs.t_phase = gtimer();
     }
     if (vb() == 0) {
