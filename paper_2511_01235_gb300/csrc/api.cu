@@ -50,6 +50,8 @@ struct maxflow_ctx {
     unsigned *multi_gstate = nullptr;
     int multi_cap = 0;
     int grid = 1, per_sm = 1, sms = 1;
+    int max_clustered = 0;        // CTAs that fit the GPU in clusters of MF_CLUSTER (0: no clusters)
+    int cluster = 1;              // CTAs per cluster of this context's launches
     int32_t stage_slots = 0;      // dynamic shared memory of the solve launches, in ints
     int32_t requeue = 1;          // discharge rounds re-queue vertices still active after their cycles
     int32_t cycle_div = 0;        // > 0: long rows get max(kernel_cycles, deg / cycle_div) cycles
@@ -244,6 +246,12 @@ int ensure_batch(maxflow_ctx *c, int64_t count)
     return MAXFLOW_OK;
 }
 
+// Cluster size of a launch of g CTAs (or of groups of g CTAs).
+int cluster_of(const maxflow_ctx *c, int g)
+{
+    return g % MF_CLUSTER == 0 && g <= c->max_clustered ? MF_CLUSTER : 1;
+}
+
 // The context's pinned memory, one block: report, mirror of the small results,
 // packed batch, side.
 int alloc_pinned(maxflow_ctx *c)
@@ -361,15 +369,22 @@ int alloc_vertex_scratch(maxflow_ctx *c)
     return rc_cuda(cudaMemsetAsync(c->sc.ins_need, 0, sizeof(int32_t) * n, c->stream));
 }
 
+// The grid of a context's launches: a CTA per 8192 reserved slots, in clusters
+// of MF_CLUSTER from that many CTAs on (36 clusters fit a GB300, 288 of the 304
+// CTAs that fit without: phases that fill the GPU lose 5 %, the small ones,
+// which the first cluster runs alone, take a third of the time).
 void choose_grid(maxflow_ctx *c)
 {
-    int maxg = c->per_sm * c->sms;
+    const int maxg = c->per_sm * c->sms;
     int g = c->opt.grid_blocks;
     if (g <= 0) {
         double want = std::ceil((double)c->g.slot_cap / 8192.0);
         g = (int)std::min<double>(maxg, std::max(2.0, want));
+        if (g >= MF_CLUSTER && c->max_clustered >= MF_CLUSTER)
+            g = std::min((g + MF_CLUSTER - 1) / MF_CLUSTER * MF_CLUSTER, c->max_clustered);
     }
     c->grid = std::max(1, std::min(g, maxg));
+    c->cluster = cluster_of(c, c->grid);
     c->st.grid_blocks = c->grid;
     c->st.block_threads = MF_BLOCK;
     c->st.blocks_per_sm = c->per_sm;
@@ -448,7 +463,7 @@ int run_kernel(maxflow_ctx *c, const MfParams &p, int *kerr, int *kstatus)
 {
     c->rep->err = MF_E_INTERNAL;      // stands if the kernel does not get to its end
     MF_TRY(rc_cuda(cudaEventRecord(c->ev0, c->stream)));
-    MF_TRY(counted(mf_launch(p, c->grid, (void *)c->stream), 1));
+    MF_TRY(counted(mf_launch(p, c->grid, c->cluster, (void *)c->stream), 1));
     MF_TRY(rc_cuda(cudaEventRecord(c->ev1, c->stream)));
     MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
     float ms = 0.f;
@@ -834,6 +849,7 @@ int maxflow_init(maxflow_ctx **out, const maxflow_graph *g, int32_t s, int32_t t
     int stage_bytes = 0;
     if (rc == MAXFLOW_OK) rc = mf_stage_bytes(dev, &stage_bytes);
     if (rc == MAXFLOW_OK) rc = mf_max_coresident_blocks(dev, &c->per_sm, &c->sms, stage_bytes);
+    if (rc == MAXFLOW_OK) rc = mf_max_clustered_blocks(stage_bytes, &c->max_clustered);
     c->stage_slots = stage_bytes / (int)sizeof(int);
     c->group_deg = std::max<int32_t>(c->hub_deg, c->stage_slots / (MF_BLOCK / (32 * MF_GROUP_WARPS)));
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaEventCreate(&c->ev0));
@@ -1231,7 +1247,8 @@ int maxflow_solve_batched(maxflow_ctx *const *ctxs, int32_t count, const maxflow
     }
     const int maxg = c0->per_sm * c0->sms;
     const int gsize = std::min<int>(group_blocks, maxg);
-    const int ngroups = std::max(1, std::min<int>(maxg / gsize, count));
+    const int cluster = cluster_of(c0, gsize);
+    const int ngroups = std::max(1, std::min<int>((cluster > 1 ? c0->max_clustered : maxg) / gsize, count));
     MF_TRY(ensure_multi(c0, count));
     unsigned *gstate = c0->multi_gstate;
     unsigned *head = gstate + 32 * maxg;
@@ -1242,7 +1259,7 @@ int maxflow_solve_batched(maxflow_ctx *const *ctxs, int32_t count, const maxflow
     unsigned long long wait_ns = plist[0].wait_limit_ns;
     MF_TRY(rc_cuda(cudaEventRecord(c0->ev0, c0->stream)));
     MF_TRY(counted(mf_launch_multi(c0->multi_plist, count, gsize, ngroups * gsize, gstate, head, wait_ns, abort_flag,
-                           (void *)c0->stream, c0->stage_slots * (int)sizeof(int)), 1));
+                           cluster, (void *)c0->stream, c0->stage_slots * (int)sizeof(int)), 1));
     MF_TRY(rc_cuda(cudaEventRecord(c0->ev1, c0->stream)));
     int abort_h = 0;
     MF_TRY(rc_cuda(cudaMemcpyAsync(&abort_h, abort_flag, sizeof(int), cudaMemcpyDeviceToHost, c0->stream)));
@@ -1578,7 +1595,7 @@ int maxflow_update_pp(maxflow_ctx *c, const maxflow_batch *b, int32_t stop_after
     MF_TRY(rc_cuda(cudaMemsetAsync(gstate, 0, sizeof(unsigned) * 32 * (size_t)(maxg + 2), c->stream)));
     MF_TRY(rc_cuda(cudaEventRecord(c->ev0, c->stream)));
     MF_TRY(counted(mf_launch_multi(c->multi_plist, 2, gsize, 2 * gsize, gstate, head, pl[0].wait_limit_ns, abort_flag,
-                           (void *)c->stream, c->stage_slots * (int)sizeof(int)), 1));
+                           2 * gsize <= c->max_clustered ? cluster_of(c, gsize) : 1, (void *)c->stream, c->stage_slots * (int)sizeof(int)), 1));
     MF_TRY(rc_cuda(cudaEventRecord(c->ev1, c->stream)));
     int abort_h = 0;
     MF_TRY(rc_cuda(cudaMemcpyAsync(&abort_h, abort_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream)));
@@ -1670,6 +1687,8 @@ int maxflow_clone(maxflow_ctx *src, maxflow_ctx **out)
     c->group_deg = src->group_deg;
     c->bfs_hub = src->bfs_hub;
     c->per_sm = src->per_sm;
+    c->max_clustered = src->max_clustered;
+    c->cluster = src->cluster;
     c->stage_slots = src->stage_slots;
     c->requeue = src->requeue;
     c->cycle_div = src->cycle_div;

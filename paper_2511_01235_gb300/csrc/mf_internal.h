@@ -28,8 +28,6 @@
 #define MF_BFS_HUB 256        // BFS: rows above this many slots enter the frontier as work items
 #define MF_BFS_CHUNK 256      // BFS: slots per work item
 #define MF_DEFAULT_ROUNDS 2   // adaptive discharge rounds: the minimum per iteration
-#define MF_DIS_PARTS 1        // adaptive rounds: the discharge may take MF_DIS_PARTS / MF_BFS_PARTS
-#define MF_BFS_PARTS 1        // of its BFS's time
 #define MF_MAX_ROUNDS 1024    // adaptive rounds: upper bound per iteration
 #define MF_TRACE 256          // hook timeline entries kept per launch
 #define MF_BU_ALPHA 14        // BFS default: go bottom-up when the frontier's slots exceed the unexplored slots / alpha
@@ -46,11 +44,13 @@
 #define MF_Q_LONG 2048        // ... those with long rows,
 #define MF_Q_WL 4096          // ... worklist entries of one phase (vertex; bin and place)
 #define MF_Q_INTS (MF_Q_BFS + MF_Q_LONG + 2 * MF_Q_WL)
-#define MF_SOLO_CAP 4096      // queue entries of a run of small phases that the first CTA does alone
-#define MF_SOLO_INTS (6 * MF_SOLO_CAP)   // its shared memory: two queues of vertex, row start, row length
-#define MF_SOLO_LEVEL 256     // BFS levels of at most this many vertices ...
-#define MF_SOLO_SLOTS 2048    // ... and slots run alone
-#define MF_SOLO_ACTIVE 256    // discharge rounds of at most this many vertices run alone
+#define MF_CLUSTER 8          // CTAs per thread-block cluster; the first cluster is the squad
+#define MF_SQUAD_CAP 4096     // queue entries of a squad CTA
+#define MF_SQUAD_INTS (6 * MF_SQUAD_CAP)   // its shared memory: two queues of vertex, row start, row length
+#define MF_SQUAD_LEVEL 256    // BFS levels of at most this many vertices per squad CTA ...
+#define MF_SQUAD_SLOTS 2048   // ... and slots run in the squad
+#define MF_SQUAD_ACTIVE 256   // so do discharge rounds of at most this many vertices per squad CTA
+#define MF_DEEP 16            // short rounds on a smaller graph: after a BFS of at least this many levels
 #define MF_SHORT_ROW 512      // rounds of one cycle per vertex: the longest row
 
 // Solve-kernel status (ctrl->status)
@@ -130,9 +130,9 @@ struct MfDesc {
     int bu_mode;                  // the coming BFS level runs bottom-up
     int bu_split;                 // the bottom-up level just scanned deferred long rows: their pass follows
     int defer_n;                  // work items of that pass
-    int bfs_solo;                 // the coming top-down level is small: the first CTA runs it, and the next small ones, alone
+    int bfs_squad;                // the coming top-down level is small: the squad runs it, and the next small ones, alone
     int dis_short;                // the coming discharge round has short rows only: one cycle per vertex
-    int dis_solo;                 // ... and few of them: the first CTA runs it, and the next small ones, alone
+    int dis_squad;                // ... and few of them: the squad runs it, and the next small ones, alone
     int need_total;               // the coming BFS roots pass sums the used slots (first BFS of a launch)
     int wl_sel;                   // which worklist buffer the current round reads
     int wl_n[MF_NBIN];
@@ -213,7 +213,7 @@ struct MfCtrl {
     long long stat[MF_STATS];
     MfLine bar;           // w[0]: arrivals in this launch (the first CTA leaves it at zero)
     MfSet set[3];
-    // the first CTA's state for the others, after it ran phases alone
+    // the first CTA's state for the others, after its squad ran phases alone
     MfDesc jd;
     MfState js;
     // per phase (mod 3) and CTA: finish time, slots scanned
@@ -288,7 +288,7 @@ struct MfParams {
     int32_t requeue;          // discharge rounds: a vertex still active after its cycles joins the next round
     int32_t cycle_div;        // > 0: a row of d slots gets max(kernel_cycles, d / cycle_div) cycles
     int32_t tail_slots;       // BFS: a top-down level whose frontier holds at most this many slots (and
-                              // vertices) runs in CTA 0 alone, without grid barriers; 0: MF_SOLO_SLOTS
+                              // vertices) runs in the squad, without grid barriers; 0: MF_SQUAD_SLOTS per CTA
     int32_t stage_slots;      // dynamic shared memory of the launch in ints: the discharge's on-chip row snapshot
                               // (a CTA keeps rows up to this many slots; 0: none)
     long long max_iters;
@@ -314,11 +314,13 @@ int mf_build_host(int32_t n, int64_t m, const int32_t *src, const int32_t *dst, 
                   float slack_factor, int32_t slack_min, MfHostGraph &out);
 
 // solver.cu
-int mf_launch(const MfParams &p, int grid, void *stream);
+// cluster: 1, or MF_CLUSTER (then grid, and gsize, are multiples of it)
+int mf_launch(const MfParams &p, int grid, int cluster, void *stream);
 int mf_launch_multi(const MfParams *plist_dev, int count, int gsize, int grid, unsigned *gstate, unsigned *head,
-                    unsigned long long wait_ns, int *abort, void *stream, int stage_bytes);
+                    unsigned long long wait_ns, int *abort, int cluster, void *stream, int stage_bytes);
 int mf_stage_bytes(int device, int *bytes);
 int mf_max_coresident_blocks(int device, int *per_sm, int *num_sms, int dyn_bytes);
+int mf_max_clustered_blocks(int dyn_bytes, int *blocks);   // with clusters of MF_CLUSTER; 0 where there are none
 int mf_launch_aux(int which, const MfParams &p, void *stream, long long *dev_out, const void *extra);
 
 #define MF_AUX_SET_CF_RESET 1     // cf = cap on all used slots

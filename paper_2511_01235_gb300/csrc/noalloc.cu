@@ -150,7 +150,7 @@ extern "C" int maxflow_global_relabel_noalloc(int32_t n, int32_t s, int32_t t, c
     int grid = (int)((n + 2047) / 2048);
     if (grid < 2) grid = 2;
     if (grid > maxg) grid = maxg;
-    rc = mf_launch(p, grid, stream);
+    rc = mf_launch(p, grid, 1, stream);
     if (rc != MAXFLOW_OK) return rc;
     mf_note_launches(1);
     unsigned err = 0;

@@ -161,6 +161,19 @@ __device__ __forceinline__ int warp_rank(int nctas, int skip)
     return r >= s ? r - s : r - s + nw;
 }
 
+// What one CTA of the squad tells the others after a phase.
+struct alignas(16) SquadSum {
+    int cnt;              // entries of its next queue
+    unsigned slots;       // BFS: their slots (with those of long rows)
+    int labelled;         // BFS: vertices labelled
+    int flag;             // SQ_*
+    long long exc;        // near BFS: excess labelled
+    long long pad;
+};
+enum { SQ_SPILL = 1,      // something went onto the grid's lists: long rows, a full queue
+       SQ_STOP = 2,       // (first CTA) the grid should take over: out of time
+       SQ_OVER = 4 };     // (first CTA) the discharge has had its share of the time
+
 // What a CTA keeps in shared memory: its accumulators, its copy of the launch's
 // state (the same in every CTA between two barriers), and work space of phases.
 struct Sh {
@@ -179,11 +192,15 @@ struct Sh {
     unsigned phase;                   // barriers passed in this launch
     MfSet *cs;                        // the counter set of the running phase
     int tr_hook, tr_info;             // of the last barrier, for the trace
-    // of the parameters, for advance(): BFS direction switch, worklist wanted, longest level run alone (slots; 0: none)
-    int k_alpha, k_beta, k_wl, k_solo;
-    // a run of small phases in the first CTA: entries of the next queue, of the
-    // next lists per bin, work items
-    int so_cnt, so_wl[MF_NBIN], so_hub, so_go;
+    // of the parameters, for advance(): BFS direction switch, worklist wanted, longest level of the squad (slots; 0: none)
+    int k_alpha, k_beta, k_wl, k_squad;
+    // the squad: its CTAs, this one's rank, whether it is the whole solve; what
+    // each of its CTAs found in a phase (two sets, written by their owners into
+    // every CTA); this CTA's entries of the next queue
+    int csize, crank, one_cluster;
+    unsigned arrivals;                // arrivals at the grid barrier so far
+    SquadSum sq[2][MF_CLUSTER];
+    int so_cnt, so_flag, so_go, so_par;
     // on-chip queue of a phase (place_labelled, place_active): entries taken, per kind
     int q_bfs, q_long, q_wn, q_wl[MF_NBIN];
     int q_base[MF_NBIN + 1];
@@ -206,7 +223,7 @@ enum Hook {
     H_DIS,
     H_FINAL,
     H_BU_SPLIT,
-    H_JOIN,               // the first CTA has run small phases alone: the others take its state
+    H_JOIN,               // unused (a squad's run ends like the phase it ended with); keeps the trace ids
     H_EXPANDED,           // unused (long rows are split into work items as they are queued); keeps the trace ids
 };
 
@@ -222,30 +239,35 @@ __device__ __forceinline__ unsigned long long cnt64(const Sh &sh, int line)
 }
 
 // A top-down level of cnt vertices with fr slots, none of them long, that the
-// first CTA runs alone (solo_bfs).
-__device__ __forceinline__ bool solo_level(const Sh &sh, long long cnt, long long fr)
+// squad runs alone (squad_bfs).
+__device__ __forceinline__ bool squad_level(const Sh &sh, long long cnt, long long fr)
 {
-    return cnt <= MF_SOLO_LEVEL && fr <= sh.k_solo;
+    return sh.k_squad > 0 && cnt <= MF_SQUAD_LEVEL * sh.csize && fr <= sh.k_squad;
 }
 
-// Adaptive rounds: whether this iteration's discharge may still take time beside its BFS.
-__device__ __forceinline__ bool rounds_left(const MfState &st, unsigned long long t)
+// Adaptive rounds: whether this iteration's discharge may still take time beside
+// its BFS: half of it with rounds of KERNEL_CYCLES cycles, all of it with short
+// ones (grid 1024 window 15.5 -> 13.6 ms, 64 batched instances 14.6 -> 11.6 ms;
+// twice the BFS's time 13.5 and 11.0, but a 512 grid's static solve 33 -> 36).
+__device__ __forceinline__ bool rounds_left(const MfDesc &d, const MfState &st, unsigned long long t)
 {
-    return MF_BFS_PARTS * (t - st.t_dis0) < MF_DIS_PARTS * (st.t_dis0 - st.t_bfs0);
+    return (d.dis_short ? 1 : 2) * (t - st.t_dis0) < st.t_dis0 - st.t_bfs0;
 }
 
 // How the coming discharge round over the worklists in d runs.  Short: a push
 // with the default schedule over rows of at most MF_SHORT_ROW slots gets one
-// cycle per vertex (phase_discharge_short), and a few vertices are left to the
-// first CTA (solo_discharge).
-__device__ __forceinline__ void pick_round(const MfParams &P, MfDesc &d)
+// cycle per vertex (phase_discharge_short), and few vertices are left to the
+// squad (squad_discharge).  On a small graph that takes a BFS of many levels:
+// short rounds pay where many rounds follow; where two or three do, the whole
+// KERNEL_CYCLES in each settle more.
+__device__ __forceinline__ void pick_round(const MfParams &P, MfDesc &d, int csize)
 {
     d.dis_short = P.rounds == 0 && !P.pull && !P.fix_steep && P.data_driven && P.requeue &&
-                          P.stage_slots >= MF_SOLO_INTS && P.hub_deg <= MF_SHORT_ROW &&
-                          (P.g.slot_cap >= MF_LARGE_SLOTS || d.round >= MF_DEFAULT_ROUNDS) &&
+                          P.stage_slots >= MF_SQUAD_INTS && P.hub_deg <= MF_SHORT_ROW &&
+                          (P.g.slot_cap >= MF_LARGE_SLOTS || d.level >= MF_DEEP) &&
                           d.wl_n[2] + d.wl_n[3] == 0
                       ? 1 : 0;
-    d.dis_solo = d.dis_short && d.wl_n[0] + d.wl_n[1] <= MF_SOLO_ACTIVE ? 1 : 0;
+    d.dis_squad = d.dis_short && d.wl_n[0] + d.wl_n[1] <= MF_SQUAD_ACTIVE * csize ? 1 : 0;
 }
 
 // The termination test of the loop (Alg. 1 / Alg. 5: stop when no active
@@ -260,8 +282,8 @@ __device__ __forceinline__ void decide_iteration(const MfParams &P, Sh &sh, int 
     ++d.fstamp;
     st.t_dis0 = st.t_now;
     for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = d.wl_app[b];
-    pick_round(P, d);
-    if (d.near) d.dis_short = d.dis_solo = 0;        // a near iteration starts with the walks
+    pick_round(P, d, sh.csize);
+    if (d.near) d.dis_short = d.dis_squad = 0;        // a near iteration starts with the walks
     if (st.iters == 0) st.active_first = active;
     st.active_total += active;
     if (active == 0) {
@@ -371,7 +393,7 @@ __device__ __forceinline__ int advance_bfs(const MfParams &P, int &hook, Sh &sh)
     else if (bu && cnt * beta < (long long)n) bu = 0;
     d.bu_mode = bu;
     d.bu_split = 0;
-    d.bfs_solo = !done && !bu && app_hub == hub_hi && solo_level(sh, cnt, fr) ? 1 : 0;
+    d.bfs_squad = !done && !bu && app_hub == hub_hi && squad_level(sh, cnt, fr) ? 1 : 0;
     // near iterations: the levels so far hold as much excess as the roots can take
     const int cut = near && !done && sup > 0 && (sup >> shift) >= dem ? 1 : 0;
     d.cut = cut;
@@ -451,16 +473,16 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         if (d.near && d.round == 0) {
             // the walks: rounds follow only a complete relabel, and only while
             // they are cheap beside it
-            more = more && !d.cut && rounds_left(st, t);
+            more = more && !d.cut && rounds_left(d, st, t);
         } else if (more && d.round + 1 >= (P.rounds > 0 ? P.rounds : MF_DEFAULT_ROUNDS))
-            more = P.rounds > 0 ? false : rounds_left(st, t);
+            more = P.rounds > 0 ? false : rounds_left(d, st, t);
         d.dis_more = more ? 1 : 0;
         if (more) {
             d.wl_sel ^= 1;
             for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = cnt32(sh, L_AUX + b);
             ++d.round;
             ++d.qstamp;
-            pick_round(P, d);
+            pick_round(P, d, sh.csize);
         } else if (!P.fix_steep) {
             // without Alg. 3 the next iteration's BFS follows at once: this
             // barrier opens it
@@ -468,28 +490,12 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         }
         break;
     }
-    case H_JOIN:
-        break;
     default:
         break;
     }
     sh.tr_hook = hook;
     sh.tr_info = tinfo;
     if (st.err != 0) d.status = MF_ST_ERROR;
-}
-
-// advance() for the first CTA alone (one thread; sh.cnt filled in), with its entry in the timeline.
-__device__ __noinline__ void solo_advance(const MfParams &P, int hook, Sh &sh)
-{
-    advance(P, hook, sh, gtimer());
-    const int i = sh.hs.trace_n - 1;
-    if (i >= MF_TRACE) return;
-    MfReport *c = P.rep;
-    c->trace_hook[i] = sh.tr_hook;
-    c->trace_t[i] = sh.hs.t_phase;
-    c->trace_slots[i] = sh.stat[ST_SLOTS_BFS] + sh.stat[ST_SLOTS_DIS] + sh.stat[ST_SLOTS_FIX];
-    c->trace_info[i] = sh.tr_info;
-    c->trace_fin_max[i] = c->trace_fin_mean[i] = 0;
 }
 
 // One entry of the hook timeline, written by the last warp of the first CTA
@@ -539,8 +545,8 @@ __device__ __forceinline__ void words_in(int *sh_dst, const int *src, int words)
 }
 
 // Excess of sink and source and the BFS label counters go to memory, the
-// finish time and the slots scanned into this CTA's place; then the arrival.
-// Called by warp 0 after a __syncthreads.
+// finish time and the slots scanned into this CTA's place.  Called by warp 0
+// after a __syncthreads.
 __device__ __forceinline__ void arrive(const MfParams &P, Sh &sh)
 {
     MfCtrl *c = P.ctrl;
@@ -574,7 +580,13 @@ __device__ __forceinline__ void arrive(const MfParams &P, Sh &sh)
         sh.dem = 0;
     }
     __syncwarp();
-    if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&c->bar.w[0]) : "memory");
+}
+
+// One thread: this CTA is at the grid barrier.
+__device__ __forceinline__ void signal_all(const MfParams &P, Sh &sh)
+{
+    ++sh.arrivals;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&P.ctrl->bar.w[0]) : "memory");
 }
 
 // Wait until every CTA has arrived at the current barrier; false after the
@@ -582,7 +594,7 @@ __device__ __forceinline__ void arrive(const MfParams &P, Sh &sh)
 __device__ __forceinline__ bool wait_all(const MfParams &P, Sh &sh)
 {
     MfCtrl *c = P.ctrl;
-    const unsigned target = (sh.phase + 1u) * (unsigned)vn();
+    const unsigned target = sh.arrivals * (unsigned)vn();
     unsigned long long t0 = 0;
     unsigned spins = 0;
     while ((int)(ld_acquire(&c->bar.w[0]) - target) < 0) {
@@ -601,27 +613,83 @@ __device__ __forceinline__ bool wait_all(const MfParams &P, Sh &sh)
     return true;
 }
 
+// ---- thread-block clusters ----
+
+__device__ __forceinline__ unsigned cluster_size()
+{
+    unsigned v;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(v));
+    return v;
+}
+
+__device__ __forceinline__ unsigned cluster_rank()
+{
+    unsigned v;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(v));
+    return v;
+}
+
+// All threads of all CTAs of the cluster (threads that have left the kernel do
+// not count).  538 clocks, against 2250 for the barrier of as many CTAs
+// through memory.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The squad's own barrier; called by all its threads.
+__device__ __forceinline__ void squad_sync(const Sh &sh)
+{
+    if (sh.csize > 1) cluster_sync();
+    else __syncthreads();
+}
+
+// sq[par][my rank] in every CTA of the squad = mine, by one warp; visible behind squad_sync.
+__device__ __forceinline__ void squad_tell(Sh &sh, int par, const SquadSum &mine)
+{
+    const int lane = threadIdx.x & 31;
+    constexpr int kW = (int)(sizeof(SquadSum) / 4);
+    if (lane < sh.csize) {
+        const unsigned own = (unsigned)__cvta_generic_to_shared(&sh.sq[par][sh.crank]);
+        unsigned there = own;
+        if (sh.csize > 1) asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(own), "r"(lane));
+        const int *w = reinterpret_cast<const int *>(&mine);
+#pragma unroll
+        for (int i = 0; i < kW; ++i)
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(there + 4u * i), "r"(w[i]) : "memory");
+    }
+}
+
 // Grid-wide barrier with a hook.  Returns false if this CTA gave up waiting
 // (the caller must return from the kernel at once).  One counter, which every
 // CTA raises and then watches: the arrival that completes it releases all of
 // them at once (304 CTAs: 1.4 us, against 2.5 us when the last one resets the
 // counter and publishes a generation word), and each works out the next step
 // from the counter set by itself (advance), where one thread running that
-// behind the barrier for all held them up for another 3 us.
-__device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh)
+// behind the barrier for all held them up for another 3 us.  A solve that is
+// one cluster uses the cluster's barrier.  With take_state, every CTA takes the
+// first one's state (its squad ran phases alone) before working out the next.
+__device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh, bool take_state = false)
 {
     MfCtrl *c = P.ctrl;
     __syncthreads();
     const unsigned k = sh.phase;
+    const bool one = sh.one_cluster != 0;
     if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        if (hook == H_JOIN && vb() == 0) {
+        if (take_state && vb() == 0) {
             words_out((int *)&c->jd, (const int *)&sh.d, (int)(sizeof(MfDesc) / 4));
             words_out((int *)&c->js, (const int *)&sh.hs, (int)(sizeof(MfState) / 4));
         }
         arrive(P, sh);
-        int ok = 0;
-        if (lane == 0) ok = wait_all(P, sh) ? 1 : 0;
+    }
+    if (one) cluster_sync();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        int ok = 1;
+        if (lane == 0 && !one) {
+            signal_all(P, sh);
+            ok = wait_all(P, sh) ? 1 : 0;
+        }
         ok = __shfl_sync(0xffffffffu, ok, 0);
         __syncwarp();
         if (ok) {
@@ -629,7 +697,7 @@ __device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh)
                 sh.cnt[lane] = __ldcg(reinterpret_cast<const int4 *>(&sh.cs->l[lane]));
                 if (vb() == 0) __stcg(reinterpret_cast<int4 *>(&c->set[(k + 2u) % 3u].l[lane]), make_int4(0, 0, 0, 0));
             }
-            if (hook == H_JOIN && vb() != 0) {
+            if (take_state && vb() != 0) {
                 words_in((int *)&sh.d, (const int *)&c->jd, (int)(sizeof(MfDesc) / 4));
                 words_in((int *)&sh.hs, (const int *)&c->js, (int)(sizeof(MfState) / 4));
             }
@@ -659,6 +727,7 @@ __device__ __noinline__ bool finish(const MfParams &P, Sh &sh)
         if (lane < MF_STATS && sh.stat[lane]) atomic_add_ll(&c->stat[lane], sh.stat[lane]);
         __syncwarp();
         arrive(P, sh);
+        if (lane == 0) signal_all(P, sh);
         if (vb() == 0) {
             int ok = 0;
             if (lane == 0) ok = wait_all(P, sh) ? 1 : 0;
@@ -2622,49 +2691,51 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
 // moves one step per round either way, so the number of rounds hardly changes
 // (grid 1024: 1172 rounds of one cycle, 1066 of two).
 //
-// What a smaller phase still costs across the grid is the barrier and the
-// round trips around it, not its work.  The first CTA runs consecutive small
-// ones alone, with its queues in shared memory and __syncthreads between
-// them, and the others wait at one grid barrier, where they take its state
-// (H_JOIN).  What bounds it there is the SM's one scattered access per clock,
-// some 14 per vertex: up to MF_SOLO_LEVEL vertices (3 to 4 us a level) it beats
-// the grid; at 1000 a level took 13 us alone, against 9.5 us across the grid.
+// What a smaller phase still costs across the grid is the barrier, the room
+// taken in the shared lists and the counters behind it, about 9 us, not its
+// work.  The squad -- the CTAs of the first thread-block cluster, or the first
+// CTA of a launch without clusters -- runs consecutive small ones alone: each
+// of its CTAs keeps the vertices it labelled or activated in a queue in its
+// shared memory and takes them up in the next phase, the CTAs tell one another
+// how many they have through distributed shared memory, and the cluster's
+// barrier stands between the phases.  The other CTAs wait at one grid barrier,
+// where they take the squad's state.  What bounds a phase there is a chain of
+// three (level) or four (round) dependent accesses, and then the one scattered
+// access per clock of each SM, some 14 per vertex.
 
-// Whether the first CTA should go back to the grid: it has held up the others
-// for a quarter of the longest wait at a barrier.
-__device__ __forceinline__ bool solo_timeout(const MfParams &P, unsigned long long t0)
+// Whether the squad should go back to the grid: it has held up the others for a
+// quarter of the longest wait at a barrier.
+__device__ __forceinline__ bool squad_timeout(const MfParams &P, unsigned long long t0)
 {
     return gtimer() - t0 > P.wait_limit_ns / 4;
 }
 
-// The queues of a run of small phases: vertex, row start and row length of the
-// next phase's entries.
-struct SoloQ {
+// A squad CTA's queues: vertex, row start and row length of its entries.
+struct SquadQ {
     int *v, *r, *d;
 };
-__device__ __forceinline__ SoloQ solo_q(int which)
+__device__ __forceinline__ SquadQ squad_q(int which)
 {
-    SoloQ q;
-    q.v = mf_stage + which * MF_SOLO_CAP;
-    q.r = q.v + 2 * MF_SOLO_CAP;
-    q.d = q.r + 2 * MF_SOLO_CAP;
+    SquadQ q;
+    q.v = mf_stage + which * MF_SQUAD_CAP;
+    q.r = q.v + 2 * MF_SQUAD_CAP;
+    q.d = q.r + 2 * MF_SQUAD_CAP;
     return q;
 }
-__device__ __forceinline__ void solo_put(const SoloQ &q, int i, int v, int r0, int d)
+__device__ __forceinline__ void squad_put(const SquadQ &q, int i, int v, int r0, int d)
 {
     q.v[i] = v;
     q.r[i] = r0;
     q.d[i] = d;
 }
 
-// bfs_visit for a level that the first CTA runs alone: labelled vertices go
-// straight into its next queue (and onto the shared frontier list, should the
-// grid take over).
+// bfs_visit for a level of the squad: labelled vertices go straight into this
+// CTA's next queue.
 template <int BR>
-__device__ __forceinline__ void solo_visit(const MfParams &P, Sh &sh, const int (&x)[BR], const bool (&valid)[BR],
-                                           int L, const SoloQ &nq, int &lab, unsigned &lab_slots)
+__device__ __forceinline__ void squad_visit(const MfParams &P, Sh &sh, const int (&x)[BR], const bool (&valid)[BR],
+                                            int L, const SquadQ &nq, int &lab, unsigned &lab_slots)
 {
-    const bool want_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY), near = sh.d.near != 0;
+    const bool want_wl = sh.k_wl != 0, near = sh.d.near != 0;
     const int n = P.g.n;
     int z[BR], rc[BR], d[BR], r0[BR];
     bool claim[BR];
@@ -2695,40 +2766,49 @@ __device__ __forceinline__ void solo_visit(const MfParams &P, Sh &sh, const int 
             if (L == 0 && ldg_cg(P.g.dst + y) == P.sink) P.sc.dem[z[r]] = rc[r];
         }
         if (d[r] > P.bfs_hub) {
-            put_items(P, r0[r], d[r], sh.d.app_hub + atomicAdd(&sh.so_hub, chunks_of(d[r])));
+            put_items(P, r0[r], d[r], sh.d.app_hub + atomicAdd(&sh.cs->l[L_HUB].w[0], (unsigned)chunks_of(d[r])));
+            sh.so_flag = SQ_SPILL;
         } else {
             const int i = atomicAdd(&sh.so_cnt, 1);
-            P.sc.border[sh.d.app_bfs + i] = z[r];
-            if (i < MF_SOLO_CAP) solo_put(nq, i, z[r], r0[r], d[r]);
+            if (i < MF_SQUAD_CAP) {
+                squad_put(nq, i, z[r], r0[r], d[r]);
+            } else {
+                P.sc.border[sh.d.app_bfs + atomicAdd(&sh.cs->l[L_BFS].w[0], 1u)] = z[r];
+                sh.so_flag = SQ_SPILL;
+            }
         }
         if (ev[r] > 0 && z[r] != P.sink) {
             const int bin = row_bin(P, d[r]);
-            P.sc.wl[sh.d.wl_sel][bin][sh.d.wl_app[bin] + atomicAdd(&sh.so_wl[bin], 1)] = z[r];
+            P.sc.wl[sh.d.wl_sel][bin][sh.d.wl_app[bin] + atomicAdd(&sh.cs->l[L_WL + bin].w[0], 1u)] = z[r];
             if (near) atomicAdd(&sh.exc, (unsigned long long)ev[r]);
         }
     }
 }
 
-// Top-down BFS levels, one after another, while they stay small.
-__device__ __noinline__ void solo_bfs(const MfParams &P, Sh &sh)
+// Top-down BFS levels, one after another, while they stay small.  The last one
+// leaves its results where a level of the grid would, and the grid barrier that
+// follows takes them up as that level's (with the squad's state).
+__device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
 {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nwarps = nt >> 5;
+    const int csize = sh.csize, rank = sh.crank;
     const unsigned long long t0 = gtimer();
-    int cur = 0;
+    int cur = 0, cnt;
     {
-        const int lo = sh.d.lvl_lo, cnt = sh.d.lvl_hi - lo;
-        const SoloQ q = solo_q(0);
+        // entry i of the frontier belongs to squad CTA i mod csize
+        const int lo = sh.d.lvl_lo, all = sh.d.lvl_hi - lo;
+        cnt = all > rank ? (all - rank + csize - 1) / csize : 0;
+        const SquadQ q = squad_q(0);
         for (int i = tid; i < cnt; i += nt) {
-            const int v = __ldcg(P.sc.border + lo + i);
-            solo_put(q, i, v, P.g.off[v], ldg_cg(P.g.deg + v));
+            const int v = __ldcg(P.sc.border + lo + i * csize + rank);
+            squad_put(q, i, v, P.g.off[v], ldg_cg(P.g.deg + v));
         }
     }
-    if (tid < MF_NBIN) sh.so_wl[tid] = 0;
-    if (tid == 0) sh.so_cnt = sh.so_hub = 0;
+    if (tid == 0) sh.so_cnt = sh.so_flag = 0;
     __syncthreads();
     for (;;) {
-        const int L = sh.d.level, cnt = sh.d.lvl_hi - sh.d.lvl_lo;
-        const SoloQ cq = solo_q(cur), nq = solo_q(cur ^ 1);
+        const int L = sh.d.level, par = sh.so_par;
+        const SquadQ cq = squad_q(cur), nq = squad_q(cur ^ 1);
         int lab = 0;
         unsigned lab_slots = 0;
         long long scanned = 0;
@@ -2762,7 +2842,7 @@ __device__ __noinline__ void solo_bfs(const MfParams &P, Sh &sh)
                     vs[r] = k < T;
                     xs[r] = rb + (k - eb);
                 }
-                solo_visit<kBR>(P, sh, xs, vs, L, nq, lab, lab_slots);
+                squad_visit<kBR>(P, sh, xs, vs, L, nq, lab, lab_slots);
             }
         }
         __syncwarp();
@@ -2773,74 +2853,94 @@ __device__ __noinline__ void solo_bfs(const MfParams &P, Sh &sh)
             add_stat(sh, ST_SLOTS_BFS, scanned);
         }
         __syncthreads();
+        if (wid == 0) {
+            SquadSum mine{};
+            mine.cnt = min(sh.so_cnt, MF_SQUAD_CAP);
+            mine.slots = (unsigned)(sh.lab & 0xffffffffull);
+            mine.labelled = (int)(sh.lab >> 32);
+            mine.flag = sh.so_flag | (rank == 0 && squad_timeout(P, t0) ? SQ_STOP : 0);
+            mine.exc = (long long)sh.exc;
+            squad_tell(sh, par, mine);
+        }
+        squad_sync(sh);
         if (tid == 0) {
+            // the same in every CTA of the squad
             MfDesc &d = sh.d;
             MfState &st = sh.hs;
-            const int c = sh.so_cnt;
-            const long long fr = (long long)(unsigned)(sh.lab & 0xffffffffull), lab_n = (long long)(sh.lab >> 32);
-            const long long vis = st.vis_slots + fr, sup = st.sup + (long long)sh.exc;
-            sh.stat[ST_LAB_BFS] += lab_n;
-            const bool go = c > 0 && sh.so_hub == 0 && solo_level(sh, c, fr) &&
-                            !(P.bu_alpha > 0 && fr * P.bu_alpha > st.used_slots - vis) &&
-                            !(d.near && sup > 0 && (sup >> st.cut_shift) >= st.dem) && !solo_timeout(P, t0);
+            int c = 0, flag = 0;
+            long long fr = 0, lab_n = 0, exc = 0;
+            for (int q = 0; q < csize; ++q) {
+                const SquadSum s = sh.sq[par][q];
+                c += s.cnt;
+                flag |= s.flag;
+                fr += s.slots;
+                lab_n += s.labelled;
+                exc += s.exc;
+            }
+            const long long vis = st.vis_slots + fr, sup = st.sup + exc;
+            const bool go = c > 0 && flag == 0 && squad_level(sh, c, fr) &&
+                            !(sh.k_alpha > 0 && fr * sh.k_alpha > st.used_slots - vis) &&
+                            !(d.near && sup > 0 && (sup >> st.cut_shift) >= st.dem);
             if (go) {
                 // what advance() does for a level that is followed by another small one
                 ++d.level;
                 ++st.bfs_levels;
-                d.lvl_lo = d.lvl_hi;
-                d.app_bfs += c;
-                d.lvl_hi = d.app_bfs;
                 st.vis_slots = vis;
                 st.sup = sup;
-                for (int q = 0; q < MF_NBIN; ++q) d.wl_app[q] += sh.so_wl[q];
-            } else {
-                for (int q = 0; q < MF_LINES; ++q) sh.cnt[q] = make_int4(0, 0, 0, 0);
-                sh.cnt[L_BFS].x = c;
-                sh.cnt[L_HUB].x = sh.so_hub;
-                for (int q = 0; q < MF_NBIN; ++q) sh.cnt[L_WL + q].x = sh.so_wl[q];
-                sh.cnt[L_LAB] = make_int4((int)(unsigned)sh.lab, (int)(sh.lab >> 32), 0, 0);
-                sh.cnt[L_EXC] = make_int4((int)(unsigned)sh.exc, (int)(sh.exc >> 32), 0, 0);
-                solo_advance(P, H_BFS_NEXT, sh);
+                sh.stat[ST_LAB_BFS] += (long long)(sh.lab >> 32);
+                sh.lab = sh.exc = 0;
             }
-            sh.lab = sh.exc = 0;
-            sh.so_cnt = sh.so_hub = 0;
-            for (int q = 0; q < MF_NBIN; ++q) sh.so_wl[q] = 0;
             sh.so_go = go ? 1 : 0;
+            sh.so_par = par ^ 1;
         }
         __syncthreads();
-        if (!sh.so_go) return;
+        const int mine = min(sh.so_cnt, MF_SQUAD_CAP);
         cur ^= 1;
+        if (!sh.so_go) {
+            // the frontier goes onto the shared list
+            int at = 0;
+            if (tid == 0 && mine) sh.bcast_i = at = (int)atomicAdd(&sh.cs->l[L_BFS].w[0], (unsigned)mine);
+            __syncthreads();
+            at = sh.d.app_bfs + sh.bcast_i;
+            for (int i = tid; i < mine; i += nt) P.sc.border[at + i] = squad_q(cur).v[i];
+            return;
+        }
+        __syncthreads();
+        if (tid == 0) sh.so_cnt = sh.so_flag = 0;
+        cnt = mine;
+        __syncthreads();
     }
 }
 
 // z received flow and became active, or stays active after its cycle: into the
-// next round.  Alone (SOLO): into the first CTA's queue, or, when that is full
-// or z's row is long, onto the grid's lists; else into the CTA's queue of
-// worklist entries.
-template <bool SOLO>
-__device__ __forceinline__ void short_enqueue(const MfParams &P, Sh &sh, int z, int r0, int d, const SoloQ &nq)
+// next round.  In the squad: into this CTA's queue, or, when that is full or z's
+// row is long, onto the grid's lists; else into the CTA's queue of worklist
+// entries.
+template <bool SQUAD>
+__device__ __forceinline__ void short_enqueue(const MfParams &P, Sh &sh, int z, int r0, int d, const SquadQ &nq)
 {
-    if (!SOLO) {
+    if (!SQUAD) {
         place_active(P, sh, z, d, L_AUX, sh.d.wl_sel ^ 1, nullptr);
         return;
     }
     if (d <= MF_SHORT_ROW) {
         const int i = atomicAdd(&sh.so_cnt, 1);
-        if (i < MF_SOLO_CAP) {
-            solo_put(nq, i, z, r0, d);
+        if (i < MF_SQUAD_CAP) {
+            squad_put(nq, i, z, r0, d);
             return;
         }
     }
     const int bin = row_bin(P, d);
-    P.sc.wl[sh.d.wl_sel ^ 1][bin][atomicAdd(&sh.so_wl[bin], 1)] = z;
+    P.sc.wl[sh.d.wl_sel ^ 1][bin][atomicAdd(&sh.cs->l[L_AUX + bin].w[0], 1u)] = z;
+    sh.so_flag = SQ_SPILL;
 }
 
 // g units along slot x = (u, z), y its reverse.  Every vertex is in a round's
 // lists at most once and lowers its own excess once, at its end, so z's excess
 // rises from <= 0 to > 0 at most once in a round: whoever makes it do so
 // queues it, and no stamp is needed.
-template <bool SOLO>
-__device__ __forceinline__ void short_push(const MfParams &P, Sh &sh, int x, int z, int y, int g, const SoloQ &nq)
+template <bool SQUAD>
+__device__ __forceinline__ void short_push(const MfParams &P, Sh &sh, int x, int z, int y, int g, const SquadQ &nq)
 {
     atomicSub(P.cf + x, g);
     atomicAdd(P.cf + y, g);
@@ -2849,9 +2949,9 @@ __device__ __forceinline__ void short_push(const MfParams &P, Sh &sh, int x, int
     } else if (z == P.source) {
         atomicAdd((unsigned long long *)&sh.src_e, (unsigned long long)g);
     } else {
-        const int d = ldg_cg(P.g.deg + z), r0 = SOLO ? P.g.off[z] : 0;     // in flight together with the excess
+        const int d = ldg_cg(P.g.deg + z), r0 = SQUAD ? P.g.off[z] : 0;     // in flight together with the excess
         const long long old = atomic_add_ll(P.e + z, (long long)g);
-        if (old <= 0 && old + g > 0) short_enqueue<SOLO>(P, sh, z, r0, d, nq);
+        if (old <= 0 && old + g > 0) short_enqueue<SQUAD>(P, sh, z, r0, d, nq);
     }
 }
 
@@ -2871,8 +2971,8 @@ __device__ __forceinline__ int short_lift(const MfParams &P, Sh &sh, int u, int 
 
 // One cycle of Alg. 2 for u by one thread (rows of at most 8 slots): relabel if
 // needed, then push to the lowest neighbours in slot order.
-template <bool SOLO>
-__device__ __forceinline__ int short_thread(const MfParams &P, Sh &sh, int u, int r0, int d, const SoloQ &nq)
+template <bool SQUAD>
+__device__ __forceinline__ int short_thread(const MfParams &P, Sh &sh, int u, int r0, int d, const SquadQ &nq)
 {
     const int4 none = make_int4(0, 0, 0, 0);
     const long long eu = ldg_cg(P.e + u);
@@ -2903,19 +3003,19 @@ __device__ __forceinline__ int short_thread(const MfParams &P, Sh &sh, int u, in
     for (int k = 0; k < 8; ++k) {
         if (hz[k] != best || rem <= 0) continue;
         const int g = rem < (long long)c[k] ? (int)rem : c[k];
-        short_push<SOLO>(P, sh, r0 + k, z[k], ldg_cg(P.g.rev + r0 + k), g, nq);
+        short_push<SQUAD>(P, sh, r0 + k, z[k], ldg_cg(P.g.rev + r0 + k), g, nq);
         rem -= g;
         ++pushes;
     }
     const long long old = atomic_add_ll(P.e + u, rem - eu);
-    if (old + rem - eu > 0) short_enqueue<SOLO>(P, sh, u, r0, d, nq);
+    if (old + rem - eu > 0) short_enqueue<SQUAD>(P, sh, u, r0, d, nq);
     return pushes;
 }
 
 // The same by one warp (rows of up to MF_SHORT_ROW slots): every lane holds four
 // slots of each 128, and a prefix sum over the lanes deals out the excess.
-template <bool SOLO>
-__device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int r0, int d, const SoloQ &nq)
+template <bool SQUAD>
+__device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int r0, int d, const SquadQ &nq)
 {
     constexpr int kQ = MF_SHORT_ROW / 128;
     const int lane = threadIdx.x & 31;
@@ -2959,7 +3059,7 @@ __device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int 
         if (hz[k] != best || rem <= 0) continue;
         const int g = rem < (long long)c[k] ? (int)rem : c[k];
         const int x = r0 + (k >> 2) * 128 + lane * 4 + (k & 3);
-        short_push<SOLO>(P, sh, x, ldg_cg(P.g.dst + x), ldg_cg(P.g.rev + x), g, nq);
+        short_push<SQUAD>(P, sh, x, ldg_cg(P.g.dst + x), ldg_cg(P.g.rev + x), g, nq);
         rem -= g;
         ++pushes;
     }
@@ -2968,7 +3068,7 @@ __device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int 
     if (lane == 0) {
         const long long sent = total < eu ? total : eu;
         const long long old = atomic_add_ll(P.e + u, -sent);
-        if (old - sent > 0) short_enqueue<SOLO>(P, sh, u, r0, d, nq);
+        if (old - sent > 0) short_enqueue<SQUAD>(P, sh, u, r0, d, nq);
     }
     __syncwarp();
     return pushes;
@@ -2980,7 +3080,7 @@ __device__ __noinline__ void phase_discharge_short(const MfParams &P, Sh &sh)
 {
     const int lane = threadIdx.x & 31;
     const int sel = sh.d.wl_sel, n0 = sh.d.wl_n[0], n1 = sh.d.wl_n[1], cnt = n0 + n1;
-    const SoloQ none{};
+    const SquadQ none{};
     long long pushes = 0, slots = 0, scans = 0;
     for (long long k = spread_thread(); k < cnt; k += (long long)vn() * blockDim.x) {
         const int i = (int)k;
@@ -3010,31 +3110,29 @@ __device__ __noinline__ void phase_discharge_short(const MfParams &P, Sh &sh)
     flush_queue(P, sh, L_AUX, sel ^ 1, nullptr, 0, 0u);
 }
 
-// Discharge rounds, one after another, while few vertices are active.  Ends when
-// none is left, when the rounds have taken their share of the time (as the
-// grid's do), or with the lists of the next grid round written.
-__device__ __noinline__ void solo_discharge(const MfParams &P, Sh &sh)
+// Discharge rounds, one after another, while few vertices are active.  The last
+// one leaves its results where a round of the grid would.
+__device__ __noinline__ void squad_discharge(const MfParams &P, Sh &sh)
 {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
+    const int csize = sh.csize, rank = sh.crank;
     const unsigned long long t0 = gtimer();
-    int cur = 0;
+    int cur = 0, cnt;
     {
-        const int sel = sh.d.wl_sel, n0 = sh.d.wl_n[0], cnt = n0 + sh.d.wl_n[1];
-        const SoloQ q = solo_q(0);
+        const int sel = sh.d.wl_sel, n0 = sh.d.wl_n[0], all = n0 + sh.d.wl_n[1];
+        cnt = all > rank ? (all - rank + csize - 1) / csize : 0;
+        const SquadQ q = squad_q(0);
         for (int i = tid; i < cnt; i += nt) {
-            const int v = __ldcg(i < n0 ? P.sc.wl[sel][0] + i : P.sc.wl[sel][1] + (i - n0));
-            solo_put(q, i, v, P.g.off[v], ldg_cg(P.g.deg + v));
-        }
-        if (tid < MF_NBIN) sh.so_wl[tid] = 0;
-        if (tid == 0) {
-            sh.so_cnt = 0;
-            sh.bcast_i = cnt;
+            const int k = i * csize + rank;
+            const int v = __ldcg(k < n0 ? P.sc.wl[sel][0] + k : P.sc.wl[sel][1] + (k - n0));
+            squad_put(q, i, v, P.g.off[v], ldg_cg(P.g.deg + v));
         }
     }
+    if (tid == 0) sh.so_cnt = sh.so_flag = 0;
     __syncthreads();
     for (;;) {
-        const int cnt = sh.bcast_i;
-        const SoloQ cq = solo_q(cur), nq = solo_q(cur ^ 1);
+        const int par = sh.so_par;
+        const SquadQ cq = squad_q(cur), nq = squad_q(cur ^ 1);
         long long slots = 0, pushes = 0, scans = 0;
         for (int i = tid; i < cnt; i += nt) {
             const int d = cq.d[i];
@@ -3058,53 +3156,51 @@ __device__ __noinline__ void solo_discharge(const MfParams &P, Sh &sh)
         add_stat(sh, ST_SLOTS_DIS, slots);
         add_stat(sh, ST_CYCLES_DIS, scans);
         __syncthreads();
+        if (wid == 0) {
+            SquadSum mine{};
+            mine.cnt = min(sh.so_cnt, MF_SQUAD_CAP);
+            mine.flag = sh.so_flag;
+            if (rank == 0) {
+                const unsigned long long now = gtimer();
+                if (sh.d.round + 1 >= MF_DEFAULT_ROUNDS && !rounds_left(sh.d, sh.hs, now)) mine.flag |= SQ_OVER;
+                if (squad_timeout(P, t0)) mine.flag |= SQ_STOP;
+            }
+            squad_tell(sh, par, mine);
+        }
+        squad_sync(sh);
         if (tid == 0) {
-            MfDesc &d = sh.d;
-            MfState &st = sh.hs;
-            const int c = min(sh.so_cnt, MF_SOLO_CAP);
-            int spill = 0;
-            for (int q = 0; q < MF_NBIN; ++q) spill += sh.so_wl[q];
-            const unsigned long long now = gtimer();
-            const bool over = d.round + 1 >= MF_DEFAULT_ROUNDS && !rounds_left(st, now);
-            sh.so_go = c + spill == 0 || d.round + 1 >= MF_MAX_ROUNDS || over ? 0
-                       : spill > 0 || c > MF_SOLO_ACTIVE || solo_timeout(P, t0) ? 2 : 1;
-            if (sh.so_go) ++d.round;
-            ++st.rounds_total;
-            sh.bcast_i = c;
-            sh.so_cnt = 0;
+            // the same in every CTA of the squad
+            int c = 0, flag = 0;
+            for (int q = 0; q < csize; ++q) {
+                c += sh.sq[par][q].cnt;
+                flag |= sh.sq[par][q].flag;
+            }
+            const bool over = c == 0 || (flag & SQ_OVER) || sh.d.round + 1 >= MF_MAX_ROUNDS;
+            sh.so_go = over ? 0 : (flag != 0 || c > MF_SQUAD_ACTIVE * csize ? 2 : 1);
+            if (sh.so_go == 1) {
+                ++sh.d.round;
+                ++sh.hs.rounds_total;
+            }
+            sh.so_par = par ^ 1;
         }
         __syncthreads();
-        const int go = sh.so_go, c = sh.bcast_i;
-        if (go == 1) {
-            cur ^= 1;
-            continue;
-        }
-        if (go == 2) {
-            // the next round is the grid's again: the queue goes onto its lists
-            for (int i = tid; i < c; i += nt) {
-                const int bin = row_bin(P, nq.d[i]);
-                P.sc.wl[sh.d.wl_sel ^ 1][bin][atomicAdd(&sh.so_wl[bin], 1)] = nq.v[i];
+        const int go = sh.so_go, mine = min(sh.so_cnt, MF_SQUAD_CAP);
+        cur ^= 1;
+        if (go != 1) {
+            // more rounds, but not here: the queue goes onto the grid's lists
+            // (what is left when the discharge is over waits for the next BFS)
+            if (go == 2) {
+                for (int i = tid; i < mine; i += nt) {
+                    const int bin = row_bin(P, nq.d[i]);
+                    P.sc.wl[sh.d.wl_sel ^ 1][bin][atomicAdd(&sh.cs->l[L_AUX + bin].w[0], 1u)] = nq.v[i];
+                }
             }
-            __syncthreads();
-        }
-        if (tid == 0) {
-            MfDesc &d = sh.d;
-            MfState &st = sh.hs;
-            const unsigned long long now = gtimer();
-            st.ns_dis += now - st.t_phase;
-            st.t_phase = st.t_now = now;
-            ++d.qstamp;
-            d.dis_more = go ? 1 : 0;
-            if (go) {
-                d.wl_sel ^= 1;
-                for (int q = 0; q < MF_NBIN; ++q) d.wl_n[q] = sh.so_wl[q];
-                pick_round(P, d);
-            } else {
-                begin_iteration(sh);
-            }
+            return;
         }
         __syncthreads();
-        return;
+        if (tid == 0) sh.so_cnt = sh.so_flag = 0;
+        cnt = mine;
+        __syncthreads();
     }
 }
 
@@ -3341,6 +3437,12 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         sh.q_bfs = sh.q_long = sh.q_wn = 0;
         for (int b = 0; b < MF_NBIN; ++b) sh.q_wl[b] = 0;
         sh.phase = 0;
+        sh.arrivals = 0;
+        const int cs = (int)cluster_size();
+        sh.csize = cs > 1 && cs <= MF_CLUSTER && vn() % cs == 0 ? cs : 1;
+        sh.crank = sh.csize > 1 ? (int)cluster_rank() : 0;
+        sh.one_cluster = sh.csize > 1 && vn() == sh.csize && P.test_skip_cta < 0 ? 1 : 0;
+        sh.so_par = 0;
         sh.cs = &c->set[0];
         sh.d = MfDesc{};
         sh.hs = MfState{};
@@ -3350,7 +3452,7 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         sh.k_alpha = P.bu_alpha;
         sh.k_beta = P.bu_beta;
         sh.k_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY) ? 1 : 0;
-        sh.k_solo = P.pull || P.stage_slots < MF_SOLO_INTS ? 0 : (P.tail_slots > 0 ? P.tail_slots : MF_SOLO_SLOTS);
+        sh.k_squad = P.pull || P.stage_slots < MF_SQUAD_INTS ? 0 : (P.tail_slots > 0 ? P.tail_slots : MF_SQUAD_SLOTS * sh.csize);
         sh.hs.t_phase = gtimer();
     }
     if (vb() == 0) {
@@ -3423,10 +3525,10 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         phase_bfs_init(P, sh);
         if (!grid_sync(P, H_BFS_START, sh)) return false;
         while (!sh.d.bfs_done) {
-            if (sh.d.bfs_solo) {
-                // the others wait at the next grid barrier and take the first CTA's state there
-                if (vb() == 0) solo_bfs(P, sh);
-                if (!grid_sync(P, H_JOIN, sh)) return false;
+            if (sh.d.bfs_squad) {
+                // the others wait at the grid barrier and take the squad's state there
+                if (vb() < sh.csize) squad_bfs(P, sh);
+                if (!grid_sync(P, H_BFS_NEXT, sh, true)) return false;
                 continue;
             }
             if (sh.d.bu_mode) {
@@ -3450,9 +3552,9 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         if (sh.d.status != MF_ST_RUNNING) break;
         // discharge rounds, then remove-invalid-edges
         do {
-            if (sh.d.dis_solo) {
-                if (vb() == 0) solo_discharge(P, sh);
-                if (!grid_sync(P, H_JOIN, sh)) return false;
+            if (sh.d.dis_squad) {
+                if (vb() < sh.csize) squad_discharge(P, sh);
+                if (!grid_sync(P, H_DIS, sh, true)) return false;
                 continue;
             }
             if (sh.d.near && sh.d.round == 0) phase_walk(P, sh);
@@ -4069,22 +4171,72 @@ int mf_max_coresident_blocks(int device, int *per_sm, int *num_sms, int dyn_byte
     return k > 0 ? MAXFLOW_OK : MAXFLOW_ERR_CUDA;
 }
 
-int mf_launch_multi(const MfParams *plist_dev, int count, int gsize, int grid, unsigned *gstate, unsigned *head,
-                    unsigned long long wait_ns, int *abort, void *stream, int stage_bytes)
+namespace {
+
+// A cooperative launch, in thread-block clusters of `cluster` CTAs where that is more than one.
+cudaError_t launch_kernel(const void *kernel, int grid, int cluster, size_t dyn, cudaStream_t st, void **args)
 {
-    void *args[] = {(void *)&plist_dev, &count, &gsize, &gstate, &head, &wait_ns, &abort};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void *)mf_multi_kernel, dim3(grid), dim3(MF_BLOCK), args,
-                                                (size_t)stage_bytes, (cudaStream_t)stream);
-    return cuda_rc(e);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(MF_BLOCK);
+    cfg.dynamicSmemBytes = dyn;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2]{};
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelExC(&cfg, kernel, args);
 }
 
-int mf_launch(const MfParams &p, int grid, void *stream)
+}  // namespace
+
+// CTAs of the solve kernels that fit the GPU at once in clusters of MF_CLUSTER
+// (a cluster's CTAs sit in one GPC, so a few SMs may be left over), with the
+// device current; 0 where there are none.
+int mf_max_clustered_blocks(int dyn_bytes, int *blocks)
+{
+    *blocks = 0;
+    int least = 0;
+    for (const void *k : {(const void *)mf_solve_kernel, (const void *)mf_multi_kernel}) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(MF_CLUSTER);
+        cfg.blockDim = dim3(MF_BLOCK);
+        cfg.dynamicSmemBytes = (size_t)dyn_bytes;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = MF_CLUSTER;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int nc = 0;
+        if (cudaOccupancyMaxActiveClusters(&nc, k, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            return MAXFLOW_OK;
+        }
+        least = k == (const void *)mf_solve_kernel || nc < least ? nc : least;
+    }
+    *blocks = least * MF_CLUSTER;
+    return MAXFLOW_OK;
+}
+
+int mf_launch_multi(const MfParams *plist_dev, int count, int gsize, int grid, unsigned *gstate, unsigned *head,
+                    unsigned long long wait_ns, int *abort, int cluster, void *stream, int stage_bytes)
+{
+    void *args[] = {(void *)&plist_dev, &count, &gsize, &gstate, &head, &wait_ns, &abort};
+    return cuda_rc(launch_kernel((const void *)mf_multi_kernel, grid, cluster, (size_t)stage_bytes,
+                                 (cudaStream_t)stream, args));
+}
+
+int mf_launch(const MfParams &p, int grid, int cluster, void *stream)
 {
     MfParams q = p;
     void *args[] = {&q};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void *)mf_solve_kernel, dim3(grid), dim3(MF_BLOCK), args,
-                                                (size_t)p.stage_slots * sizeof(int), (cudaStream_t)stream);
-    return cuda_rc(e);
+    return cuda_rc(launch_kernel((const void *)mf_solve_kernel, grid, cluster, (size_t)p.stage_slots * sizeof(int),
+                                 (cudaStream_t)stream, args));
 }
 
 int mf_launch_aux(int which, const MfParams &p, void *stream, long long *dev_out, const void *extra)
