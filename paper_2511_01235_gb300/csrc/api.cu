@@ -304,17 +304,17 @@ void free_graph(maxflow_ctx *c)
     c->x_cf = c->x_cf2 = nullptr;
 }
 
-// Upload a host layout into freshly allocated slot arrays (vertex arrays kept).
-int upload_graph(maxflow_ctx *c, const MfHostGraph &hg)
+// Freshly allocated slot arrays for S reserved slots, and the BFS lists sized by
+// them (vertex arrays kept).  with_deg: off, deg and bdeg too.
+int alloc_slots(maxflow_ctx *c, int32_t n, int64_t S, bool with_deg)
 {
-    free_graph(c);
-    int64_t S = hg.slot_cap;
-    int32_t n = hg.n;
     c->g.n = n;
     c->g.slot_cap = S;
     c->g.off = dalloc_n<int32_t>(c, n + 1);
-    c->g.deg = dalloc_n<int32_t>(c, n);
-    c->g.bdeg = dalloc_n<int32_t>(c, n);
+    if (with_deg) {
+        c->g.deg = dalloc_n<int32_t>(c, n);
+        c->g.bdeg = dalloc_n<int32_t>(c, n);
+    }
     c->g.dst = dalloc_n<int32_t>(c, S);
     c->g.cf = dalloc_n<int32_t>(c, S);
     c->g.cap = dalloc_n<int32_t>(c, S);
@@ -322,6 +322,26 @@ int upload_graph(maxflow_ctx *c, const MfHostGraph &hg)
     c->g.pcap = dalloc_n<int32_t>(c, S);
     if (!c->g.off || !c->g.deg || !c->g.bdeg || !c->g.dst || !c->g.cf || !c->g.cap || !c->g.rev || !c->g.pcap)
         return MAXFLOW_ERR_OOM;
+    return MAXFLOW_OK;
+}
+
+int alloc_items(maxflow_ctx *c)
+{
+    dfree(c, c->sc.bitem);
+    dfree(c, c->sc.bdefer);
+    const int64_t k = (int64_t)c->g.n + c->g.slot_cap / MF_BFS_CHUNK + 64;
+    c->sc.bitem = dalloc_n<int2>(c, k);
+    c->sc.bdefer = dalloc_n<int2>(c, k);
+    return c->sc.bitem && c->sc.bdefer ? MAXFLOW_OK : MAXFLOW_ERR_OOM;
+}
+
+// Upload a host layout into freshly allocated slot arrays (vertex arrays kept).
+int upload_graph(maxflow_ctx *c, const MfHostGraph &hg)
+{
+    free_graph(c);
+    int64_t S = hg.slot_cap;
+    int32_t n = hg.n;
+    MF_TRY(alloc_slots(c, n, S, true));
     cudaStream_t st = c->stream;
     MF_TRY(rc_cuda(cudaMemcpyAsync(c->g.off, hg.off, sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, st)));
     MF_TRY(rc_cuda(cudaMemcpyAsync(c->g.deg, hg.deg, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st)));
@@ -333,14 +353,51 @@ int upload_graph(maxflow_ctx *c, const MfHostGraph &hg)
     if (hg.pcap) MF_TRY(rc_cuda(cudaMemcpyAsync(c->g.pcap, hg.pcap, sizeof(int32_t) * S, cudaMemcpyHostToDevice, st)));
     // the host arrays must stay valid until the copies complete
     MF_TRY(rc_cuda(cudaStreamSynchronize(st)));
-    dfree(c, c->sc.bitem);
-    dfree(c, c->sc.bdefer);
-    c->sc.bitem = dalloc_n<int2>(c, (int64_t)n + S / MF_BFS_CHUNK + 64);
-    c->sc.bdefer = dalloc_n<int2>(c, (int64_t)n + S / MF_BFS_CHUNK + 64);
-    if (!c->sc.bitem || !c->sc.bdefer) return MAXFLOW_ERR_OOM;
+    MF_TRY(alloc_items(c));
     c->st.slot_capacity = S;
     c->st.slots = hg.slots;
     c->st.m_edges = hg.m_merged;
+    return MAXFLOW_OK;
+}
+
+// The layout of g made on the device.  *made stays false, with nothing
+// allocated, when there is no room for its scratch memory: the host builds then.
+int build_on_device(maxflow_ctx *c, const maxflow_graph *g, bool *made)
+{
+    *made = false;
+    const size_t need = mf_build_scratch(g->n, g->m);
+    if (g->m < MF_BUILD_MIN || (long long)need > MF_BUILD_SCRATCH) return MAXFLOW_OK;
+    MfBuild b;
+    b.scratch = dalloc(c, need);
+    if (!b.scratch) {
+        cudaGetLastError();
+        return MAXFLOW_OK;
+    }
+    *made = true;
+    c->g.deg = b.deg = dalloc_n<int32_t>(c, g->n);
+    c->g.bdeg = b.bdeg = dalloc_n<int32_t>(c, g->n);
+    int rc = b.deg && b.bdeg ? MAXFLOW_OK : MAXFLOW_ERR_OOM;
+    if (rc == MAXFLOW_OK)
+        rc = mf_build_sizes(b, g->n, g->m, g->src, g->dst, g->cap, c->opt.slack_factor, c->opt.slack_min,
+                            (void *)c->stream);
+    if (rc == MAXFLOW_OK) rc = alloc_slots(c, g->n, b.slots, false);
+    if (rc == MAXFLOW_ERR_OOM) {
+        // the state may still fit without the scratch memory beside it
+        cudaGetLastError();
+        *made = false;
+        rc = MAXFLOW_OK;
+        free_graph(c);
+    } else if (rc == MAXFLOW_OK) {
+        rc = mf_build_fill(b, g->n, g->m, c->g, (void *)c->stream);
+    }
+    mf_note_launches(b.launches);
+    dfree(c, b.scratch);
+    if (rc != MAXFLOW_OK || !*made) return rc;
+    MF_TRY(alloc_items(c));
+    c->st.slot_capacity = b.slots;
+    c->st.slots = b.pairs;
+    c->st.m_edges = b.merged;
+    c->mean_cap = (float)(b.cap_sum / (double)g->m);
     return MAXFLOW_OK;
 }
 
@@ -823,15 +880,8 @@ int maxflow_init(maxflow_ctx **out, const maxflow_graph *g, int32_t s, int32_t t
     if (dev < 0 && cudaGetDevice(&dev) != cudaSuccess) return MAXFLOW_ERR_CUDA;
     if (dev >= ndev) return MAXFLOW_ERR_INVALID;
 
-    MfHostGraph hg;
-    int rc = mf_build_host(g->n, g->m, g->src, g->dst, g->cap, o.slack_factor, o.slack_min, hg);
-    if (rc != MAXFLOW_OK) return rc;
-
     maxflow_ctx *c = new (std::nothrow) maxflow_ctx();
-    if (!c) {
-        hg.release();
-        return MAXFLOW_ERR_OOM;
-    }
+    if (!c) return MAXFLOW_ERR_OOM;
     c->opt = o;
     c->device = dev;
     c->stream = (cudaStream_t)o.stream;
@@ -839,13 +889,8 @@ int maxflow_init(maxflow_ctx **out, const maxflow_graph *g, int32_t s, int32_t t
     c->s = s;
     c->t = t;
     c->st.n = g->n;
-    {
-        double sum = 0;
-        for (int64_t i = 0; i < g->m; ++i) sum += g->cap[i];
-        c->mean_cap = g->m > 0 ? (float)(sum / (double)g->m) : 0.f;
-    }
     DeviceGuard dg(dev);
-    rc = dg.ok ? MAXFLOW_OK : MAXFLOW_ERR_CUDA;
+    int rc = dg.ok ? MAXFLOW_OK : MAXFLOW_ERR_CUDA;
     int stage_bytes = 0;
     if (rc == MAXFLOW_OK) rc = mf_stage_bytes(dev, &stage_bytes);
     if (rc == MAXFLOW_OK) rc = mf_max_coresident_blocks(dev, &c->per_sm, &c->sms, stage_bytes);
@@ -855,8 +900,19 @@ int maxflow_init(maxflow_ctx **out, const maxflow_graph *g, int32_t s, int32_t t
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaEventCreate(&c->ev0));
     if (rc == MAXFLOW_OK) rc = rc_cuda(cudaEventCreate(&c->ev1));
     if (rc == MAXFLOW_OK) rc = alloc_pinned(c);
-    if (rc == MAXFLOW_OK) rc = upload_graph(c, hg);
-    hg.release();
+    bool made = false;
+    if (rc == MAXFLOW_OK) rc = build_on_device(c, g, &made);
+    if (rc == MAXFLOW_OK && !made) {
+        MfHostGraph hg;
+        rc = mf_build_host(g->n, g->m, g->src, g->dst, g->cap, o.slack_factor, o.slack_min, hg);
+        if (rc == MAXFLOW_OK) {
+            double sum = 0;
+            for (int64_t i = 0; i < g->m; ++i) sum += g->cap[i];
+            c->mean_cap = g->m > 0 ? (float)(sum / (double)g->m) : 0.f;
+            rc = upload_graph(c, hg);
+        }
+        hg.release();
+    }
     if (rc == MAXFLOW_OK) {
         int32_t n = c->n;
         c->g.h = dalloc_n<int32_t>(c, n);

@@ -46,16 +46,6 @@ void parallel_rows(int32_t n, F fn)
     for (auto &x : th) x.join();
 }
 
-int32_t slack_of(int64_t deg, float factor, int32_t smin)
-{
-    double want = (double)deg * (double)factor;
-    int64_t s = (int64_t)want;
-    if ((double)s < want) ++s;
-    if (s < smin) s = smin;
-    if (s > (1 << 24)) s = 1 << 24;
-    return (int32_t)s;
-}
-
 // rows[u] holds (v, cap, cf) records; entries are unique per (u, v) after
 // merge_row.  Builds the device layout.
 int layout(int32_t n, std::vector<int64_t> &rstart, std::vector<SlotRec> &recs, float slack_factor,
@@ -66,10 +56,7 @@ int layout(int32_t n, std::vector<int64_t> &rstart, std::vector<SlotRec> &recs, 
     // kernels can read a row's slot fields four at a time with 16-byte loads
     std::vector<int64_t> offs((size_t)n + 1, 0);
     for (int32_t u = 0; u < n; ++u) {
-        int64_t d = rstart[u + 1] - rstart[u];
-        int64_t r = d + slack_of(d, slack_factor, slack_min);
-        r = (r + MF_ROW_ALIGN - 1) / MF_ROW_ALIGN * MF_ROW_ALIGN;
-        offs[u + 1] = offs[u] + r;
+        offs[u + 1] = offs[u] + mf_row_size(rstart[u + 1] - rstart[u], slack_factor, slack_min);
     }
     if (offs[n] >= (int64_t)INT32_MAX - 1) return MAXFLOW_ERR_TOO_LARGE;
     out.slot_cap = offs[n];

@@ -313,7 +313,43 @@ struct MfHostGraph {
 int mf_build_host(int32_t n, int64_t m, const int32_t *src, const int32_t *dst, const int32_t *cap,
                   float slack_factor, int32_t slack_min, MfHostGraph &out);
 
+// Reserved slots of a row with d used ones: slack of max(smin, ceil(d * factor)), rounded up
+// so that the next row starts on a 16-byte boundary.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline long long mf_row_size(long long d, float factor, int smin)
+{
+    const double want = (double)d * (double)factor;
+    long long sl = (long long)want;
+    if ((double)sl < want) ++sl;
+    if (sl < smin) sl = smin;
+    if (sl > (1 << 24)) sl = 1 << 24;
+    return (d + sl + MF_ROW_ALIGN - 1) / MF_ROW_ALIGN * MF_ROW_ALIGN;
+}
+
+// build.cu: the same layout, made on the device.  mf_build_sizes uploads, checks and
+// sorts the edges and sizes the rows; the caller then allocates the slot arrays
+// (slots entries each) and mf_build_fill writes them.  Both wait for the stream.
+#define MF_BUILD_MIN 16384            // edge lists shorter than this are built on the host
+#define MF_BUILD_SCRATCH (4ll << 30)  // ... and those that would need more scratch memory than this
+struct MfBuild {
+    void *scratch = nullptr;          // device, mf_build_scratch(n, m) bytes
+    int32_t *deg = nullptr, *bdeg = nullptr;   // device, [n]
+    long long pairs = 0;              // used slots
+    long long slots = 0;              // reserved slots
+    long long merged = 0;             // directed edges with a capacity
+    double cap_sum = 0;
+    int bits = 0, launches = 0;
+};
+size_t mf_build_scratch(int n, long long m);
+int mf_build_sizes(MfBuild &b, int n, long long m, const int32_t *src, const int32_t *dst, const int32_t *cap,
+                   float slack_factor, int slack_min, void *stream);
+int mf_build_fill(MfBuild &b, int n, long long m, const MfGraph &g, void *stream);
+
 // solver.cu
+// Exclusive scan of a[0 .. n) in place, its total into a[n]; mf_rebuild_scratch(n) values.  Three kernels.
+int mf_scan64(long long *a, long long n, void *stream);
 // cluster: 1, or MF_CLUSTER (then grid, and gsize, are multiples of it)
 int mf_launch(const MfParams &p, int grid, int cluster, void *stream);
 int mf_launch_multi(const MfParams *plist_dev, int count, int gsize, int grid, unsigned *gstate, unsigned *head,

@@ -3901,13 +3901,7 @@ __global__ void k_row_capacity(MfParams P, float slack_factor, int slack_min, lo
 {
     for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < P.g.n;
          u += (long long)gridDim.x * blockDim.x) {
-        long long need = (long long)P.g.deg[u] + P.sc.ins_need[u];
-        double want = (double)need * (double)slack_factor;
-        long long sl = (long long)want;
-        if ((double)sl < want) ++sl;
-        if (sl < slack_min) sl = slack_min;
-        if (sl > (1 << 24)) sl = 1 << 24;
-        cap_out[u] = (need + sl + MF_ROW_ALIGN - 1) / MF_ROW_ALIGN * MF_ROW_ALIGN;   // rows stay 16-byte aligned
+        cap_out[u] = mf_row_size((long long)P.g.deg[u] + P.sc.ins_need[u], slack_factor, slack_min);
     }
 }
 
@@ -4316,14 +4310,20 @@ int mf_rebuild_capacity(const MfParams &p, void *stream, float slack_factor, int
     if (g < 1) g = 1;
     k_row_capacity<<<g, 256, 0, st>>>(p, slack_factor, slack_min, noff);
     if (cudaGetLastError() != cudaSuccess) return MAXFLOW_ERR_CUDA;
-    // the tile totals sit behind the n + 1 row starts (mf_rebuild_scratch)
-    const long long nt = mf_scan_tiles(p.g.n);
-    long long *part = noff + p.g.n + 1;
-    k_scan_tiles<<<(int)nt, kScanThreads, 0, st>>>(noff, p.g.n, part);
+    return mf_scan64(noff, p.g.n, stream);
+}
+
+// The tile totals sit behind the n + 1 values (mf_rebuild_scratch).
+int mf_scan64(long long *a, long long n, void *stream)
+{
+    cudaStream_t st = (cudaStream_t)stream;
+    const long long nt = mf_scan_tiles(n);
+    long long *part = a + n + 1;
+    k_scan_tiles<<<(int)nt, kScanThreads, 0, st>>>(a, n, part);
     if (cudaGetLastError() != cudaSuccess) return MAXFLOW_ERR_CUDA;
     k_scan_parts<<<1, kScanThreads, 0, st>>>(part, nt);
     if (cudaGetLastError() != cudaSuccess) return MAXFLOW_ERR_CUDA;
-    k_scan_add<<<(int)nt, kScanThreads, 0, st>>>(noff, p.g.n, part, nt);
+    k_scan_add<<<(int)nt, kScanThreads, 0, st>>>(a, n, part, nt);
     return cuda_rc(cudaGetLastError());
 }
 
