@@ -178,6 +178,7 @@ enum { SQ_SPILL = 1,      // something went onto the grid's lists: long rows, a 
 // state (the same in every CTA between two barriers), and work space of phases.
 struct Sh {
     long long sink_e, src_e;          // excess of the sink and the source, added to memory before every barrier
+    long long value;                  // this CTA's share of the value
     long long stat[MF_STATS];         // work counters, added to memory at the end of the launch
     unsigned long long lab;           // BFS: vertices labelled this phase << 32 | their slots
     unsigned long long exc, dem;      // near BFS: excess labelled, what the roots can take, this phase
@@ -227,9 +228,25 @@ enum Hook {
     H_EXPANDED,           // unused (long rows are split into work items as they are queued); keeps the trace ids
 };
 
+// x += v, x in shared memory, as two 32-bit additions with the carry between
+// them.  A 64-bit atomic on shared memory is a loop of compare and swap, which
+// the threads of a CTA that add to one word run one after another, dozens of
+// clocks each; 32-bit additions to one word are combined in hardware (512
+// threads: 42 clocks).
+template <class T>
+__device__ __forceinline__ void add_shared(T &x, long long v)
+{
+    static_assert(sizeof(T) == 8, "a 64-bit word");
+    unsigned *w = reinterpret_cast<unsigned *>(&x);
+    const unsigned lo = (unsigned)v;
+    const unsigned old = atomicAdd(w, lo);
+    const unsigned hi = (unsigned)((unsigned long long)v >> 32) + (old + lo < old ? 1u : 0u);
+    if (hi) atomicAdd(w + 1, hi);
+}
+
 __device__ __forceinline__ void add_stat(Sh &sh, MfStat i, long long v)
 {
-    if (v) atomicAdd((unsigned long long *)&sh.stat[i], (unsigned long long)v);
+    if (v) add_shared(sh.stat[i], v);
 }
 
 __device__ __forceinline__ int cnt32(const Sh &sh, int line) { return sh.cnt[line].x; }
@@ -725,6 +742,7 @@ __device__ __noinline__ bool finish(const MfParams &P, Sh &sh)
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
         if (lane < MF_STATS && sh.stat[lane]) atomic_add_ll(&c->stat[lane], sh.stat[lane]);
+        if (lane == 31 && sh.value) atomic_add_ll(&c->value, sh.value);
         __syncwarp();
         arrive(P, sh);
         if (lane == 0) signal_all(P, sh);
@@ -785,9 +803,9 @@ __device__ __noinline__ bool finish(const MfParams &P, Sh &sh)
 __device__ __forceinline__ void add_excess(const MfParams &P, Sh &sh, int z, long long d)
 {
     if (z == P.sink)
-        atomicAdd((unsigned long long *)&sh.sink_e, (unsigned long long)d);
+        add_shared(sh.sink_e, d);
     else if (z == P.source)
-        atomicAdd((unsigned long long *)&sh.src_e, (unsigned long long)d);
+        add_shared(sh.src_e, d);
     else
         atomic_add_ll(P.e + z, d);
 }
@@ -836,12 +854,12 @@ __device__ __noinline__ void phase_saturate_source(const MfParams &P, Sh &sh)
         P.cf[y] = ldg_cg(P.g.pcap + x);
         int z = ldg_cg(P.g.dst + x);
         if (z == P.sink)
-            atomicAdd((unsigned long long *)&sh.sink_e, (unsigned long long)(long long)c);
+            add_shared(sh.sink_e, c);
         else
             P.e[z] = c;
         acc -= c;
     }
-    if (acc) atomicAdd((unsigned long long *)&sh.src_e, (unsigned long long)acc);
+    if (acc) add_shared(sh.src_e, acc);
 }
 
 // Static push-pull (Sec. 5.2.2): every edge into t is saturated as well; its
@@ -863,7 +881,7 @@ __device__ __noinline__ void phase_saturate_sink(const MfParams &P, Sh &sh)
             acc += c;
         }
     }
-    if (acc) atomicAdd((unsigned long long *)&sh.sink_e, (unsigned long long)acc);
+    if (acc) add_shared(sh.sink_e, acc);
 }
 
 // Dynamic push-pull (Sec. 5.2.2): the sides of the last cut, read from the
@@ -1204,7 +1222,7 @@ __device__ __noinline__ void phase_resaturate(const MfParams &P, Sh &sh)
             acc -= c;
         }
     }
-    if (acc) atomicAdd((unsigned long long *)&sh.src_e, (unsigned long long)acc);
+    if (acc) add_shared(sh.src_e, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -1268,7 +1286,7 @@ __device__ __forceinline__ void place_labelled(const MfParams &P, Sh &sh, int z,
     }
     if (ev > 0) {
         place_active(P, sh, z, d, L_WL, sh.d.wl_sel, sh.d.wl_app);
-        if (sh.d.near) atomicAdd(&sh.exc, (unsigned long long)ev);
+        if (sh.d.near) add_shared(sh.exc, ev);
     }
 }
 
@@ -1282,7 +1300,7 @@ __device__ __forceinline__ void flush_queue(const MfParams &P, Sh &sh, int line,
     __syncwarp();
     lab = __reduce_add_sync(0xffffffffu, lab);
     lab_slots = __reduce_add_sync(0xffffffffu, lab_slots);
-    if (lane == 0 && lab) atomicAdd(&sh.lab, ((unsigned long long)(unsigned)lab << 32) | lab_slots);
+    if (lane == 0 && lab) add_shared(sh.lab, ((long long)lab << 32) | lab_slots);
     __syncthreads();
     const int nb = min(sh.q_bfs, MF_Q_BFS), nl = min(sh.q_long, MF_Q_LONG), nw = min(sh.q_wn, MF_Q_WL);
     if (nb + nw > 0) {
@@ -1366,7 +1384,7 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
         }
         total += dall;
     }
-    if (take) atomicAdd(&sh.dem, (unsigned long long)take);
+    if (take) add_shared(sh.dem, take);
     flush_labelled(P, sh, lab, lab_slots);
     if (need_total) {
         // one atomic per CTA for the used-slot total
@@ -1810,9 +1828,9 @@ __device__ __forceinline__ void move_flow(const MfParams &P, Sh &sh, int x, int 
     }
     const long long dz = PULL ? -amt : amt;
     if (z == P.sink) {
-        atomicAdd((unsigned long long *)&sh.sink_e, (unsigned long long)dz);
+        add_shared(sh.sink_e, dz);
     } else if (z == P.source) {
-        atomicAdd((unsigned long long *)&sh.src_e, (unsigned long long)dz);
+        add_shared(sh.src_e, dz);
     } else {
         const long long old = atomic_add_ll(P.e + z, dz);
         const bool became = PULL ? (old >= 0 && old + dz < 0) : (old <= 0 && old + dz > 0);
@@ -2780,7 +2798,7 @@ __device__ __forceinline__ void squad_visit(const MfParams &P, Sh &sh, const int
         if (ev[r] > 0 && z[r] != P.sink) {
             const int bin = row_bin(P, d[r]);
             P.sc.wl[sh.d.wl_sel][bin][sh.d.wl_app[bin] + atomicAdd(&sh.cs->l[L_WL + bin].w[0], 1u)] = z[r];
-            if (near) atomicAdd(&sh.exc, (unsigned long long)ev[r]);
+            if (near) add_shared(sh.exc, ev[r]);
         }
     }
 }
@@ -2849,7 +2867,7 @@ __device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
         lab = __reduce_add_sync(0xffffffffu, lab);
         lab_slots = __reduce_add_sync(0xffffffffu, lab_slots);
         if (lane == 0) {
-            if (lab) atomicAdd(&sh.lab, ((unsigned long long)(unsigned)lab << 32) | lab_slots);
+            if (lab) add_shared(sh.lab, ((long long)lab << 32) | lab_slots);
             add_stat(sh, ST_SLOTS_BFS, scanned);
         }
         __syncthreads();
@@ -2945,9 +2963,9 @@ __device__ __forceinline__ void short_push(const MfParams &P, Sh &sh, int x, int
     atomicSub(P.cf + x, g);
     atomicAdd(P.cf + y, g);
     if (z == P.sink) {
-        atomicAdd((unsigned long long *)&sh.sink_e, (unsigned long long)g);
+        add_shared(sh.sink_e, g);
     } else if (z == P.source) {
-        atomicAdd((unsigned long long *)&sh.src_e, (unsigned long long)g);
+        add_shared(sh.src_e, g);
     } else {
         const int d = ldg_cg(P.g.deg + z), r0 = SQUAD ? P.g.off[z] : 0;     // in flight together with the excess
         const long long old = atomic_add_ll(P.e + z, (long long)g);
@@ -3407,7 +3425,7 @@ __device__ __noinline__ void phase_fix(const MfParams &P, Sh &sh)
 // Value (Alg. 5 last lines, reading R3)
 // ---------------------------------------------------------------------------
 
-__device__ __noinline__ void phase_value(const MfParams &P)
+__device__ __noinline__ void phase_value(const MfParams &P, Sh &sh)
 {
     // push (R3): sum of e(v) over v != s with h(v) < n; pull (Sec. 5.2.2, the
     // mirror): sum of -e(v) over v != t with h(v) < n
@@ -3418,7 +3436,7 @@ __device__ __noinline__ void phase_value(const MfParams &P)
     for (long long v = (long long)vb() * blockDim.x + threadIdx.x; v < n; v += (long long)vn() * blockDim.x)
         if ((int)v != skip && ldg_cg(P.h + v) < n) acc += pull ? -ldg_cg(P.e + v) : ldg_cg(P.e + v);
     acc = warp_sum_ll(acc);
-    if ((threadIdx.x & 31) == 0 && acc) atomic_add_ll(&P.ctrl->value, acc);
+    if ((threadIdx.x & 31) == 0 && acc) add_shared(sh.value, acc);
 }
 
 // One whole solve of one instance by the vn() CTAs of the caller: the
@@ -3432,7 +3450,7 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
     if (threadIdx.x < MF_STATS) sh.stat[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         MfCtrl *c = P.ctrl;
-        sh.sink_e = sh.src_e = 0;
+        sh.sink_e = sh.src_e = sh.value = 0;
         sh.lab = sh.exc = sh.dem = 0;
         sh.q_bfs = sh.q_long = sh.q_wn = 0;
         for (int b = 0; b < MF_NBIN; ++b) sh.q_wl[b] = 0;
@@ -3569,7 +3587,7 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
             if (!grid_sync(P, H_ITER, sh)) return false;
         }
     }
-    if (sh.d.status != MF_ST_ERROR && !(P.mode & MF_M_NO_VALUE)) phase_value(P);
+    if (sh.d.status != MF_ST_ERROR && !(P.mode & MF_M_NO_VALUE)) phase_value(P, sh);
     return finish(P, sh);
 }
 
