@@ -25,8 +25,8 @@
 #define MF_HUB_DEG 512        // discharge: rows above this many slots get a 4-warp group (or a whole CTA)
 #define MF_NBIN 4             // discharge row kinds: thread, warp, 4-warp group, CTA
 #define MF_GROUP_WARPS 4      // warps of a group; a group keeps rows up to a quarter of the snapshot
-#define MF_BFS_HUB 256        // BFS: rows above this many slots enter the frontier as work items
-#define MF_BFS_CHUNK 256      // BFS: slots per work item
+#define MF_BFS_HUB 128        // BFS: rows above this many slots enter the frontier as work items
+#define MF_BFS_CHUNK 128      // BFS: slots per work item
 #define MF_DEFAULT_ROUNDS 2   // adaptive discharge rounds: the minimum per iteration
 #define MF_MAX_ROUNDS 1024    // adaptive rounds: upper bound per iteration
 #define MF_TRACE 256          // hook timeline entries kept per launch
@@ -46,7 +46,8 @@
 #define MF_Q_INTS (MF_Q_BFS + MF_Q_LONG + 2 * MF_Q_WL)
 #define MF_CLUSTER 8          // CTAs per thread-block cluster; the first cluster is the squad
 #define MF_SQUAD_CAP 4096     // queue entries of a squad CTA
-#define MF_SQUAD_INTS (6 * MF_SQUAD_CAP)   // its shared memory: two queues of vertex, row start, row length
+#define MF_SQUAD_LONG 1024    // long-row vertices a squad CTA keeps on chip
+#define MF_SQUAD_INTS (6 * MF_SQUAD_CAP + MF_SQUAD_LONG)   // two queues of vertex, row start, row length; long rows
 #define MF_SQUAD_LEVEL 256    // BFS levels of at most this many vertices per squad CTA ...
 #define MF_SQUAD_SLOTS 2048   // ... and slots run in the squad
 #define MF_SQUAD_ACTIVE 256   // so do discharge rounds of at most this many vertices per squad CTA

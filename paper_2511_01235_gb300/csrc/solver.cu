@@ -38,6 +38,14 @@ constexpr unsigned long long kEmpty = ~0ull;
 // vb() in [0, vn()), and the grid barrier waits for vn() CTAs.
 __shared__ int g_vb, g_vn;
 
+// The parameters of the running solve, in shared memory: the phases read them
+// often.  P and sh (below) are variables of the file and not arguments, so that
+// the compiler knows that they are shared memory: through a pointer every
+// access is a generic one and every addition to a counter a choice between two
+// kinds of atomics, which had made a single phase 20 to 80 KB of code, more than
+// the instruction cache holds beside the rest of an iteration.
+__shared__ MfParams P;
+
 // Dynamic shared memory of the persistent kernels: the on-chip snapshot of a
 // row during its discharge (P.stage_slots ints).
 extern __shared__ __align__(16) int mf_stage[];
@@ -50,7 +58,7 @@ __device__ __forceinline__ int vn() { return g_vn; }
 // every SM's memory pipeline busy instead of crowding onto the first CTAs.
 // spread_warp keeps 32 consecutive indices in one warp (warp-uniform loops).
 // Row kind of a vertex with d used slots: 0 thread, 1 warp, 2 four-warp group, 3 CTA.
-__device__ __forceinline__ int row_bin(const MfParams &P, int d)
+__device__ __forceinline__ int row_bin(int d)
 {
     return d <= P.small_deg ? 0 : (d <= P.hub_deg ? 1 : (d <= P.group_deg ? 2 : 3));
 }
@@ -201,7 +209,7 @@ struct Sh {
     int csize, crank, one_cluster;
     unsigned arrivals;                // arrivals at the grid barrier so far
     SquadSum sq[2][MF_CLUSTER];
-    int so_cnt, so_flag, so_go, so_par;
+    int so_cnt, so_long, so_flag, so_go, so_par;
     // on-chip queue of a phase (place_labelled, place_active): entries taken, per kind
     int q_bfs, q_long, q_wn, q_wl[MF_NBIN];
     int q_base[MF_NBIN + 1];
@@ -209,6 +217,8 @@ struct Sh {
     MfDesc d;
     MfState hs;
 };
+
+__shared__ Sh sh;
 
 enum Hook {
     H_START = 0,          // unused (a launch starts without a barrier); keeps the trace ids
@@ -244,20 +254,20 @@ __device__ __forceinline__ void add_shared(T &x, long long v)
     if (hi) atomicAdd(w + 1, hi);
 }
 
-__device__ __forceinline__ void add_stat(Sh &sh, MfStat i, long long v)
+__device__ __forceinline__ void add_stat(MfStat i, long long v)
 {
     if (v) add_shared(sh.stat[i], v);
 }
 
-__device__ __forceinline__ int cnt32(const Sh &sh, int line) { return sh.cnt[line].x; }
-__device__ __forceinline__ unsigned long long cnt64(const Sh &sh, int line)
+__device__ __forceinline__ int cnt32(int line) { return sh.cnt[line].x; }
+__device__ __forceinline__ unsigned long long cnt64(int line)
 {
     return (unsigned long long)(unsigned)sh.cnt[line].x | ((unsigned long long)(unsigned)sh.cnt[line].y << 32);
 }
 
 // A top-down level of cnt vertices with fr slots, none of them long, that the
 // squad runs alone (squad_bfs).
-__device__ __forceinline__ bool squad_level(const Sh &sh, long long cnt, long long fr)
+__device__ __forceinline__ bool squad_level(long long cnt, long long fr)
 {
     return sh.k_squad > 0 && cnt <= MF_SQUAD_LEVEL * sh.csize && fr <= sh.k_squad;
 }
@@ -277,7 +287,7 @@ __device__ __forceinline__ bool rounds_left(const MfDesc &d, const MfState &st, 
 // squad (squad_discharge).  On a small graph that takes a BFS of many levels:
 // short rounds pay where many rounds follow; where two or three do, the whole
 // KERNEL_CYCLES in each settle more.
-__device__ __forceinline__ void pick_round(const MfParams &P, MfDesc &d, int csize)
+__device__ __forceinline__ void pick_round(MfDesc &d, int csize)
 {
     d.dis_short = P.rounds == 0 && !P.pull && !P.fix_steep && P.data_driven && P.requeue &&
                           P.stage_slots >= MF_SQUAD_INTS && P.hub_deg <= MF_SHORT_ROW &&
@@ -289,7 +299,7 @@ __device__ __forceinline__ void pick_round(const MfParams &P, MfDesc &d, int csi
 
 // The termination test of the loop (Alg. 1 / Alg. 5: stop when no active
 // vertex remains), taken right after a complete backward BFS.
-__device__ __forceinline__ void decide_iteration(const MfParams &P, Sh &sh, int active)
+__device__ __forceinline__ void decide_iteration(int active)
 {
     MfDesc &d = sh.d;
     MfState &st = sh.hs;
@@ -299,7 +309,7 @@ __device__ __forceinline__ void decide_iteration(const MfParams &P, Sh &sh, int 
     ++d.fstamp;
     st.t_dis0 = st.t_now;
     for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = d.wl_app[b];
-    pick_round(P, d, sh.csize);
+    pick_round(d, sh.csize);
     if (d.near) d.dis_short = d.dis_squad = 0;        // a near iteration starts with the walks
     if (st.iters == 0) st.active_first = active;
     st.active_total += active;
@@ -317,7 +327,7 @@ __device__ __forceinline__ void decide_iteration(const MfParams &P, Sh &sh, int 
 // longer sink row (grids: every pixel has an edge to t) what the sink can take
 // exceeds any excess, no relabel would be cut, and the bookkeeping would only
 // cost.
-__device__ __forceinline__ int near_allowed(const MfParams &P)
+__device__ __forceinline__ int near_allowed()
 {
     if (P.sc.par == nullptr || !(P.mode & MF_M_SOLVE) || (P.mode & MF_M_NO_DEFICIT_ROOTS) || P.pull ||
         P.side_root >= 0 || P.rounds != 0 || P.fix_steep || !P.data_driven || P.g.slot_cap < MF_LARGE_SLOTS)
@@ -326,7 +336,7 @@ __device__ __forceinline__ int near_allowed(const MfParams &P)
 }
 
 // Opens an iteration of the loop (its BFS comes next).
-__device__ __forceinline__ void begin_iteration(Sh &sh)
+__device__ __forceinline__ void begin_iteration()
 {
     MfDesc &d = sh.d;
     sh.hs.t_bfs0 = sh.hs.t_now;
@@ -343,13 +353,13 @@ __device__ __forceinline__ void begin_iteration(Sh &sh)
 // After a phase of the BFS.  On the critical path of every level: all it needs
 // is read before anything is written, so its shared-memory accesses overlap
 // instead of following one another.  Returns what the trace shows.
-__device__ __forceinline__ int advance_bfs(const MfParams &P, int &hook, Sh &sh)
+__device__ __forceinline__ int advance_bfs(int &hook)
 {
     MfDesc &d = sh.d;
     MfState &st = sh.hs;
-    const int c_bfs = cnt32(sh, L_BFS), c_hub = cnt32(sh, L_HUB), c_defer = cnt32(sh, L_DEFER);
-    const int c_w0 = cnt32(sh, L_WL), c_w1 = cnt32(sh, L_WL + 1), c_w2 = cnt32(sh, L_WL + 2), c_w3 = cnt32(sh, L_WL + 3);
-    const unsigned long long lab = cnt64(sh, L_LAB), exc = cnt64(sh, L_EXC);
+    const int c_bfs = cnt32(L_BFS), c_hub = cnt32(L_HUB), c_defer = cnt32(L_DEFER);
+    const int c_w0 = cnt32(L_WL), c_w1 = cnt32(L_WL + 1), c_w2 = cnt32(L_WL + 2), c_w3 = cnt32(L_WL + 3);
+    const unsigned long long lab = cnt64(L_LAB), exc = cnt64(L_EXC);
     const int alpha = sh.k_alpha, beta = sh.k_beta, want_wl = sh.k_wl, n = P.g.n, near = d.near;
     const int app_bfs = d.app_bfs + c_bfs, app_hub = d.app_hub + c_hub;
     const int w0 = d.wl_app[0] + c_w0, w1 = d.wl_app[1] + c_w1, w2 = d.wl_app[2] + c_w2, w3 = d.wl_app[3] + c_w3;
@@ -381,12 +391,12 @@ __device__ __forceinline__ int advance_bfs(const MfParams &P, int &hook, Sh &sh)
     }
     const bool first = hook == H_BFS_START;
     if (first) {
-        if (d.need_total) st.used_slots = used = (long long)cnt64(sh, L_TOTAL);
+        if (d.need_total) st.used_slots = used = (long long)cnt64(L_TOTAL);
         if (near) {
             // a cut-short relabel whose walks settled less than half of what was
             // open looks for more excess this time, so that after a few of them
             // the relabel is a complete one
-            dem = (long long)cnt64(sh, L_DEM);
+            dem = (long long)cnt64(L_DEM);
             if (st.cut_prev && 2 * dem > st.dem_prev) shift = min(shift + MF_NEAR_STEP, 60);
             st.cut_shift = shift;
             st.dem = st.dem_prev = dem;
@@ -410,13 +420,13 @@ __device__ __forceinline__ int advance_bfs(const MfParams &P, int &hook, Sh &sh)
     else if (bu && cnt * beta < (long long)n) bu = 0;
     d.bu_mode = bu;
     d.bu_split = 0;
-    d.bfs_squad = !done && !bu && app_hub == hub_hi && squad_level(sh, cnt, fr) ? 1 : 0;
+    d.bfs_squad = !done && !bu && app_hub == hub_hi && squad_level(cnt, fr) ? 1 : 0;
     // near iterations: the levels so far hold as much excess as the roots can take
     const int cut = near && !done && sup > 0 && (sup >> shift) >= dem ? 1 : 0;
     d.cut = cut;
     st.cut_prev = cut;
     d.bfs_done = done || cut ? 1 : 0;
-    if ((done || cut) && want_wl) decide_iteration(P, sh, w0 + w1 + w2 + w3);
+    if ((done || cut) && want_wl) decide_iteration(w0 + w1 + w2 + w3);
     return ((first ? 0 : bu_was) << 30) | ((first ? 0 : min(hub_hi - hub_lo, 1023)) << 20) |
            (int)min(cnt, (long long)((1 << 20) - 1));
 }
@@ -425,7 +435,7 @@ __device__ __forceinline__ int advance_bfs(const MfParams &P, int &hook, Sh &sh)
 // counters of the phase that ended (sh.cnt) and the state all CTAs share, in
 // shared memory only, so all of them arrive at the same answer.  t: the first
 // CTA's clock.
-__device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsigned long long t)
+__device__ __noinline__ void advance(int hook, unsigned long long t)
 {
     MfDesc &d = sh.d;
     MfState &st = sh.hs;
@@ -442,7 +452,7 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
     int tinfo = 0;
     if (hook == H_BU_SPLIT || hook == H_BFS_START || hook == H_BFS_NEXT) {
         st.ns_bfs += dt;
-        sh.tr_info = advance_bfs(P, hook, sh);
+        sh.tr_info = advance_bfs(hook);
         sh.tr_hook = hook;
         if (err != 0) d.status = MF_ST_ERROR;
         return;
@@ -464,12 +474,12 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
     case H_ITER:
         if (P.mode & (MF_M_STATIC_INIT | MF_M_APPLY) && st.iters == 0) st.ns_apply += dt;
         else st.ns_fix += dt;
-        begin_iteration(sh);
+        begin_iteration();
         break;
     case H_WL:
         st.ns_wl += dt;
-        for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] = cnt32(sh, L_WL + b);
-        decide_iteration(P, sh, cnt32(sh, L_ACT));
+        for (int b = 0; b < MF_NBIN; ++b) d.wl_app[b] = cnt32(L_WL + b);
+        decide_iteration(cnt32(L_ACT));
         break;
     case H_DIS: {
         // after a discharge round: run another one over the vertices that
@@ -478,10 +488,10 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         tinfo = (min(d.wl_n[2] + d.wl_n[3], 1023) << 20) |
                 min(d.wl_n[0] + d.wl_n[1] + d.wl_n[2] + d.wl_n[3], (1 << 20) - 1);
         ++st.rounds_total;
-        d.fix_n[0] += cnt32(sh, L_FIX);
-        d.fix_n[1] += cnt32(sh, L_FIX + 1);
+        d.fix_n[0] += cnt32(L_FIX);
+        d.fix_n[1] += cnt32(L_FIX + 1);
         int nxt = 0;
-        for (int b = 0; b < MF_NBIN; ++b) nxt += cnt32(sh, L_AUX + b);
+        for (int b = 0; b < MF_NBIN; ++b) nxt += cnt32(L_AUX + b);
         // fixed: P.rounds rounds; adaptive (P.rounds == 0): at least
         // MF_DEFAULT_ROUNDS, then more while this iteration's discharge has
         // taken less than half of its BFS -- a global relabel that costs much
@@ -496,14 +506,14 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
         d.dis_more = more ? 1 : 0;
         if (more) {
             d.wl_sel ^= 1;
-            for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = cnt32(sh, L_AUX + b);
+            for (int b = 0; b < MF_NBIN; ++b) d.wl_n[b] = cnt32(L_AUX + b);
             ++d.round;
             ++d.qstamp;
-            pick_round(P, d, sh.csize);
+            pick_round(d, sh.csize);
         } else if (!P.fix_steep) {
             // without Alg. 3 the next iteration's BFS follows at once: this
             // barrier opens it
-            begin_iteration(sh);
+            begin_iteration();
         }
         break;
     }
@@ -518,7 +528,7 @@ __device__ __noinline__ void advance(const MfParams &P, int hook, Sh &sh, unsign
 // One entry of the hook timeline, written by the last warp of the first CTA
 // beside the phase that follows: the barrier, when it was reached, and from
 // what every CTA left before arriving when they finished and the slots scanned.
-__device__ __noinline__ void write_trace(const MfParams &P, Sh &sh, unsigned phase)
+__device__ __noinline__ void write_trace(unsigned phase)
 {
     MfCtrl *c = P.ctrl;
     const int lane = threadIdx.x & 31;
@@ -564,7 +574,7 @@ __device__ __forceinline__ void words_in(int *sh_dst, const int *src, int words)
 // Excess of sink and source and the BFS label counters go to memory, the
 // finish time and the slots scanned into this CTA's place.  Called by warp 0
 // after a __syncthreads.
-__device__ __forceinline__ void arrive(const MfParams &P, Sh &sh)
+__device__ __forceinline__ void arrive()
 {
     MfCtrl *c = P.ctrl;
     const int lane = threadIdx.x & 31;
@@ -600,7 +610,7 @@ __device__ __forceinline__ void arrive(const MfParams &P, Sh &sh)
 }
 
 // One thread: this CTA is at the grid barrier.
-__device__ __forceinline__ void signal_all(const MfParams &P, Sh &sh)
+__device__ __forceinline__ void signal_all()
 {
     ++sh.arrivals;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&P.ctrl->bar.w[0]) : "memory");
@@ -608,7 +618,7 @@ __device__ __forceinline__ void signal_all(const MfParams &P, Sh &sh)
 
 // Wait until every CTA has arrived at the current barrier; false after the
 // wait limit (MF_E_WAIT is recorded).  One thread.
-__device__ __forceinline__ bool wait_all(const MfParams &P, Sh &sh)
+__device__ __forceinline__ bool wait_all()
 {
     MfCtrl *c = P.ctrl;
     const unsigned target = sh.arrivals * (unsigned)vn();
@@ -655,14 +665,14 @@ __device__ __forceinline__ void cluster_sync()
 }
 
 // The squad's own barrier; called by all its threads.
-__device__ __forceinline__ void squad_sync(const Sh &sh)
+__device__ __forceinline__ void squad_sync()
 {
     if (sh.csize > 1) cluster_sync();
     else __syncthreads();
 }
 
 // sq[par][my rank] in every CTA of the squad = mine, by one warp; visible behind squad_sync.
-__device__ __forceinline__ void squad_tell(Sh &sh, int par, const SquadSum &mine)
+__device__ __forceinline__ void squad_tell(int par, const SquadSum &mine)
 {
     const int lane = threadIdx.x & 31;
     constexpr int kW = (int)(sizeof(SquadSum) / 4);
@@ -686,7 +696,7 @@ __device__ __forceinline__ void squad_tell(Sh &sh, int par, const SquadSum &mine
 // behind the barrier for all held them up for another 3 us.  A solve that is
 // one cluster uses the cluster's barrier.  With take_state, every CTA takes the
 // first one's state (its squad ran phases alone) before working out the next.
-__device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh, bool take_state = false)
+__device__ __noinline__ bool grid_sync(int hook, bool take_state = false)
 {
     MfCtrl *c = P.ctrl;
     __syncthreads();
@@ -697,15 +707,15 @@ __device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh, bool
             words_out((int *)&c->jd, (const int *)&sh.d, (int)(sizeof(MfDesc) / 4));
             words_out((int *)&c->js, (const int *)&sh.hs, (int)(sizeof(MfState) / 4));
         }
-        arrive(P, sh);
+        arrive();
     }
     if (one) cluster_sync();
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
         int ok = 1;
         if (lane == 0 && !one) {
-            signal_all(P, sh);
-            ok = wait_all(P, sh) ? 1 : 0;
+            signal_all();
+            ok = wait_all() ? 1 : 0;
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
         __syncwarp();
@@ -719,7 +729,7 @@ __device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh, bool
                 words_in((int *)&sh.hs, (const int *)&c->js, (int)(sizeof(MfState) / 4));
             }
             __syncwarp();
-            if (lane == 0) advance(P, hook, sh, cnt64(sh, L_TIME));
+            if (lane == 0) advance(hook, cnt64(L_TIME));
         }
         if (lane == 0) {
             sh.ok = ok;
@@ -728,14 +738,14 @@ __device__ __noinline__ bool grid_sync(const MfParams &P, int hook, Sh &sh, bool
         }
     }
     __syncthreads();
-    if (vb() == 0 && (threadIdx.x >> 5) == (blockDim.x >> 5) - 1 && sh.ok) write_trace(P, sh, k);
+    if (vb() == 0 && (threadIdx.x >> 5) == (blockDim.x >> 5) - 1 && sh.ok) write_trace(k);
     return sh.ok != 0;
 }
 
 // The end of a launch: the counters go to the control block, every CTA arrives
 // once more, and the first one alone waits for the others, writes the results
 // down and leaves barrier and counter sets at zero for the next launch.
-__device__ __noinline__ bool finish(const MfParams &P, Sh &sh)
+__device__ __noinline__ bool finish()
 {
     MfCtrl *c = P.ctrl;
     __syncthreads();
@@ -744,11 +754,11 @@ __device__ __noinline__ bool finish(const MfParams &P, Sh &sh)
         if (lane < MF_STATS && sh.stat[lane]) atomic_add_ll(&c->stat[lane], sh.stat[lane]);
         if (lane == 31 && sh.value) atomic_add_ll(&c->value, sh.value);
         __syncwarp();
-        arrive(P, sh);
-        if (lane == 0) signal_all(P, sh);
+        arrive();
+        if (lane == 0) signal_all();
         if (vb() == 0) {
             int ok = 0;
-            if (lane == 0) ok = wait_all(P, sh) ? 1 : 0;
+            if (lane == 0) ok = wait_all() ? 1 : 0;
             ok = __shfl_sync(0xffffffffu, ok, 0);
             __syncwarp();
             if (lane == 0) {
@@ -762,7 +772,7 @@ __device__ __noinline__ bool finish(const MfParams &P, Sh &sh)
             }
             __syncwarp();
             if (ok) {
-                write_trace(P, sh, sh.phase);
+                write_trace(sh.phase);
                 const int4 zero = make_int4(0, 0, 0, 0);
                 if (lane < MF_LINES)
                     for (int q = 0; q < 3; ++q) __stcg(reinterpret_cast<int4 *>(&c->set[q].l[lane]), zero);
@@ -800,7 +810,7 @@ __device__ __noinline__ bool finish(const MfParams &P, Sh &sh)
 }
 
 // Add d to the excess of z (sink and source go to the CTA accumulators).
-__device__ __forceinline__ void add_excess(const MfParams &P, Sh &sh, int z, long long d)
+__device__ __forceinline__ void add_excess(int z, long long d)
 {
     if (z == P.sink)
         add_shared(sh.sink_e, d);
@@ -816,7 +826,7 @@ __device__ __forceinline__ void add_excess(const MfParams &P, Sh &sh, int z, lon
 
 // c_f = c on every slot, e = h = 0: a streaming copy, 16-byte vectors with four
 // in flight per thread (the slot arrays start on 256-byte boundaries).
-__device__ __noinline__ void phase_static_reset(const MfParams &P)
+__device__ __noinline__ void phase_static_reset()
 {
     const long long gt = (long long)vb() * blockDim.x + threadIdx.x;
     const long long gs = (long long)vn() * blockDim.x;
@@ -840,7 +850,7 @@ __device__ __noinline__ void phase_static_reset(const MfParams &P)
     }
 }
 
-__device__ __noinline__ void phase_saturate_source(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_saturate_source()
 {
     const int s = P.source;
     const int r0 = P.g.off[s];
@@ -864,7 +874,7 @@ __device__ __noinline__ void phase_saturate_source(const MfParams &P, Sh &sh)
 
 // Static push-pull (Sec. 5.2.2): every edge into t is saturated as well; its
 // tail keeps the deficit, and the deficient vertices then act as sinks.
-__device__ __noinline__ void phase_saturate_sink(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_saturate_sink()
 {
     const int t = P.sink;
     const int r0 = P.g.off[t];
@@ -877,7 +887,7 @@ __device__ __noinline__ void phase_saturate_sink(const MfParams &P, Sh &sh)
         if (c > 0) {
             P.cf[y] = 0;
             P.cf[x] = ldg_cg(P.cf + x) + c;
-            add_excess(P, sh, ldg_cg(P.g.dst + x), -(long long)c);
+            add_excess(ldg_cg(P.g.dst + x), -(long long)c);
             acc += c;
         }
     }
@@ -887,7 +897,7 @@ __device__ __noinline__ void phase_saturate_sink(const MfParams &P, Sh &sh)
 // Dynamic push-pull (Sec. 5.2.2): the sides of the last cut, read from the
 // heights the previous solve ended with (1: the vertex reached t or a
 // deficit, 0: it did not) ...
-__device__ __noinline__ void phase_cut_side(const MfParams &P)
+__device__ __noinline__ void phase_cut_side()
 {
     const int n = P.g.n;
     const long long gs = (long long)vn() * blockDim.x;
@@ -901,7 +911,7 @@ __device__ __noinline__ void phase_cut_side(const MfParams &P)
 
 // ... then every residual edge from side 0 to side 1 sends all it can, so
 // that no residual path leads from side 0 to side 1.  One warp per row.
-__device__ __noinline__ void phase_saturate_cut(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_saturate_cut()
 {
     const int n = P.g.n;
     const int lane = threadIdx.x & 31;
@@ -918,11 +928,11 @@ __device__ __noinline__ void phase_saturate_cut(const MfParams &P, Sh &sh)
             if (P.side[z] != 1) continue;
             P.cf[x] = 0;
             atomicAdd(P.cf + ldg_cg(P.g.rev + x), c);
-            add_excess(P, sh, z, (long long)c);
+            add_excess(z, (long long)c);
             out += c;
         }
         out = warp_sum_ll(out);
-        if (lane == 0 && out) add_excess(P, sh, (int)u, -out);
+        if (lane == 0 && out) add_excess((int)u, -out);
     }
 }
 
@@ -944,7 +954,7 @@ __device__ __forceinline__ void warp_append(unsigned *tail, int *arr, bool take,
 // Batch apply and repair (Alg. 5)
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ bool batch_entry(const MfParams &P, long long i, int &u, int &v, int &c)
+__device__ __forceinline__ bool batch_entry(long long i, int &u, int &v, int &c)
 {
     u = __ldcg(P.bu + i);
     v = __ldcg(P.bv + i);
@@ -954,7 +964,7 @@ __device__ __forceinline__ bool batch_entry(const MfParams &P, long long i, int 
 
 // Validate every entry; insert the directed key into the dedup table, where
 // the largest batch index (the last update of the pair) wins.
-__device__ __noinline__ void phase_apply_validate(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_apply_validate()
 {
     MfSet *cs = sh.cs;
     const int bits = P.sc.hash_bits;
@@ -967,7 +977,7 @@ __device__ __noinline__ void phase_apply_validate(const MfParams &P, Sh &sh)
         unsigned pos = 0;
         int u, v, c;
         if (i < P.bcount) {
-            if (!batch_entry(P, i, u, v, c)) {
+            if (!batch_entry(i, u, v, c)) {
                 atomicCAS(&cs->l[L_MISC].w[3], 0u, (unsigned)MF_E_INVALID);
             } else if (u != v) {
                 unsigned long long key = ((unsigned long long)(unsigned)u << 32) | (unsigned)v;
@@ -991,7 +1001,7 @@ __device__ __noinline__ void phase_apply_validate(const MfParams &P, Sh &sh)
 // (seven pivots loaded together per round, so a row of 2^15 slots takes five
 // dependent rounds instead of fifteen), then a scan of the inserted slots.
 // *probes counts the dst entries read.
-__device__ __forceinline__ int find_slot(const MfParams &P, int u, int v, int *probes = nullptr)
+__device__ __noinline__ int find_slot(const MfParams &P, int u, int v, int *probes = nullptr)
 {
     const int r0 = P.g.off[u];
     const int bd = ldg_cg(P.g.bdeg + u);
@@ -1029,6 +1039,17 @@ __device__ __forceinline__ int find_slot(const MfParams &P, int u, int v, int *p
     return found;
 }
 
+// Slot of (u, v), or -1, looked for in the shorter of the two rows: the pair has a
+// slot in both, and on power-law graphs one end of most edges is a hub.
+__device__ __forceinline__ int find_pair(int u, int v, int *probes)
+{
+    if (2ll * ldg_cg(P.g.bdeg + v) < ldg_cg(P.g.bdeg + u)) {
+        const int y = find_slot(P, v, u, probes);
+        return y < 0 ? -1 : ldg_cg(P.g.rev + y);
+    }
+    return find_slot(P, u, v, probes);
+}
+
 __device__ __forceinline__ unsigned hash_find(const unsigned long long *keys, int bits, unsigned long long key)
 {
     const unsigned mask = (1u << bits) - 1u;
@@ -1050,7 +1071,7 @@ __device__ __forceinline__ unsigned hash_find(const unsigned long long *keys, in
 // pair -- must fit int32 (residual capacities are int32 and c_f(u,v) +
 // c_f(v,u) equals that sum).  A batch that breaks it sets MF_E_TOO_LARGE and
 // is refused whole.
-__device__ __noinline__ void phase_apply_locate(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_apply_locate()
 {
     MfSet *cs = sh.cs;
     const int bits = P.sc.hash_bits;
@@ -1062,7 +1083,7 @@ __device__ __noinline__ void phase_apply_locate(const MfParams &P, Sh &sh)
         bool fresh = false;
         unsigned pp = 0;
         int u = 0, v = 0, c = 0;
-        if (i < P.bcount) batch_entry(P, i, u, v, c);
+        if (i < P.bcount) batch_entry(i, u, v, c);
         unsigned long long key = ((unsigned long long)(unsigned)u << 32) | (unsigned)v;
         const unsigned pos = (i < P.bcount && u != v) ? hash_find(P.sc.hkey, bits, key) : 0xffffffffu;
         if (i >= P.bcount) {
@@ -1070,7 +1091,7 @@ __device__ __noinline__ void phase_apply_locate(const MfParams &P, Sh &sh)
         } else if (pos == 0xffffffffu || __ldcg(P.sc.hval + pos) != (int)i) {
             P.sc.bslot[i] = -2;     // a self-loop, or a later update of the same pair wins
         } else {
-            const int x = find_slot(P, u, v, &probes);
+            const int x = find_pair(u, v, &probes);
             P.sc.bslot[i] = x;
             {
                 const unsigned long long rkey = ((unsigned long long)(unsigned)v << 32) | (unsigned)u;
@@ -1105,12 +1126,12 @@ __device__ __noinline__ void phase_apply_locate(const MfParams &P, Sh &sh)
         }
         warp_append(&cs->l[L_MISC].w[0], P.sc.ins_list, fresh, (int)pp);   // each new pair once
     }
-    add_stat(sh, ST_SLOTS_APPLY, probes);
+    add_stat(ST_SLOTS_APPLY, probes);
 }
 
 // Winning new capacity of the directed pair (a, b) in the batch, or -1 if the
 // batch does not set it.
-__device__ __forceinline__ int batch_cap_of(const MfParams &P, int a, int b)
+__device__ __forceinline__ int batch_cap_of(int a, int b)
 {
     const unsigned long long key = ((unsigned long long)(unsigned)a << 32) | (unsigned)b;
     const unsigned pos = hash_find(P.sc.hkey, P.sc.hash_bits, key);
@@ -1126,7 +1147,7 @@ __device__ __forceinline__ int batch_cap_of(const MfParams &P, int a, int b)
 // of c_f(u,v) is the owner of (v,u), and the two clamps cannot both fire (the
 // pair's residuals sum to the new c(u,v) + c(v,u) >= 0), so the order of the
 // atomics does not matter.
-__device__ __noinline__ void phase_apply_change(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_apply_change()
 {
     const int nins = sh.d.ins_n;
     long long applied = 0, clamped = 0;
@@ -1134,7 +1155,7 @@ __device__ __noinline__ void phase_apply_change(const MfParams &P, Sh &sh)
         int pp = __ldcg(P.sc.ins_list + k);
         unsigned long long pk = __ldcg(P.sc.pkey + pp);
         int a = (int)(pk >> 32), b = (int)(pk & 0xffffffffu);
-        const int ca = batch_cap_of(P, a, b), cb = batch_cap_of(P, b, a);
+        const int ca = batch_cap_of(a, b), cb = batch_cap_of(b, a);
         const int xa = P.g.off[a] + atomicAdd(P.g.deg + a, 1);
         const int xb = P.g.off[b] + atomicAdd(P.g.deg + b, 1);
         const int va = ca > 0 ? ca : 0, vb2 = cb > 0 ? cb : 0;
@@ -1156,7 +1177,7 @@ __device__ __noinline__ void phase_apply_change(const MfParams &P, Sh &sh)
         const int x = __ldcg(P.sc.bslot + i);
         if (x < 0) continue;                 // superseded, ignored, or a new pair (set above)
         int u, v, c;
-        batch_entry(P, i, u, v, c);
+        batch_entry(i, u, v, c);
         const int old = ldg_cg(P.g.cap + x);
         const int delta = c - old;
         ++applied;
@@ -1170,18 +1191,18 @@ __device__ __noinline__ void phase_apply_change(const MfParams &P, Sh &sh)
             const int d = -cf_new;
             atomicAdd(P.cf + x, d);
             atomicAdd(P.cf + y, -d);
-            add_excess(P, sh, u, (long long)d);
-            add_excess(P, sh, v, -(long long)d);
+            add_excess(u, (long long)d);
+            add_excess(v, -(long long)d);
             ++clamped;
         }
     }
-    add_stat(sh, ST_N_APPLY, applied);
-    add_stat(sh, ST_CLAMPS_APPLY, clamped);
+    add_stat(ST_N_APPLY, applied);
+    add_stat(ST_CLAMPS_APPLY, clamped);
 }
 
 // keep_need: leave ins_need[] as it is (the rows' demand of spare slots after
 // an overflow; the rebuild that follows reads and clears it).
-__device__ __noinline__ void phase_apply_cleanup(const MfParams &P, const Sh &sh, bool keep_need)
+__device__ __noinline__ void phase_apply_cleanup(bool keep_need)
 {
     const int nused = sh.d.hused_n;
     const int nins = sh.d.ins_n;
@@ -1205,20 +1226,20 @@ __device__ __noinline__ void phase_apply_cleanup(const MfParams &P, const Sh &sh
 
 // The source step of Alg. 5 (reading: push the remaining residual of every edge out
 // of the source and add it to the head's excess).
-__device__ __noinline__ void phase_resaturate(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_resaturate()
 {
     const int s = P.source;
     const int r0 = P.g.off[s];
     const int d = ldg_cg(P.g.deg + s);
     long long acc = 0;
-    if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_SLOTS_APPLY, d);
+    if (vb() == 0 && threadIdx.x == 0) add_stat(ST_SLOTS_APPLY, d);
     for (int j = vb() * blockDim.x + threadIdx.x; j < d; j += vn() * blockDim.x) {
         int x = r0 + j;
         int c = ldg_cg(P.cf + x);
         if (c > 0) {
             P.cf[x] = 0;
             atomicAdd(P.cf + ldg_cg(P.g.rev + x), c);
-            add_excess(P, sh, ldg_cg(P.g.dst + x), (long long)c);
+            add_excess(ldg_cg(P.g.dst + x), (long long)c);
             acc -= c;
         }
     }
@@ -1230,7 +1251,7 @@ __device__ __noinline__ void phase_resaturate(const MfParams &P, Sh &sh)
 // ---------------------------------------------------------------------------
 
 // The work items of vertex z (d slots from r0), by one thread: where a queue has no room.
-__device__ __forceinline__ void put_items(const MfParams &P, int r0, int d, unsigned at)
+__device__ __forceinline__ void put_items(int r0, int d, unsigned at)
 {
     for (int j = 0; j < d; j += MF_BFS_CHUNK)
         P.sc.bitem[at++] = make_int2(r0 + j, d - j < MF_BFS_CHUNK ? d - j : MF_BFS_CHUNK);
@@ -1244,10 +1265,10 @@ __device__ __forceinline__ int chunks_of(int d) { return (d + MF_BFS_CHUNK - 1) 
 // room in the shared lists with one atomic per list: returning atomics on one
 // word are served one after another, about 2.4 clocks each, and a level whose
 // 4864 warps append alone spends some 5 us on that.
-__device__ __forceinline__ void place_active(const MfParams &P, Sh &sh, int z, int d, int line, int sel,
+__device__ __forceinline__ void place_active(int z, int d, int line, int sel,
                                              const int *app)
 {
-    const int bin = row_bin(P, d);
+    const int bin = row_bin(d);
     if (P.stage_slots >= MF_Q_INTS) {
         const int j = atomicAdd(&sh.q_wn, 1);
         if (j < MF_Q_WL) {
@@ -1268,7 +1289,7 @@ __device__ __forceinline__ void place_active(const MfParams &P, Sh &sh, int z, i
 // coming discharge (Sec. 5.2.1 O1): it is active exactly when this BFS labels
 // it, so no separate pass over all vertices is needed.  The entries wait in the
 // CTA's queue (flush_labelled).
-__device__ __forceinline__ void place_labelled(const MfParams &P, Sh &sh, int z, int d, long long ev)
+__device__ __forceinline__ void place_labelled(int z, int d, long long ev)
 {
     const bool room = P.stage_slots >= MF_Q_INTS;
     if (d > P.bfs_hub) {
@@ -1276,7 +1297,7 @@ __device__ __forceinline__ void place_labelled(const MfParams &P, Sh &sh, int z,
         if (i < MF_Q_LONG)
             mf_stage[MF_Q_BFS + i] = z;
         else
-            put_items(P, P.g.off[z], d, sh.d.app_hub + atomicAdd(&sh.cs->l[L_HUB].w[0], (unsigned)chunks_of(d)));
+            put_items(P.g.off[z], d, sh.d.app_hub + atomicAdd(&sh.cs->l[L_HUB].w[0], (unsigned)chunks_of(d)));
     } else {
         const int i = room ? atomicAdd(&sh.q_bfs, 1) : MF_Q_BFS;
         if (i < MF_Q_BFS)
@@ -1285,18 +1306,54 @@ __device__ __forceinline__ void place_labelled(const MfParams &P, Sh &sh, int z,
             P.sc.border[sh.d.app_bfs + atomicAdd(&sh.cs->l[L_BFS].w[0], 1u)] = z;
     }
     if (ev > 0) {
-        place_active(P, sh, z, d, L_WL, sh.d.wl_sel, sh.d.wl_app);
+        place_active(z, d, L_WL, sh.d.wl_sel, sh.d.wl_app);
         if (sh.d.near) add_shared(sh.exc, ev);
+    }
+}
+
+// The work items of nl long-row vertices (in shared memory), by the whole CTA: a
+// warp takes 32 vertices, makes room for all their items at once and writes
+// them together, each lane finding the vertex that owns its item.  (A warp per
+// vertex took 5 us where three CTAs had labelled 270 hubs between them.)
+__device__ __forceinline__ void write_long(const int *list, int nl)
+{
+    const int lane = threadIdx.x & 31;
+    for (int b = (int)(threadIdx.x & ~31u); b < nl; b += blockDim.x) {
+        const int z = b + lane < nl ? list[b + lane] : -1;
+        const int d = z >= 0 ? ldg_cg(P.g.deg + z) : 0, r0 = z >= 0 ? P.g.off[z] : 0, nc = chunks_of(d);
+        int incl = nc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int excl = incl - nc, tot = __shfl_sync(0xffffffffu, incl, 31);
+        unsigned at = 0;
+        if (lane == 0) at = sh.d.app_hub + atomicAdd(&sh.cs->l[L_HUB].w[0], (unsigned)tot);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        for (int i0 = 0; i0 < tot; i0 += 32) {
+            const int i = i0 + lane;
+            int owner = 0;
+#pragma unroll
+            for (int st = 16; st >= 1; st >>= 1) {
+                const int cand = owner + st;
+                const int ec = __shfl_sync(0xffffffffu, excl, cand & 31);
+                if (cand < 32 && ec <= i) owner = cand;
+            }
+            const int rb = __shfl_sync(0xffffffffu, r0, owner), rd_ = __shfl_sync(0xffffffffu, d, owner);
+            const int j = (i - __shfl_sync(0xffffffffu, excl, owner)) * MF_BFS_CHUNK;
+            if (i < tot) P.sc.bitem[at + i] = make_int2(rb + j, rd_ - j < MF_BFS_CHUNK ? rd_ - j : MF_BFS_CHUNK);
+        }
     }
 }
 
 // The end of a phase: the CTA's queue goes onto the shared lists, and what its
 // threads labelled (vertices, slots) to the counters.  Long rows' work items
-// are written here by whole warps.
-__device__ __forceinline__ void flush_queue(const MfParams &P, Sh &sh, int line, int sel, const int *app, int lab,
+// are written here.
+__device__ __forceinline__ void flush_queue(int line, int sel, const int *app, int lab,
                                             unsigned lab_slots)
 {
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
     __syncwarp();
     lab = __reduce_add_sync(0xffffffffu, lab);
     lab_slots = __reduce_add_sync(0xffffffffu, lab_slots);
@@ -1319,25 +1376,15 @@ __device__ __forceinline__ void flush_queue(const MfParams &P, Sh &sh, int line,
             P.sc.wl[sel][b >> 28][sh.q_base[b >> 28] + (b & 0x0fffffff)] = q[i];
         }
     }
-    for (int i = wid; i < nl; i += nt >> 5) {
-        const int z = mf_stage[MF_Q_BFS + i];
-        const int r0 = P.g.off[z], d = ldg_cg(P.g.deg + z), nc = chunks_of(d);
-        unsigned at = 0;
-        if (lane == 0) at = sh.d.app_hub + atomicAdd(&sh.cs->l[L_HUB].w[0], (unsigned)nc);
-        at = __shfl_sync(0xffffffffu, at, 0);
-        for (int c = lane; c < nc; c += 32) {
-            const int len = d - c * MF_BFS_CHUNK;
-            P.sc.bitem[at + c] = make_int2(r0 + c * MF_BFS_CHUNK, len < MF_BFS_CHUNK ? len : MF_BFS_CHUNK);
-        }
-    }
+    write_long(mf_stage + MF_Q_BFS, nl);
 }
 
-__device__ __forceinline__ void flush_labelled(const MfParams &P, Sh &sh, int lab, unsigned lab_slots)
+__device__ __forceinline__ void flush_labelled(int lab, unsigned lab_slots)
 {
-    flush_queue(P, sh, L_WL, sh.d.wl_sel, sh.d.wl_app, lab, lab_slots);
+    flush_queue(L_WL, sh.d.wl_sel, sh.d.wl_app, lab, lab_slots);
 }
 
-__device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_bfs_init()
 {
     const int n = P.g.n;
     const bool deficit_roots = (P.mode & MF_M_NO_DEFICIT_ROOTS) == 0;
@@ -1354,7 +1401,7 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
         for (long long j = (long long)vb() * blockDim.x + threadIdx.x; j < d; j += gs)
             take += ldg_cg(P.g.pcap + r0 + j) - ldg_cg(P.cf + r0 + j);
     }
-    if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_VERTS_BFS, n);     // every vertex: e read, h written
+    if (vb() == 0 && threadIdx.x == 0) add_stat(ST_VERTS_BFS, n);     // every vertex: e read, h written
     for (long long base = (long long)vb() * blockDim.x + threadIdx.x - lane; base < n; base += gs) {
         const int v = (int)base + lane;
         bool root = false;
@@ -1379,13 +1426,13 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
                 const int d = need_total ? dall : ldg_cg(P.g.deg + v);
                 ++lab;
                 lab_slots += (unsigned)d;
-                place_labelled(P, sh, v, d, 0);
+                place_labelled(v, d, 0);
             }
         }
         total += dall;
     }
     if (take) add_shared(sh.dem, take);
-    flush_labelled(P, sh, lab, lab_slots);
+    flush_labelled(lab, lab_slots);
     if (need_total) {
         // one atomic per CTA for the used-slot total
         total = warp_sum_ll(total);
@@ -1406,7 +1453,7 @@ __device__ __noinline__ void phase_bfs_init(const MfParams &P, Sh &sh)
 // claims, degree/excess loads) is issued for all BR slots together, so each
 // lane keeps BR independent requests in flight.
 template <int BR>
-__device__ __forceinline__ void bfs_visit(const MfParams &P, Sh &sh, const int (&x)[BR], const bool (&valid)[BR], int L,
+__device__ __forceinline__ void bfs_visit(const int (&x)[BR], const bool (&valid)[BR], int L,
                                           int &lab, unsigned &lab_slots)
 {
     const bool with_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY);
@@ -1443,13 +1490,13 @@ __device__ __forceinline__ void bfs_visit(const MfParams &P, Sh &sh, const int (
         if (!claim[r]) continue;
         ++lab;
         lab_slots += (unsigned)d[r];
-        place_labelled(P, sh, z[r], d[r], ev[r]);
+        place_labelled(z[r], d[r], ev[r]);
     }
 }
 
 constexpr int kBR = 4;
 
-__device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_bfs_level()
 {
     MfSet *cs = sh.cs;
     const int L = sh.d.level;
@@ -1459,82 +1506,78 @@ __device__ __noinline__ void phase_bfs_level(const MfParams &P, Sh &sh)
     int lab = 0;
     unsigned lab_slots = 0;
     const int nwarps = nctas * (int)(blockDim.x >> 5);
-    // chunks of long rows: one warp per item (at most MF_BFS_CHUNK slots)
+    // first the chunks of long rows, one per warp, then the regular frontier:
+    // warps take up to 32 vertices at a time and expand their rows together
+    // (each lane finds the entry that owns its slot).  A frontier of fewer is
+    // dealt out evenly and at once, so that its rows spread over all warps and
+    // nobody comes back for more (a level of 5116 vertices, one for each of 4864
+    // warps and a rush of all of them on the head for the rest, took 19 us, one
+    // of 4438 took 11).  One copy of the expansion serves both: the code of a
+    // level has to come through the instruction cache before its few warps can
+    // run it.
     const int ilo = sh.d.hub_lo, icnt = sh.d.hub_hi - ilo;
-    bool first = true;
-    const int rank_i = warp_rank(nctas, 0);
-    for (;;) {
-        const int i = warp_deal(&cs->l[L_HEAD1].w[0], icnt, 1u, rank_i, nwarps, first);
-        if (i >= icnt) break;
-        const int2 it = __ldcg(P.sc.bitem + ilo + i);
-        if (lane == 0) slots += it.y;
-        for (int kb = 0; kb < it.y; kb += 32 * kBR) {
-            int xs[kBR];
-            bool vs[kBR];
-#pragma unroll
-            for (int r = 0; r < kBR; ++r) {
-                int k = kb + r * 32 + lane;
-                vs[r] = k < it.y;
-                xs[r] = it.x + k;
-            }
-            bfs_visit<kBR>(P, sh, xs, vs, L, lab, lab_slots);
-        }
-    }
-    // regular frontier: warps take up to 32 vertices at a time and expand their
-    // rows together (each lane finds the vertex that owns its slot); a frontier
-    // of fewer is dealt out evenly and at once, so that its rows spread over all
-    // warps and nobody comes back for more (a level of 5116 vertices, one for
-    // each of 4864 warps and a rush of all of them on the head for the rest,
-    // took 19 us, one of 4438 took 11)
     const int lo = sh.d.lvl_lo, cnt = sh.d.lvl_hi - lo;
     const int take = max(1, min(32, (cnt + nwarps - 1) / nwarps));
-    first = true;
-    const int rank_f = warp_rank(nctas, icnt);
-    for (;;) {
-        const int b = warp_deal(&cs->l[L_HEAD0].w[0], cnt, (unsigned)take, rank_f, nwarps, first);
-        if (b >= cnt) break;
-        int idx = b + lane;
-        int u = (lane < take && idx < cnt) ? __ldcg(P.sc.border + lo + idx) : -1;
-        int d = u >= 0 ? ldg_cg(P.g.deg + u) : 0;
-        int r0 = u >= 0 ? P.g.off[u] : 0;
-        int incl = d;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const int excl = incl - d;
-        const int T = __shfl_sync(0xffffffffu, incl, 31);
-        if (lane == 0) slots += T;
-        for (int kb = 0; kb < T; kb += 32 * kBR) {
-            int xs[kBR];
-            bool vs[kBR];
-#pragma unroll
-            for (int r = 0; r < kBR; ++r) {
-                const int k = kb + r * 32 + lane;
-                int owner = 0;
-#pragma unroll
-                for (int step = 16; step >= 1; step >>= 1) {
-                    int cand = owner + step;
-                    int ec = __shfl_sync(0xffffffffu, excl, cand & 31);
-                    if (cand < 32 && ec <= k) owner = cand;
+    for (int kind = icnt > 0 ? 0 : 1; kind < 2; ++kind) {
+        bool first = true;
+        const int rank = warp_rank(nctas, kind ? icnt : 0);
+        for (;;) {
+            int d = 0, r0 = 0;
+            if (kind == 0) {
+                const int i = warp_deal(&cs->l[L_HEAD1].w[0], icnt, 1u, rank, nwarps, first);
+                if (i >= icnt) break;
+                if (lane == 0) {
+                    const int2 it = __ldcg(P.sc.bitem + ilo + i);
+                    r0 = it.x;
+                    d = it.y;
                 }
-                int rb = __shfl_sync(0xffffffffu, r0, owner);
-                int eb = __shfl_sync(0xffffffffu, excl, owner);
-                vs[r] = k < T;
-                xs[r] = rb + (k - eb);
+            } else {
+                const int b = warp_deal(&cs->l[L_HEAD0].w[0], cnt, (unsigned)take, rank, nwarps, first);
+                if (b >= cnt) break;
+                const int idx = b + lane;
+                const int u = (lane < take && idx < cnt) ? __ldcg(P.sc.border + lo + idx) : -1;
+                d = u >= 0 ? ldg_cg(P.g.deg + u) : 0;
+                r0 = u >= 0 ? P.g.off[u] : 0;
             }
-            bfs_visit<kBR>(P, sh, xs, vs, L, lab, lab_slots);
+            int incl = d;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int excl = incl - d;
+            const int T = __shfl_sync(0xffffffffu, incl, 31);
+            if (lane == 0) slots += T;
+            for (int kb = 0; kb < T; kb += 32 * kBR) {
+                int xs[kBR];
+                bool vs[kBR];
+#pragma unroll
+                for (int r = 0; r < kBR; ++r) {
+                    const int k = kb + r * 32 + lane;
+                    int owner = 0;
+#pragma unroll
+                    for (int step = 16; step >= 1; step >>= 1) {
+                        int cand = owner + step;
+                        int ec = __shfl_sync(0xffffffffu, excl, cand & 31);
+                        if (cand < 32 && ec <= k) owner = cand;
+                    }
+                    int rb = __shfl_sync(0xffffffffu, r0, owner);
+                    int eb = __shfl_sync(0xffffffffu, excl, owner);
+                    vs[r] = k < T;
+                    xs[r] = rb + (k - eb);
+                }
+                bfs_visit<kBR>(xs, vs, L, lab, lab_slots);
+            }
         }
     }
-    add_stat(sh, ST_SLOTS_BFS, slots);
-    flush_labelled(P, sh, lab, lab_slots);
+    add_stat(ST_SLOTS_BFS, slots);
+    flush_labelled(lab, lab_slots);
 }
 
 // Near BFS, bottom-up: slot x = (v, z) with residual c leads v down to z at
 // level L.  Several lanes may find a slot for the same v; any of them will do
 // (there is one slot (v, sink) at most, so dem[v] fits par[v] either way).
-__device__ __forceinline__ void note_parent(const MfParams &P, int v, int x, int z, int c, int L)
+__device__ __forceinline__ void note_parent(int v, int x, int z, int c, int L)
 {
     P.sc.par[v] = x;
     if (L == 0 && z == P.sink) P.sc.dem[v] = c;
@@ -1548,7 +1591,7 @@ __device__ __forceinline__ void note_parent(const MfParams &P, int v, int x, int
 // labelled L + 1 exactly when it has such a neighbour); the work follows the
 // unlabelled vertices' rows up to the first hit instead of the frontier's
 // rows, which pays off once the frontier holds most of the graph.
-__device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_bfs_bottom_up()
 {
     MfSet *cs = sh.cs;
     const int n = P.g.n;
@@ -1571,7 +1614,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
     long long slots = 0, unl = 0;
     int lab = 0;
     unsigned lab_slots = 0;
-    if (vb() == 0 && threadIdx.x == 0) add_stat(sh, ST_HSCAN_BFS, n);    // every vertex's height is read
+    if (vb() == 0 && threadIdx.x == 0) add_stat(ST_HSCAN_BFS, n);    // every vertex's height is read
     for (long long base = (long long)vb() * blockDim.x + threadIdx.x - lane; base < n; base += gs) {
         const int v = (int)base + lane;
         const bool ok = v < n && v != skip;
@@ -1594,7 +1637,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
             for (int r = 0; r < kA; ++r) {
                 const bool hitr = c[r] > 0 && ldg_cg(P.h + z[r]) == L;
                 take |= hitr;
-                if (near && hitr) note_parent(P, v, r0 + r, z[r], c[r], L);
+                if (near && hitr) note_parent(v, r0 + r, z[r], c[r], L);
             }
             slots += d < kA ? d : kA;
         }
@@ -1638,7 +1681,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
             for (int r = 0; r < kA; ++r)
                 if (c[r] > 0 && ldg_cg(P.h + z[r]) == L) {
                     mine |= 1u << ow[r];
-                    if (near) note_parent(P, (int)base + ow[r], xs[r], z[r], c[r], L);
+                    if (near) note_parent((int)base + ow[r], xs[r], z[r], c[r], L);
                 }
             hit |= __reduce_or_sync(0xffffffffu, mine);
         }
@@ -1649,7 +1692,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
             const long long ev = with_wl && v != P.sink && v != P.source ? (pull ? -ldg_cg(P.e + v) : ldg_cg(P.e + v)) : 0;
             ++lab;
             lab_slots += (unsigned)d;
-            place_labelled(P, sh, v, d, ev);
+            place_labelled(v, d, ev);
         } else if (open && d > lim) {
             nitem = (d - lim + MF_BU_CHUNK - 1) / MF_BU_CHUNK;
             x0 = r0 + lim;
@@ -1668,9 +1711,9 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
             for (int cc = 0; cc < nitem; ++cc) P.sc.bdefer[at + cc] = make_int2(v, x0 + cc * MF_BU_CHUNK);
         }
     }
-    add_stat(sh, ST_SLOTS_BFS, slots);
-    flush_labelled(P, sh, lab, lab_slots);
-    add_stat(sh, ST_VERTS_BFS, unl);
+    add_stat(ST_SLOTS_BFS, slots);
+    flush_labelled(lab, lab_slots);
+    add_stat(ST_VERTS_BFS, unl);
 }
 
 // Second pass of a bottom-up level: the deferred chunks of long rows whose
@@ -1678,7 +1721,7 @@ __device__ __noinline__ void phase_bfs_bottom_up(const MfParams &P, Sh &sh)
 // towards it.  One warp per chunk of MF_BU_CHUNK slots, 8 per lane; the first
 // chunk of a row that finds one labels the vertex (a claim by CAS, as other
 // chunks of the same row may find one too).
-__device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_bfs_bottom_up_long()
 {
     MfSet *cs = sh.cs;
     const int n = P.g.n;
@@ -1718,26 +1761,26 @@ __device__ __noinline__ void phase_bfs_bottom_up_long(const MfParams &P, Sh &sh)
         for (int r = 0; r < kR; ++r) {
             const bool hitr = c[r] > 0 && ldg_cg(P.h + z[r]) == L;
             hit |= hitr;
-            if (near && hitr) note_parent(P, v, it.y + r * 32 + lane, z[r], c[r], L);
+            if (near && hitr) note_parent(v, it.y + r * 32 + lane, z[r], c[r], L);
         }
         if (lane == 0) slots += len;
         if (__any_sync(0xffffffffu, hit) && lane == 0 && atomicCAS(P.h + v, n, L + 1) == n) {
             const long long ev = with_wl && v != P.sink && v != P.source ? (pull ? -ldg_cg(P.e + v) : ldg_cg(P.e + v)) : 0;
             ++lab;
             lab_slots += (unsigned)d;
-            place_labelled(P, sh, v, d, ev);
+            place_labelled(v, d, ev);
         }
         __syncwarp();
     }
-    add_stat(sh, ST_SLOTS_BFS, slots);
-    flush_labelled(P, sh, lab, lab_slots);
+    add_stat(ST_SLOTS_BFS, slots);
+    flush_labelled(lab, lab_slots);
 }
 
 // ---------------------------------------------------------------------------
 // Worklist of active vertices (Sec. 5.2.1 O1) with the termination count
 // ---------------------------------------------------------------------------
 
-__device__ __noinline__ void phase_worklist(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_worklist()
 {
     MfSet *cs = sh.cs;
     const int sel = sh.d.wl_sel;
@@ -1751,7 +1794,7 @@ __device__ __noinline__ void phase_worklist(const MfParams &P, Sh &sh)
         bool act = cand && ldg_cg(P.h + v) < n && (P.pull ? ev < 0 : ev > 0);
         bool listed = P.data_driven ? act : cand;
         int bin = 0;
-        if (listed) bin = row_bin(P, ldg_cg(P.g.deg + v));
+        if (listed) bin = row_bin(ldg_cg(P.g.deg + v));
         unsigned am = __ballot_sync(0xffffffffu, act);
         if (lane == 0 && am) atomicAdd(&cs->l[L_ACT].w[0], (unsigned)__popc(am));
 #pragma unroll
@@ -1779,11 +1822,11 @@ struct DisCtx {
 // z just became active (its excess went from <= 0 to > 0 during this round):
 // give it to the next round (Alg. 2's kernel checks e(u) > 0 on every cycle,
 // so a vertex that receives flow while the kernel runs is discharged too).
-__device__ __forceinline__ void enqueue_active(const MfParams &P, int z, const DisCtx &dc)
+__device__ __forceinline__ void enqueue_active(int z, const DisCtx &dc)
 {
     const int dz = ldg_cg(P.g.deg + z);      // in flight together with the stamp exchange
     if (atomicExch(P.sc.vmark + z, dc.qstamp) == dc.qstamp) return;
-    const int bin = row_bin(P, dz);
+    const int bin = row_bin(dz);
     const unsigned pos = atomicAdd(&dc.cs->l[L_AUX + bin].w[0], 1u);
     P.sc.wl[dc.nsel][bin][pos] = z;
 }
@@ -1792,16 +1835,16 @@ __device__ __forceinline__ void enqueue_active(const MfParams &P, int z, const D
 // push, a deficit for a pull) and a height below n: with P.requeue it joins the
 // next round's queue too, instead of waiting for the next global relabel.
 template <bool PULL>
-__device__ __forceinline__ void requeue_if_active(const MfParams &P, int u, const DisCtx &dc)
+__device__ __forceinline__ void requeue_if_active(int u, const DisCtx &dc)
 {
     if (!P.requeue || !dc.queue) return;
     const long long eu = ldg_cg(P.e + u);
-    if ((PULL ? eu < 0 : eu > 0) && ldg_cg(P.h + u) < P.g.n) enqueue_active(P, u, dc);
+    if ((PULL ? eu < 0 : eu > 0) && ldg_cg(P.h + u) < P.g.n) enqueue_active(u, dc);
 }
 
 // u was relabelled: list it (once per iteration) for remove-invalid-edges;
 // only relabelled vertices can have steep residual edges.
-__device__ __forceinline__ void note_relabel(const MfParams &P, int u, const DisCtx &dc)
+__device__ __forceinline__ void note_relabel(int u, const DisCtx &dc)
 {
     if (atomicExch(P.sc.fixmark + u, dc.fstamp) == dc.fstamp) return;
     const int d = ldg_cg(P.g.deg + u);
@@ -1816,7 +1859,7 @@ __device__ __forceinline__ void note_relabel(const MfParams &P, int u, const Dis
 // caller updates e(u).  Only u's owner lowers the slot it moves through, so
 // an amount read from that slot can always be moved.
 template <bool PULL>
-__device__ __forceinline__ void move_flow(const MfParams &P, Sh &sh, int x, int y, int z, long long amt,
+__device__ __forceinline__ void move_flow(int x, int y, int z, long long amt,
                                           const DisCtx &dc)
 {
     if (PULL) {
@@ -1834,21 +1877,21 @@ __device__ __forceinline__ void move_flow(const MfParams &P, Sh &sh, int x, int 
     } else {
         const long long old = atomic_add_ll(P.e + z, dz);
         const bool became = PULL ? (old >= 0 && old + dz < 0) : (old <= 0 && old + dz > 0);
-        if (dc.queue && became) enqueue_active(P, z, dc);
+        if (dc.queue && became) enqueue_active(z, dc);
     }
 }
 
 // Residual of slot x in the direction of the move, from the slot's own row:
 // c_f(u, z) for a push, c_f(z, u) = pcap - c_f(u, z) for a pull.
 template <bool PULL>
-__device__ __forceinline__ int residual_dir(const MfParams &P, int x)
+__device__ __forceinline__ int residual_dir(int x)
 {
     return PULL ? ldg_cg(P.g.pcap + x) - ldg_cg(P.cf + x) : ldg_cg(P.cf + x);
 }
 
 // The amount slot x of u can move now (exact): c_f(u, z) for a push, c_f(z, u) for a pull.
 template <bool PULL>
-__device__ __forceinline__ int movable(const MfParams &P, int x, int y)
+__device__ __forceinline__ int movable(int x, int y)
 {
     return PULL ? ldg_cg(P.cf + y) : ldg_cg(P.cf + x);
 }
@@ -1858,7 +1901,7 @@ __device__ __forceinline__ int movable(const MfParams &P, int x, int y)
 // lowest slot index.  Slots are read kU at a time with their loads issued
 // together.
 template <int kU, bool PULL>
-__device__ __forceinline__ unsigned long long scan_lowest(const MfParams &P, int r0, int d, int j0, int step)
+__device__ __forceinline__ unsigned long long scan_lowest(int r0, int d, int j0, int step)
 {
     unsigned long long best = kEmpty;
     for (int jb = j0; jb < d; jb += step * kU) {
@@ -1895,7 +1938,7 @@ constexpr int kNoRes = 0x7fffffff;
 // KERNEL_CYCLES of Alg. 2 for a row of d slots: P.kernel_cycles, or with
 // P.cycle_div > 0 at least d / P.cycle_div, so that a long row, whose first
 // scan dominates its discharge, makes more of its pushes per scan.
-__device__ __forceinline__ int cycles_for(const MfParams &P, int d)
+__device__ __forceinline__ int cycles_for(int d)
 {
     if (P.cycle_div <= 0) return P.kernel_cycles;
     const int k = d / P.cycle_div;
@@ -1908,7 +1951,7 @@ constexpr int kStaleMax = 8;
 // The first scan of a row: the lowest residual height as scan_lowest does, and
 // the snapshot of every slot of the row in stg.
 template <int kU, bool PULL>
-__device__ __forceinline__ unsigned long long scan_and_stage(const MfParams &P, int r0, int d, int j0, int step,
+__device__ __forceinline__ unsigned long long scan_and_stage(int r0, int d, int j0, int step,
                                                              int *stg)
 {
     unsigned long long best = kEmpty;
@@ -1945,7 +1988,7 @@ __device__ __forceinline__ int comp4(const int4 &a, int e)
 // each slot array.  Thread t of nt takes groups t, t + nt, ... two at a time
 // (eight slots in flight).  Same result as scan_and_stage.
 template <bool PULL>
-__device__ __forceinline__ unsigned long long scan_and_stage_v4(const MfParams &P, int r0, int d, int t, int nt,
+__device__ __forceinline__ unsigned long long scan_and_stage_v4(int r0, int d, int t, int nt,
                                                                 int *stg)
 {
     unsigned long long best = kEmpty;
@@ -2014,14 +2057,14 @@ __device__ __forceinline__ unsigned long long scan_staged(const int *stg, int d,
 // a head of height want: 0 unless the head still has that height and the slot
 // still has residual capacity; the snapshot entry is corrected on the way.
 template <bool PULL>
-__device__ __forceinline__ int staged_amount(const MfParams &P, int x, int want, int &sj)
+__device__ __forceinline__ int staged_amount(int x, int want, int &sj)
 {
     const int hz = ldg_cg(P.h + ldg_cg(P.g.dst + x));
     if (hz != want) {
         sj = hz;
         return 0;
     }
-    const int c = movable<PULL>(P, x, ldg_cg(P.g.rev + x));
+    const int c = movable<PULL>(x, ldg_cg(P.g.rev + x));
     if (c <= 0) {
         sj = kNoRes;
         return 0;
@@ -2035,7 +2078,7 @@ __device__ __forceinline__ int staged_amount(const MfParams &P, int x, int want,
 // Rows of at most kTS slots keep the heads' heights in registers after the
 // first scan.
 template <bool PULL>
-__device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, const DisCtx &dc)
+__device__ __noinline__ bool discharge_thread(int u, const DisCtx &dc)
 {
     constexpr int kTS = 8;
     bool lifted = false;
@@ -2061,7 +2104,7 @@ __device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, 
                     int c[kTS], z[kTS];
 #pragma unroll
                     for (int j = 0; j < kTS; ++j) {
-                        c[j] = j < d ? residual_dir<PULL>(P, r0 + j) : 0;
+                        c[j] = j < d ? residual_dir<PULL>(r0 + j) : 0;
                         z[j] = j < d ? ldg_cg(P.g.dst + r0 + j) : 0;
                     }
 #pragma unroll
@@ -2087,7 +2130,7 @@ __device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, 
                 hu = (best == kEmpty || best_h >= n - 1) ? n : best_h + 1;
                 P.h[u] = hu;
                 lifted = true;
-                add_stat(sh, ST_RELABELS, 1);
+                add_stat(ST_RELABELS, 1);
                 ++cyc;
                 if (hu >= n || cyc >= P.kernel_cycles) continue;
             }
@@ -2101,12 +2144,12 @@ __device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, 
                 if (j < jstart || j >= d || rem <= 0 || cyc + k >= P.kernel_cycles || hc[j] != best_h) continue;
                 const int x = r0 + j;
                 int sj = hc[j];
-                const int c = staged_amount<PULL>(P, x, best_h, sj);
+                const int c = staged_amount<PULL>(x, best_h, sj);
                 hc[j] = sj;
                 ++fused;
                 if (c <= 0) continue;
                 const long long a = rem < (long long)c ? rem : (long long)c;
-                move_flow<PULL>(P, sh, x, ldg_cg(P.g.rev + x), ldg_cg(P.g.dst + x), a, dc);
+                move_flow<PULL>(x, ldg_cg(P.g.rev + x), ldg_cg(P.g.dst + x), a, dc);
                 if (a == c) hc[j] = kNoRes;
                 rem -= a;
                 sent += a;
@@ -2124,13 +2167,13 @@ __device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, 
             if (!(hu < n && eu > 0)) break;
             ++scans;
             gscan += d;
-            unsigned long long best = scan_lowest<4, PULL>(P, r0, d, 0, 1);
+            unsigned long long best = scan_lowest<4, PULL>(r0, d, 0, 1);
             int best_h = best == kEmpty ? 0x7fffffff : (int)(best >> 32);
             if (best == kEmpty || hu <= best_h) {
                 hu = (best == kEmpty || best_h >= n - 1) ? n : best_h + 1;
                 P.h[u] = hu;
                 lifted = true;
-                add_stat(sh, ST_RELABELS, 1);
+                add_stat(ST_RELABELS, 1);
                 ++cyc;
                 if (hu >= n || cyc >= P.kernel_cycles) continue;
             }
@@ -2140,14 +2183,14 @@ __device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, 
             const int jstart = j;
             for (; j < d && rem > 0 && cyc + k < P.kernel_cycles; ++j) {
                 const int x = r0 + j;
-                if (residual_dir<PULL>(P, x) <= 0) continue;
+                if (residual_dir<PULL>(x) <= 0) continue;
                 const int z = ldg_cg(P.g.dst + x);
                 if (ldg_cg(P.h + z) != best_h) continue;
                 const int y = ldg_cg(P.g.rev + x);
-                const int c = movable<PULL>(P, x, y);
+                const int c = movable<PULL>(x, y);
                 if (c <= 0) continue;
                 const long long a = rem < (long long)c ? rem : (long long)c;
-                move_flow<PULL>(P, sh, x, y, z, a, dc);
+                move_flow<PULL>(x, y, z, a, dc);
                 rem -= a;
                 sent += a;
                 ++k;
@@ -2159,23 +2202,23 @@ __device__ __noinline__ bool discharge_thread(const MfParams &P, Sh &sh, int u, 
         }
     }
     if (scans) {
-        add_stat(sh, ST_CYCLES_DIS, scans);
-        add_stat(sh, ST_SLOTS_DIS, gscan + fused);
+        add_stat(ST_CYCLES_DIS, scans);
+        add_stat(ST_SLOTS_DIS, gscan + fused);
     }
-    add_stat(sh, ST_PUSHES, moves);
+    add_stat(ST_PUSHES, moves);
     return lifted;
 }
 
 // One warp per vertex; ST: the row's heads are kept in stg (this warp's slice
 // of the on-chip snapshot) after the first scan.
 template <bool PULL, bool ST>
-__device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int u, int d, const DisCtx &dc, int *stg)
+__device__ __noinline__ bool discharge_warp_rows(int u, int d, const DisCtx &dc, int *stg)
 {
     bool lifted = false;
     const int n = P.g.n;
     const int lane = threadIdx.x & 31;
     const int r0 = P.g.off[u];
-    const int kcyc = cycles_for(P, d);
+    const int kcyc = cycles_for(d);
     constexpr bool st = ST;
     bool have = false;
     int stale = 0;
@@ -2188,10 +2231,10 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
         ++scans;
         unsigned long long best;
         if (!st) {
-            best = warp_min_u64(scan_lowest<8, PULL>(P, r0, d, lane, 32));
+            best = warp_min_u64(scan_lowest<8, PULL>(r0, d, lane, 32));
             gscan += d;
         } else if (!have) {
-            best = warp_min_u64(scan_and_stage_v4<PULL>(P, r0, d, lane, 32, stg));
+            best = warp_min_u64(scan_and_stage_v4<PULL>(r0, d, lane, 32, stg));
             have = true;
             gscan += d;
             __syncwarp();
@@ -2201,7 +2244,7 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
             if (best == kEmpty || hu <= bh) {
                 // a relabel is decided on fresh values: refresh the snapshot first
                 __syncwarp();
-                best = warp_min_u64(scan_and_stage_v4<PULL>(P, r0, d, lane, 32, stg));
+                best = warp_min_u64(scan_and_stage_v4<PULL>(r0, d, lane, 32, stg));
                 gscan += d;
                 __syncwarp();
             }
@@ -2213,7 +2256,7 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
             lifted = true;
             if (lane == 0) {
                 P.h[u] = hu;
-                add_stat(sh, ST_RELABELS, 1);
+                add_stat(ST_RELABELS, 1);
             }
             ++cyc;
             if (hu >= n || cyc >= kcyc) {
@@ -2246,7 +2289,7 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
                     for (int r = 0; r < kSeg; ++r) {
                         if (a[r]) {
                             int sj = stg[js + r];
-                            a[r] = staged_amount<PULL>(P, r0 + js + r, best_h, sj);
+                            a[r] = staged_amount<PULL>(r0 + js + r, best_h, sj);
                             stg[js + r] = sj;
                             ++fused;
                             tsum += a[r];
@@ -2258,7 +2301,7 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
                     for (int r = 0; r < kSeg; ++r) {
                         a[r] = 0;
                         const int j = js + r;
-                        if (r < seg && j < d && residual_dir<PULL>(P, r0 + j) > 0) a[r] = 1;
+                        if (r < seg && j < d && residual_dir<PULL>(r0 + j) > 0) a[r] = 1;
                     }
 #pragma unroll
                     for (int r = 0; r < kSeg; ++r) {
@@ -2271,7 +2314,7 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
                     for (int r = 0; r < kSeg; ++r) {
                         if (a[r]) {
                             const int x = r0 + js + r;
-                            const int c = movable<PULL>(P, x, ldg_cg(P.g.rev + x));
+                            const int c = movable<PULL>(x, ldg_cg(P.g.rev + x));
                             a[r] = c > 0 ? c : 0;
                             tsum += a[r];
                             tcnt += a[r] > 0 ? 1 : 0;
@@ -2301,7 +2344,7 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
                         if (off < rem && cyc + k + coff < kcyc) {
                             const long long g = a[r] < rem - off ? a[r] : rem - off;
                             const int x = r0 + js + r;
-                            move_flow<PULL>(P, sh, x, ldg_cg(P.g.rev + x), ldg_cg(P.g.dst + x), g, dc);
+                            move_flow<PULL>(x, ldg_cg(P.g.rev + x), ldg_cg(P.g.dst + x), g, dc);
                             if (st && g == a[r]) stg[js + r] = kNoRes;
                             mine += g;
                             ++mk;
@@ -2328,10 +2371,10 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
     fused = warp_sum_ll(fused);
     if (lane == 0) {
         if (scans) {
-            add_stat(sh, ST_CYCLES_DIS, scans);
-            add_stat(sh, ST_SLOTS_DIS, gscan + fused);
+            add_stat(ST_CYCLES_DIS, scans);
+            add_stat(ST_SLOTS_DIS, gscan + fused);
         }
-        add_stat(sh, ST_PUSHES, moves);
+        add_stat(ST_PUSHES, moves);
     }
     return lifted;
 }
@@ -2339,11 +2382,11 @@ __device__ __noinline__ bool discharge_warp_rows(const MfParams &P, Sh &sh, int 
 // One warp per vertex (returns the same value in every lane).  stg: this
 // warp's slice of the on-chip snapshot (wcap entries), used when the row fits.
 template <bool PULL>
-__device__ __forceinline__ bool discharge_warp(const MfParams &P, Sh &sh, int u, const DisCtx &dc, int *stg, int wcap)
+__device__ __forceinline__ bool discharge_warp(int u, const DisCtx &dc, int *stg, int wcap)
 {
     const int d = ldg_cg(P.g.deg + u);
-    if (stg != nullptr && d <= wcap) return discharge_warp_rows<PULL, true>(P, sh, u, d, dc, stg);
-    return discharge_warp_rows<PULL, false>(P, sh, u, d, dc, nullptr);
+    if (stg != nullptr && d <= wcap) return discharge_warp_rows<PULL, true>(u, d, dc, stg);
+    return discharge_warp_rows<PULL, false>(u, d, dc, nullptr);
 }
 
 // The threads that discharge one long row together: the whole CTA, or a group
@@ -2371,14 +2414,14 @@ struct GroupTeam {
 // One team per vertex; ST: the row's heads are kept in stg (the team's share of
 // the on-chip snapshot) after the first scan.
 template <bool PULL, bool ST, class Team>
-__device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int u, int d, const DisCtx &dc, int *stg)
+__device__ __noinline__ bool discharge_team_rows(int u, int d, const DisCtx &dc, int *stg)
 {
     const Team T;
     bool lifted = false;
     const int n = P.g.n;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int r0 = P.g.off[u];
-    const int kcyc = cycles_for(P, d);
+    const int kcyc = cycles_for(d);
     constexpr bool st = ST;
     bool have = false;
     int stale = 0;
@@ -2398,8 +2441,8 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
         }
         unsigned long long best;
         bool global_scan = !st || !have;
-        if (!st) best = scan_lowest<8, PULL>(P, r0, d, T.tid, T.n);
-        else if (!have) best = scan_and_stage_v4<PULL>(P, r0, d, T.tid, T.n, stg);
+        if (!st) best = scan_lowest<8, PULL>(r0, d, T.tid, T.n);
+        else if (!have) best = scan_and_stage_v4<PULL>(r0, d, T.tid, T.n, stg);
         else best = scan_staged(stg, d, T.tid, T.n);
         have = true;
         best = warp_min_u64(best);
@@ -2410,7 +2453,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
         if (!global_scan && (b == kEmpty || hu <= (int)(b >> 32))) {
             // a relabel is decided on fresh values: refresh the snapshot first
             T.sync();               // every warp has read sh.red
-            best = warp_min_u64(scan_and_stage_v4<PULL>(P, r0, d, T.tid, T.n, stg));
+            best = warp_min_u64(scan_and_stage_v4<PULL>(r0, d, T.tid, T.n, stg));
             if (lane == 0) sh.red[wid] = best;
             T.sync();
             b = kEmpty;
@@ -2419,8 +2462,8 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
         }
         const int best_h = b == kEmpty ? 0x7fffffff : (int)(b >> 32);
         if (T.tid == 0) {
-            add_stat(sh, ST_CYCLES_DIS, 1);
-            if (global_scan) add_stat(sh, ST_SLOTS_DIS, d);
+            add_stat(ST_CYCLES_DIS, 1);
+            if (global_scan) add_stat(ST_SLOTS_DIS, d);
         }
         bool go = b != kEmpty && hu > best_h;
         if (!go) {
@@ -2428,7 +2471,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
             const int nh = (b == kEmpty || best_h >= n - 1) ? n : best_h + 1;
             if (T.tid == 0) {
                 P.h[u] = nh;
-                add_stat(sh, ST_RELABELS, 1);
+                add_stat(ST_RELABELS, 1);
             }
             lifted = true;
             ++cyc;
@@ -2462,7 +2505,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
                     for (int r = 0; r < kSeg; ++r) {
                         if (a[r]) {
                             int sj = stg[js + r];
-                            a[r] = staged_amount<PULL>(P, r0 + js + r, best_h, sj);
+                            a[r] = staged_amount<PULL>(r0 + js + r, best_h, sj);
                             stg[js + r] = sj;
                             ++cand;
                             tsum += a[r];
@@ -2474,7 +2517,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
                     for (int r = 0; r < kSeg; ++r) {
                         a[r] = 0;
                         const int j = js + r;
-                        if (r < seg && j < d && residual_dir<PULL>(P, r0 + j) > 0) a[r] = 1;   // candidate
+                        if (r < seg && j < d && residual_dir<PULL>(r0 + j) > 0) a[r] = 1;   // candidate
                     }
 #pragma unroll
                     for (int r = 0; r < kSeg; ++r) {
@@ -2488,14 +2531,14 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
                     for (int r = 0; r < kSeg; ++r) {
                         if (a[r]) {
                             const int x = r0 + js + r;
-                            const int c = movable<PULL>(P, x, ldg_cg(P.g.rev + x));
+                            const int c = movable<PULL>(x, ldg_cg(P.g.rev + x));
                             a[r] = c > 0 ? c : 0;
                             tsum += a[r];
                             tcnt += a[r] > 0 ? 1 : 0;
                         }
                     }
                     if (T.tid == 0)
-                        add_stat(sh, ST_SLOTS_DIS, seg * T.n);
+                        add_stat(ST_SLOTS_DIS, seg * T.n);
                 }
                 long long incl = tsum;
                 int cincl = tcnt;
@@ -2528,7 +2571,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
                         if (off < rem && cyc + k + coff < kcyc) {
                             const long long g = a[r] < rem - off ? a[r] : rem - off;
                             const int x = r0 + js + r;
-                            move_flow<PULL>(P, sh, x, ldg_cg(P.g.rev + x), ldg_cg(P.g.dst + x), g, dc);
+                            move_flow<PULL>(x, ldg_cg(P.g.rev + x), ldg_cg(P.g.dst + x), g, dc);
                             if (st && g == a[r]) stg[js + r] = kNoRes;
                             mine += g;
                             ++mk;
@@ -2558,7 +2601,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
             }
             if (T.tid == 0) {
                 if (sent) atomic_add_ll(P.e + u, PULL ? sent : -sent);
-                add_stat(sh, ST_PUSHES, k);
+                add_stat(ST_PUSHES, k);
             }
             // staged: a pass that found only stale entries corrected them and costs no cycle (bounded)
             if (k > 0) cyc += k;
@@ -2566,7 +2609,7 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
         }
         T.sync();
     }
-    if (cand) add_stat(sh, ST_SLOTS_DIS, cand);
+    if (cand) add_stat(ST_SLOTS_DIS, cand);
     return lifted;
 }
 
@@ -2574,26 +2617,26 @@ __device__ __noinline__ bool discharge_team_rows(const MfParams &P, Sh &sh, int 
 // the return value is meaningful in thread 0.  stg: the CTA's on-chip
 // snapshot (ccap entries), used when the row fits.
 template <bool PULL>
-__device__ __forceinline__ bool discharge_cta(const MfParams &P, Sh &sh, int u, const DisCtx &dc, int *stg, int ccap)
+__device__ __forceinline__ bool discharge_cta(int u, const DisCtx &dc, int *stg, int ccap)
 {
     const int d = ldg_cg(P.g.deg + u);
-    if (stg != nullptr && d <= ccap) return discharge_team_rows<PULL, true, CtaTeam>(P, sh, u, d, dc, stg);
-    return discharge_team_rows<PULL, false, CtaTeam>(P, sh, u, d, dc, nullptr);
+    if (stg != nullptr && d <= ccap) return discharge_team_rows<PULL, true, CtaTeam>(u, d, dc, stg);
+    return discharge_team_rows<PULL, false, CtaTeam>(u, d, dc, nullptr);
 }
 
 // One 4-warp group per vertex (rows up to group_deg slots, which fit the
 // group's share of the snapshot).  All threads of the group call this
 // together; the return value is meaningful in the group's thread 0.
 template <bool PULL>
-__device__ __forceinline__ bool discharge_group(const MfParams &P, Sh &sh, int u, const DisCtx &dc, int *stg, int gcap)
+__device__ __forceinline__ bool discharge_group(int u, const DisCtx &dc, int *stg, int gcap)
 {
     const int d = ldg_cg(P.g.deg + u);
-    if (stg != nullptr && d <= gcap) return discharge_team_rows<PULL, true, GroupTeam>(P, sh, u, d, dc, stg);
-    return discharge_team_rows<PULL, false, GroupTeam>(P, sh, u, d, dc, nullptr);
+    if (stg != nullptr && d <= gcap) return discharge_team_rows<PULL, true, GroupTeam>(u, d, dc, stg);
+    return discharge_team_rows<PULL, false, GroupTeam>(u, d, dc, nullptr);
 }
 
 template <bool PULL>
-__device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_discharge()
 {
     MfSet *cs = sh.cs;
     const int lane = threadIdx.x & 31;
@@ -2623,10 +2666,10 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
         __syncthreads();
         if (i >= nh) break;
         const int u = __ldcg(wl3 + i);
-        const bool lifted = discharge_cta<PULL>(P, sh, u, dc, stage, P.stage_slots);
+        const bool lifted = discharge_cta<PULL>(u, dc, stage, P.stage_slots);
         if (threadIdx.x == 0) {
-            if (lifted) note_relabel(P, u, dc);
-            requeue_if_active<PULL>(P, u, dc);
+            if (lifted) note_relabel(u, dc);
+            requeue_if_active<PULL>(u, dc);
         }
     }
     // long rows up to group_deg: one 4-warp group each, four side by side per
@@ -2646,15 +2689,15 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
             T.sync();
             if (i >= ng) break;
             const int u = __ldcg(wl2 + i);
-            const bool lifted = discharge_group<PULL>(P, sh, u, dc, gstage, gcap);
+            const bool lifted = discharge_group<PULL>(u, dc, gstage, gcap);
             if (T.tid == 0) {
-                if (lifted) note_relabel(P, u, dc);
-                requeue_if_active<PULL>(P, u, dc);
+                if (lifted) note_relabel(u, dc);
+                requeue_if_active<PULL>(u, dc);
             }
         }
     }
     const unsigned long long t_b = gtimer();
-    if (lane == 0) add_stat(sh, ST_NS_CTA, (long long)(t_b - t_a));
+    if (lane == 0) add_stat(ST_NS_CTA, (long long)(t_b - t_a));
     // mid-degree rows: one warp each, on a slice of its own group's quarter of
     // the snapshot buffer (free once the group has left the loop above, while
     // the other groups may still be on their rows)
@@ -2668,10 +2711,10 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
         const int i = warp_grab(&cs->l[L_HEAD1].w[0], nm, 1u);
         if (i >= nm) break;
         const int u = __ldcg(wl1 + i);
-        const bool lifted = discharge_warp<PULL>(P, sh, u, dc, wstage, wcap);
+        const bool lifted = discharge_warp<PULL>(u, dc, wstage, wcap);
         if (lane == 0) {
-            if (lifted) note_relabel(P, u, dc);
-            requeue_if_active<PULL>(P, u, dc);
+            if (lifted) note_relabel(u, dc);
+            requeue_if_active<PULL>(u, dc);
         }
     }
     const unsigned long long t_c = gtimer();
@@ -2682,16 +2725,16 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
         if (b >= ns) break;
         if (b + lane < ns) {
             const int u = __ldcg(wl0 + b + lane);
-            if (discharge_thread<PULL>(P, sh, u, dc)) note_relabel(P, u, dc);
-            requeue_if_active<PULL>(P, u, dc);
+            if (discharge_thread<PULL>(u, dc)) note_relabel(u, dc);
+            requeue_if_active<PULL>(u, dc);
         }
     }
     __syncwarp();
     const unsigned long long t_d = gtimer();
     if (lane == 0) {
         // per warp, into the CTA's counters
-        add_stat(sh, ST_NS_WARP, (long long)(t_c - t_b));
-        add_stat(sh, ST_NS_THREAD, (long long)(t_d - t_c));
+        add_stat(ST_NS_WARP, (long long)(t_c - t_b));
+        add_stat(ST_NS_THREAD, (long long)(t_d - t_c));
     }
 }
 
@@ -2723,7 +2766,7 @@ __device__ __noinline__ void phase_discharge(const MfParams &P, Sh &sh)
 
 // Whether the squad should go back to the grid: it has held up the others for a
 // quarter of the longest wait at a barrier.
-__device__ __forceinline__ bool squad_timeout(const MfParams &P, unsigned long long t0)
+__device__ __forceinline__ bool squad_timeout(unsigned long long t0)
 {
     return gtimer() - t0 > P.wait_limit_ns / 4;
 }
@@ -2750,7 +2793,7 @@ __device__ __forceinline__ void squad_put(const SquadQ &q, int i, int v, int r0,
 // bfs_visit for a level of the squad: labelled vertices go straight into this
 // CTA's next queue.
 template <int BR>
-__device__ __forceinline__ void squad_visit(const MfParams &P, Sh &sh, const int (&x)[BR], const bool (&valid)[BR],
+__device__ __forceinline__ void squad_visit(const int (&x)[BR], const bool (&valid)[BR],
                                             int L, const SquadQ &nq, int &lab, unsigned &lab_slots)
 {
     const bool want_wl = sh.k_wl != 0, near = sh.d.near != 0;
@@ -2784,7 +2827,11 @@ __device__ __forceinline__ void squad_visit(const MfParams &P, Sh &sh, const int
             if (L == 0 && ldg_cg(P.g.dst + y) == P.sink) P.sc.dem[z[r]] = rc[r];
         }
         if (d[r] > P.bfs_hub) {
-            put_items(P, r0[r], d[r], sh.d.app_hub + atomicAdd(&sh.cs->l[L_HUB].w[0], (unsigned)chunks_of(d[r])));
+            const int i = atomicAdd(&sh.so_long, 1);
+            if (i < MF_SQUAD_LONG)
+                mf_stage[6 * MF_SQUAD_CAP + i] = z[r];
+            else
+                put_items(r0[r], d[r], sh.d.app_hub + atomicAdd(&sh.cs->l[L_HUB].w[0], (unsigned)chunks_of(d[r])));
             sh.so_flag = SQ_SPILL;
         } else {
             const int i = atomicAdd(&sh.so_cnt, 1);
@@ -2796,7 +2843,7 @@ __device__ __forceinline__ void squad_visit(const MfParams &P, Sh &sh, const int
             }
         }
         if (ev[r] > 0 && z[r] != P.sink) {
-            const int bin = row_bin(P, d[r]);
+            const int bin = row_bin(d[r]);
             P.sc.wl[sh.d.wl_sel][bin][sh.d.wl_app[bin] + atomicAdd(&sh.cs->l[L_WL + bin].w[0], 1u)] = z[r];
             if (near) add_shared(sh.exc, ev[r]);
         }
@@ -2806,7 +2853,7 @@ __device__ __forceinline__ void squad_visit(const MfParams &P, Sh &sh, const int
 // Top-down BFS levels, one after another, while they stay small.  The last one
 // leaves its results where a level of the grid would, and the grid barrier that
 // follows takes them up as that level's (with the squad's state).
-__device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
+__device__ __noinline__ void squad_bfs()
 {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nwarps = nt >> 5;
     const int csize = sh.csize, rank = sh.crank;
@@ -2822,7 +2869,7 @@ __device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
             squad_put(q, i, v, P.g.off[v], ldg_cg(P.g.deg + v));
         }
     }
-    if (tid == 0) sh.so_cnt = sh.so_flag = 0;
+    if (tid == 0) sh.so_cnt = sh.so_long = sh.so_flag = 0;
     __syncthreads();
     for (;;) {
         const int L = sh.d.level, par = sh.so_par;
@@ -2860,7 +2907,7 @@ __device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
                     vs[r] = k < T;
                     xs[r] = rb + (k - eb);
                 }
-                squad_visit<kBR>(P, sh, xs, vs, L, nq, lab, lab_slots);
+                squad_visit<kBR>(xs, vs, L, nq, lab, lab_slots);
             }
         }
         __syncwarp();
@@ -2868,7 +2915,7 @@ __device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
         lab_slots = __reduce_add_sync(0xffffffffu, lab_slots);
         if (lane == 0) {
             if (lab) add_shared(sh.lab, ((long long)lab << 32) | lab_slots);
-            add_stat(sh, ST_SLOTS_BFS, scanned);
+            add_stat(ST_SLOTS_BFS, scanned);
         }
         __syncthreads();
         if (wid == 0) {
@@ -2876,11 +2923,11 @@ __device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
             mine.cnt = min(sh.so_cnt, MF_SQUAD_CAP);
             mine.slots = (unsigned)(sh.lab & 0xffffffffull);
             mine.labelled = (int)(sh.lab >> 32);
-            mine.flag = sh.so_flag | (rank == 0 && squad_timeout(P, t0) ? SQ_STOP : 0);
+            mine.flag = sh.so_flag | (rank == 0 && squad_timeout(t0) ? SQ_STOP : 0);
             mine.exc = (long long)sh.exc;
-            squad_tell(sh, par, mine);
+            squad_tell(par, mine);
         }
-        squad_sync(sh);
+        squad_sync();
         if (tid == 0) {
             // the same in every CTA of the squad
             MfDesc &d = sh.d;
@@ -2896,7 +2943,7 @@ __device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
                 exc += s.exc;
             }
             const long long vis = st.vis_slots + fr, sup = st.sup + exc;
-            const bool go = c > 0 && flag == 0 && squad_level(sh, c, fr) &&
+            const bool go = c > 0 && flag == 0 && squad_level(c, fr) &&
                             !(sh.k_alpha > 0 && fr * sh.k_alpha > st.used_slots - vis) &&
                             !(d.near && sup > 0 && (sup >> st.cut_shift) >= st.dem);
             if (go) {
@@ -2921,6 +2968,7 @@ __device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
             __syncthreads();
             at = sh.d.app_bfs + sh.bcast_i;
             for (int i = tid; i < mine; i += nt) P.sc.border[at + i] = squad_q(cur).v[i];
+            write_long(mf_stage + 6 * MF_SQUAD_CAP, min(sh.so_long, MF_SQUAD_LONG));
             return;
         }
         __syncthreads();
@@ -2935,10 +2983,10 @@ __device__ __noinline__ void squad_bfs(const MfParams &P, Sh &sh)
 // row is long, onto the grid's lists; else into the CTA's queue of worklist
 // entries.
 template <bool SQUAD>
-__device__ __forceinline__ void short_enqueue(const MfParams &P, Sh &sh, int z, int r0, int d, const SquadQ &nq)
+__device__ __forceinline__ void short_enqueue(int z, int r0, int d, const SquadQ &nq)
 {
     if (!SQUAD) {
-        place_active(P, sh, z, d, L_AUX, sh.d.wl_sel ^ 1, nullptr);
+        place_active(z, d, L_AUX, sh.d.wl_sel ^ 1, nullptr);
         return;
     }
     if (d <= MF_SHORT_ROW) {
@@ -2948,7 +2996,7 @@ __device__ __forceinline__ void short_enqueue(const MfParams &P, Sh &sh, int z, 
             return;
         }
     }
-    const int bin = row_bin(P, d);
+    const int bin = row_bin(d);
     P.sc.wl[sh.d.wl_sel ^ 1][bin][atomicAdd(&sh.cs->l[L_AUX + bin].w[0], 1u)] = z;
     sh.so_flag = SQ_SPILL;
 }
@@ -2958,7 +3006,7 @@ __device__ __forceinline__ void short_enqueue(const MfParams &P, Sh &sh, int z, 
 // rises from <= 0 to > 0 at most once in a round: whoever makes it do so
 // queues it, and no stamp is needed.
 template <bool SQUAD>
-__device__ __forceinline__ void short_push(const MfParams &P, Sh &sh, int x, int z, int y, int g, const SquadQ &nq)
+__device__ __forceinline__ void short_push(int x, int z, int y, int g, const SquadQ &nq)
 {
     atomicSub(P.cf + x, g);
     atomicAdd(P.cf + y, g);
@@ -2969,20 +3017,20 @@ __device__ __forceinline__ void short_push(const MfParams &P, Sh &sh, int x, int
     } else {
         const int d = ldg_cg(P.g.deg + z), r0 = SQUAD ? P.g.off[z] : 0;     // in flight together with the excess
         const long long old = atomic_add_ll(P.e + z, (long long)g);
-        if (old <= 0 && old + g > 0) short_enqueue<SQUAD>(P, sh, z, r0, d, nq);
+        if (old <= 0 && old + g > 0) short_enqueue<SQUAD>(z, r0, d, nq);
     }
 }
 
 // u's new height when its lowest residual neighbour has height best (INT_MAX:
 // none): Alg. 2's relabel if u is not above it.
-__device__ __forceinline__ int short_lift(const MfParams &P, Sh &sh, int u, int hu, int best, bool write)
+__device__ __forceinline__ int short_lift(int u, int hu, int best, bool write)
 {
     const int n = P.g.n;
     if (best < hu) return hu;
     const int nh = best >= n - 1 ? n : best + 1;
     if (write) {
         P.h[u] = nh;
-        add_stat(sh, ST_RELABELS, 1);
+        add_stat(ST_RELABELS, 1);
     }
     return nh;
 }
@@ -2990,7 +3038,7 @@ __device__ __forceinline__ int short_lift(const MfParams &P, Sh &sh, int u, int 
 // One cycle of Alg. 2 for u by one thread (rows of at most 8 slots): relabel if
 // needed, then push to the lowest neighbours in slot order.
 template <bool SQUAD>
-__device__ __forceinline__ int short_thread(const MfParams &P, Sh &sh, int u, int r0, int d, const SquadQ &nq)
+__device__ __forceinline__ int short_thread(int u, int r0, int d, const SquadQ &nq)
 {
     const int4 none = make_int4(0, 0, 0, 0);
     const long long eu = ldg_cg(P.e + u);
@@ -3013,7 +3061,7 @@ __device__ __forceinline__ int short_thread(const MfParams &P, Sh &sh, int u, in
     for (int k = 0; k < 8; ++k) hz[k] = c[k] > 0 ? ldg_cg(P.h + z[k]) : 0x7fffffff;
 #pragma unroll
     for (int k = 0; k < 8; ++k) best = min(best, hz[k]);
-    hu = short_lift(P, sh, u, hu, best, true);
+    hu = short_lift(u, hu, best, true);
     if (hu >= P.g.n) return 0;
     long long rem = eu;
     int pushes = 0;
@@ -3021,19 +3069,19 @@ __device__ __forceinline__ int short_thread(const MfParams &P, Sh &sh, int u, in
     for (int k = 0; k < 8; ++k) {
         if (hz[k] != best || rem <= 0) continue;
         const int g = rem < (long long)c[k] ? (int)rem : c[k];
-        short_push<SQUAD>(P, sh, r0 + k, z[k], ldg_cg(P.g.rev + r0 + k), g, nq);
+        short_push<SQUAD>(r0 + k, z[k], ldg_cg(P.g.rev + r0 + k), g, nq);
         rem -= g;
         ++pushes;
     }
     const long long old = atomic_add_ll(P.e + u, rem - eu);
-    if (old + rem - eu > 0) short_enqueue<SQUAD>(P, sh, u, r0, d, nq);
+    if (old + rem - eu > 0) short_enqueue<SQUAD>(u, r0, d, nq);
     return pushes;
 }
 
 // The same by one warp (rows of up to MF_SHORT_ROW slots): every lane holds four
 // slots of each 128, and a prefix sum over the lanes deals out the excess.
 template <bool SQUAD>
-__device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int r0, int d, const SquadQ &nq)
+__device__ __forceinline__ int short_warp(int u, int r0, int d, const SquadQ &nq)
 {
     constexpr int kQ = MF_SHORT_ROW / 128;
     const int lane = threadIdx.x & 31;
@@ -3058,7 +3106,7 @@ __device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int 
 #pragma unroll
     for (int k = 0; k < 4 * kQ; ++k) best = min(best, hz[k]);
     best = __reduce_min_sync(0xffffffffu, best);
-    hu = short_lift(P, sh, u, hu, best, lane == 0);
+    hu = short_lift(u, hu, best, lane == 0);
     if (hu >= P.g.n) return 0;
     long long mine = 0;
 #pragma unroll
@@ -3077,7 +3125,7 @@ __device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int 
         if (hz[k] != best || rem <= 0) continue;
         const int g = rem < (long long)c[k] ? (int)rem : c[k];
         const int x = r0 + (k >> 2) * 128 + lane * 4 + (k & 3);
-        short_push<SQUAD>(P, sh, x, ldg_cg(P.g.dst + x), ldg_cg(P.g.rev + x), g, nq);
+        short_push<SQUAD>(x, ldg_cg(P.g.dst + x), ldg_cg(P.g.rev + x), g, nq);
         rem -= g;
         ++pushes;
     }
@@ -3086,7 +3134,7 @@ __device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int 
     if (lane == 0) {
         const long long sent = total < eu ? total : eu;
         const long long old = atomic_add_ll(P.e + u, -sent);
-        if (old - sent > 0) short_enqueue<SQUAD>(P, sh, u, r0, d, nq);
+        if (old - sent > 0) short_enqueue<SQUAD>(u, r0, d, nq);
     }
     __syncwarp();
     return pushes;
@@ -3094,7 +3142,7 @@ __device__ __forceinline__ int short_warp(const MfParams &P, Sh &sh, int u, int 
 
 // A discharge round of one cycle per vertex across the grid: a thread for a row
 // of at most 8 slots, a warp for a longer one.
-__device__ __noinline__ void phase_discharge_short(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_discharge_short()
 {
     const int lane = threadIdx.x & 31;
     const int sel = sh.d.wl_sel, n0 = sh.d.wl_n[0], n1 = sh.d.wl_n[1], cnt = n0 + n1;
@@ -3105,7 +3153,7 @@ __device__ __noinline__ void phase_discharge_short(const MfParams &P, Sh &sh)
         const int u = __ldcg(i < n0 ? P.sc.wl[sel][0] + i : P.sc.wl[sel][1] + (i - n0));
         const int d = ldg_cg(P.g.deg + u), r0 = P.g.off[u];
         if (d > 8) continue;
-        pushes += short_thread<false>(P, sh, u, r0, d, none);
+        pushes += short_thread<false>(u, r0, d, none);
         slots += d;
         ++scans;
     }
@@ -3115,22 +3163,22 @@ __device__ __noinline__ void phase_discharge_short(const MfParams &P, Sh &sh)
         const int u = __ldcg(i < n0 ? P.sc.wl[sel][0] + i : P.sc.wl[sel][1] + (i - n0));
         const int d = ldg_cg(P.g.deg + u), r0 = P.g.off[u];
         if (d <= 8) continue;
-        const int p = short_warp<false>(P, sh, u, r0, d, none);
+        const int p = short_warp<false>(u, r0, d, none);
         if (lane == 0) {
             pushes += p;
             slots += d;
             ++scans;
         }
     }
-    add_stat(sh, ST_PUSHES, pushes);
-    add_stat(sh, ST_SLOTS_DIS, slots);
-    add_stat(sh, ST_CYCLES_DIS, scans);
-    flush_queue(P, sh, L_AUX, sel ^ 1, nullptr, 0, 0u);
+    add_stat(ST_PUSHES, pushes);
+    add_stat(ST_SLOTS_DIS, slots);
+    add_stat(ST_CYCLES_DIS, scans);
+    flush_queue(L_AUX, sel ^ 1, nullptr, 0, 0u);
 }
 
 // Discharge rounds, one after another, while few vertices are active.  The last
 // one leaves its results where a round of the grid would.
-__device__ __noinline__ void squad_discharge(const MfParams &P, Sh &sh)
+__device__ __noinline__ void squad_discharge()
 {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
     const int csize = sh.csize, rank = sh.crank;
@@ -3155,7 +3203,7 @@ __device__ __noinline__ void squad_discharge(const MfParams &P, Sh &sh)
         for (int i = tid; i < cnt; i += nt) {
             const int d = cq.d[i];
             if (d > 8) continue;
-            pushes += short_thread<true>(P, sh, cq.v[i], cq.r[i], d, nq);
+            pushes += short_thread<true>(cq.v[i], cq.r[i], d, nq);
             slots += d;
             ++scans;
         }
@@ -3163,16 +3211,16 @@ __device__ __noinline__ void squad_discharge(const MfParams &P, Sh &sh)
         for (int i = wid; i < cnt; i += nt >> 5) {
             const int d = cq.d[i];
             if (d <= 8) continue;
-            const int p = short_warp<true>(P, sh, cq.v[i], cq.r[i], d, nq);
+            const int p = short_warp<true>(cq.v[i], cq.r[i], d, nq);
             if (lane == 0) {
                 pushes += p;
                 slots += d;
                 ++scans;
             }
         }
-        add_stat(sh, ST_PUSHES, pushes);
-        add_stat(sh, ST_SLOTS_DIS, slots);
-        add_stat(sh, ST_CYCLES_DIS, scans);
+        add_stat(ST_PUSHES, pushes);
+        add_stat(ST_SLOTS_DIS, slots);
+        add_stat(ST_CYCLES_DIS, scans);
         __syncthreads();
         if (wid == 0) {
             SquadSum mine{};
@@ -3181,11 +3229,11 @@ __device__ __noinline__ void squad_discharge(const MfParams &P, Sh &sh)
             if (rank == 0) {
                 const unsigned long long now = gtimer();
                 if (sh.d.round + 1 >= MF_DEFAULT_ROUNDS && !rounds_left(sh.d, sh.hs, now)) mine.flag |= SQ_OVER;
-                if (squad_timeout(P, t0)) mine.flag |= SQ_STOP;
+                if (squad_timeout(t0)) mine.flag |= SQ_STOP;
             }
-            squad_tell(sh, par, mine);
+            squad_tell(par, mine);
         }
-        squad_sync(sh);
+        squad_sync();
         if (tid == 0) {
             // the same in every CTA of the squad
             int c = 0, flag = 0;
@@ -3209,7 +3257,7 @@ __device__ __noinline__ void squad_discharge(const MfParams &P, Sh &sh)
             // (what is left when the discharge is over waits for the next BFS)
             if (go == 2) {
                 for (int i = tid; i < mine; i += nt) {
-                    const int bin = row_bin(P, nq.d[i]);
+                    const int bin = row_bin(nq.d[i]);
                     P.sc.wl[sh.d.wl_sel ^ 1][bin][atomicAdd(&sh.cs->l[L_AUX + bin].w[0], 1u)] = nq.v[i];
                 }
             }
@@ -3263,7 +3311,7 @@ __device__ __forceinline__ int draw(int *cf, long long a)
 // active vertex under way at once.  A discharge round over the same vertices
 // scans their whole rows: on R-MAT 20 with 10 K updates two rounds read some
 // 5 M slots of hub rows and took 120-190 us, the walks take about 10 us.
-__device__ __noinline__ void phase_walk(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_walk()
 {
     const int sel = sh.d.wl_sel;
     DisCtx dc;
@@ -3299,11 +3347,11 @@ __device__ __noinline__ void phase_walk(const MfParams &P, Sh &sh)
             a = got;
         }
         if (a <= 0) {
-            if (dc.queue) enqueue_active(P, u, dc);
+            if (dc.queue) enqueue_active(u, dc);
             continue;
         }
         atomic_add_ll(P.e + u, -a);
-        if (dc.queue && eu > a) enqueue_active(P, u, dc);
+        if (dc.queue && eu > a) enqueue_active(u, dc);
         int v = u;
         do {
             const int y = ldg_cg(P.sc.par + v);
@@ -3315,14 +3363,14 @@ __device__ __noinline__ void phase_walk(const MfParams &P, Sh &sh)
             }
             if (g < a) {
                 atomic_add_ll(P.e + v, a - g);
-                if (dc.queue) enqueue_active(P, v, dc);
+                if (dc.queue) enqueue_active(v, dc);
             }
             a = g;
             v = w;
         } while (a > 0 && v != P.sink && ldg_cg(P.h + v) > 0);
-        if (a > 0) add_excess(P, sh, v, a);
+        if (a > 0) add_excess(v, a);
     }
-    add_stat(sh, ST_PUSHES, pushes);
+    add_stat(ST_PUSHES, pushes);
 }
 
 // ---------------------------------------------------------------------------
@@ -3336,7 +3384,7 @@ __device__ __noinline__ void phase_walk(const MfParams &P, Sh &sh)
 // PULL (Sec. 5.2.2): a steep in-residual c_f(v, u) is pulled whole, and the
 // return value is minus the flow received.
 template <bool PULL>
-__device__ __forceinline__ long long fix_scan(const MfParams &P, Sh &sh, int hu, int r0, int d, int j0, int step)
+__device__ __forceinline__ long long fix_scan(int hu, int r0, int d, int j0, int step)
 {
     constexpr int kF = 4;
     long long out = 0;
@@ -3359,16 +3407,16 @@ __device__ __forceinline__ long long fix_scan(const MfParams &P, Sh &sh, int hu,
                     const int old = atomicExch(P.cf + y, 0);
                     if (old > 0) {
                         atomicAdd(P.cf + x, old);
-                        add_excess(P, sh, z[r], -(long long)old);
-                        add_stat(sh, ST_STEEP, 1);
+                        add_excess(z[r], -(long long)old);
+                        add_stat(ST_STEEP, 1);
                         out -= old;
                     }
                 } else {
                     const int old = atomicExch(P.cf + x, 0);
                     if (old > 0) {
                         atomicAdd(P.cf + ldg_cg(P.g.rev + x), old);
-                        add_excess(P, sh, z[r], (long long)old);
-                        add_stat(sh, ST_STEEP, 1);
+                        add_excess(z[r], (long long)old);
+                        add_stat(ST_STEEP, 1);
                         out += old;
                     }
                 }
@@ -3379,7 +3427,7 @@ __device__ __forceinline__ long long fix_scan(const MfParams &P, Sh &sh, int hu,
 }
 
 template <bool PULL>
-__device__ __noinline__ void phase_fix(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_fix()
 {
     MfSet *cs = sh.cs;
     const int lane = threadIdx.x & 31;
@@ -3398,7 +3446,7 @@ __device__ __noinline__ void phase_fix(const MfParams &P, Sh &sh)
         const int u = __ldcg(P.sc.fixl[1] + i);
         const int hu = ldg_cg(P.h + u);
         const int r0 = P.g.off[u], d = ldg_cg(P.g.deg + u);
-        long long out = fix_scan<PULL>(P, sh, hu, r0, d, threadIdx.x, blockDim.x);
+        long long out = fix_scan<PULL>(hu, r0, d, threadIdx.x, blockDim.x);
         if (out) atomic_add_ll(P.e + u, -out);
         if (threadIdx.x == 0) { slots += d; ++verts; }
     }
@@ -3410,22 +3458,22 @@ __device__ __noinline__ void phase_fix(const MfParams &P, Sh &sh)
         const int u = __ldcg(P.sc.fixl[0] + i);
         const int hu = ldg_cg(P.h + u);
         const int r0 = P.g.off[u], d = ldg_cg(P.g.deg + u);
-        long long out = warp_sum_ll(fix_scan<PULL>(P, sh, hu, r0, d, lane, 32));
+        long long out = warp_sum_ll(fix_scan<PULL>(hu, r0, d, lane, 32));
         if (lane == 0) {
             if (out) atomic_add_ll(P.e + u, -out);
             slots += d;
             ++verts;
         }
     }
-    add_stat(sh, ST_SLOTS_FIX, slots);
-    add_stat(sh, ST_VERTS_FIX, verts);
+    add_stat(ST_SLOTS_FIX, slots);
+    add_stat(ST_VERTS_FIX, verts);
 }
 
 // ---------------------------------------------------------------------------
 // Value (Alg. 5 last lines, reading R3)
 // ---------------------------------------------------------------------------
 
-__device__ __noinline__ void phase_value(const MfParams &P, Sh &sh)
+__device__ __noinline__ void phase_value()
 {
     // push (R3): sum of e(v) over v != s with h(v) < n; pull (Sec. 5.2.2, the
     // mirror): sum of -e(v) over v != t with h(v) < n
@@ -3444,7 +3492,7 @@ __device__ __noinline__ void phase_value(const MfParams &P, Sh &sh)
 // the value.  Returns false only if this CTA gave up waiting at a barrier
 // (the caller must then leave the kernel); every other exit is taken by all
 // CTAs together.
-__device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
+__device__ __noinline__ bool solve_instance()
 {
     __syncthreads();          // the parameters are in shared memory
     if (threadIdx.x < MF_STATS) sh.stat[threadIdx.x] = 0;
@@ -3466,7 +3514,7 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
         sh.hs = MfState{};
         sh.d.qstamp = __ldcg(&c->qstamp);
         sh.d.fstamp = __ldcg(&c->fstamp);
-        sh.d.near = near_allowed(P);
+        sh.d.near = near_allowed();
         sh.k_alpha = P.bu_alpha;
         sh.k_beta = P.bu_beta;
         sh.k_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY) ? 1 : 0;
@@ -3491,118 +3539,116 @@ __device__ __noinline__ bool solve_instance(const MfParams &P, Sh &sh)
     bool opened = false;      // the last barrier opened the first iteration
     if (P.mode & MF_M_STATIC_INIT) {
         const bool sat = !(P.mode & MF_M_NO_SRC_SAT), sink = (P.mode & MF_M_SAT_SINK) != 0;
-        phase_static_reset(P);
-        if (!grid_sync(P, sat || sink || !loops ? H_NONE : H_ITER, sh)) return false;
+        phase_static_reset();
+        if (!grid_sync(sat || sink || !loops ? H_NONE : H_ITER)) return false;
         if (sat) {
-            phase_saturate_source(P, sh);
-            if (!grid_sync(P, sink || !loops ? H_NONE : H_ITER, sh)) return false;
+            phase_saturate_source();
+            if (!grid_sync(sink || !loops ? H_NONE : H_ITER)) return false;
         }
         if (sink) {
-            phase_saturate_sink(P, sh);
-            if (!grid_sync(P, loops ? H_ITER : H_NONE, sh)) return false;
+            phase_saturate_sink();
+            if (!grid_sync(loops ? H_ITER : H_NONE)) return false;
         }
         opened = loops;
     }
     if (P.mode & MF_M_APPLY) {
-        phase_apply_validate(P, sh);
-        if (!grid_sync(P, H_APPLY_VALID, sh)) return false;
+        phase_apply_validate();
+        if (!grid_sync(H_APPLY_VALID)) return false;
         if (sh.d.status != MF_ST_RUNNING) {
-            phase_apply_cleanup(P, sh, false);
-            return finish(P, sh);
+            phase_apply_cleanup(false);
+            return finish();
         }
-        phase_apply_locate(P, sh);
-        if (!grid_sync(P, H_APPLY_LOCATED, sh)) return false;
+        phase_apply_locate();
+        if (!grid_sync(H_APPLY_LOCATED)) return false;
         if (sh.d.status != MF_ST_RUNNING) {
             // a row overflow keeps the rows' demand for the rebuild that follows;
             // a refused batch (pair sum) leaves nothing behind
-            phase_apply_cleanup(P, sh, sh.hs.err == MF_E_OVERFLOW);
-            return finish(P, sh);
+            phase_apply_cleanup(sh.hs.err == MF_E_OVERFLOW);
+            return finish();
         }
-        phase_apply_change(P, sh);
-        if (!grid_sync(P, H_APPLY_DELTA, sh)) return false;
+        phase_apply_change();
+        if (!grid_sync(H_APPLY_DELTA)) return false;
         // the source step reads the final residuals; the tables are cleared beside it
-        phase_apply_cleanup(P, sh, false);
-        if (!(P.mode & MF_M_SKIP_SOURCE_SAT)) phase_resaturate(P, sh);
+        phase_apply_cleanup(false);
+        if (!(P.mode & MF_M_SKIP_SOURCE_SAT)) phase_resaturate();
         // straight on to the loop: this barrier opens its first iteration
         opened = loops && !(P.mode & MF_M_CUT);
-        if (!opened && !(P.mode & MF_M_CUT) && !loops) return finish(P, sh);
-        if (!grid_sync(P, opened ? H_ITER : H_NONE, sh)) return false;
+        if (!opened && !(P.mode & MF_M_CUT) && !loops) return finish();
+        if (!grid_sync(opened ? H_ITER : H_NONE)) return false;
         if (P.mode & MF_M_CUT) {
-            phase_cut_side(P);
-            if (!grid_sync(P, H_NONE, sh)) return false;
-            phase_saturate_cut(P, sh);
-            if (!grid_sync(P, H_NONE, sh)) return false;
+            phase_cut_side();
+            if (!grid_sync(H_NONE)) return false;
+            phase_saturate_cut();
+            if (!grid_sync(H_NONE)) return false;
         }
-        if (sh.d.status != MF_ST_RUNNING) return finish(P, sh);
+        if (sh.d.status != MF_ST_RUNNING) return finish();
     }
-    if (!loops) return finish(P, sh);
+    if (!loops) return finish();
 
-    if (!opened && !grid_sync(P, H_ITER, sh)) return false;
+    if (!opened && !grid_sync(H_ITER)) return false;
     for (;;) {
         // backward BFS
-        phase_bfs_init(P, sh);
-        if (!grid_sync(P, H_BFS_START, sh)) return false;
+        phase_bfs_init();
+        if (!grid_sync(H_BFS_START)) return false;
         while (!sh.d.bfs_done) {
             if (sh.d.bfs_squad) {
                 // the others wait at the grid barrier and take the squad's state there
-                if (vb() < sh.csize) squad_bfs(P, sh);
-                if (!grid_sync(P, H_BFS_NEXT, sh, true)) return false;
+                if (vb() < sh.csize) squad_bfs();
+                if (!grid_sync(H_BFS_NEXT, true)) return false;
                 continue;
             }
             if (sh.d.bu_mode) {
-                phase_bfs_bottom_up(P, sh);
-                if (!grid_sync(P, H_BU_SPLIT, sh)) return false;     // ends the level if nothing was deferred
+                phase_bfs_bottom_up();
+                if (!grid_sync(H_BU_SPLIT)) return false;     // ends the level if nothing was deferred
                 if (sh.d.bu_split) {
-                    phase_bfs_bottom_up_long(P, sh);
-                    if (!grid_sync(P, H_BFS_NEXT, sh)) return false;
+                    phase_bfs_bottom_up_long();
+                    if (!grid_sync(H_BFS_NEXT)) return false;
                 }
             } else {
-                phase_bfs_level(P, sh);
-                if (!grid_sync(P, H_BFS_NEXT, sh)) return false;
+                phase_bfs_level();
+                if (!grid_sync(H_BFS_NEXT)) return false;
             }
         }
-        if (P.mode & MF_M_BFS_ONLY) return finish(P, sh);
+        if (P.mode & MF_M_BFS_ONLY) return finish();
         // worklist and termination test (built during the BFS when data-driven)
         if (!P.data_driven) {
-            phase_worklist(P, sh);
-            if (!grid_sync(P, H_WL, sh)) return false;
+            phase_worklist();
+            if (!grid_sync(H_WL)) return false;
         }
         if (sh.d.status != MF_ST_RUNNING) break;
         // discharge rounds, then remove-invalid-edges
         do {
             if (sh.d.dis_squad) {
-                if (vb() < sh.csize) squad_discharge(P, sh);
-                if (!grid_sync(P, H_DIS, sh, true)) return false;
+                if (vb() < sh.csize) squad_discharge();
+                if (!grid_sync(H_DIS, true)) return false;
                 continue;
             }
-            if (sh.d.near && sh.d.round == 0) phase_walk(P, sh);
-            else if (sh.d.dis_short) phase_discharge_short(P, sh);
-            else if (P.pull) phase_discharge<true>(P, sh);
-            else phase_discharge<false>(P, sh);
-            if (!grid_sync(P, H_DIS, sh)) return false;
+            if (sh.d.near && sh.d.round == 0) phase_walk();
+            else if (sh.d.dis_short) phase_discharge_short();
+            else if (P.pull) phase_discharge<true>();
+            else phase_discharge<false>();
+            if (!grid_sync(H_DIS)) return false;
         } while (sh.d.dis_more);
         if (P.fix_steep) {
-            if (P.pull) phase_fix<true>(P, sh);
-            else phase_fix<false>(P, sh);
-            if (!grid_sync(P, H_ITER, sh)) return false;
+            if (P.pull) phase_fix<true>();
+            else phase_fix<false>();
+            if (!grid_sync(H_ITER)) return false;
         }
     }
-    if (sh.d.status != MF_ST_ERROR && !(P.mode & MF_M_NO_VALUE)) phase_value(P, sh);
-    return finish(P, sh);
+    if (sh.d.status != MF_ST_ERROR && !(P.mode & MF_M_NO_VALUE)) phase_value();
+    return finish();
 }
 
-__global__ void __launch_bounds__(MF_BLOCK, 2) mf_solve_kernel(const __grid_constant__ MfParams P)
+__global__ void __launch_bounds__(MF_BLOCK, 2) mf_solve_kernel(const __grid_constant__ MfParams params)
 {
-    __shared__ Sh sh;
-    __shared__ MfParams sP;       // the phases read the parameters often: from shared memory
     for (int i = threadIdx.x; i < (int)(sizeof(MfParams) / 4); i += blockDim.x)
-        reinterpret_cast<int *>(&sP)[i] = reinterpret_cast<const int *>(&P)[i];
+        reinterpret_cast<int *>(&P)[i] = reinterpret_cast<const int *>(&params)[i];
     if (threadIdx.x == 0) {
         g_vb = blockIdx.x;
         g_vn = gridDim.x;
     }
     __syncthreads();
-    solve_instance(sP, sh);
+    solve_instance();
 }
 
 // Barrier of one group of CTAs (no hook): w[0] arrivals, w[1] generation.
@@ -3653,8 +3699,6 @@ __global__ void __launch_bounds__(MF_BLOCK, 2) mf_multi_kernel(const MfParams *_
                                                                int gsize, unsigned *gstate, unsigned *head,
                                                                unsigned long long wait_ns, int *abort)
 {
-    __shared__ Sh sh;
-    __shared__ MfParams sP;
     __shared__ unsigned ggen;
     const int grp = blockIdx.x / gsize;
     unsigned *gw = gstate + 32 * grp;
@@ -3670,8 +3714,8 @@ __global__ void __launch_bounds__(MF_BLOCK, 2) mf_multi_kernel(const MfParams *_
         const int i = (int)__ldcg(gw + 2);
         if (i >= count) return;
         for (int w = threadIdx.x; w < (int)(sizeof(MfParams) / 4); w += blockDim.x)
-            reinterpret_cast<int *>(&sP)[w] = __ldcg(reinterpret_cast<const int *>(plist + i) + w);
-        if (!solve_instance(sP, sh)) {
+            reinterpret_cast<int *>(&P)[w] = __ldcg(reinterpret_cast<const int *>(plist + i) + w);
+        if (!solve_instance()) {
             atomicExch(abort, 1);
             return;
         }
