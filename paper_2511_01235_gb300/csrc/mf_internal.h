@@ -38,7 +38,7 @@
 #define MF_BU_CHUNK 256       // bottom-up BFS: slots per deferred work item (one warp, 8 per lane)
 #define MF_NEAR_SINK 8        // near iterations: the sink's row holds at most 1/8 of the vertices
 #define MF_LARGE_SLOTS 65536  // near iterations and short rounds: graphs of at least this many reserved slots
-#define MF_NEAR_STEP 3        // near iterations: a cut that settled less than half asks for 2^3 times the excess next
+#define MF_NEAR_STEP 2        // near iterations: a cut that settled less than half asks for 2^2 times the excess next
 #define MF_NEAR_SUB 8192      // walks: residuals up to this are taken with one atomic subtraction
 #define MF_Q_BFS 8192         // on-chip queue of a CTA: labelled vertices of one BFS phase,
 #define MF_Q_LONG 2048        // ... those with long rows,
@@ -158,6 +158,7 @@ struct MfState {
     long long used_slots;         // used slots of the graph (0: not summed yet)
     long long sup, dem, dem_prev; // this BFS: excess labelled, what the roots can take (and the BFS before)
     int cut_prev, cut_shift;      // the iteration before was cut short; how much more excess a cut asks for
+    int full_run, pad0;           // complete relabels in a row that left excess to move (near)
     long long iters, bfs_levels, rounds_total, barriers, active_first, active_total;
     int err;                      // MF_E_*
     int trace_n;

@@ -498,9 +498,11 @@ __device__ __noinline__ void advance(int hook, unsigned long long t)
         // (deep BFS, e.g. grids) is amortised over more rounds
         bool more = nxt > 0 && st.err == 0 && d.round + 1 < MF_MAX_ROUNDS;
         if (d.near && d.round == 0) {
-            // the walks: rounds follow only a complete relabel, and only while
-            // they are cheap beside it
-            more = more && !d.cut && rounds_left(d, st, t);
+            // the walks: rounds, which scan hub rows whole, follow only when a
+            // second complete relabel in a row has left something to do, and
+            // only while they are cheap beside it
+            more = more && !d.cut && st.full_run > 0 && rounds_left(d, st, t);
+            st.full_run = d.cut ? 0 : st.full_run + 1;
         } else if (more && d.round + 1 >= (P.rounds > 0 ? P.rounds : MF_DEFAULT_ROUNDS))
             more = P.rounds > 0 ? false : rounds_left(d, st, t);
         d.dis_more = more ? 1 : 0;
