@@ -192,9 +192,15 @@ int maxflow_set_kernel_cycles(maxflow_ctx *c, int32_t k);
  * rounds, before the next BFS -- as in the paper's kernel, where every vertex
  * checks e(u) > 0 on each of its cycles.  0 (the default) is adaptive, not in
  * the paper: at least 2 rounds, then more while the discharge of the current
- * iteration has taken less than half the time of its BFS, at most 1024, so
- * that a global relabel that costs much (a deep BFS, as on grids) is spread
- * over more discharge work.  MAXFLOW_ERR_INVALID below 0. */
+ * iteration has taken less than half the time of its BFS (rounds of one cycle
+ * per vertex, which push solves run where every active row has at most 512
+ * slots and the graph is large or its BFS deep: less than all of it), at most
+ * 1024, so that a global relabel that costs much (a deep BFS, as on grids) is
+ * spread over more discharge work.  On large graphs whose sink has a short row,
+ * 0 also lets a push solve end a global relabel once it has labelled as much
+ * excess as its roots can take, and send that excess down the BFS tree before
+ * any round; the solve still ends only behind a complete BFS.
+ * MAXFLOW_ERR_INVALID below 0. */
 int maxflow_set_rounds(maxflow_ctx *c, int32_t rounds);
 
 /* With on = 1 (the default), a vertex that still has excess and a height
@@ -213,14 +219,14 @@ int maxflow_set_requeue(maxflow_ctx *c, int32_t on);
  * work only).  MAXFLOW_ERR_INVALID below 0. */
 int maxflow_set_cycle_div(maxflow_ctx *c, int32_t div);
 
-/* Small BFS levels on one CTA: a top-down level whose frontier holds at most
- * `slots` slots (and at most as many vertices) runs in the first CTA alone,
- * level after level, without a grid barrier between levels (the labels are
- * those of Alg. 4 / Alg. 6 either way); the grid meets again when a frontier
- * grows past the limit, the BFS ends, or after 256 such levels.  0 (the
- * default) turns it off: measured on R-MAT, grids and the batched instances it
- * did not pay (a level of a few hundred slots costs about as much in one CTA as
- * the grid's barrier does).  Not in the paper.  MAXFLOW_ERR_INVALID below 0. */
+/* Small BFS levels on one thread-block cluster: a top-down level whose
+ * frontier holds at most `slots` slots (and at most 256 vertices per CTA) runs
+ * in the first cluster of eight CTAs alone, level after level, with the
+ * cluster's barrier between levels instead of the grid's (the labels are those
+ * of Alg. 4 / Alg. 6 either way); the grid meets again when a frontier grows
+ * past a limit or the BFS ends.  0 (the default) is the library's own limit,
+ * 2048 slots per CTA.  Launches without clusters use their first CTA.  Not in
+ * the paper.  MAXFLOW_ERR_INVALID below 0. */
 int maxflow_set_bfs_tail(maxflow_ctx *c, int32_t slots);
 
 /* Run remove-invalid-edges (Alg. 3) after each iteration's discharge rounds
@@ -290,7 +296,7 @@ int maxflow_mlp_train(maxflow_mlp *m, const float *x, const float *target, const
 
 /* Compute the batch's features, let the network predict each action's log
  * time, and run the action with the smallest prediction (written to
- * *action_out, may be NULL).  The network must have 16 inputs and one output
+ * *action_out, may be NULL), all in the launch that applies the batch.  The network must have 16 inputs and one output
  * per action (else MAXFLOW_ERR_INVALID).  Every action gives the same maximum
  * flow; errors as maxflow_run_action. */
 int maxflow_update_scheduled(maxflow_ctx *c, const maxflow_batch *b, maxflow_mlp *m, int32_t *action_out);
@@ -300,11 +306,11 @@ int maxflow_update_scheduled(maxflow_ctx *c, const maxflow_batch *b, maxflow_mlp
  * one warp, longer rows a 4-warp group up to a quarter of the CTA's snapshot
  * buffer (about 7.2 K slots) and the longest a whole CTA (remove-invalid-edges:
  * a warp up to warp_max_slots, then a CTA); the BFS splits rows longer than
- * bfs_item_min_slots into 256-slot work items.  All three 0: the defaults,
+ * bfs_item_min_slots into 128-slot work items.  All three 0: the defaults,
  * thread_max_slots 8, or 4 on a graph of at most 8 merged directed edges per
  * vertex (grids, geometric and layered graphs: many short discharge rounds,
  * where a warp's parallel scan of a short row beats one thread's), then 512
- * and 256.  Not in the paper (it steers work only).  MAXFLOW_ERR_INVALID for
+ * and 128.  Not in the paper (it steers work only).  MAXFLOW_ERR_INVALID for
  * NULL c, a zero or negative threshold (unless all three are 0) or
  * warp_max_slots < thread_max_slots. */
 int maxflow_set_tuning(maxflow_ctx *c, int32_t thread_max_slots, int32_t warp_max_slots, int32_t bfs_item_min_slots);

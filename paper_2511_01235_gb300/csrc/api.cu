@@ -55,7 +55,7 @@ struct maxflow_ctx {
     int32_t stage_slots = 0;      // dynamic shared memory of the solve launches, in ints
     int32_t requeue = 1;          // discharge rounds re-queue vertices still active after their cycles
     int32_t cycle_div = 0;        // > 0: long rows get max(kernel_cycles, deg / cycle_div) cycles
-    int32_t tail_slots = 0;       // BFS frontiers of at most this many slots run in one CTA (0: off)
+    int32_t tail_slots = 0;       // BFS frontiers of at most this many slots run in the squad (0: MF_SQUAD_SLOTS per CTA)
     MfGraph g{};
     MfScratch sc{};
     MfCtrl *ctrl = nullptr;
@@ -81,7 +81,6 @@ struct maxflow_ctx {
     int64_t inc_iters = 0, inc_active_first = 0, inc_levels = 0;
     double inc_ms = 0;
     float *feat = nullptr;        // [MF_FEATURES] device
-    float *sched_y = nullptr;     // [64] device
     // eviction: the state parked in host memory while the device memory is released
     // (one pinned block, kept after a restore so that the next eviction reuses it)
     bool evicted = false;
@@ -105,7 +104,8 @@ struct maxflow_ctx {
 
 // exported by mlp.cu (C linkage)
 extern "C" {
-int mlp_forward_device(maxflow_mlp *m, const float *x_dev, int32_t rows, float *y_dev, cudaStream_t st);
+int mlp_params_device(maxflow_mlp *m, const float **p);
+int mlp_hidden(const maxflow_mlp *m);
 int mlp_n_out(const maxflow_mlp *m);
 int mlp_n_in(const maxflow_mlp *m);
 }
@@ -174,6 +174,12 @@ int rc_cuda(cudaError_t e) { return e == cudaSuccess ? MAXFLOW_OK : MAXFLOW_ERR_
         if (_rc != MAXFLOW_OK) return _rc;    \
     } while (0)
 
+// KERNEL_CYCLES by the average degree (Sec. 6.1).
+int32_t avg_cycles(const maxflow_ctx *c)
+{
+    return (int32_t)std::max<int64_t>(1, (c->st.m_edges + c->n - 1) / c->n);
+}
+
 MfParams base_params(maxflow_ctx *c)
 {
     MfParams p{};
@@ -187,6 +193,7 @@ MfParams base_params(maxflow_ctx *c)
     p.sink = c->t;
     p.source = c->s;
     p.kernel_cycles = c->kernel_cycles;
+    p.avg_cycles = avg_cycles(c);
     p.rounds = c->rounds;
     p.small_deg = c->small_deg;
     p.hub_deg = c->hub_deg;
@@ -452,7 +459,7 @@ void choose_grid(maxflow_ctx *c)
 // and layered graphs), where the rounds are many and short and a warp's
 // parallel scan of a 5-8 slot row beats one thread's; then warps up to 512
 // slots, 4-warp groups up to a quarter of the snapshot buffer, CTAs above; BFS
-// work items for rows of more than 256 slots.
+// work items for rows of more than 128 slots.
 void default_split(maxflow_ctx *c)
 {
     const int64_t m = c->st.m_edges;
@@ -671,15 +678,21 @@ int check_host_batch(maxflow_ctx *c, const maxflow_batch *b)
 }
 
 // Apply (and optionally solve) a batch.
-int do_batch(maxflow_ctx *c, const maxflow_batch *b, int mode)
+int do_batch(maxflow_ctx *c, const maxflow_batch *b, int mode, const MfNet *net = nullptr)
 {
     c->acc_ms = 0;
+    c->rep->action = -1;
     if (!b || b->count < 0) return MAXFLOW_ERR_INVALID;
     if (b->count > 0 && (!b->u || !b->v || !b->new_cap)) return MAXFLOW_ERR_INVALID;
     if (!b->on_device) MF_TRY(check_host_batch(c, b));
     MF_TRY(ensure_batch(c, b->count));
     MfParams p = base_params(c);
     p.mode = mode;
+    if (net) {
+        p.net = *net;
+        p.rounds = p.cycle_div = p.fix_steep = 0;      // until the choice
+        p.kernel_cycles = p.avg_cycles;
+    }
     p.bcount = b->count;
     if (b->count > 0) {
         if (b->on_device) {
@@ -943,8 +956,7 @@ int maxflow_init(maxflow_ctx **out, const maxflow_graph *g, int32_t s, int32_t t
     }
     if (rc == MAXFLOW_OK) {
         c->feat = dalloc_n<float>(c, MF_FEATURES);
-        c->sched_y = dalloc_n<float>(c, 64);
-        if (!c->feat || !c->sched_y) rc = MAXFLOW_ERR_OOM;
+        if (!c->feat) rc = MAXFLOW_ERR_OOM;
     }
     if (rc != MAXFLOW_OK) {
         maxflow_destroy(c);
@@ -1063,8 +1075,7 @@ int maxflow_trace_work(maxflow_ctx *c, int64_t *slots, int32_t *info, double *ct
 int maxflow_set_kernel_cycles(maxflow_ctx *c, int32_t k)
 {
     if (!c || k < 0) return MAXFLOW_ERR_INVALID;
-    int64_t m = c->st.m_edges;
-    c->kernel_cycles = k > 0 ? k : (int32_t)std::max<int64_t>(1, (m + c->n - 1) / c->n);
+    c->kernel_cycles = k > 0 ? k : avg_cycles(c);
     c->st.kernel_cycles = c->kernel_cycles;
     return MAXFLOW_OK;
 }
@@ -1073,26 +1084,21 @@ int maxflow_set_kernel_cycles(maxflow_ctx *c, int32_t k)
 
 namespace {
 
-struct SchedAction {
-    int32_t mode;      // 0: incremental (Alg. 5), 1: apply the batch, then re-solve from zero flow (Alg. 1)
-    int32_t rounds;    // discharge rounds per global relabel (0: adaptive)
-    int32_t cycles;    // KERNEL_CYCLES (0: the average-degree heuristic of Sec. 6.1)
-    int32_t cycle_div; // > 0: rows of d slots get max(cycles, d / cycle_div) cycles
-    int32_t fix;       // 1: remove-invalid-edges (Alg. 3) after each iteration's discharge
-};
-
-// Index 0 is the library's default schedule, 5 the paper's fixed one (one
-// round, KERNEL_CYCLES = average degree, Alg. 3 after every discharge) and 18
-// the paper's static re-solve.
-const SchedAction kActions[] = {
-    {0, 0, 0, 0, 0},   {0, 0, 0, 256, 0}, {0, 0, 4, 0, 0},   {0, 0, 64, 0, 0},  {0, 0, 64, 256, 0},
-    {0, 1, 0, 0, 1},   {0, 1, 16, 0, 0},  {0, 1, 64, 0, 0},  {0, 4, 4, 0, 0},   {0, 4, 16, 0, 0},
-    {0, 4, 64, 0, 0},  {0, 16, 4, 0, 0},  {0, 16, 16, 0, 0}, {0, 16, 64, 0, 0}, {0, 64, 16, 0, 0},
-    {0, 64, 64, 0, 0}, {1, 0, 0, 0, 0},   {1, 0, 64, 0, 0},  {1, 1, 0, 0, 1},   {1, 16, 16, 0, 0},
-};
+const MfAction kActions[] = {MF_ACTIONS};
 constexpr int kNumActions = (int)(sizeof(kActions) / sizeof(kActions[0]));
 
 float lg(double x) { return (float)std::log2(1.0 + (x > 0 ? x : 0)); }
+
+// Features 9..14, known on the host.
+void host_features(const maxflow_ctx *c, float *x)
+{
+    x[0] = lg((double)c->inc_iters) / 8.f;
+    x[1] = lg(c->inc_ms * 1000.0) / 16.f;
+    x[2] = lg((double)c->inc_active_first) / 20.f;
+    x[3] = lg((double)c->init_iters) / 8.f;
+    x[4] = lg(c->init_ms * 1000.0) / 16.f;
+    x[5] = lg((double)c->inc_levels) / 12.f;
+}
 
 // Stage the batch on the device (copying a host batch) and compute its features.
 int stage_and_features(maxflow_ctx *c, const maxflow_batch *b, maxflow_batch *dev_view)
@@ -1120,21 +1126,15 @@ int stage_and_features(maxflow_ctx *c, const maxflow_batch *b, maxflow_batch *de
     f.t = c->t;
     f.m = c->st.m_edges;
     f.mean_cap = c->mean_cap;
-    f.host[0] = lg((double)c->inc_iters) / 8.f;
-    f.host[1] = lg(c->inc_ms * 1000.0) / 16.f;
-    f.host[2] = lg((double)c->inc_active_first) / 20.f;
-    f.host[3] = lg((double)c->init_iters) / 8.f;
-    f.host[4] = lg(c->init_ms * 1000.0) / 16.f;
-    f.host[5] = lg((double)c->inc_levels) / 12.f;
+    host_features(c, f.host);
     return counted(mf_features(f, c->feat, (void *)c->stream), 1);
 }
 
 int run_action(maxflow_ctx *c, const maxflow_batch *dev_batch, int a)
 {
-    const SchedAction &A = kActions[a];
+    const MfAction &A = kActions[a];
     const int32_t keep_k = c->kernel_cycles, keep_r = c->rounds, keep_div = c->cycle_div, keep_fix = c->opt.fix_steep;
-    int64_t m = c->st.m_edges;
-    c->kernel_cycles = A.cycles > 0 ? A.cycles : (int32_t)std::max<int64_t>(1, (m + c->n - 1) / c->n);
+    c->kernel_cycles = A.cycles > 0 ? A.cycles : avg_cycles(c);
     c->rounds = A.rounds;
     c->cycle_div = A.cycle_div;
     c->opt.fix_steep = A.fix;
@@ -1206,17 +1206,20 @@ int maxflow_update_scheduled(maxflow_ctx *c, const maxflow_batch *b, maxflow_mlp
     if (mlp_n_in(m) != MF_FEATURES || mlp_n_out(m) != kNumActions) return MAXFLOW_ERR_INVALID;
     DeviceGuard dg(c->device);
     if (!dg.ok) return MAXFLOW_ERR_CUDA;
-    maxflow_batch view;
-    MF_TRY(stage_and_features(c, b, &view));
-    MF_TRY(mlp_forward_device(m, c->feat, 1, c->sched_y, c->stream));
-    float y[64];
-    MF_TRY(rc_cuda(cudaMemcpyAsync(y, c->sched_y, sizeof(float) * kNumActions, cudaMemcpyDeviceToHost, c->stream)));
-    MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
-    int best = 0;
-    for (int i = 1; i < kNumActions; ++i)
-        if (y[i] < y[best]) best = i;
+    if (mlp_hidden(m) > MF_NET_HIDDEN) return MAXFLOW_ERR_INVALID;
+    MfNet net{};
+    MF_TRY(mlp_params_device(m, &net.p));
+    net.hidden = mlp_hidden(m);
+    net.n_out = kNumActions;
+    net.m = c->st.m_edges;
+    net.mean_cap = c->mean_cap;
+    host_features(c, net.host);
+    const int rc = do_batch(c, b, MF_M_APPLY | MF_M_SOLVE | MF_M_SCHED, &net);
+    const int best = c->rep->action;
+    if (best < 0 || best >= kNumActions) return rc;          // refused before the choice
     if (action_out) *action_out = best;
-    return run_action(c, &view, best);
+    if (rc == MAXFLOW_OK && kActions[best].mode == 0) note_incremental(c);
+    return rc;
 }
 
 int maxflow_set_tuning(maxflow_ctx *c, int32_t thread_max_slots, int32_t warp_max_slots, int32_t bfs_item_min_slots)
@@ -1488,7 +1491,7 @@ static void release_device(maxflow_ctx *c)
     c->sc = MfScratch{};
     c->ctrl = nullptr;
     c->dbuf = nullptr;
-    c->feat = c->sched_y = nullptr;
+    c->feat = nullptr;
     c->x_cf = c->x_cf2 = c->x_h = nullptr;
     c->x_e = nullptr;
     c->multi_plist = nullptr;
@@ -1550,8 +1553,7 @@ int maxflow_restore(maxflow_ctx *c)
         c->ctrl = (MfCtrl *)dalloc(c, sizeof(MfCtrl));
         c->dbuf = dalloc_n<long long>(c, 16);
         c->feat = dalloc_n<float>(c, MF_FEATURES);
-        c->sched_y = dalloc_n<float>(c, 64);
-        if (!c->g.h || !c->g.e || !c->ctrl || !c->dbuf || !c->feat || !c->sched_y) rc = MAXFLOW_ERR_OOM;
+        if (!c->g.h || !c->g.e || !c->ctrl || !c->dbuf || !c->feat) rc = MAXFLOW_ERR_OOM;
     }
     if (rc == MAXFLOW_OK)
         rc = counted(mf_launch_aux(MF_AUX_PCAP, base_params(c), (void *)c->stream, nullptr, nullptr), 1);
@@ -1783,9 +1785,8 @@ int maxflow_clone(maxflow_ctx *src, maxflow_ctx **out)
         c->ctrl = (MfCtrl *)dalloc(c, sizeof(MfCtrl));
         c->dbuf = dalloc_n<long long>(c, 16);
         c->feat = dalloc_n<float>(c, MF_FEATURES);
-        c->sched_y = dalloc_n<float>(c, 64);
         if (!c->g.off || !c->g.deg || !c->g.bdeg || !c->g.dst || !c->g.cf || !c->g.cap || !c->g.rev || !c->g.pcap ||
-            !c->g.h || !c->g.e || !c->sc.bitem || !c->sc.bdefer || !c->ctrl || !c->dbuf || !c->feat || !c->sched_y)
+            !c->g.h || !c->g.e || !c->sc.bitem || !c->sc.bdefer || !c->ctrl || !c->dbuf || !c->feat)
             rc = MAXFLOW_ERR_OOM;
     }
     if (rc == MAXFLOW_OK) rc = alloc_vertex_scratch(c);

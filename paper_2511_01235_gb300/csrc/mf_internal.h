@@ -78,6 +78,7 @@
 #define MF_M_SAT_SINK 64          // static init also saturates every edge into the sink (Sec. 5.2.2 static push-pull)
 #define MF_M_NO_SRC_SAT 128       // static init leaves the source edges alone (the pull-only static solve)
 #define MF_M_CUT 256              // after the batch: record the sides of the last cut, saturate the edges S -> T
+#define MF_M_SCHED 1024            // after the batch: the network picks the schedule (MfParams.net)
 #define MF_M_NO_VALUE 512         // skip the value phase (the side-limited push / pull parts)
 
 struct alignas(128) MfLine {
@@ -103,6 +104,8 @@ enum MfLineId {
     L_AUX = L_WL + MF_NBIN,       // [MF_NBIN] next-round worklist entries per bin
     L_FIX = L_AUX + MF_NBIN,      // [2] remove-invalid lists (warp / CTA)
     L_ACT = L_FIX + 2,    // active vertices (only when the worklist is a pass of its own)
+    L_FEAT,               // learned schedule: updates touching s, touching t, deleting
+    L_FCAP,               // learned schedule: 64-bit sum of the batch's capacities; w[2]: 1 + the action it picked
     L_MISC,               // w[0] new pairs, w[1] a row without room, w[2] dedup entries, w[3] error (MF_E_*)
     L_LAB,                // 64-bit: labelled vertices << 32 | their slots
     L_TOTAL,              // 64-bit: used slots of the whole graph (summed by the BFS roots pass)
@@ -140,6 +143,7 @@ struct MfDesc {
     int ins_n, hused_n;           // batch: new pairs, dedup table entries
     int round;                    // discharge round within the iteration
     int dis_more;                 // another discharge round follows
+    int resolve;                  // the picked action re-solves from zero flow
     int near;                     // this launch may cut its global relabels short and walk the excess down
     int cut;                      // ... and this iteration's was cut short
     int fix_n[2];                 // vertices for remove-invalid-edges (warp list, CTA list); grows over the rounds
@@ -185,6 +189,7 @@ enum MfStat {
 struct MfReport {
     int err;              // MF_E_*
     int status;           // MF_ST_*
+    int action, pad;      // the action the network picked (MF_M_SCHED)
     long long iters, value;
     long long bfs_levels, active_total, active_first;
     long long cut_slots, used_slots;      // slots of the vertices the last BFS labelled; of all
@@ -223,6 +228,34 @@ struct MfCtrl {
 };
 // The part the host clears after a launch that ended in a barrier that gave up.
 #define MF_CTRL_SYNC_BYTES (sizeof(MfLine) + sizeof(MfSet) * 3)
+
+// A schedule (action) of the learned scheduler; the table is fixed.
+struct MfAction {
+    int32_t mode;      // 0: incremental (Alg. 5), 1: apply the batch, then re-solve from zero flow (Alg. 1)
+    int32_t rounds;    // discharge rounds per global relabel (0: adaptive)
+    int32_t cycles;    // KERNEL_CYCLES (0: the average-degree heuristic of Sec. 6.1)
+    int32_t cycle_div; // > 0: rows of d slots get max(cycles, d / cycle_div) cycles
+    int32_t fix;       // 1: remove-invalid-edges (Alg. 3) after each iteration's discharge
+};
+// Index 0 is the library's default schedule, 5 the paper's fixed one (one
+// round, KERNEL_CYCLES = average degree, Alg. 3 after every discharge) and 18
+// the paper's static re-solve.
+#define MF_ACTIONS                                                                                      \
+    {0, 0, 0, 0, 0},   {0, 0, 0, 256, 0}, {0, 0, 4, 0, 0},   {0, 0, 64, 0, 0},  {0, 0, 64, 256, 0},     \
+    {0, 1, 0, 0, 1},   {0, 1, 16, 0, 0},  {0, 1, 64, 0, 0},  {0, 4, 4, 0, 0},   {0, 4, 16, 0, 0},       \
+    {0, 4, 64, 0, 0},  {0, 16, 4, 0, 0},  {0, 16, 16, 0, 0}, {0, 16, 64, 0, 0}, {0, 64, 16, 0, 0},      \
+    {0, 64, 64, 0, 0}, {1, 0, 0, 0, 0},   {1, 0, 64, 0, 0},  {1, 1, 0, 0, 1},   {1, 16, 16, 0, 0},
+
+// The network that picks one, and what it looks at besides the batch.
+#define MF_FEATURES 16
+#define MF_NET_HIDDEN 256
+struct MfNet {
+    const float *p;           // its parameters (mlp.cu's layout); nullptr: none
+    int32_t hidden, n_out;
+    long long m;              // merged directed edges
+    float mean_cap;
+    float host[6];            // features 9..14
+};
 
 struct MfGraph {
     int32_t n;
@@ -296,6 +329,8 @@ struct MfParams {
     long long max_iters;
     unsigned long long time_limit_ns;
     unsigned long long wait_limit_ns;
+    int32_t avg_cycles;       // KERNEL_CYCLES by the average degree
+    MfNet net;                // MF_M_SCHED
     // batch
     int64_t bcount;
     const int32_t *bu, *bv, *bc;
@@ -393,7 +428,6 @@ int mf_rebuild_move(const MfParams &p, void *stream, const long long *noff, int3
                     int32_t *cap, int32_t *rev, int32_t *pcap, long long slot_cap, int2 *items, unsigned *nitems);
 
 // scheduler features of a batch (16 floats)
-#define MF_FEATURES 16
 struct MfFeatIn {
     const int32_t *bu, *bv, *bc;
     long long count;

@@ -264,16 +264,15 @@ int maxflow_mlp_forward(maxflow_mlp *m, const float *x, int32_t rows, float *y)
     return rc;
 }
 
-// Device-side forward for the scheduler (x, y device pointers, no sync).
-int mlp_forward_device(maxflow_mlp *m, const float *x_dev, int32_t rows, float *y_dev, cudaStream_t st)
+// The parameters on the device, for the solver's own forward pass; what was
+// issued on the network's stream (training) is waited for.
+int mlp_params_device(maxflow_mlp *m, const float **p)
 {
-    Layout L{m->n_in, m->H, m->n_out};
-    k_mlp_fwd_bwd<<<rows, threads_for(m), 0, st>>>(L, m->p, x_dev, nullptr, nullptr, 0.f, y_dev, nullptr, nullptr);
-    int rc = ok(cudaGetLastError());
-    if (rc == MAXFLOW_OK) mf_note_launches(1);
-    return rc;
+    *p = m->p;
+    return ok(cudaStreamSynchronize(m->stream));
 }
 
+int mlp_hidden(const maxflow_mlp *m) { return m->H; }
 int mlp_n_out(const maxflow_mlp *m) { return m->n_out; }
 int mlp_n_in(const maxflow_mlp *m) { return m->n_in; }
 

@@ -11,6 +11,15 @@
 // launch.  Every barrier wait is bounded in time: on expiry the CTA records
 // MF_E_WAIT and returns, and the host reports MAXFLOW_ERR_INTERNAL.
 //
+// A solve is bound by its chain of phases, each a few dependent trips to L2
+// (302 clocks; DRAM 824) and a barrier, and not by bytes: most of what follows
+// shortens that chain.  Every CTA takes the decisions between phases itself
+// from the phase's counters (advance); a phase's results are queued on chip and
+// appended with one reservation per CTA (flush_queue); small levels and rounds
+// stay in one cluster (squad); rounds on short rows are one cycle per vertex;
+// and on graphs with a short sink row a relabel ends early and the excess walks
+// down its tree (near iterations).
+//
 // Readings of the paper used here (the same as the CPU oracle's):
 //   - BFS roots are the sink and every vertex other than s, t with e < 0
 //     (Alg. 6), in the static solve too, and h(s) = n always;
@@ -52,17 +61,17 @@ extern __shared__ __align__(16) int mf_stage[];
 __device__ __forceinline__ int vb() { return g_vb; }
 __device__ __forceinline__ int vn() { return g_vn; }
 
-// First work index of this thread in a grid-stride loop (stride vn() *
-// blockDim.x) that spreads a short list over the whole grid: consecutive
-// indices go to different CTAs, so a batch of a few thousand updates keeps
-// every SM's memory pipeline busy instead of crowding onto the first CTAs.
-// spread_warp keeps 32 consecutive indices in one warp (warp-uniform loops).
 // Row kind of a vertex with d used slots: 0 thread, 1 warp, 2 four-warp group, 3 CTA.
 __device__ __forceinline__ int row_bin(int d)
 {
     return d <= P.small_deg ? 0 : (d <= P.hub_deg ? 1 : (d <= P.group_deg ? 2 : 3));
 }
 
+// First work index of this thread in a grid-stride loop (stride vn() *
+// blockDim.x) that spreads a short list over the whole grid: consecutive
+// indices go to different CTAs, so a batch of a few thousand updates keeps
+// every SM's memory pipeline busy instead of crowding onto the first CTAs.
+// spread_warp keeps 32 consecutive indices in one warp (warp-uniform loops).
 __device__ __forceinline__ long long spread_thread() { return (long long)threadIdx.x * vn() + vb(); }
 __device__ __forceinline__ long long spread_warp()
 {
@@ -187,6 +196,10 @@ enum { SQ_SPILL = 1,      // something went onto the grid's lists: long rows, a 
 struct Sh {
     long long sink_e, src_e;          // excess of the sink and the source, added to memory before every barrier
     long long value;                  // this CTA's share of the value
+    unsigned ft_s, ft_t, ft_del;      // learned schedule: this CTA's updates touching s, touching t, deleting
+    long long ft_cap;                 // ... and their capacities' sum
+    float x[MF_FEATURES], h1[MF_NET_HIDDEN], h2[MF_NET_HIDDEN], y[64];   // the network's layers
+    int action;                       // what it picked (-1: nothing yet)
     long long stat[MF_STATS];         // work counters, added to memory at the end of the launch
     unsigned long long lab;           // BFS: vertices labelled this phase << 32 | their slots
     unsigned long long exc, dem;      // near BFS: excess labelled, what the roots can take, this phase
@@ -335,6 +348,86 @@ __device__ __forceinline__ int near_allowed()
     return (long long)ldg_cg(P.g.deg + P.sink) * MF_NEAR_SINK <= (long long)P.g.n ? 1 : 0;
 }
 
+// ---- learned schedule ----
+//
+// The network is asked inside the launch that applies the batch: the phase that
+// validates the batch sums what the features need, the last CTA runs the 16 ->
+// H -> H -> n_out network beside the phase that locates the slots (which takes
+// longer), and behind that phase's barrier every CTA sets its parameters to the
+// picked action's.  As kernels of their own, features, network and the host's
+// read of the choice cost 28 held-out updates of ER, R-MAT and grid graphs 35.7
+// ms against 26.5 with the default schedule; here both take 21 ms.
+
+__constant__ MfAction kActionTable[] = {MF_ACTIONS};
+
+// One thread: the features of the batch (k_features has them too, for the call that returns them).
+__device__ __noinline__ void batch_features()
+{
+    const float B = (float)P.bcount, m = (float)(P.net.m > 0 ? P.net.m : 1), n = (float)P.g.n;
+    const float inv = P.bcount > 0 ? 1.f / B : 0.f;
+    float *x = sh.x;
+    x[0] = log2f(1.f + B) / 20.f;
+    x[1] = fminf(B / m, 1.f);
+    x[2] = log2f(n) / 24.f;
+    x[3] = log2f(1.f + m) / 28.f;
+    x[4] = (m / n) / 16.f;
+    x[5] = (float)(unsigned)sh.cnt[L_FEAT].x * inv;
+    x[6] = (float)(unsigned)sh.cnt[L_FEAT].y * inv;
+    x[7] = (float)(unsigned)sh.cnt[L_FEAT].z * inv;
+    x[8] = P.bcount > 0 && P.net.mean_cap > 0.f
+               ? fminf((float)(long long)cnt64(L_FCAP) * inv / P.net.mean_cap, 4.f) / 4.f : 0.f;
+    for (int k = 0; k < 6; ++k) x[9 + k] = P.net.host[k];
+    x[15] = 1.f;
+}
+
+// Forward pass and choice, by one CTA; 1 + the action goes to the counter set.
+__device__ __noinline__ void pick_action()
+{
+    const int j = threadIdx.x, H = P.net.hidden, no = P.net.n_out;
+    const float *w1 = P.net.p, *b1 = w1 + H * MF_FEATURES, *w2 = b1 + H, *b2 = w2 + H * H, *w3 = b2 + H,
+                *b3 = w3 + no * H;
+    if (j < H) {
+        float a = b1[j];
+        for (int i = 0; i < MF_FEATURES; ++i) a += w1[j * MF_FEATURES + i] * sh.x[i];
+        sh.h1[j] = a > 0.f ? a : 0.f;
+    }
+    __syncthreads();
+    if (j < H) {
+        float a = b2[j];
+        for (int k = 0; k < H; ++k) a += w2[j * H + k] * sh.h1[k];
+        sh.h2[j] = a > 0.f ? a : 0.f;
+    }
+    __syncthreads();
+    if (j < no) {
+        float a = b3[j];
+        for (int k = 0; k < H; ++k) a += w3[j * H + k] * sh.h2[k];
+        sh.y[j] = a;
+    }
+    __syncthreads();
+    if (j == 0) {
+        int best = 0;
+        for (int i = 1; i < no; ++i)
+            if (sh.y[i] < sh.y[best]) best = i;
+        sh.cs->l[L_FCAP].w[2] = (unsigned)(1 + best);
+    }
+}
+
+// One thread of every CTA: the launch goes on with this action.
+__device__ __noinline__ void take_action(int action)
+{
+    const int k = min(max(action, 0), (int)(sizeof(kActionTable) / sizeof(MfAction)) - 1);
+    const MfAction A = kActionTable[k];
+    sh.action = k;
+    P.kernel_cycles = A.cycles > 0 ? A.cycles : P.avg_cycles;
+    P.rounds = A.rounds;
+    P.cycle_div = A.cycle_div;
+    P.fix_steep = A.fix;
+    sh.d.resolve = A.mode;
+    // near_allowed() for these rounds; the sink's row, which the next phase may
+    // already be changing, was read at the launch's start
+    if (A.rounds != 0 || A.fix != 0) sh.d.near = 0;
+}
+
 // Opens an iteration of the loop (its BFS comes next).
 __device__ __forceinline__ void begin_iteration()
 {
@@ -413,7 +506,7 @@ __device__ __forceinline__ int advance_bfs(int &hook)
     st.lvl_slots = st.lvl_cnt = 0;
     // direction of the coming level (Beamer's test): bottom-up once the
     // frontier's slots exceed 1/alpha of the unexplored slots, back to
-    // top-down once it holds fewer than n/beta vertices
+    // top-down once it holds fewer than n/beta vertices.
     int bu = bu_was;
     if (alpha <= 0) bu = 0;
     else if (!bu && fr * alpha > used - vis) bu = 1;
@@ -461,11 +554,13 @@ __device__ __noinline__ void advance(int hook, unsigned long long t)
     case H_APPLY_VALID:
         st.ns_apply += dt;
         d.hused_n = sh.cnt[L_MISC].z;
+        if (P.mode & MF_M_SCHED) batch_features();
         break;
     case H_APPLY_LOCATED:
         st.ns_apply += dt;
         d.ins_n = sh.cnt[L_MISC].x;
         if (sh.cnt[L_MISC].y != 0 && st.err == 0) st.err = MF_E_OVERFLOW;   // a row has no room for its new pairs
+        if (P.mode & MF_M_SCHED) take_action(sh.cnt[L_FCAP].z - 1);
         break;
     case H_APPLY_DELTA:
     case H_NONE:
@@ -601,6 +696,13 @@ __device__ __forceinline__ void arrive()
     } else if (lane == 4) {
         if (sh.exc) atomicAdd((unsigned long long *)sh.cs->l[L_EXC].w, sh.exc);
         sh.exc = 0;
+    } else if (lane == 7) {
+        if (sh.ft_s) atomicAdd(&sh.cs->l[L_FEAT].w[0], sh.ft_s);
+        if (sh.ft_t) atomicAdd(&sh.cs->l[L_FEAT].w[1], sh.ft_t);
+        if (sh.ft_del) atomicAdd(&sh.cs->l[L_FEAT].w[2], sh.ft_del);
+        if (sh.ft_cap) atomicAdd((unsigned long long *)sh.cs->l[L_FCAP].w, (unsigned long long)sh.ft_cap);
+        sh.ft_s = sh.ft_t = sh.ft_del = 0;
+        sh.ft_cap = 0;
     } else if (lane == 6) {
         sh.q_bfs = sh.q_long = sh.q_wn = 0;
         for (int b = 0; b < MF_NBIN; ++b) sh.q_wl[b] = 0;
@@ -787,6 +889,7 @@ __device__ __noinline__ bool finish()
                     c->fstamp = sh.d.fstamp;
                     r->err = st.err;
                     r->status = sh.d.status;
+                    r->action = sh.action;
                     r->value = __ldcg(&c->value);
                     r->iters = st.iters;
                     r->bfs_levels = st.bfs_levels;
@@ -972,6 +1075,9 @@ __device__ __noinline__ void phase_apply_validate()
     const int bits = P.sc.hash_bits;
     const unsigned mask = (1u << bits) - 1u;
     const int lane = threadIdx.x & 31;
+    const bool sched = (P.mode & MF_M_SCHED) != 0;
+    unsigned fs = 0, ft = 0, fz = 0;
+    long long fcap = 0;
     // warp-uniform loop: the positions taken in the table are appended with one atomic per warp
     for (long long base = spread_warp() - lane; base < P.bcount; base += (long long)vn() * blockDim.x) {
         const long long i = base + lane;
@@ -979,7 +1085,14 @@ __device__ __noinline__ void phase_apply_validate()
         unsigned pos = 0;
         int u, v, c;
         if (i < P.bcount) {
-            if (!batch_entry(i, u, v, c)) {
+            const bool fine = batch_entry(i, u, v, c);
+            if (sched) {
+                fs += u == P.source || v == P.source;
+                ft += u == P.sink || v == P.sink;
+                fz += c == 0;
+                fcap += c;
+            }
+            if (!fine) {
                 atomicCAS(&cs->l[L_MISC].w[3], 0u, (unsigned)MF_E_INVALID);
             } else if (u != v) {
                 unsigned long long key = ((unsigned long long)(unsigned)u << 32) | (unsigned)v;
@@ -996,6 +1109,18 @@ __device__ __noinline__ void phase_apply_validate()
             }
         }
         warp_append(&cs->l[L_MISC].w[2], P.sc.hused, fresh, (int)pos);   // positions to clear afterwards
+    }
+    if (sched) {
+        fs = __reduce_add_sync(0xffffffffu, fs);
+        ft = __reduce_add_sync(0xffffffffu, ft);
+        fz = __reduce_add_sync(0xffffffffu, fz);
+        fcap = warp_sum_ll(fcap);
+        if (lane == 0) {
+            if (fs) atomicAdd(&sh.ft_s, fs);
+            if (ft) atomicAdd(&sh.ft_t, ft);
+            if (fz) atomicAdd(&sh.ft_del, fz);
+            if (fcap) add_shared(sh.ft_cap, fcap);
+        }
     }
 }
 
@@ -3500,7 +3625,9 @@ __device__ __noinline__ bool solve_instance()
     if (threadIdx.x < MF_STATS) sh.stat[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         MfCtrl *c = P.ctrl;
-        sh.sink_e = sh.src_e = sh.value = 0;
+        sh.sink_e = sh.src_e = sh.value = sh.ft_cap = 0;
+        sh.ft_s = sh.ft_t = sh.ft_del = 0;
+        sh.action = -1;
         sh.lab = sh.exc = sh.dem = 0;
         sh.q_bfs = sh.q_long = sh.q_wn = 0;
         for (int b = 0; b < MF_NBIN; ++b) sh.q_wl[b] = 0;
@@ -3560,6 +3687,7 @@ __device__ __noinline__ bool solve_instance()
             phase_apply_cleanup(false);
             return finish();
         }
+        if ((P.mode & MF_M_SCHED) && vb() == vn() - 1) pick_action();
         phase_apply_locate();
         if (!grid_sync(H_APPLY_LOCATED)) return false;
         if (sh.d.status != MF_ST_RUNNING) {
@@ -3572,7 +3700,14 @@ __device__ __noinline__ bool solve_instance()
         if (!grid_sync(H_APPLY_DELTA)) return false;
         // the source step reads the final residuals; the tables are cleared beside it
         phase_apply_cleanup(false);
-        if (!(P.mode & MF_M_SKIP_SOURCE_SAT)) phase_resaturate();
+        if (!(P.mode & MF_M_SKIP_SOURCE_SAT) && !sh.d.resolve) phase_resaturate();
+        if (sh.d.resolve) {
+            // the picked action re-solves the changed graph from zero flow
+            if (!grid_sync(H_NONE)) return false;
+            phase_static_reset();
+            if (!grid_sync(H_NONE)) return false;
+            phase_saturate_source();
+        }
         // straight on to the loop: this barrier opens its first iteration
         opened = loops && !(P.mode & MF_M_CUT);
         if (!opened && !(P.mode & MF_M_CUT) && !loops) return finish();
