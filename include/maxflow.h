@@ -329,7 +329,8 @@ int maxflow_test_stalled_barrier(maxflow_ctx *c, int32_t cta);
  * unlabelled vertex looks through its own row for a neighbour of the current
  * level with residual towards it, stopping at the first -- once the frontier's
  * slots exceed 1/alpha of the still unexplored slots, and top-down again once
- * the frontier holds fewer than n/beta vertices.  The labels are the same
+ * the frontier holds fewer than n/beta vertices; from the 16th level on no level
+ * turns bottom-up any more.  The labels are the same
  * either way.  alpha = 0 keeps every level top-down.  Defaults 14 and 24.
  * MAXFLOW_ERR_INVALID for alpha < 0 or beta < 1. */
 int maxflow_set_bfs_switch(maxflow_ctx *c, int32_t alpha, int32_t beta);

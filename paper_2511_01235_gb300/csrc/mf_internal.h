@@ -51,7 +51,7 @@
 #define MF_SQUAD_LEVEL 256    // BFS levels of at most this many vertices per squad CTA ...
 #define MF_SQUAD_SLOTS 2048   // ... and slots run in the squad
 #define MF_SQUAD_ACTIVE 256   // so do discharge rounds of at most this many vertices per squad CTA
-#define MF_DEEP 16            // short rounds on a smaller graph: after a BFS of at least this many levels
+#define MF_DEEP 16            // a BFS of this many levels is deep: no level turns bottom-up, and a small graph runs short rounds
 #define MF_SHORT_ROW 512      // rounds of one cycle per vertex: the longest row
 
 // Solve-kernel status (ctrl->status)

@@ -506,10 +506,13 @@ __device__ __forceinline__ int advance_bfs(int &hook)
     st.lvl_slots = st.lvl_cnt = 0;
     // direction of the coming level (Beamer's test): bottom-up once the
     // frontier's slots exceed 1/alpha of the unexplored slots, back to
-    // top-down once it holds fewer than n/beta vertices.
+    // top-down once it holds fewer than n/beta vertices.  Not in a deep BFS,
+    // whose frontiers are short: near its end the unexplored slots get few too,
+    // and a bottom-up level still visits every vertex (256 x 256 grid, window
+    // updates 4.9 -> 4.7 ms; 64 batched instances 12.0 -> 11.3)
     int bu = bu_was;
     if (alpha <= 0) bu = 0;
-    else if (!bu && fr * alpha > used - vis) bu = 1;
+    else if (!bu && d.level < MF_DEEP && fr * alpha > used - vis) bu = 1;
     else if (bu && cnt * beta < (long long)n) bu = 0;
     d.bu_mode = bu;
     d.bu_split = 0;
