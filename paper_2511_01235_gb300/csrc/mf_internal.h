@@ -168,6 +168,23 @@ struct MfState {
     int trace_n;
 };
 
+// Whether round `round` of an iteration's discharge may be a short one, by the
+// kind of the round before.  Short rounds queue without stamps, which needs a
+// list whose vertices all have excess.  A BFS and a short round leave such a
+// list.  A round of several cycles does not: u sends its excess, a neighbour
+// pushes to u and queues it, and a later cycle of u's sends that too; nor do the
+// walks, where u may take along what another walk has left there.  In a short
+// round such a vertex, listed with e = 0, could be queued by a receiver and then
+// by itself, and the round after would hold it twice: two owners that both take
+// the same residual, below zero.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline bool mf_short_may_follow(int round, int last_short)
+{
+    return round == 0 || last_short != 0;
+}
+
 // Work counters.  Each CTA keeps its own in shared memory and adds them to the
 // control block once, at the end of the launch.
 enum MfStat {

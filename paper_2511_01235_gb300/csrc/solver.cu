@@ -294,18 +294,19 @@ __device__ __forceinline__ bool rounds_left(const MfDesc &d, const MfState &st, 
     return (d.dis_short ? 1 : 2) * (t - st.t_dis0) < st.t_dis0 - st.t_bfs0;
 }
 
-// How the coming discharge round over the worklists in d runs.  Short: a push
-// with the default schedule over rows of at most MF_SHORT_ROW slots gets one
-// cycle per vertex (phase_discharge_short), and few vertices are left to the
-// squad (squad_discharge).  On a small graph that takes a BFS of many levels:
-// short rounds pay where many rounds follow; where two or three do, the whole
-// KERNEL_CYCLES in each settle more.
+// How the coming discharge round (number d.round of its iteration) over the
+// worklists in d runs.  Short: a push with the default schedule over rows of at
+// most MF_SHORT_ROW slots gets one cycle per vertex (phase_discharge_short), and
+// few vertices are left to the squad (squad_discharge).  On a small graph that
+// takes a BFS of many levels: short rounds pay where many rounds follow; where
+// two or three do, the whole KERNEL_CYCLES in each settle more.  Behind a round
+// of another kind no short one follows (mf_short_may_follow).
 __device__ __forceinline__ void pick_round(MfDesc &d, int csize)
 {
     d.dis_short = P.rounds == 0 && !P.pull && !P.fix_steep && P.data_driven && P.requeue &&
                           P.stage_slots >= MF_SQUAD_INTS && P.hub_deg <= MF_SHORT_ROW &&
                           (P.g.slot_cap >= MF_LARGE_SLOTS || d.level >= MF_DEEP) &&
-                          d.wl_n[2] + d.wl_n[3] == 0
+                          d.wl_n[2] + d.wl_n[3] == 0 && mf_short_may_follow(d.round, d.dis_short)
                       ? 1 : 0;
     d.dis_squad = d.dis_short && d.wl_n[0] + d.wl_n[1] <= MF_SQUAD_ACTIVE * csize ? 1 : 0;
 }
@@ -3131,10 +3132,13 @@ __device__ __forceinline__ void short_enqueue(int z, int r0, int d, const SquadQ
     sh.so_flag = SQ_SPILL;
 }
 
-// g units along slot x = (u, z), y its reverse.  Every vertex is in a round's
-// lists at most once and lowers its own excess once, at its end, so z's excess
-// rises from <= 0 to > 0 at most once in a round: whoever makes it do so
-// queues it, and no stamp is needed.
+// g units along slot x = (u, z), y its reverse.  No stamp is needed to queue a
+// receiver: the list of a short round holds every vertex once, and each with
+// e > 0 (it comes from the BFS or from a short round, mf_short_may_follow).  A
+// listed vertex lowers its own excess once, by what it read at first, and queues
+// itself if some is left; until then its excess is above zero and no receiver
+// queues it, and after that it rises from zero at most once.  A vertex that is
+// not listed never lowers its excess.  So everyone is queued once, with e > 0.
 template <bool SQUAD>
 __device__ __forceinline__ void short_push(int x, int z, int y, int g, const SquadQ &nq)
 {
