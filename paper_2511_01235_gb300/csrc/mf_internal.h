@@ -51,6 +51,7 @@
 #define MF_SQUAD_LEVEL 256    // BFS levels of at most this many vertices per squad CTA ...
 #define MF_SQUAD_SLOTS 2048   // ... and slots run in the squad
 #define MF_SQUAD_ACTIVE 256   // so do discharge rounds of at most this many vertices per squad CTA
+#define MF_HANDOVER 2         // copies of the state that the first CTA hands over at a barrier (MfCtrl)
 #define MF_DEEP 16            // a BFS of this many levels is deep: no level turns bottom-up, and a small graph runs short rounds
 #define MF_SHORT_ROW 512      // rounds of one cycle per vertex: the longest row
 
@@ -237,9 +238,13 @@ struct MfCtrl {
     long long stat[MF_STATS];
     MfLine bar;           // w[0]: arrivals in this launch (the first CTA leaves it at zero)
     MfSet set[3];
-    // the first CTA's state for the others, after its squad ran phases alone
-    MfDesc jd;
-    MfState js;
+    // the first CTA's state for the others, after its squad ran phases alone.
+    // Barrier k uses copy k mod MF_HANDOVER: a CTA may still be reading copy k
+    // when the first one, which only needs its own cluster to get there, writes
+    // the copy of barrier k + 1; it writes copy k again only for barrier k + 2,
+    // after every CTA has arrived at k + 1 and so has read it.
+    MfDesc jd[MF_HANDOVER];
+    MfState js[MF_HANDOVER];
     // per phase (mod 3) and CTA: finish time, slots scanned
     unsigned fin[3][MF_MAX_CTAS], scanned[3][MF_MAX_CTAS];
 };

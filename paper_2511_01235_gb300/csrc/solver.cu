@@ -803,7 +803,8 @@ __device__ __forceinline__ void squad_tell(int par, const SquadSum &mine)
 // from the counter set by itself (advance), where one thread running that
 // behind the barrier for all held them up for another 3 us.  A solve that is
 // one cluster uses the cluster's barrier.  With take_state, every CTA takes the
-// first one's state (its squad ran phases alone) before working out the next.
+// first one's state (its squad ran phases alone) before working out the next;
+// two such barriers may follow one another, so the state has two copies (MfCtrl).
 __device__ __noinline__ bool grid_sync(int hook, bool take_state = false)
 {
     MfCtrl *c = P.ctrl;
@@ -812,8 +813,8 @@ __device__ __noinline__ bool grid_sync(int hook, bool take_state = false)
     const bool one = sh.one_cluster != 0;
     if (threadIdx.x < 32) {
         if (take_state && vb() == 0) {
-            words_out((int *)&c->jd, (const int *)&sh.d, (int)(sizeof(MfDesc) / 4));
-            words_out((int *)&c->js, (const int *)&sh.hs, (int)(sizeof(MfState) / 4));
+            words_out((int *)&c->jd[k % MF_HANDOVER], (const int *)&sh.d, (int)(sizeof(MfDesc) / 4));
+            words_out((int *)&c->js[k % MF_HANDOVER], (const int *)&sh.hs, (int)(sizeof(MfState) / 4));
         }
         arrive();
     }
@@ -833,8 +834,8 @@ __device__ __noinline__ bool grid_sync(int hook, bool take_state = false)
                 if (vb() == 0) __stcg(reinterpret_cast<int4 *>(&c->set[(k + 2u) % 3u].l[lane]), make_int4(0, 0, 0, 0));
             }
             if (take_state && vb() != 0) {
-                words_in((int *)&sh.d, (const int *)&c->jd, (int)(sizeof(MfDesc) / 4));
-                words_in((int *)&sh.hs, (const int *)&c->js, (int)(sizeof(MfState) / 4));
+                words_in((int *)&sh.d, (const int *)&c->jd[k % MF_HANDOVER], (int)(sizeof(MfDesc) / 4));
+                words_in((int *)&sh.hs, (const int *)&c->js[k % MF_HANDOVER], (int)(sizeof(MfState) / 4));
             }
             __syncwarp();
             if (lane == 0) advance(hook, cnt64(L_TIME));
