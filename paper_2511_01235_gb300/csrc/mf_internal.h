@@ -59,9 +59,9 @@
 #define MF_ST_RUNNING 0
 #define MF_ST_CONVERGED 1
 #define MF_ST_CAP 2           // iteration or time cap
-#define MF_ST_ERROR 3         // ctrl->err holds the error
+#define MF_ST_ERROR 3         // MfReport.err holds the error
 
-// ctrl->err values
+// MfReport.err values
 #define MF_E_NONE 0
 #define MF_E_INVALID 1        // batch entry out of range / negative capacity
 #define MF_E_OVERFLOW 2       // insertion needs more slack than a row has
@@ -232,11 +232,11 @@ struct MfReport {
 
 struct MfCtrl {
     MfReport rep;         // of launches without pinned memory to report to
-    MfLine err;           // w[0]: a barrier gave up (MF_E_WAIT)
     int qstamp, fstamp;   // carried over from launch to launch
     long long value;
     long long stat[MF_STATS];
-    MfLine bar;           // w[0]: arrivals in this launch (the first CTA leaves it at zero)
+    MfLine bar;           // w[0]: arrivals in this launch (the first CTA leaves it at zero);
+                          // w[1]: a CTA of the first cluster gave up at a barrier
     MfSet set[3];
     // the first CTA's state for the others, after its squad ran phases alone.
     // Barrier k uses copy k mod MF_HANDOVER: a CTA may still be reading copy k

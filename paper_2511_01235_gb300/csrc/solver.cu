@@ -8,8 +8,11 @@
 // (Alg. 3, when enabled: off by default) }, then the value formula of Alg. 5.
 // Phases are separated by a grid barrier instead of kernel launches, so the
 // termination test never leaves the device and a small update costs one
-// launch.  Every barrier wait is bounded in time: on expiry the CTA records
-// MF_E_WAIT and returns, and the host reports MAXFLOW_ERR_INTERNAL.
+// launch.  Every wait at a barrier in memory (grid, group) is bounded in time: on
+// expiry the CTA records MF_E_WAIT and returns, and the host reports
+// MAXFLOW_ERR_INTERNAL.  A cluster's barrier is the hardware's and has no limit
+// of its own; it ends because each CTA of the cluster reaches it after bounded
+// work and bounded waits, or has left the kernel, which counts as having arrived.
 //
 // A solve is bound by its chain of phases, each a few dependent trips to L2
 // (302 clocks; DRAM 824) and a barrier, and not by bytes: most of what follows
@@ -738,7 +741,7 @@ __device__ __forceinline__ bool wait_all()
             if (t0 == 0) {
                 t0 = now;
             } else if (now - t0 > P.wait_limit_ns) {
-                atomicExch(&c->err.w[0], (unsigned)MF_E_WAIT);
+                if (vb() < sh.csize) atomicExch(&c->bar.w[1], 1u);      // squad_entered
                 *(volatile int *)&P.rep->err = MF_E_WAIT;
                 return false;
             }
@@ -777,6 +780,32 @@ __device__ __forceinline__ void squad_sync()
 {
     if (sh.csize > 1) cluster_sync();
     else __syncthreads();
+}
+
+// Before the squad runs phases alone, all its CTAs make sure that none has given
+// up at the barrier before (it may have, and left the kernel, just as the others
+// saw that barrier complete): they write into one another's shared memory, which
+// has to be there.  A CTA of the first cluster that gives up leaves a mark in
+// memory and passes the cluster's barrier once more before it leaves
+// (grid_sync); the others read the mark behind that barrier, which they pass
+// here, and then all of them leave.  Only CTAs of this cluster set the mark, so
+// nobody can set it between two reads.  squad_enter and squad_entered are the
+// barrier's two halves; what the squad reads first is loaded between them.
+__device__ __forceinline__ void squad_enter()
+{
+    if (sh.csize > 1 && !sh.one_cluster) {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    }
+}
+__device__ __forceinline__ bool squad_entered()
+{
+    if (sh.csize > 1 && !sh.one_cluster) {
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (threadIdx.x == 0) sh.ok = __ldcg(&P.ctrl->bar.w[1]) == 0 ? 1 : 0;
+        __syncthreads();
+    }
+    return sh.ok != 0;
 }
 
 // sq[par][my rank] in every CTA of the squad = mine, by one warp; visible behind squad_sync.
@@ -848,6 +877,7 @@ __device__ __noinline__ bool grid_sync(int hook, bool take_state = false)
     }
     __syncthreads();
     if (vb() == 0 && (threadIdx.x >> 5) == (blockDim.x >> 5) - 1 && sh.ok) write_trace(k);
+    if (sh.ok == 0 && sh.csize > 1 && !one && vb() < sh.csize) cluster_sync();    // squad_entered
     return sh.ok != 0;
 }
 
@@ -2984,13 +3014,15 @@ __device__ __forceinline__ void squad_visit(const int (&x)[BR], const bool (&val
 
 // Top-down BFS levels, one after another, while they stay small.  The last one
 // leaves its results where a level of the grid would, and the grid barrier that
-// follows takes them up as that level's (with the squad's state).
-__device__ __noinline__ void squad_bfs()
+// follows takes them up as that level's (with the squad's state).  False: a CTA of
+// the squad is gone, and the caller leaves the kernel too.
+__device__ __noinline__ bool squad_bfs()
 {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nwarps = nt >> 5;
     const int csize = sh.csize, rank = sh.crank;
     const unsigned long long t0 = gtimer();
     int cur = 0, cnt;
+    squad_enter();
     {
         // entry i of the frontier belongs to squad CTA i mod csize
         const int lo = sh.d.lvl_lo, all = sh.d.lvl_hi - lo;
@@ -3003,6 +3035,7 @@ __device__ __noinline__ void squad_bfs()
     }
     if (tid == 0) sh.so_cnt = sh.so_long = sh.so_flag = 0;
     __syncthreads();
+    if (!squad_entered()) return false;
     for (;;) {
         const int L = sh.d.level, par = sh.so_par;
         const SquadQ cq = squad_q(cur), nq = squad_q(cur ^ 1);
@@ -3101,7 +3134,7 @@ __device__ __noinline__ void squad_bfs()
             at = sh.d.app_bfs + sh.bcast_i;
             for (int i = tid; i < mine; i += nt) P.sc.border[at + i] = squad_q(cur).v[i];
             write_long(mf_stage + 6 * MF_SQUAD_CAP, min(sh.so_long, MF_SQUAD_LONG));
-            return;
+            return true;
         }
         __syncthreads();
         if (tid == 0) sh.so_cnt = sh.so_flag = 0;
@@ -3312,13 +3345,14 @@ __device__ __noinline__ void phase_discharge_short()
 }
 
 // Discharge rounds, one after another, while few vertices are active.  The last
-// one leaves its results where a round of the grid would.
-__device__ __noinline__ void squad_discharge()
+// one leaves its results where a round of the grid would.  False as squad_bfs.
+__device__ __noinline__ bool squad_discharge()
 {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
     const int csize = sh.csize, rank = sh.crank;
     const unsigned long long t0 = gtimer();
     int cur = 0, cnt;
+    squad_enter();
     {
         const int sel = sh.d.wl_sel, n0 = sh.d.wl_n[0], all = n0 + sh.d.wl_n[1];
         cnt = all > rank ? (all - rank + csize - 1) / csize : 0;
@@ -3331,6 +3365,7 @@ __device__ __noinline__ void squad_discharge()
     }
     if (tid == 0) sh.so_cnt = sh.so_flag = 0;
     __syncthreads();
+    if (!squad_entered()) return false;
     for (;;) {
         const int par = sh.so_par;
         const SquadQ cq = squad_q(cur), nq = squad_q(cur ^ 1);
@@ -3396,7 +3431,7 @@ __device__ __noinline__ void squad_discharge()
                     P.sc.wl[sh.d.wl_sel ^ 1][bin][atomicAdd(&sh.cs->l[L_AUX + bin].w[0], 1u)] = nq.v[i];
                 }
             }
-            return;
+            return true;
         }
         __syncthreads();
         if (tid == 0) sh.so_cnt = sh.so_flag = 0;
@@ -3738,7 +3773,7 @@ __device__ __noinline__ bool solve_instance()
         while (!sh.d.bfs_done) {
             if (sh.d.bfs_squad) {
                 // the others wait at the grid barrier and take the squad's state there
-                if (vb() < sh.csize) squad_bfs();
+                if (vb() < sh.csize && !squad_bfs()) return false;
                 if (!grid_sync(H_BFS_NEXT, true)) return false;
                 continue;
             }
@@ -3764,7 +3799,7 @@ __device__ __noinline__ bool solve_instance()
         // discharge rounds, then remove-invalid-edges
         do {
             if (sh.d.dis_squad) {
-                if (vb() < sh.csize) squad_discharge();
+                if (vb() < sh.csize && !squad_discharge()) return false;
                 if (!grid_sync(H_DIS, true)) return false;
                 continue;
             }
@@ -3796,7 +3831,11 @@ __global__ void __launch_bounds__(MF_BLOCK, 2) mf_solve_kernel(const __grid_cons
     solve_instance();
 }
 
-// Barrier of one group of CTAs (no hook): w[0] arrivals, w[1] generation.
+// Barrier of one group of CTAs (no hook): w[0] arrivals, w[1] generation.  In
+// clusters, a CTA that gives up sets its cluster's bit (w[3], w[4]) and the whole
+// cluster leaves: the squads of the instance that follows write into one
+// another's shared memory.  Only a cluster's own CTAs set its bit, before the
+// cluster's barrier behind which all of them read it.
 __device__ bool group_sync(unsigned *w, unsigned &gen_local, unsigned long long wait_ns, int *abort)
 {
     __shared__ int ok;
@@ -3820,6 +3859,8 @@ __device__ bool group_sync(unsigned *w, unsigned &gen_local, unsigned long long 
                     if (t0 == 0) {
                         t0 = now;
                     } else if (now - t0 > wait_ns) {
+                        const unsigned q = (unsigned)vb() / cluster_size();
+                        if (cluster_size() > 1) atomicOr(w + 3 + (q >> 5), 1u << (q & 31u));
                         atomicExch(abort, 1);
                         good = 0;
                         break;
@@ -3832,6 +3873,12 @@ __device__ bool group_sync(unsigned *w, unsigned &gen_local, unsigned long long 
         ok = good;
     }
     __syncthreads();
+    if (cluster_size() > 1) {
+        const unsigned q = (unsigned)vb() / cluster_size();
+        cluster_sync();
+        if (threadIdx.x == 0 && (__ldcg(w + 3 + (q >> 5)) >> (q & 31u) & 1u)) ok = 0;
+        __syncthreads();
+    }
     return ok != 0;
 }
 
@@ -3839,7 +3886,7 @@ __device__ bool group_sync(unsigned *w, unsigned &gen_local, unsigned long long 
 // gsize CTAs; each group takes the next instance from a shared queue (the host
 // orders it largest first) and runs its whole solve, then takes another.
 // gstate holds, per group, 32 words: w[0] arrivals, w[1] generation, w[2] the
-// instance the group's first CTA took.
+// instance the group's first CTA took, w[3] and w[4] the clusters that left.
 __global__ void __launch_bounds__(MF_BLOCK, 2) mf_multi_kernel(const MfParams *__restrict__ plist, int count,
                                                                int gsize, unsigned *gstate, unsigned *head,
                                                                unsigned long long wait_ns, int *abort)
