@@ -138,6 +138,7 @@ struct MfDesc {
     int bfs_squad;                // the coming top-down level is small: the squad runs it, and the next small ones, alone
     int dis_short;                // the coming discharge round has short rows only: one cycle per vertex
     int dis_squad;                // ... and few of them: the squad runs it, and the next small ones, alone
+    int dis_stamp;                // a short round queues behind stamps (mf_round_stamps)
     int need_total;               // the coming BFS roots pass sums the used slots (first BFS of a launch)
     int wl_sel;                   // which worklist buffer the current round reads
     int wl_n[MF_NBIN];
@@ -169,21 +170,21 @@ struct MfState {
     int trace_n;
 };
 
-// Whether round `round` of an iteration's discharge may be a short one, by the
-// kind of the round before.  Short rounds queue without stamps, which needs a
-// list whose vertices all have excess.  A BFS and a short round leave such a
-// list.  A round of several cycles does not: u sends its excess, a neighbour
-// pushes to u and queues it, and a later cycle of u's sends that too; nor do the
-// walks, where u may take along what another walk has left there.  In a short
-// round such a vertex, listed with e = 0, could be queued by a receiver and then
-// by itself, and the round after would hold it twice: two owners that both take
-// the same residual, below zero.
+// Whether round `round` of an iteration's discharge, if it is a short one, has to
+// queue behind stamps, by the round before.  Without stamps a short round needs a
+// list whose vertices all have excess.  A BFS and an unstamped short round leave
+// such a list.  A round of several cycles does not: u sends its excess, a
+// neighbour pushes to u and queues it, and a later cycle of u's sends that too;
+// nor do the walks, where u may take along what another walk has left there.  In
+// an unstamped round such a vertex, listed with e = 0, could be queued by a
+// receiver and then by itself, and the round after would hold it twice: two
+// owners that both take the same residual, below zero.
 #ifdef __CUDACC__
 __host__ __device__
 #endif
-inline bool mf_short_may_follow(int round, int last_short)
+inline int mf_round_stamps(int round, int last_short, int last_stamped)
 {
-    return round == 0 || last_short != 0;
+    return round > 0 && (last_stamped || !last_short) ? 1 : 0;
 }
 
 // Work counters.  Each CTA keeps its own in shared memory and adds them to the

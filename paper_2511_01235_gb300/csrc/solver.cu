@@ -303,13 +303,15 @@ __device__ __forceinline__ bool rounds_left(const MfDesc &d, const MfState &st, 
 // few vertices are left to the squad (squad_discharge).  On a small graph that
 // takes a BFS of many levels: short rounds pay where many rounds follow; where
 // two or three do, the whole KERNEL_CYCLES in each settle more.  Behind a round
-// of another kind no short one follows (mf_short_may_follow).
+// of another kind it queues behind stamps (64 batched instances: 11.9 ms, and
+// 17.5 without short rounds there).
 __device__ __forceinline__ void pick_round(MfDesc &d, int csize)
 {
+    d.dis_stamp = mf_round_stamps(d.round, d.dis_short, d.dis_stamp);
     d.dis_short = P.rounds == 0 && !P.pull && !P.fix_steep && P.data_driven && P.requeue &&
                           P.stage_slots >= MF_SQUAD_INTS && P.hub_deg <= MF_SHORT_ROW &&
                           (P.g.slot_cap >= MF_LARGE_SLOTS || d.level >= MF_DEEP) &&
-                          d.wl_n[2] + d.wl_n[3] == 0 && mf_short_may_follow(d.round, d.dis_short)
+                          d.wl_n[2] + d.wl_n[3] == 0
                       ? 1 : 0;
     d.dis_squad = d.dis_short && d.wl_n[0] + d.wl_n[1] <= MF_SQUAD_ACTIVE * csize ? 1 : 0;
 }
@@ -3144,12 +3146,13 @@ __device__ __noinline__ bool squad_bfs()
 }
 
 // z received flow and became active, or stays active after its cycle: into the
-// next round.  In the squad: into this CTA's queue, or, when that is full or z's
+// next round, once (by the stamp or by the reasons at short_push).  In the squad: into this CTA's queue, or, when that is full or z's
 // row is long, onto the grid's lists; else into the CTA's queue of worklist
 // entries.
 template <bool SQUAD>
 __device__ __forceinline__ void short_enqueue(int z, int r0, int d, const SquadQ &nq)
 {
+    if (sh.d.dis_stamp && atomicExch(P.sc.vmark + z, sh.d.qstamp) == sh.d.qstamp) return;
     if (!SQUAD) {
         place_active(z, d, L_AUX, sh.d.wl_sel ^ 1, nullptr);
         return;
@@ -3166,13 +3169,13 @@ __device__ __forceinline__ void short_enqueue(int z, int r0, int d, const SquadQ
     sh.so_flag = SQ_SPILL;
 }
 
-// g units along slot x = (u, z), y its reverse.  No stamp is needed to queue a
-// receiver: the list of a short round holds every vertex once, and each with
-// e > 0 (it comes from the BFS or from a short round, mf_short_may_follow).  A
-// listed vertex lowers its own excess once, by what it read at first, and queues
-// itself if some is left; until then its excess is above zero and no receiver
-// queues it, and after that it rises from zero at most once.  A vertex that is
-// not listed never lowers its excess.  So everyone is queued once, with e > 0.
+// g units along slot x = (u, z), y its reverse.  A round straight behind the BFS,
+// or behind other such short rounds, needs no stamp to queue a receiver: its list
+// holds every vertex once, and each with e > 0.  A listed vertex lowers its own
+// excess once, by what it read at first, and queues itself if some is left; until
+// then its excess is above zero and no receiver queues it, and after that it
+// rises from zero at most once.  A vertex that is not listed never lowers its
+// excess.  So everyone is queued once, with e > 0.
 template <bool SQUAD>
 __device__ __forceinline__ void short_push(int x, int z, int y, int g, const SquadQ &nq)
 {
@@ -3415,6 +3418,7 @@ __device__ __noinline__ bool squad_discharge()
             sh.so_go = over ? 0 : (flag != 0 || c > MF_SQUAD_ACTIVE * csize ? 2 : 1);
             if (sh.so_go == 1) {
                 ++sh.d.round;
+                ++sh.d.qstamp;
                 ++sh.hs.rounds_total;
             }
             sh.so_par = par ^ 1;

@@ -3,7 +3,7 @@
 Bipartite matching graphs whose right side has rows of 600 to 2100 slots (a round
 with one of them active is never a short one) beside short rows, and a sink row
 above n / 8 (no near iterations): rounds over hub rows are followed by rounds
-without any.  Exact against the oracle, and no residual below zero.
+without any, which queue behind stamps.  Exact against the oracle, and no residual below zero.
 """
 import numpy as np
 import pytest
@@ -33,7 +33,9 @@ def _matching(left, hubs, small, seed):
     cap = rng.integers(1, 8, src.size)
     cap[src == s] = rng.integers(1, 20, left)
     cap[(dst == t) & (src > left)] = rng.integers(1, 30, hubs + small)
-    keep = src != dst
+    keep = np.zeros(src.size, bool)
+    keep[np.unique(src * n + dst, return_index=True)[1]] = True       # each pair once
+    keep &= src != dst
     return W.Graph(n, src[keep].astype(np.int32), dst[keep].astype(np.int32), cap[keep].astype(np.int32), s, t)
 
 

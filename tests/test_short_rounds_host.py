@@ -1,10 +1,10 @@
-"""Which discharge rounds may be short ones, on the CPU.
+"""Short discharge rounds queue every vertex once, on the CPU.
 
-A short round queues vertices without stamps.  The model below runs two vertices
-through a round of several cycles (queued behind a stamp) and through short
-rounds, over every interleaving of their accesses, and asks the header's own rule
-(mf_short_may_follow, compiled here) what may come next: a short round's list
-never holds a vertex twice, and never one without excess.
+A short round queues behind stamps or without.  The model below runs two vertices
+through a round of several cycles (always behind stamps) and through short rounds,
+over every interleaving of their accesses, and asks the header's own rule
+(mf_round_stamps, compiled here) which kind a short round is: its list never holds
+a vertex twice, and without stamps never one that has no excess.
 """
 import os
 import subprocess
@@ -17,22 +17,20 @@ PROBE = """
 #include <cstdio>
 #include "mf_internal.h"
 int main() {
-    for (int round = 0; round < 4; ++round)
-        for (int last = 0; last < 2; ++last) std::printf("%d\\n", mf_short_may_follow(round, last) ? 1 : 0);
+    for (int i = 0; i < 16; ++i) std::printf("%d\\n", mf_round_stamps(i >> 2, i >> 1 & 1, i & 1));
 }
 """
 
 
 @pytest.fixture(scope="module")
-def may_follow(tmp_path_factory):
+def stamps(tmp_path_factory):
     d = tmp_path_factory.mktemp("short")
     (d / "probe.cpp").write_text(PROBE)
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(build_ext._nvcc())))
     subprocess.check_call(["g++", "-std=c++17", "-I", os.path.join(cuda, "include"), "-I", build_ext.CSRC,
                            str(d / "probe.cpp"), "-o", str(d / "probe")])
     out = subprocess.check_output([str(d / "probe")], text=True).split()
-    table = {(r, k): out[2 * r + k] == "1" for r in range(4) for k in range(2)}
-    return lambda round_, last_short: table[min(round_, 3), int(last_short)]
+    return lambda round_, last_short, last_stamped: out[4 * min(round_, 3) + 2 * last_short + last_stamped] == "1"
 
 
 # p above u above w: p's slots to u (a slot is one push), u's to w
@@ -61,17 +59,17 @@ def _long(v):
         yield ("queue", v, True)
 
 
-def _short(v):
-    """One cycle on the excess read at first; queueing without a stamp."""
+def _short(v, stamp):
+    """One cycle on the excess read at first."""
     eu = yield ("read", v)
     if eu <= 0:
         return
     sent = 0
     for _ in range(2):                     # the slots of the lowest neighbour
         if sent < eu:
-            sent += yield ("push", v, eu - sent, False)
+            sent += yield ("push", v, eu - sent, stamp)
     if (yield ("take", v, sent)) > 0:
-        yield ("queue", v, False)
+        yield ("queue", v, stamp)
 
 
 def _outcomes(state, body):
@@ -123,27 +121,29 @@ def _outcomes(state, body):
 
 
 @pytest.mark.parametrize("first", ["long", "short"])
-def test_a_short_rounds_list_holds_every_vertex_once_and_with_excess(may_follow, first):
-    states = [(dict(START, list=["u", "p"]), first == "short")]
-    shorts = bare = 0
-    for round_ in range(3):
+def test_a_short_rounds_list_holds_every_vertex_once(stamps, first):
+    kind0 = (True, stamps(0, 0, 0)) if first == "short" else (False, False)
+    states = [(dict(START, list=["u", "p"]), kind0)]
+    plain = stamped = bare = 0
+    for round_ in range(4):
         nxt = {}
-        for st, short in states:
-            if short:
-                shorts += 1
-                assert len(set(st["list"])) == len(st["list"]), st
+        for st, (short, stamp) in states:
+            assert len(set(st["list"])) == len(st["list"]), st
+            if short and not stamp:
                 assert all(st["e"][v] > 0 for v in st["list"]), st
-            else:
-                bare += any(st["e"][v] <= 0 for v in st["list"])
-            for o in _outcomes(st, _short if short else _long):
+            plain += short and not stamp
+            stamped += short and stamp
+            bare += any(st["e"][v] <= 0 for v in st["list"])
+            for o in _outcomes(st, (lambda v: _short(v, stamp)) if short else _long):
                 assert min(o["e"].values()) >= 0
-                if o["list"]:
-                    # a round with short rows only: short wherever the rule lets it
-                    kind = may_follow(round_ + 1, short)
+                for again in (True, False) if o["list"] and not short else (True,) if o["list"] else ():
+                    kind = (again, again and stamps(round_ + 1, short, stamp))     # a long round may follow too
                     nxt[(tuple(sorted(o["e"].items())), tuple(o["cf"].items()), tuple(o["list"]), kind)] = (o, kind)
-        states = list(nxt.values())[:60]
-    assert shorts > 3 if first == "short" else bare     # the model reaches what the rule is about
+        states = list(nxt.values())[:80]
+    # the model reaches what the rule is about
+    assert plain > 3 and not stamped if first == "short" else stamped > 3 and bare
 
 
-def test_an_iteration_may_open_with_a_short_round(may_follow):
-    assert may_follow(0, 0) and may_follow(0, 1) and may_follow(2, 1)
+def test_rounds_behind_a_relabel_need_no_stamps(stamps):
+    assert not any(stamps(0, a, b) for a in (0, 1) for b in (0, 1))
+    assert not stamps(1, 1, 0) and stamps(1, 0, 0) and stamps(2, 1, 1)
