@@ -1204,10 +1204,14 @@ __device__ __noinline__ int find_slot(const MfParams &P, int u, int v, int *prob
 }
 
 // Slot of (u, v), or -1, looked for in the shorter of the two rows: the pair has a
-// slot in both, and on power-law graphs one end of most edges is a hub.
+// slot in both, and on power-law graphs one end of most edges is a hub.  A row's
+// base slots are searched, its inserted ones read one by one, so the other row
+// is only taken if it has no more of those.
 __device__ __forceinline__ int find_pair(int u, int v, int *probes)
 {
-    if (2ll * ldg_cg(P.g.bdeg + v) < ldg_cg(P.g.bdeg + u)) {
+    const int bu = ldg_cg(P.g.bdeg + u), bv = ldg_cg(P.g.bdeg + v);
+    const int iu = ldg_cg(P.g.deg + u) - bu, iv = ldg_cg(P.g.deg + v) - bv;
+    if (2ll * bv < bu && iv <= iu) {
         const int y = find_slot(P, v, u, probes);
         return y < 0 ? -1 : ldg_cg(P.g.rev + y);
     }
