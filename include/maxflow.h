@@ -224,9 +224,10 @@ int maxflow_set_cycle_div(maxflow_ctx *c, int32_t div);
  * in the first cluster of eight CTAs alone, level after level, with the
  * cluster's barrier between levels instead of the grid's (the labels are those
  * of Alg. 4 / Alg. 6 either way); the grid meets again when a frontier grows
- * past a limit or the BFS ends.  0 (the default) is the library's own limit,
- * 2048 slots per CTA.  Launches without clusters use their first CTA.  Not in
- * the paper.  MAXFLOW_ERR_INVALID below 0. */
+ * past a limit or the BFS ends.  0 turns it off: every level runs across the
+ * grid.  Until this is called the limit is the library's own, 2048 slots per
+ * CTA.  Launches without clusters use their first CTA.  Not in the paper.
+ * MAXFLOW_ERR_INVALID below 0. */
 int maxflow_set_bfs_tail(maxflow_ctx *c, int32_t slots);
 
 /* Run remove-invalid-edges (Alg. 3) after each iteration's discharge rounds

@@ -55,7 +55,7 @@ struct maxflow_ctx {
     int32_t stage_slots = 0;      // dynamic shared memory of the solve launches, in ints
     int32_t requeue = 1;          // discharge rounds re-queue vertices still active after their cycles
     int32_t cycle_div = 0;        // > 0: long rows get max(kernel_cycles, deg / cycle_div) cycles
-    int32_t tail_slots = 0;       // BFS frontiers of at most this many slots run in the squad (0: MF_SQUAD_SLOTS per CTA)
+    int32_t tail_slots = -1;      // BFS frontiers of at most this many slots run in the squad (0: none; -1: MF_SQUAD_SLOTS per CTA)
     MfGraph g{};
     MfScratch sc{};
     MfCtrl *ctrl = nullptr;

@@ -346,7 +346,7 @@ struct MfParams {
     int32_t requeue;          // discharge rounds: a vertex still active after its cycles joins the next round
     int32_t cycle_div;        // > 0: a row of d slots gets max(kernel_cycles, d / cycle_div) cycles
     int32_t tail_slots;       // BFS: a top-down level whose frontier holds at most this many slots (and
-                              // vertices) runs in the squad, without grid barriers; 0: MF_SQUAD_SLOTS per CTA
+                              // vertices) runs in the squad, without grid barriers; 0: none does; -1: MF_SQUAD_SLOTS per CTA
     int32_t stage_slots;      // dynamic shared memory of the launch in ints: the discharge's on-chip row snapshot
                               // (a CTA keeps rows up to this many slots; 0: none)
     long long max_iters;

@@ -3698,7 +3698,7 @@ __device__ __noinline__ bool solve_instance()
         sh.k_alpha = P.bu_alpha;
         sh.k_beta = P.bu_beta;
         sh.k_wl = P.data_driven && !(P.mode & MF_M_BFS_ONLY) ? 1 : 0;
-        sh.k_squad = P.pull || P.stage_slots < MF_SQUAD_INTS ? 0 : (P.tail_slots > 0 ? P.tail_slots : MF_SQUAD_SLOTS * sh.csize);
+        sh.k_squad = P.pull || P.stage_slots < MF_SQUAD_INTS ? 0 : (P.tail_slots >= 0 ? P.tail_slots : MF_SQUAD_SLOTS * sh.csize);
         sh.hs.t_phase = gtimer();
     }
     if (vb() == 0) {
