@@ -199,7 +199,8 @@ int maxflow_set_kernel_cycles(maxflow_ctx *c, int32_t k);
  * spread over more discharge work.  On large graphs whose sink has a short row,
  * 0 also lets a push solve end a global relabel once it has labelled as much
  * excess as its roots can take, and send that excess down the BFS tree before
- * any round; the solve still ends only behind a complete BFS.
+ * any round; the solve still ends only behind a complete BFS.  Not under a cap
+ * on iterations (maxflow_opts.max_iters), which counts complete relabels.
  * MAXFLOW_ERR_INVALID below 0. */
 int maxflow_set_rounds(maxflow_ctx *c, int32_t rounds);
 

@@ -211,6 +211,7 @@ MfParams base_params(maxflow_ctx *c)
     p.cycle_div = c->cycle_div;
     p.tail_slots = c->tail_slots;
     p.side = c->pp.side;
+    p.allow_near = c->opt.max_iters > 0 ? 0 : 1;
     p.max_iters = c->opt.max_iters > 0 ? c->opt.max_iters : 4LL * c->n + 1000;
     double tl = c->opt.time_limit_s > 0 ? c->opt.time_limit_s : 120.0;
     double wl = c->opt.wait_limit_s > 0 ? c->opt.wait_limit_s : 1.0;

@@ -349,6 +349,7 @@ struct MfParams {
                               // vertices) runs in the squad, without grid barriers; 0: none does; -1: MF_SQUAD_SLOTS per CTA
     int32_t stage_slots;      // dynamic shared memory of the launch in ints: the discharge's on-chip row snapshot
                               // (a CTA keeps rows up to this many slots; 0: none)
+    int32_t allow_near;       // 0: no near iterations (the caller has set a cap on iterations, which counts complete relabels)
     long long max_iters;
     unsigned long long time_limit_ns;
     unsigned long long wait_limit_ns;

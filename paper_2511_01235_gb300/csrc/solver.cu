@@ -345,10 +345,11 @@ __device__ __forceinline__ void decide_iteration(int active)
 // schedule, and a sink that can be reached from few vertices directly.  With a
 // longer sink row (grids: every pixel has an edge to t) what the sink can take
 // exceeds any excess, no relabel would be cut, and the bookkeeping would only
-// cost.
+// cost.  Nor under the caller's own cap on iterations: those behind a cut relabel
+// settle less, so a cap that sufficed would not.
 __device__ __forceinline__ int near_allowed()
 {
-    if (P.sc.par == nullptr || !(P.mode & MF_M_SOLVE) || (P.mode & MF_M_NO_DEFICIT_ROOTS) || P.pull ||
+    if (!P.allow_near || P.sc.par == nullptr || !(P.mode & MF_M_SOLVE) || (P.mode & MF_M_NO_DEFICIT_ROOTS) || P.pull ||
         P.side_root >= 0 || P.rounds != 0 || P.fix_steep || !P.data_driven || P.g.slot_cap < MF_LARGE_SLOTS)
         return 0;
     return (long long)ldg_cg(P.g.deg + P.sink) * MF_NEAR_SINK <= (long long)P.g.n ? 1 : 0;
@@ -523,8 +524,12 @@ __device__ __forceinline__ int advance_bfs(int &hook)
     d.bu_mode = bu;
     d.bu_split = 0;
     d.bfs_squad = !done && !bu && app_hub == hub_hi && squad_level(cnt, fr) ? 1 : 0;
-    // near iterations: the levels so far hold as much excess as the roots can take
-    const int cut = near && !done && sup > 0 && (sup >> shift) >= dem ? 1 : 0;
+    // near iterations: the levels so far hold as much excess as the roots can
+    // take.  Not when the solve is to end at a cap behind this BFS: it leaves a
+    // complete labelling then, and the value is summed over it
+    const int cut = near && !done && sup > 0 && (sup >> shift) >= dem && st.iters < P.max_iters &&
+                            st.t_now - st.t_start <= P.time_limit_ns
+                        ? 1 : 0;
     d.cut = cut;
     st.cut_prev = cut;
     d.bfs_done = done || cut ? 1 : 0;
