@@ -1219,6 +1219,7 @@ int maxflow_update_scheduled(maxflow_ctx *c, const maxflow_batch *b, maxflow_mlp
     const int best = c->rep->action;
     if (best < 0 || best >= kNumActions) return rc;          // refused before the choice
     if (action_out) *action_out = best;
+    c->st.kernel_cycles = kActions[best].cycles > 0 ? kActions[best].cycles : avg_cycles(c);   // as run_action leaves it
     if (rc == MAXFLOW_OK && kActions[best].mode == 0) note_incremental(c);
     return rc;
 }
