@@ -288,6 +288,17 @@ __device__ __forceinline__ bool squad_level(long long cnt, long long fr)
     return sh.k_squad > 0 && cnt <= MF_SQUAD_LEVEL * sh.csize && fr <= sh.k_squad;
 }
 
+// Direction of a BFS level that follows a top-down one (Beamer's test): bottom-up
+// once the frontier's slots (fr) exceed 1/alpha of the unexplored ones.  Not in a
+// deep BFS, whose frontiers are short: near its end the unexplored slots get few
+// too, and a bottom-up level still visits every vertex (256 x 256 grid, window
+// updates 4.9 -> 4.7 ms; 64 batched instances 12.0 -> 11.3).  The squad asks the
+// same: what it leaves for a bottom-up level has to become one.
+__device__ __forceinline__ bool turns_bottom_up(int alpha, int level, long long fr, long long unexplored)
+{
+    return alpha > 0 && level < MF_DEEP && fr * alpha > unexplored;
+}
+
 // Adaptive rounds: whether this iteration's discharge may still take time beside
 // its BFS: half of it with rounds of KERNEL_CYCLES cycles, all of it with short
 // ones (grid 1024 window 15.5 -> 13.6 ms, 64 batched instances 14.6 -> 11.6 ms;
@@ -511,16 +522,12 @@ __device__ __forceinline__ int advance_bfs(int &hook)
     d.level = first ? 0 : level + 1;
     st.vis_slots = vis;
     st.lvl_slots = st.lvl_cnt = 0;
-    // direction of the coming level (Beamer's test): bottom-up once the
-    // frontier's slots exceed 1/alpha of the unexplored slots, back to
-    // top-down once it holds fewer than n/beta vertices.  Not in a deep BFS,
-    // whose frontiers are short: near its end the unexplored slots get few too,
-    // and a bottom-up level still visits every vertex (256 x 256 grid, window
-    // updates 4.9 -> 4.7 ms; 64 batched instances 12.0 -> 11.3)
+    // direction of the coming level: back to top-down once the frontier holds
+    // fewer than n/beta vertices
     int bu = bu_was;
     if (alpha <= 0) bu = 0;
-    else if (!bu && d.level < MF_DEEP && fr * alpha > used - vis) bu = 1;
-    else if (bu && cnt * beta < (long long)n) bu = 0;
+    else if (!bu) bu = turns_bottom_up(alpha, d.level, fr, used - vis) ? 1 : 0;
+    else if (cnt * beta < (long long)n) bu = 0;
     d.bu_mode = bu;
     d.bu_split = 0;
     d.bfs_squad = !done && !bu && app_hub == hub_hi && squad_level(cnt, fr) ? 1 : 0;
@@ -3120,7 +3127,7 @@ __device__ __noinline__ bool squad_bfs()
             }
             const long long vis = st.vis_slots + fr, sup = st.sup + exc;
             const bool go = c > 0 && flag == 0 && squad_level(c, fr) &&
-                            !(sh.k_alpha > 0 && fr * sh.k_alpha > st.used_slots - vis) &&
+                            !turns_bottom_up(sh.k_alpha, sh.d.level + 1, fr, st.used_slots - vis) &&
                             !(d.near && sup > 0 && (sup >> st.cut_shift) >= st.dem);
             if (go) {
                 // what advance() does for a level that is followed by another small one
