@@ -264,12 +264,13 @@ int maxflow_mlp_forward(maxflow_mlp *m, const float *x, int32_t rows, float *y)
     return rc;
 }
 
-// The parameters on the device, for the solver's own forward pass; what was
-// issued on the network's stream (training) is waited for.
+// The parameters on the device, for the solver's own forward pass; what is still
+// under way on the network's stream (training) is waited for.
 int mlp_params_device(maxflow_mlp *m, const float **p)
 {
     *p = m->p;
-    return ok(cudaStreamSynchronize(m->stream));
+    const cudaError_t e = cudaStreamQuery(m->stream);
+    return ok(e == cudaErrorNotReady ? cudaStreamSynchronize(m->stream) : e);
 }
 
 int mlp_hidden(const maxflow_mlp *m) { return m->H; }

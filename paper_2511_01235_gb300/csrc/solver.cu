@@ -76,9 +76,9 @@ __device__ __forceinline__ int row_bin(int d)
 // every SM's memory pipeline busy instead of crowding onto the first CTAs.
 // spread_warp keeps 32 consecutive indices in one warp (warp-uniform loops).
 __device__ __forceinline__ long long spread_thread() { return (long long)threadIdx.x * vn() + vb(); }
-__device__ __forceinline__ long long spread_warp()
+__device__ __forceinline__ long long spread_warp(int nctas)
 {
-    return ((long long)(threadIdx.x >> 5) * vn() + vb()) * 32 + (threadIdx.x & 31);
+    return ((long long)(threadIdx.x >> 5) * nctas + vb()) * 32 + (threadIdx.x & 31);
 }
 
 __device__ __forceinline__ int ldg_cg(const int *p) { return __ldcg(p); }
@@ -398,31 +398,34 @@ __device__ __noinline__ void batch_features()
     x[15] = 1.f;
 }
 
+// y = w x + b by one CTA (relu: not below zero), a warp per output with its lanes
+// over the inputs, so that the weights come in whole lines.
+__device__ __forceinline__ void net_layer(const float *__restrict__ w, const float *__restrict__ b, const float *x,
+                                          int n_in, int n_out, float *y, bool relu)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll 4
+    for (int j = (int)(threadIdx.x >> 5); j < n_out; j += MF_WARPS) {
+        float a = 0.f;
+        for (int k = lane; k < n_in; k += 32) a += __ldg(w + j * n_in + k) * x[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        a += __ldg(b + j);
+        if (lane == 0) y[j] = !relu || a > 0.f ? a : 0.f;
+    }
+    __syncthreads();
+}
+
 // Forward pass and choice, by one CTA; 1 + the action goes to the counter set.
 __device__ __noinline__ void pick_action()
 {
-    const int j = threadIdx.x, H = P.net.hidden, no = P.net.n_out;
+    const int H = P.net.hidden, no = P.net.n_out;
     const float *w1 = P.net.p, *b1 = w1 + H * MF_FEATURES, *w2 = b1 + H, *b2 = w2 + H * H, *w3 = b2 + H,
                 *b3 = w3 + no * H;
-    if (j < H) {
-        float a = b1[j];
-        for (int i = 0; i < MF_FEATURES; ++i) a += w1[j * MF_FEATURES + i] * sh.x[i];
-        sh.h1[j] = a > 0.f ? a : 0.f;
-    }
-    __syncthreads();
-    if (j < H) {
-        float a = b2[j];
-        for (int k = 0; k < H; ++k) a += w2[j * H + k] * sh.h1[k];
-        sh.h2[j] = a > 0.f ? a : 0.f;
-    }
-    __syncthreads();
-    if (j < no) {
-        float a = b3[j];
-        for (int k = 0; k < H; ++k) a += w3[j * H + k] * sh.h2[k];
-        sh.y[j] = a;
-    }
-    __syncthreads();
-    if (j == 0) {
+    net_layer(w1, b1, sh.x, MF_FEATURES, H, sh.h1, true);
+    net_layer(w2, b2, sh.h1, H, H, sh.h2, true);
+    net_layer(w3, b3, sh.h2, H, no, sh.y, false);
+    if (threadIdx.x == 0) {
         int best = 0;
         for (int i = 1; i < no; ++i)
             if (sh.y[i] < sh.y[best]) best = i;
@@ -1128,7 +1131,7 @@ __device__ __noinline__ void phase_apply_validate()
     unsigned fs = 0, ft = 0, fz = 0;
     long long fcap = 0;
     // warp-uniform loop: the positions taken in the table are appended with one atomic per warp
-    for (long long base = spread_warp() - lane; base < P.bcount; base += (long long)vn() * blockDim.x) {
+    for (long long base = spread_warp(vn()) - lane; base < P.bcount; base += (long long)vn() * blockDim.x) {
         const long long i = base + lane;
         bool fresh = false;
         unsigned pos = 0;
@@ -1250,15 +1253,15 @@ __device__ __forceinline__ unsigned hash_find(const unsigned long long *keys, in
 // update of (v, u) if it has one, else the current c(v, u), else 0 for a new
 // pair -- must fit int32 (residual capacities are int32 and c_f(u,v) +
 // c_f(v,u) equals that sum).  A batch that breaks it sets MF_E_TOO_LARGE and
-// is refused whole.
-__device__ __noinline__ void phase_apply_locate()
+// is refused whole.  Done by the first nctas CTAs.
+__device__ __noinline__ void phase_apply_locate(int nctas)
 {
     MfSet *cs = sh.cs;
     const int bits = P.sc.hash_bits;
     const unsigned mask = (1u << bits) - 1u;
     const int lane = threadIdx.x & 31;
     int probes = 0;
-    for (long long base = spread_warp() - lane; base < P.bcount; base += (long long)vn() * blockDim.x) {
+    for (long long base = spread_warp(nctas) - lane; base < P.bcount; base += (long long)nctas * blockDim.x) {
         const long long i = base + lane;
         bool fresh = false;
         unsigned pp = 0;
@@ -3750,8 +3753,10 @@ __device__ __noinline__ bool solve_instance()
             phase_apply_cleanup(false);
             return finish();
         }
+        // the last CTA asks the network while the others locate the slots
+        const int finders = (P.mode & MF_M_SCHED) && vn() > 1 ? vn() - 1 : vn();
         if ((P.mode & MF_M_SCHED) && vb() == vn() - 1) pick_action();
-        phase_apply_locate();
+        if (vb() < finders) phase_apply_locate(finders);
         if (!grid_sync(H_APPLY_LOCATED)) return false;
         if (sh.d.status != MF_ST_RUNNING) {
             // a row overflow keeps the rows' demand for the rebuild that follows;
