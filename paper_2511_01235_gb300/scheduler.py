@@ -166,7 +166,8 @@ def train(X, T, M, hidden=64, steps=3000, lr=3e-3, seed=0):
 def prefer_default(mlp: native.MLP, margin):
     """Shift the outputs so that a schedule other than the default has to be predicted `margin` (log time)
     faster: where schedules tie, timing noise in the traces would pick one, and a wrong pick costs more
-    than a tie gains."""
+    than a tie gains.  On the current kernel the default is within 4 % of the best schedule of every
+    family, and on held-out batches predictions are off by up to 0.5."""
     p = mlp.params.copy()
     b3 = p[p.size - mlp.n_out:]
     b3[np.arange(mlp.n_out) != ACTION_DEFAULT] += margin
@@ -215,7 +216,7 @@ def main():
     ap.add_argument("--steps", type=int, default=1200)
     ap.add_argument("--traces", default=None, help="save traces (npz) here")
     ap.add_argument("--reps", type=int, default=3, help="runs per action and batch (the fastest counts)")
-    ap.add_argument("--margin", type=float, default=0.1,
+    ap.add_argument("--margin", type=float, default=0.6,
                     help="log time another schedule has to be predicted faster than the default")
     args = ap.parse_args()
     import torch
