@@ -562,6 +562,10 @@ def scheduler_comparison(S, wl, count):
         batches.append(b)
     out = {"batches": len(batches), "sizes": sizes}
     picks = []
+    C = S.clone()               # once through untimed: the first arm would pay for the first use of batches and sizes
+    for b in batches:
+        C.update(b.u, b.v, b.cap)
+    C.close()
     for key in ("learned", "paper", "default"):
         C = S.clone()
         ts = []
