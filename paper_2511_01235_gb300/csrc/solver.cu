@@ -1067,29 +1067,58 @@ __device__ __noinline__ void phase_cut_side()
 }
 
 // ... then every residual edge from side 0 to side 1 sends all it can, so
-// that no residual path leads from side 0 to side 1.  One warp per row.
+// that no residual path leads from side 0 to side 1.  Slots j0, j0 + step, ... of
+// a row; returns what its vertex sent.
+__device__ __forceinline__ long long saturate_row(int r0, int d, int j0, int step)
+{
+    long long out = 0;
+    for (int j = j0; j < d; j += step) {
+        const int x = r0 + j;
+        const int c = ldg_cg(P.cf + x);
+        if (c <= 0) continue;
+        const int z = ldg_cg(P.g.dst + x);
+        if (P.side[z] != 1) continue;
+        P.cf[x] = 0;
+        atomicAdd(P.cf + ldg_cg(P.g.rev + x), c);
+        add_excess(z, (long long)c);
+        out += c;
+    }
+    return out;
+}
+
+// One warp per row, consecutive rows in different CTAs; rows of more than
+// MF_HUB_DEG slots wait in a list for their whole CTA.  The longest chain of a
+// warp's rows bounds it: with hub rows walked by one warp each, the longest on
+// R-MAT 20 was 6578 steps of 32 slots when 4864 warps shared the rows and 9402
+// when 4608 did (whose count has more factors of two, as the hubs' numbers do),
+// 7.7 and 9.3 ms of an update by push-pull; the whole update now takes 3.4 ms.
 __device__ __noinline__ void phase_saturate_cut()
 {
     const int n = P.g.n;
     const int lane = threadIdx.x & 31;
     const long long nw = ((long long)vn() * blockDim.x) >> 5;
-    for (long long u = ((long long)vb() * blockDim.x + threadIdx.x) >> 5; u < n; u += nw) {
+    if (threadIdx.x == 0) sh.bcast_i = 0;
+    __syncthreads();
+    for (long long u = warp_rank(vn(), 0); u < n; u += nw) {
         if (P.side[u] != 0) continue;
         const int r0 = P.g.off[u], d = ldg_cg(P.g.deg + u);
-        long long out = 0;
-        for (int j = lane; j < d; j += 32) {
-            const int x = r0 + j;
-            const int c = ldg_cg(P.cf + x);
-            if (c <= 0) continue;
-            const int z = ldg_cg(P.g.dst + x);
-            if (P.side[z] != 1) continue;
-            P.cf[x] = 0;
-            atomicAdd(P.cf + ldg_cg(P.g.rev + x), c);
-            add_excess(z, (long long)c);
-            out += c;
+        if (d > MF_HUB_DEG) {
+            int at = 0;
+            if (lane == 0) {
+                at = atomicAdd(&sh.bcast_i, 1);
+                if (at < P.stage_slots) mf_stage[at] = (int)u;
+            }
+            if (__shfl_sync(0xffffffffu, at, 0) < P.stage_slots) continue;
         }
-        out = warp_sum_ll(out);
+        const long long out = warp_sum_ll(saturate_row(r0, d, lane, 32));
         if (lane == 0 && out) add_excess((int)u, -out);
+    }
+    __syncthreads();
+    const int nl = min(sh.bcast_i, P.stage_slots);
+    for (int i = 0; i < nl; ++i) {
+        const int u = mf_stage[i];
+        const long long out = warp_sum_ll(saturate_row(P.g.off[u], ldg_cg(P.g.deg + u), threadIdx.x, blockDim.x));
+        if (lane == 0 && out) add_excess(u, -out);
     }
 }
 
