@@ -230,25 +230,23 @@ int ensure_batch(maxflow_ctx *c, int64_t count)
     int bits = 1;
     while ((1LL << bits) < 2 * cap) ++bits;
     MF_TRY(rc_cuda(cudaStreamSynchronize(c->stream)));
-    void *olds[] = {c->sc.hkey, c->sc.hval, c->sc.pkey, c->sc.pval, c->sc.bslot, c->sc.ins_list,
+    void *olds[] = {c->sc.hkey, c->sc.hval, c->sc.pkey, c->sc.bslot, c->sc.ins_list,
                     c->sc.hused, c->sc.bu};
     for (void *p : olds) dfree(c, p);
     int64_t hs = 1LL << bits;
     c->sc.hkey = dalloc_n<unsigned long long>(c, hs);
     c->sc.hval = dalloc_n<int32_t>(c, hs);
     c->sc.pkey = dalloc_n<unsigned long long>(c, hs);
-    c->sc.pval = dalloc_n<int32_t>(c, hs);
     c->sc.bslot = dalloc_n<int32_t>(c, cap);
     c->sc.ins_list = dalloc_n<int32_t>(c, cap);
     c->sc.hused = dalloc_n<int32_t>(c, cap);
     c->sc.bu = dalloc_n<int32_t>(c, 3 * cap);
-    if (!c->sc.hkey || !c->sc.hval || !c->sc.pkey || !c->sc.pval || !c->sc.bslot || !c->sc.ins_list ||
+    if (!c->sc.hkey || !c->sc.hval || !c->sc.pkey || !c->sc.bslot || !c->sc.ins_list ||
         !c->sc.hused || !c->sc.bu)
         return MAXFLOW_ERR_OOM;
     MF_TRY(rc_cuda(cudaMemsetAsync(c->sc.hkey, 0xff, sizeof(unsigned long long) * hs, c->stream)));
     MF_TRY(rc_cuda(cudaMemsetAsync(c->sc.hval, 0xff, sizeof(int32_t) * hs, c->stream)));
     MF_TRY(rc_cuda(cudaMemsetAsync(c->sc.pkey, 0xff, sizeof(unsigned long long) * hs, c->stream)));
-    MF_TRY(rc_cuda(cudaMemsetAsync(c->sc.pval, 0xff, sizeof(int32_t) * hs, c->stream)));
     c->sc.batch_cap = cap;
     c->sc.hash_bits = bits;
     return MAXFLOW_OK;

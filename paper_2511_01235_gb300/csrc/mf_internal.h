@@ -307,7 +307,6 @@ struct MfScratch {
     unsigned long long *hkey; // [1 << hash_bits] directed-pair dedup
     int32_t *hval;
     unsigned long long *pkey; // [1 << hash_bits] new-pair dedup
-    int32_t *pval;
     int32_t *bslot;           // [batch_cap] slot of each update (-2: superseded or ignored)
     int32_t *ins_list;        // [batch_cap] new-pair table positions
     int32_t *hused;           // [batch_cap] dedup table positions in use

@@ -378,24 +378,32 @@ __device__ __forceinline__ int near_allowed()
 
 __constant__ MfAction kActionTable[] = {MF_ACTIONS};
 
-// One thread: the features of the batch (k_features has them too, for the call that returns them).
-__device__ __noinline__ void batch_features()
+// The features of a batch (with updates touching s, touching t and deleting, and
+// the sum of its capacities) on a graph of n vertices and m edges.
+__device__ __forceinline__ void make_features(float *x, long long count, long long edges, int vertices, unsigned at_s,
+                                              unsigned at_t, unsigned deleting, long long cap_sum, float mean_cap,
+                                              const float *host)
 {
-    const float B = (float)P.bcount, m = (float)(P.net.m > 0 ? P.net.m : 1), n = (float)P.g.n;
-    const float inv = P.bcount > 0 ? 1.f / B : 0.f;
-    float *x = sh.x;
+    const float B = (float)count, m = (float)(edges > 0 ? edges : 1), n = (float)vertices;
+    const float inv = count > 0 ? 1.f / B : 0.f;
     x[0] = log2f(1.f + B) / 20.f;
     x[1] = fminf(B / m, 1.f);
     x[2] = log2f(n) / 24.f;
     x[3] = log2f(1.f + m) / 28.f;
     x[4] = (m / n) / 16.f;
-    x[5] = (float)(unsigned)sh.cnt[L_FEAT].x * inv;
-    x[6] = (float)(unsigned)sh.cnt[L_FEAT].y * inv;
-    x[7] = (float)(unsigned)sh.cnt[L_FEAT].z * inv;
-    x[8] = P.bcount > 0 && P.net.mean_cap > 0.f
-               ? fminf((float)(long long)cnt64(L_FCAP) * inv / P.net.mean_cap, 4.f) / 4.f : 0.f;
-    for (int k = 0; k < 6; ++k) x[9 + k] = P.net.host[k];
+    x[5] = (float)at_s * inv;
+    x[6] = (float)at_t * inv;
+    x[7] = (float)deleting * inv;
+    x[8] = count > 0 && mean_cap > 0.f ? fminf((float)cap_sum * inv / mean_cap, 4.f) / 4.f : 0.f;
+    for (int k = 0; k < 6; ++k) x[9 + k] = host[k];
     x[15] = 1.f;
+}
+
+// One thread: the features of the launch's batch.
+__device__ __noinline__ void batch_features()
+{
+    make_features(sh.x, P.bcount, P.net.m, P.g.n, (unsigned)sh.cnt[L_FEAT].x, (unsigned)sh.cnt[L_FEAT].y,
+                  (unsigned)sh.cnt[L_FEAT].z, (long long)cnt64(L_FCAP), P.net.mean_cap, P.net.host);
 }
 
 // y = w x + b by one CTA (relu: not below zero), a warp per output with its lanes
@@ -1380,7 +1388,6 @@ __device__ __noinline__ void phase_apply_change()
         P.g.pcap[xa] = P.g.pcap[xb] = va + vb2;
         P.cf[xa] = va;
         P.cf[xb] = vb2;
-        P.sc.pval[pp] = xa;
         P.sc.ins_need[a] = 0;
         P.sc.ins_need[b] = 0;
         applied += (ca >= 0 ? 1 : 0) + (cb >= 0 ? 1 : 0);
@@ -1432,7 +1439,6 @@ __device__ __noinline__ void phase_apply_cleanup(bool keep_need)
             P.sc.ins_need[b] = 0;
         }
         P.sc.pkey[pp] = kEmpty;
-        P.sc.pval[pp] = -1;
     }
 }
 
@@ -2160,47 +2166,18 @@ __device__ __forceinline__ int cycles_for(int d)
 // without using up a cycle (each such pass corrects at least one entry upward)
 constexpr int kStaleMax = 8;
 
-// The first scan of a row: the lowest residual height as scan_lowest does, and
-// the snapshot of every slot of the row in stg.
-template <int kU, bool PULL>
-__device__ __forceinline__ unsigned long long scan_and_stage(int r0, int d, int j0, int step,
-                                                             int *stg)
-{
-    unsigned long long best = kEmpty;
-    for (int jb = j0; jb < d; jb += step * kU) {
-        int c[kU], z[kU], hz[kU];
-#pragma unroll
-        for (int r = 0; r < kU; ++r) {
-            const int j = jb + r * step;
-            c[r] = j < d ? (PULL ? ldg_cg(P.g.pcap + r0 + j) - ldg_cg(P.cf + r0 + j) : ldg_cg(P.cf + r0 + j)) : 0;
-            z[r] = j < d ? ldg_cg(P.g.dst + r0 + j) : 0;
-        }
-#pragma unroll
-        for (int r = 0; r < kU; ++r) hz[r] = c[r] > 0 ? ldg_cg(P.h + z[r]) : kNoRes;
-#pragma unroll
-        for (int r = 0; r < kU; ++r) {
-            const int j = jb + r * step;
-            if (j < d) stg[j] = hz[r];
-            if (c[r] > 0) {
-                const unsigned long long key = ((unsigned long long)(unsigned)hz[r] << 32) | (unsigned)j;
-                best = key < best ? key : best;
-            }
-        }
-    }
-    return best;
-}
-
 __device__ __forceinline__ int comp4(const int4 &a, int e)
 {
     return e == 0 ? a.x : (e == 1 ? a.y : (e == 2 ? a.z : a.w));
 }
 
-// The first scan of a row with 16-byte loads: rows start on multiples of four
-// slots (MF_ROW_ALIGN), so slot group g (slots 4g .. 4g+3) is one int4 of
-// each slot array.  Thread t of nt takes groups t, t + nt, ... two at a time
-// (eight slots in flight).  Same result as scan_and_stage.
+// The first scan of a row: the lowest residual height as scan_lowest does, and the
+// snapshot of every slot of the row in stg.  With 16-byte loads: rows start on
+// multiples of four slots (MF_ROW_ALIGN), so slot group g (slots 4g .. 4g+3) is
+// one int4 of each slot array.  Thread t of nt takes groups t, t + nt, ... two at
+// a time (eight slots in flight).
 template <bool PULL>
-__device__ __forceinline__ unsigned long long scan_and_stage_v4(int r0, int d, int t, int nt,
+__device__ __forceinline__ unsigned long long scan_and_stage(int r0, int d, int t, int nt,
                                                                 int *stg)
 {
     unsigned long long best = kEmpty;
@@ -2446,7 +2423,7 @@ __device__ __noinline__ bool discharge_warp_rows(int u, int d, const DisCtx &dc,
             best = warp_min_u64(scan_lowest<8, PULL>(r0, d, lane, 32));
             gscan += d;
         } else if (!have) {
-            best = warp_min_u64(scan_and_stage_v4<PULL>(r0, d, lane, 32, stg));
+            best = warp_min_u64(scan_and_stage<PULL>(r0, d, lane, 32, stg));
             have = true;
             gscan += d;
             __syncwarp();
@@ -2456,7 +2433,7 @@ __device__ __noinline__ bool discharge_warp_rows(int u, int d, const DisCtx &dc,
             if (best == kEmpty || hu <= bh) {
                 // a relabel is decided on fresh values: refresh the snapshot first
                 __syncwarp();
-                best = warp_min_u64(scan_and_stage_v4<PULL>(r0, d, lane, 32, stg));
+                best = warp_min_u64(scan_and_stage<PULL>(r0, d, lane, 32, stg));
                 gscan += d;
                 __syncwarp();
             }
@@ -2654,7 +2631,7 @@ __device__ __noinline__ bool discharge_team_rows(int u, int d, const DisCtx &dc,
         unsigned long long best;
         bool global_scan = !st || !have;
         if (!st) best = scan_lowest<8, PULL>(r0, d, T.tid, T.n);
-        else if (!have) best = scan_and_stage_v4<PULL>(r0, d, T.tid, T.n, stg);
+        else if (!have) best = scan_and_stage<PULL>(r0, d, T.tid, T.n, stg);
         else best = scan_staged(stg, d, T.tid, T.n);
         have = true;
         best = warp_min_u64(best);
@@ -2665,7 +2642,7 @@ __device__ __noinline__ bool discharge_team_rows(int u, int d, const DisCtx &dc,
         if (!global_scan && (b == kEmpty || hu <= (int)(b >> 32))) {
             // a relabel is decided on fresh values: refresh the snapshot first
             T.sync();               // every warp has read sh.red
-            best = warp_min_u64(scan_and_stage_v4<PULL>(r0, d, T.tid, T.n, stg));
+            best = warp_min_u64(scan_and_stage<PULL>(r0, d, T.tid, T.n, stg));
             if (lane == 0) sh.red[wid] = best;
             T.sync();
             b = kEmpty;
@@ -4663,41 +4640,28 @@ int mf_rebuild_move(const MfParams &p, void *stream, const long long *noff, int3
 // ---- scheduler features of a batch (one CTA) ----
 __global__ void __launch_bounds__(256) k_features(MfFeatIn F, float *out)
 {
-    __shared__ float red[4][8];
-    float ts = 0.f, tt = 0.f, zero = 0.f, capsum = 0.f;
+    __shared__ long long red[4][8];
+    long long vals[4] = {0, 0, 0, 0};              // touching s, touching t, deleting, capacities
     for (long long i = threadIdx.x; i < F.count; i += blockDim.x) {
         const int u = F.bu[i], v = F.bv[i], c = F.bc[i];
-        ts += (u == F.s || v == F.s) ? 1.f : 0.f;
-        tt += (u == F.t || v == F.t) ? 1.f : 0.f;
-        zero += c == 0 ? 1.f : 0.f;
-        capsum += (float)c;
+        vals[0] += u == F.s || v == F.s;
+        vals[1] += u == F.t || v == F.t;
+        vals[2] += c == 0;
+        vals[3] += c;
     }
-    float vals[4] = {ts, tt, zero, capsum};
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        float x = vals[k];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        const long long x = warp_sum_ll(vals[k]);
         if (lane == 0) red[k][w] = x;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        float tot[4] = {0.f, 0.f, 0.f, 0.f};
+        long long tot[4] = {0, 0, 0, 0};
         for (int k = 0; k < 4; ++k)
             for (int q = 0; q < (int)(blockDim.x >> 5); ++q) tot[k] += red[k][q];
-        const float B = (float)F.count, m = (float)(F.m > 0 ? F.m : 1), n = (float)F.n;
-        const float inv = F.count > 0 ? 1.f / B : 0.f;
-        out[0] = log2f(1.f + B) / 20.f;
-        out[1] = fminf(B / m, 1.f);
-        out[2] = log2f(n) / 24.f;
-        out[3] = log2f(1.f + m) / 28.f;
-        out[4] = (m / n) / 16.f;
-        out[5] = tot[0] * inv;
-        out[6] = tot[1] * inv;
-        out[7] = tot[2] * inv;
-        out[8] = F.count > 0 && F.mean_cap > 0.f ? fminf(tot[3] * inv / F.mean_cap, 4.f) / 4.f : 0.f;
-        for (int k = 0; k < 6; ++k) out[9 + k] = F.host[k];
-        out[15] = 1.f;
+        make_features(out, F.count, F.m, F.n, (unsigned)tot[0], (unsigned)tot[1], (unsigned)tot[2], tot[3], F.mean_cap,
+                      F.host);
     }
 }
 
