@@ -314,8 +314,9 @@ __device__ __forceinline__ bool rounds_left(const MfDesc &d, const MfState &st, 
 // few vertices are left to the squad (squad_discharge).  On a small graph that
 // takes a BFS of many levels: short rounds pay where many rounds follow; where
 // two or three do, the whole KERNEL_CYCLES in each settle more.  Behind a round
-// of another kind it queues behind stamps (64 batched instances: 11.9 ms, and
-// 17.5 without short rounds there).
+// of another kind it queues behind stamps, unless the squad runs it, which drops
+// the entries without excess first (64 batched instances: 11.9 ms, and 17.5
+// without short rounds there).
 __device__ __forceinline__ void pick_round(MfDesc &d, int csize)
 {
     d.dis_stamp = mf_round_stamps(d.round, d.dis_short, d.dis_stamp);
@@ -3171,14 +3172,14 @@ __device__ __noinline__ bool squad_bfs()
 }
 
 // z received flow and became active, or stays active after its cycle: into the
-// next round, once (by the stamp or by the reasons at short_push).  In the squad: into this CTA's queue, or, when that is full or z's
-// row is long, onto the grid's lists; else into the CTA's queue of worklist
-// entries.
+// next round, once (by the stamp or for the reasons at short_push).  In the squad:
+// into this CTA's queue, or, when that is full or z's row is long, onto the grid's
+// lists; else into the CTA's queue of worklist entries.
 template <bool SQUAD>
 __device__ __forceinline__ void short_enqueue(int z, int r0, int d, const SquadQ &nq)
 {
-    if (sh.d.dis_stamp && atomicExch(P.sc.vmark + z, sh.d.qstamp) == sh.d.qstamp) return;
     if (!SQUAD) {
+        if (sh.d.dis_stamp && atomicExch(P.sc.vmark + z, sh.d.qstamp) == sh.d.qstamp) return;
         place_active(z, d, L_AUX, sh.d.wl_sel ^ 1, nullptr);
         return;
     }
@@ -3383,17 +3384,29 @@ __device__ __noinline__ bool squad_discharge()
     squad_enter();
     {
         const int sel = sh.d.wl_sel, n0 = sh.d.wl_n[0], all = n0 + sh.d.wl_n[1];
+        const bool stamped = sh.d.dis_stamp != 0;
+        if (tid == 0) sh.so_cnt = 0;
+        __syncthreads();
         cnt = all > rank ? (all - rank + csize - 1) / csize : 0;
         const SquadQ q = squad_q(0);
         for (int i = tid; i < cnt; i += nt) {
             const int k = i * csize + rank;
             const int v = __ldcg(k < n0 ? P.sc.wl[sel][0] + k : P.sc.wl[sel][1] + (k - n0));
-            squad_put(q, i, v, P.g.off[v], ldg_cg(P.g.deg + v));
+            const int r0 = P.g.off[v], d = ldg_cg(P.g.deg + v);
+            if (!stamped) squad_put(q, i, v, r0, d);
+            else if (ldg_cg(P.e + v) > 0) squad_put(q, atomicAdd(&sh.so_cnt, 1), v, r0, d);
         }
+        __syncthreads();
+        if (stamped) cnt = sh.so_cnt;
+        __syncthreads();
+        if (tid == 0) sh.so_cnt = sh.so_flag = sh.d.dis_stamp = 0;
+        __syncthreads();
+        if (!squad_entered()) return false;
+        // without the vertices that have no excess the list is as a short round
+        // wants it, and no stamps are needed; nobody pushes before every CTA of
+        // the squad has looked
+        if (stamped) squad_sync();
     }
-    if (tid == 0) sh.so_cnt = sh.so_flag = 0;
-    __syncthreads();
-    if (!squad_entered()) return false;
     for (;;) {
         const int par = sh.so_par;
         const SquadQ cq = squad_q(cur), nq = squad_q(cur ^ 1);
@@ -3443,7 +3456,6 @@ __device__ __noinline__ bool squad_discharge()
             sh.so_go = over ? 0 : (flag != 0 || c > MF_SQUAD_ACTIVE * csize ? 2 : 1);
             if (sh.so_go == 1) {
                 ++sh.d.round;
-                ++sh.d.qstamp;
                 ++sh.hs.rounds_total;
             }
             sh.so_par = par ^ 1;
